@@ -14,17 +14,6 @@ namespace hikonv {
 constexpr int kThreadsTc = 256;
 constexpr int kWarpsTc = kThreadsTc / 32;
 
-// Byte `b` (0..3) of w as a 32-bit value, sign- or zero-extended: one prmt.
-template <bool SIGNED>
-__device__ __forceinline__ uint32_t extract_code(uint32_t w, int b) {
-    uint32_t r;
-    // selector nibbles: low nibble picks byte b; in the upper three, bit 3 replicates that byte's sign,
-    // or index 4 picks byte 0 of the zero second operand
-    const uint32_t sel = SIGNED ? (uint32_t)(b | ((8 | b) << 4) | ((8 | b) << 8) | ((8 | b) << 12)) : (uint32_t)(b | 0x4440);
-    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(w), "r"(0u), "r"(sel));
-    return r;
-}
-
 // Loads the words covering elements [e0 - 4 HW, e0 + 4 NWD - 4 HW) of f; e0 is a multiple of 4.
 template <int NWORDS, int HW>
 __device__ __forceinline__ void load_words(const int8_t *f, long long len, long long e0, bool fast, uint32_t (&w)[NWORDS]) {

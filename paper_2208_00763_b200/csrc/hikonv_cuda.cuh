@@ -97,6 +97,17 @@ __device__ __forceinline__ int32_t load_code(const int8_t *p) {
     return code_value<SIGNED>(__ldg(p));
 }
 
+// Byte `b` (0..3) of w as a 32-bit value, sign- or zero-extended: one prmt.
+template <bool SIGNED>
+__device__ __forceinline__ uint32_t extract_code(uint32_t w, int b) {
+    uint32_t r;
+    // selector nibbles: low nibble picks byte b; in the upper three, bit 3 replicates that byte's sign,
+    // or index 4 picks byte 0 of the zero second operand
+    const uint32_t sel = SIGNED ? (uint32_t)(b | ((8 | b) << 4) | ((8 | b) << 8) | ((8 | b) << 12)) : (uint32_t)(b | 0x4440);
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(w), "r"(0u), "r"(sel));
+    return r;
+}
+
 // Asynchronous global -> shared copies (cp.async); src_bytes < 4 zero-fills the rest of the 4-byte word.
 __device__ __forceinline__ void cp_async_4(void *smem_dst, const void *gmem_src, int src_bytes) {
     const unsigned dst = (unsigned)__cvta_generic_to_shared(smem_dst);

@@ -28,6 +28,25 @@ def test_pack_matches_eq5():
                 assert np.array_equal(got, direct.pack_words(v, S, N, wb)), (bits, S, N, wb, n, signed)
 
 
+@pytest.mark.parametrize("word_bits", [32, 64])
+def test_pack_every_block_size(word_bits):
+    # the four-words-per-thread kernel for every N it is built for and the first one past it: counts around a group of four
+    # words and around a CTA's 1024 words, both signs, and inputs that start off the alignment the kernel wants
+    rng = np.random.default_rng(3)
+    for N in range(1, 14):
+        bits = min(8, word_bits // N)
+        S = max(bits, (word_bits - bits) // (N - 1)) if N > 1 else bits
+        for signed in (False, True):
+            for n in (1, 4 * N - 1, 4 * N, 4 * N + 1, 1024 * N - 1, 1024 * N + 4 * N + 1):
+                v = inputs.uniform_codes(rng, (n,), bits, signed)
+                for off in (0, 1, 4, 8):
+                    buf = torch.zeros(n + 16, dtype=torch.int8, device="cuda")
+                    buf[off:off + n] = dev(v)
+                    got = hk.pack(buf[off:off + n], bits, signed, S, N, word_bits).cpu().numpy()
+                    got = got.view(np.uint32).astype(np.uint64) if word_bits == 32 else got.view(np.uint64)
+                    assert np.array_equal(got, direct.pack_words(v, S, N, word_bits)), (N, signed, n, off)
+
+
 def test_pack_reproduces_the_printed_multiplicands():
     vals = {}
     with open(os.path.join(GOLDEN, "worked_example_f32.txt")) as fh:
