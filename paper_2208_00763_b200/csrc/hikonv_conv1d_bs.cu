@@ -124,6 +124,8 @@ __global__ void __launch_bounds__(kThreadsTc, MINB) conv1d_bs_kernel(const Conv1
     constexpr int NW = HW + L / 4;
     const int S = MODE == 1 ? 8 : MODE == 2 ? 16 : p.S;
     __shared__ __align__(16) int32_t s_stage[kWarpsTc][32 * stage_pitch(L)];
+    grid_dependency_release();
+    grid_dependency_wait();
 
     // kernel words B_j (Eq. 5 on g), built by every lane from warp-uniform loads
     uint32_t Bw[J];

@@ -150,6 +150,9 @@ inline unsigned fast_tiles_after_first(long long len, int run, bool aligned) {
     return (aligned && whole > 1) ? (unsigned)(whole - 1) : 0u;
 }
 
+// The kernels are launched with a programmatic dependency (they release their successor and wait for their predecessor
+// first thing): the CTAs of the next call move in as this call's leave, so that neither the launch latency nor the
+// drained last tiles of a call stand between two calls of a stream.
 // Persistent launch: as many CTAs as fit on the device at once (occupancy query, cached per kernel),
 // fewer when the problem is small; each warp then walks tiles with a grid-wide stride.
 // CTAs of `kernel` that fit one SM, asked once per kernel (all instantiations share one function-pointer
@@ -174,7 +177,7 @@ inline int launch_persistent(Kernel kernel, const Params &p, cudaStream_t st) {
     const long long want = (p.n_tiles + kWarpsTc - 1) / kWarpsTc;
     const long long cap = (long long)sms * resident;
     const unsigned grid = (unsigned)(want < cap ? want : cap);
-    return launch_plain(kernel, dim3(grid), dim3(kThreadsTc), 0, st, p);
+    return launch_dependent(kernel, dim3(grid), dim3(kThreadsTc), 0, st, p);
 }
 
 }  // namespace hikonv

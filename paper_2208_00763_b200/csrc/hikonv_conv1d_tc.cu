@@ -79,6 +79,8 @@ __global__ void __launch_bounds__(kThreadsTc, ((N >= 9 && P == 0) ? 3 : 4)) conv
     constexpr int NWORDS = P == 0 ? HW + L / 4 : (NE * (P == 0 ? 8 : P) + 31) / 32;
     constexpr int FRONT = P == 0 ? 4 * HW : J * N;   // codes held in front of the run
     __shared__ __align__(16) int32_t s_stage[kWarpsTc][32 * stage_pitch(L)];
+    grid_dependency_release();
+    grid_dependency_wait();
 
     const int S = SC > 0 ? SC : p.S;
     const uint32_t mask = SC > 0 ? ((1u << (SC > 0 ? SC : 1)) - 1u) : p.mask;
@@ -187,6 +189,8 @@ __global__ void __launch_bounds__(kThreadsTc, MINB) conv1d_unpacked_tc_kernel(co
     constexpr int HW = (K - 1 + 3) / 4;
     constexpr int NWORDS = HW + L / 4;
     __shared__ __align__(16) int32_t s_stage[kWarpsTc][32 * stage_pitch(L)];
+    grid_dependency_release();
+    grid_dependency_wait();
     int32_t gk[K];
 #pragma unroll
     for (int k = 0; k < K; ++k) {
@@ -230,6 +234,8 @@ __global__ void __launch_bounds__(kThreadsTc, MINB) conv1d_dp4a_tc_kernel(const 
     constexpr int HW = KW;                       // 4 KW codes in front of the run cover the K - 1 <= 4 KW - 1 it needs
     constexpr int NWORDS = HW + L / 4;
     __shared__ __align__(16) int32_t s_stage[kWarpsTc][32 * stage_pitch(L)];
+    grid_dependency_release();
+    grid_dependency_wait();
     uint32_t gw[KW];
 #pragma unroll
     for (int t = 0; t < KW; ++t) {
