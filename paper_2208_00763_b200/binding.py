@@ -113,14 +113,21 @@ def _tune(tune: Optional[dict]):
     return ctypes.byref(t)
 
 
+# The current stream as a plain address, without building a torch.cuda.Stream around it (0.1 against 3.1 us; a short 1-D
+# call takes 9 us in all): only called with CUDA tensors at hand, so CUDA is initialised.
+_raw_stream, _current_device = (getattr(torch._C, n, None) for n in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
+
+
 def _stream(stream) -> int:
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return int(stream.cuda_stream)
+    return _raw_stream(_current_device()) if stream is None else int(stream.cuda_stream)
+
+
+_CODE_DTYPES = (torch.int8, torch.uint8)
+_INT32 = (torch.int32,)
 
 
 def _dev_i8(t: torch.Tensor, name: str) -> int:
-    if not t.is_cuda or t.dtype not in (torch.int8, torch.uint8) or not t.is_contiguous():
+    if not t.is_cuda or t.dtype not in _CODE_DTYPES or not t.is_contiguous():
         raise ValueError("%s must be a contiguous CUDA int8/uint8 tensor" % name)
     return t.data_ptr()
 
@@ -139,9 +146,6 @@ def _dev_out(t: torch.Tensor, name: str, numel: int, dtypes, like: torch.Tensor)
     if t.numel() != numel:
         raise ValueError("%s holds %d elements, the call writes %d" % (name, t.numel(), numel))
     return t.data_ptr()
-
-
-_CODE_DTYPES = (torch.int8, torch.uint8)
 
 
 # ------------------------------------------------------------------ host-only planning
@@ -214,7 +218,7 @@ def conv1d(d_f: torch.Tensor, d_g: torch.Tensor, p: int, q: int, f_signed: bool,
     if out is None:
         out = torch.empty(n + K - 1, dtype=torch.int32, device=d_f.device)
     _check(lib().hikonv_conv1d(_dev_i8(d_f, "d_f"), n, _dev_i8(d_g, "d_g"), K, p, q, int(f_signed), int(g_signed),
-                               _dev_out(out, "out", n + K - 1, (torch.int32,), d_f), algo, _tune(tune), _stream(stream)),
+                               _dev_out(out, "out", n + K - 1, _INT32, d_f), algo, _tune(tune), _stream(stream)),
            "hikonv_conv1d")
     return out
 
@@ -230,7 +234,7 @@ def conv1d_dense(d_f_dense: torch.Tensor, n: int, d_g: torch.Tensor, p: int, q: 
     if out is None:
         out = torch.empty(n + K - 1, dtype=torch.int32, device=d_f_dense.device)
     _check(lib().hikonv_conv1d_dense(d_f_dense.data_ptr(), n, _dev_i8(d_g, "d_g"), K, p, q, int(f_signed), int(g_signed),
-                                     _dev_out(out, "out", n + K - 1, (torch.int32,), d_f_dense), _tune(tune), _stream(stream)),
+                                     _dev_out(out, "out", n + K - 1, _INT32, d_f_dense), _tune(tune), _stream(stream)),
            "hikonv_conv1d_dense")
     return out
 
@@ -266,7 +270,7 @@ def conv2d(d_x: torch.Tensor, d_w: torch.Tensor, pad: int, p: int, q: int, x_sig
     if out is None:
         out = torch.empty((B, Co, max(Ho, 0), max(Wo, 0)), dtype=torch.int8 if requant else torch.int32, device=d_x.device)
     shift, lo, hi = requant if requant else (0, 0, 0)
-    out_ptr = _dev_out(out, "out", B * Co * max(Ho, 0) * max(Wo, 0), _CODE_DTYPES if requant else (torch.int32,), d_x)
+    out_ptr = _dev_out(out, "out", B * Co * max(Ho, 0) * max(Wo, 0), _CODE_DTYPES if requant else _INT32, d_x)
     if not workspace.is_cuda or workspace.device != d_x.device or not workspace.is_contiguous():
         raise ValueError("workspace must be a contiguous CUDA tensor on the inputs' device")
     _check(lib().hikonv_conv2d(_dev_i8(d_x, "d_x"), B, Ci, H, W, _dev_i8(d_w, "d_w"), Co, K, stride, pad, p, q,
@@ -310,7 +314,7 @@ def conv2d_dense(d_x: torch.Tensor, x_shape, x_store_bits: int, d_w: torch.Tenso
     if not requant:
         if out is None:
             out = torch.empty((B, Co, max(Ho, 0), max(Wo, 0)), dtype=torch.int32, device=d_x.device)
-        out_ptr, store = _dev_out(out, "out", B * Co * max(Ho, 0) * max(Wo, 0), (torch.int32,), d_x), 32
+        out_ptr, store = _dev_out(out, "out", B * Co * max(Ho, 0) * max(Wo, 0), _INT32, d_x), 32
     else:
         nbytes = (count * out_store_bits + 7) // 8
         if out is None:
@@ -350,7 +354,7 @@ def conv2d_static_scratch(d_x: torch.Tensor, d_w: torch.Tensor, pad: int, p: int
         raise ValueError("weight shape does not match the input")
     shift, lo, hi = requant if requant else (0, 0, 0)
     Ho, Wo = H + 2 * pad - K + 1, W + 2 * pad - K + 1
-    out_ptr = _dev_out(out, "out", B * Co * max(Ho, 0) * max(Wo, 0), _CODE_DTYPES if requant else (torch.int32,), d_x)
+    out_ptr = _dev_out(out, "out", B * Co * max(Ho, 0) * max(Wo, 0), _CODE_DTYPES if requant else _INT32, d_x)
     if d_w.device != d_x.device:
         raise ValueError("d_w is on %s, d_x on %s" % (d_w.device, d_x.device))
     with torch.cuda.device(d_x.device):      # the built-in buffer that is used is the current device's
