@@ -625,10 +625,10 @@ __global__ void __launch_bounds__(kMaxThreads2D, 2) conv2d_kernel(const Conv2dPa
 struct WeightPackParams {
     const int8_t *w;
     uint32_t *wp;
-    int Co, Ci, K, J, Kc, S, w_signed, CoP, total;
+    int Co, Ci, K, J, Kc, S, w_signed, CoP;
     int w_bits;                // storage: 8 = one code per byte, 1 / 2 / 4 = dense (8 / w_bits codes per byte)
-    int w_blocks;              // CTAs that pack kernel rows; the CTAs after them sum the weights of a channel (x_off != 0)
-    Div32 d_cop, d_j, d_k;     // divisions of pack_weight_word
+    int w_blocks;              // CTAs that pack kernel rows, one word per thread; the CTAs before them sum the weights of a channel (x_off != 0)
+    Div32 d_cg, d_j;           // divisions by the number of groups of eight channels and by J
     int x_off;                 // offset taken from every activation code (0: none)
     int32_t *corr;             // corr[co] = x_off * sum of the weights of channel co, CoP entries
 };
@@ -644,21 +644,20 @@ __device__ __forceinline__ int32_t load_dense_code(const int8_t *base, size_t e,
     return is_signed ? (int32_t)((v ^ sb) - sb) : (int32_t)v;
 }
 
-__device__ __forceinline__ void pack_weight_word(const WeightPackParams &q, int idx) {
-    if (idx >= q.total) return;
-    uint32_t rest = div32((uint32_t)idx, q.d_cop);
-    const int co = idx - (int)rest * q.CoP;
-    uint32_t up = div32(rest, q.d_j);
-    const int j = (int)(rest - up * q.J);
-    rest = up;
-    up = div32(rest, q.d_k);
-    const int kh = (int)(rest - up * q.K);
-    const int ci = (int)up;
+// A warp packs four neighbouring (row, chunk) words of eight channels: a channel's rows are contiguous in memory and the
+// words are contiguous over channels, so a load touches eight sectors and a store four.  (With 32 channels per warp every
+// lane's loads touched a sector of its own; with the sums below taken one load at a time, the packing launch of the
+// 256 -> 256 channel layer on 64 14x14 maps took 15.2 us, now 9.8.)
+__device__ __forceinline__ void pack_weight_words(const WeightPackParams &q, int warp, int lane) {
+    const int rg = (int)div32((uint32_t)warp, q.d_cg), cg = warp - rg * ((q.CoP + 7) / 8);
+    const int rj = rg * 4 + (lane >> 3), co = cg * 8 + (lane & 7);
+    if (rj >= q.Ci * q.K * q.J || co >= q.CoP) return;
+    const int row = (int)div32((uint32_t)rj, q.d_j), j = rj - row * q.J;
     uint32_t word = 0;
     if (co < q.Co) {
-        const size_t row_e = (((size_t)co * q.Ci + ci) * q.K + kh) * q.K;       // first code of the kernel row
+        const size_t row_e = ((size_t)co * q.Ci * q.K + row) * q.K;              // first code of the kernel row
         for (int k = 0; k < q.Kc; ++k) {
-            const int g_idx = j * q.Kc + k;              // index into the reversed row
+            const int g_idx = j * q.Kc + k;                                      // index into the reversed row
             if (g_idx < q.K) {
                 int32_t v;
                 if (q.w_bits == 8) {
@@ -671,23 +670,26 @@ __device__ __forceinline__ void pack_weight_word(const WeightPackParams &q, int 
             }
         }
     }
-    q.wp[idx] = word;
+    q.wp[(size_t)rj * q.CoP + co] = word;
 }
 
-// corr[co] = x_off * sum_{ci, kh, kw} W[co][ci][kh][kw]: one warp per output channel (its Ci K K codes are contiguous).
+// corr[co] = x_off * sum_{ci, kh, kw} W[co][ci][kh][kw]: one warp per output channel (its Ci K K codes are contiguous),
+// eight loads of a lane in flight at a time.
 __device__ __forceinline__ void sum_channel_weights(const WeightPackParams &q, int co, int lane) {
     if (co >= q.CoP) return;
     int32_t sum = 0;
     if (co < q.Co) {
         const int per_co = q.Ci * q.K * q.K;
         const size_t e0 = (size_t)co * per_co;
-        for (int e = lane; e < per_co; e += 32) {
-            if (q.w_bits == 8) {
+        if (q.w_bits == 8) {
+#pragma unroll 8
+            for (int e = lane; e < per_co; e += 32) {
                 const int8_t raw = __ldg(q.w + e0 + e);
                 sum += q.w_signed ? (int32_t)raw : (int32_t)(uint8_t)raw;
-            } else {
-                sum += load_dense_code(q.w, e0 + e, q.w_bits, q.w_signed != 0);
             }
+        } else {
+#pragma unroll 8
+            for (int e = lane; e < per_co; e += 32) sum += load_dense_code(q.w, e0 + e, q.w_bits, q.w_signed != 0);
         }
 #pragma unroll
         for (int d = 16; d > 0; d >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, d);
@@ -695,22 +697,32 @@ __device__ __forceinline__ void sum_channel_weights(const WeightPackParams &q, i
     if (lane == 0) q.corr[co] = sum * q.x_off;
 }
 
-// Packed activation rows (Eq. 5): ap[(ci * B*Hp + b*Hp + hp) * XBT + xb] packs the N input pixels of block
-// x = xb - J of padded row hp, i.e. columns (xb - J) N + K - 1 - pad + n of input row hp - pad, zero where the
-// row or a column lies in the padding.  For the comparator S == 0 and N == 1: one int32 code per word.
+// Packed activation rows (Eq. 5): ap[(ci * B*Hp + b*Hp + hp) * XBT + xb] packs the N input pixels of padded row hp that
+// start at column col_first + xb N (input row hp - pad), zero where the row or a column lies outside the image.  For the
+// comparator S == 0 and N == 1: one int32 code per word.
 // One thread packs four consecutive words of a row (one 16-byte store); threads are numbered through all
 // (ci, b) planes, so that small maps still fill their CTAs.  The first CTAs of the launch sum the channels' weights
-// (when the layer runs on shifted codes) and pack the kernel rows (one word per thread), so that a layer needs one
+// (when the layer runs on shifted codes) and pack the kernel rows, so that a layer needs one
 // packing launch and its longest serial work starts first.
-// x_bits: storage of the activations, 8 = one code per byte, 1 / 2 / 4 = dense.
+// The 4 N codes of a thread start at any byte: it loads the N + 1 aligned words around them, shifts them into place, blanks
+// the bytes outside the row with one mask per word and packs by byte permute and Horner's rule (as hikonv_pack does).
+// x_bits: storage of the activations, 8 = one code per byte, 1 / 2 / 4 = dense (code by code).
 // With wq.x_off != 0 every slot holds code - x_off, the slots outside the image included (code 0 there).
 struct ActPackDivs {
     Div32 per_plane, b, xq;    // pieces per (ci, b) plane, images, 16-byte pieces per packed row
 };
 
+// Byte mask of the bytes of word i (bytes 4 i .. 4 i + 3) whose index lies in [first, last).
+__device__ __forceinline__ uint32_t byte_range_mask(int i, int first, int last) {
+    const int lo = max(first - 4 * i, 0), n = max(last - 4 * i - lo, 0);
+    uint32_t m;
+    asm("bmsk.clamp.b32 %0, %1, %2;" : "=r"(m) : "r"(8 * lo), "r"(8 * n));      // 8 n bits from bit 8 lo on, clamped to the word
+    return m;
+}
+
 template <bool XS, int N>
 __global__ void __launch_bounds__(256) pack_operands_kernel(const int8_t *__restrict__ x, int B, int Ci, int H, int W, int Hp,
-                                                            int pad, int K, int J, int S, int XBT,
+                                                            int pad, int col_first, int S, int XBT,
                                                             uint32_t *__restrict__ ap, int weight_blocks, const WeightPackParams wq,
                                                             int x_bits, const ActPackDivs dv, unsigned act_items) {
     grid_dependency_release();
@@ -719,7 +731,7 @@ __global__ void __launch_bounds__(256) pack_operands_kernel(const int8_t *__rest
     if ((int)blockIdx.x < weight_blocks) {
         const int cb = weight_blocks - wq.w_blocks;                  // CTAs that sum weights (0 unless x_off != 0)
         if ((int)blockIdx.x < cb) sum_channel_weights(wq, (int)blockIdx.x * 8 + ((int)threadIdx.x >> 5), (int)threadIdx.x & 31);
-        else pack_weight_word(wq, ((int)blockIdx.x - cb) * 256 + (int)threadIdx.x);
+        else pack_weight_words(wq, ((int)blockIdx.x - cb) * 8 + ((int)threadIdx.x >> 5), (int)threadIdx.x & 31);
         return;
     }
     // the (plane, piece) pairs are numbered through: a CTA may span several small planes (ci * B + b)
@@ -738,18 +750,31 @@ __global__ void __launch_bounds__(256) pack_operands_kernel(const int8_t *__rest
         for (int n = 0; n < N; ++n) fill += (uint32_t)(-wq.x_off) << (S * n);
     }
     uint32_t word[4] = {fill, fill, fill, fill};
-    if (hi >= 0 && hi < H) {
+    const int col0 = col_first + 4 * q * N;                          // input column of slot 0 of the first word
+    if (hi >= 0 && hi < H && col0 + 4 * N > 0 && col0 < W) {
         const size_t row_e = (((size_t)b * Ci + ci) * H + hi) * W;  // first code of the input row
-        const int col0 = (4 * q - J) * N + K - 1 - pad;              // input column of slot 0 of the first word
         if (x_bits == 8) {
-            const int8_t *row = x + row_e;
+            const int8_t *src = x + row_e + col0;                    // not dereferenced outside the row
+            const int off = (int)((uintptr_t)src & 3);
+            const uint32_t *al = reinterpret_cast<const uint32_t *>(src - off);
+            // aligned word i holds the codes of columns col0 - off + 4 i .. + 3: loaded when one of them is in the row
+            uint32_t v[N + 1];
 #pragma unroll
-            for (int w = 0; w < 4; ++w)
+            for (int i = 0; i <= N; ++i) {
+                const int c = col0 - off + 4 * i;
+                v[i] = (c + 3 >= 0 && c < W) ? __ldg(al + i) : 0u;
+            }
 #pragma unroll
-                for (int n = 0; n < N; ++n) {
-                    const int col = col0 + w * N + n;
-                    if (col >= 0 && col < W) word[w] += (uint32_t)load_code<XS>(row + col) << (S * n);
-                }
+            for (int i = 0; i < N; ++i)
+                v[i] = __funnelshift_r(v[i], v[i + 1], 8 * off) & byte_range_mask(i, -col0, W - col0);
+            const uint32_t step = 1u << S;
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+                uint32_t a = extract_code<XS>(v[(w * N + N - 1) / 4], (w * N + N - 1) % 4);
+#pragma unroll
+                for (int n = N - 2; n >= 0; --n) a = a * step + extract_code<XS>(v[(w * N + n) / 4], (w * N + n) % 4);
+                word[w] += a;
+            }
         } else {
 #pragma unroll
             for (int w = 0; w < 4; ++w)
@@ -821,6 +846,8 @@ struct Conv2dSetup {
     bool unpacked;
     int tm;               // positions per thread of the packed kernel
 };
+
+constexpr int kSmemPerSm = 228 * 1024;   // shared memory of an SM; every resident CTA takes 1 KB more than it asks for
 
 static int sm_count() {
     int dev = 0, sms = 148;
@@ -1156,6 +1183,12 @@ static int make_setup(int B, int Ci, int H, int W, int Co, int K, int stride, in
     const int gy = ceil_div(Co, kp.TCO);
     if (gx > 0x7FFFFFFFLL || gy > 65535) return HIKONV_ERR_UNSUPPORTED;
     s->grid = dim3((unsigned)gx, (unsigned)gy, 1);
+    // A grid of less than one wave must spread over the SMs evenly.  The kernel is launched while the packing launch still
+    // runs (programmatic dependency), and its CTAs then pile up on the SMs that are free first: 111 CTAs took 32 us one to
+    // an SM and 55 to 60 us when two found room on one.  Such a grid asks for as much shared memory as lets only the
+    // even share of CTAs onto an SM.
+    const long long ctas = gx * gy, share = (ctas + sm_count() - 1) / sm_count();
+    if (share <= 4) s->smem_bytes = std::max(s->smem_bytes, (size_t)(kSmemPerSm / (share + 1) - 1024 + 256));
     return HIKONV_OK;
 }
 
@@ -1244,11 +1277,13 @@ static int conv2d_run(const void *d_x, int x_bits, int B, int Ci, int H, int W, 
     {
         WeightPackParams wq;
         wq.w = (const int8_t *)d_w; wq.wp = d_wp; wq.Co = Co; wq.Ci = Ci; wq.K = K; wq.J = s.L.J; wq.Kc = s.L.Kc; wq.S = s.L.S;
-        wq.w_signed = w_signed ? 1 : 0; wq.CoP = s.kp.CoP; wq.total = Ci * K * s.L.J * s.kp.CoP; wq.w_bits = w_bits;
+        wq.w_signed = w_signed ? 1 : 0; wq.CoP = s.kp.CoP; wq.w_bits = w_bits;
         wq.x_off = s.kp.x_off; wq.corr = d_corr;
-        wq.d_cop = make_div32((uint32_t)s.kp.CoP); wq.d_j = make_div32((uint32_t)s.L.J); wq.d_k = make_div32((uint32_t)K);
+        const size_t w_warps = (size_t)ceil_div(Ci * K * s.L.J, 4) * ceil_div(s.kp.CoP, 8);
+        wq.d_cg = make_div32((uint32_t)ceil_div(s.kp.CoP, 8));
+        wq.d_j = make_div32((uint32_t)s.L.J);
         const size_t act_items = (size_t)Ci * B * s.kp.Hp * (s.kp.XBT / 4);              // below 2^29: ap_words is below 2^31
-        const size_t act_blocks = (act_items + 255) / 256, w_blocks = (size_t)ceil_div(wq.total, 256);
+        const size_t act_blocks = (act_items + 255) / 256, w_blocks = (w_warps + 7) / 8;
         const size_t corr_blocks = s.kp.x_off ? (size_t)ceil_div(s.kp.CoP, 8) : 0;      // one warp per channel
         wq.w_blocks = (int)w_blocks;
         if (act_blocks + w_blocks + corr_blocks > 0x7FFFFFFFull) return HIKONV_ERR_UNSUPPORTED;
@@ -1259,7 +1294,7 @@ static int conv2d_run(const void *d_x, int x_bits, int B, int Ci, int H, int W, 
         dv.xq = make_div32((uint32_t)(s.kp.XBT / 4));
 #define HK_PACK(XSIGN, NN)                                                                                                 \
     rc = launch_dependent(pack_operands_kernel<XSIGN, NN>, dim3(grid), dim3(256), 0, st, (const int8_t *)d_x, B, Ci, H, W, s.kp.Hp, \
-                          pad, K, s.L.J, s.L.S, s.kp.XBT, d_ap, (int)(w_blocks + corr_blocks), wq, x_bits, dv, (unsigned)act_items)
+                          pad, K - 1 - pad - s.L.J * s.L.N, s.L.S, s.kp.XBT, d_ap, (int)(w_blocks + corr_blocks), wq, x_bits, dv, (unsigned)act_items)
         switch (s.L.N * 2 + (x_signed ? 1 : 0)) {
             case 2: HK_PACK(false, 1); break;
             case 3: HK_PACK(true, 1); break;
