@@ -1,0 +1,449 @@
+// The packed layer kernel.  A layer is computed as row-wise packed 1-D convolutions (Theorem 3) whose products are summed
+// over input channels and kernel rows in 64-bit packed accumulators before the split (Eq. 23).
+//
+// Work decomposition.  Group x of an output row is N neighbouring columns; its packed input word A_x (Eq. 5) gives
+//     Q_x = bias + sum_{ci, kh, j} A[ci][row + kh][x - j] * Bw[ci][kh][j]
+// whose slots m < N belong to group x and slots m >= N to group x + 1 (Theorem 2).  A thread owns a STRIP of TM
+// neighbouring output rows at one group and TN output channels: the TM + K - 1 activation words of a channel serve all K
+// kernel rows (a 4 x 4 tile loads 6 words and three 16-byte weight pieces for 48 multiplies; with four positions of one row
+// per thread it loaded 12), and all index arithmetic is done for one position instead of TM.  Lanes run along the row, so the
+// group in front of a lane's is in the lane before it, whatever the row of the strip.
+//
+// A CTA computes TS consecutive strips (of one or several images) of one row segment times TCO channels.  Packed activation
+// rows and kernel rows are streamed in stages of CK input channels with asynchronous copies into double-buffered shared memory.  The distance between two channels of a stage is a constant (kPlaneWords), so that the unrolled channel
+// loop needs no address arithmetic whatever the width of the rows.
+//
+// Split.  Every slot starts at a bias that makes its running sum non-negative, so slots never borrow from each other (this
+// replaces the sign-borrow increment of Eq. 29).  After CF input channels a slot could overflow; the bits of every slot above
+// its low h then move to a SECOND packed accumulator with the same layout,
+//     E += (Q >> h) & mask_high;      Q = (Q & mask_low) | bias,
+// which takes 2^h such moves.  At the end the words above the N low slots travel to the next lane still packed and are added
+// there (packed_add; where the slots do not have the room for that, as separate fields), the N slots are read by shift and
+// mask, value m = 2^h E_m + Q_m - (moves + 1) (bias_m + bias_{m + N}).
+//
+// What bounds it: instruction issue.  A warp-wide 32x32->64 multiply-add holds its scheduler for 4.1 cycles, every other
+// arithmetic instruction adds about one more.  Measured against the kernel before it (four positions of one row per thread,
+// second accumulators in shared memory, one halo word per row, run-time loops for 5x5), packing launch included:
+// 32x64x56x56 -> 64 s4 93.3 -> 87.9 us, 64x256x14x14 -> 256 u4 x s4 211 -> 166 us (205 with the new packing launch alone),
+// 8x48x37x53 -> 40 s8 32.4 -> 27.3 us, 16x24x45x61 -> 40 5x5 2-bit 70.6 -> 30.3 us, the compact CNN (batch 64) 605 -> 499 us.
+#pragma once
+
+#include <type_traits>
+
+#include "hikonv_cuda.cuh"
+#include "hikonv_conv2d_strip.h"
+#include "hikonv_conv2d_util.cuh"
+
+namespace hikonv {
+
+template <bool SP>
+__device__ __forceinline__ void packed_mac(uint64_t &acc, uint32_t a, uint32_t b) {
+    if constexpr (SP) acc += (uint64_t)((int64_t)(int32_t)a * (int64_t)(int32_t)b);
+    else acc += (uint64_t)a * (uint64_t)b;
+}
+
+template <int N, int KT, int JT>
+constexpr bool kStripPackedAdd = strip_packed_add(N, KT, JT);
+
+// N: pixels per word; KT, JT: kernel size and words per kernel row (0: run-time bounds); TM x TN: rows x channels per thread;
+// SP: signed product; HASE: with second accumulators.
+template <int N, int KT, int JT, int TM, int TN, bool SP, bool HASE>
+__global__ void __launch_bounds__(kStripThreads, 2) conv2d_strip_kernel(const __grid_constant__ StripParams p) {
+    constexpr bool PACKED_ADD = kStripPackedAdd<N, KT, JT>;
+    constexpr bool UP = N > 1 && KT != 1;                       // some products have slots above the N low ones
+    constexpr int ROWS = KT > 0 ? TM + KT - 1 : TM;            // activation rows a thread points at
+    extern __shared__ __align__(16) uint32_t smem[];
+    grid_dependency_release();
+
+    const int tid = threadIdx.x, nthreads = blockDim.x, lane = tid & 31, warp = tid >> 5;
+    const int tnx_log2 = 31 - __clz(p.TNX);                    // TNX is a power of two
+    const int tn = tid & (p.TNX - 1);
+    const int strip_tile = p.NSEG > 1 ? (int)(blockIdx.x / (unsigned)p.NSEG) : (int)blockIdx.x;
+    const int seg = (int)blockIdx.x - strip_tile * p.NSEG;
+    const int g0 = strip_tile * p.TS;                          // first strip
+    const int b0 = g0 / p.SH, s0 = g0 - b0 * p.SH;
+    const int TSe = min(p.TS, p.strips - g0);
+    const int co0 = blockIdx.y * p.TCO;
+    const int K = KT > 0 ? KT : p.K, J = JT > 0 ? JT : p.J;
+
+    // staged rows: from the first row of the first strip to the last row of the last one (rows past the last image do not exist)
+    const int r0 = b0 * p.Hp + s0 * TM;
+    const int tl = s0 + TSe - 1, dbl = fast_div(tl, p.mg_sh);
+    const int NR = min(dbl * p.Hp + (tl - dbl * p.SH) * TM - s0 * TM + TM + K - 1, p.ap_rows - r0);
+
+    // this thread's strip and group (an idle thread works on position 0; its results are dropped)
+    const int pos = tid >> tnx_log2, pos_ok = pos < TSe * p.XB, pc = pos_ok ? pos : 0;
+    const int sl = fast_div(pc, p.mg_xb), xb = pc - sl * p.XB;
+    const int db = fast_div(s0 + sl, p.mg_sh), s_img = s0 + sl - db * p.SH;
+    const uint32_t *a0 = smem + (db * p.Hp + (s_img - s0) * TM) * p.pitch + xb + J - 1;
+
+    uint64_t acc[TM][TN];
+    uint32_t e_lo[HASE ? TM : 1][TN], e_hi[HASE ? TM : 1][TN];
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int t = 0; t < TN; ++t) {
+            acc[i][t] = p.bias;
+            if constexpr (HASE) e_lo[i][t] = e_hi[i][t] = 0u;
+        }
+    auto move_upper_bits = [&]() {
+        if constexpr (HASE) {
+            const uint32_t mh_lo = (uint32_t)p.mask_high, mh_hi = (uint32_t)(p.mask_high >> 32);
+            const uint32_t ml_lo = (uint32_t)p.mask_low, ml_hi = (uint32_t)(p.mask_low >> 32);
+            const uint32_t b_lo = (uint32_t)p.bias, b_hi = (uint32_t)(p.bias >> 32);
+#pragma unroll
+            for (int i = 0; i < TM; ++i)
+#pragma unroll
+                for (int t = 0; t < TN; ++t) {
+                    const uint32_t q_lo = (uint32_t)acc[i][t], q_hi = (uint32_t)(acc[i][t] >> 32);
+                    const uint32_t h_lo = __funnelshift_r(q_lo, q_hi, p.h) & mh_lo, h_hi = (q_hi >> p.h) & mh_hi;
+                    asm("add.cc.u32 %0, %0, %2;\n\taddc.u32 %1, %1, %3;" : "+r"(e_lo[i][t]), "+r"(e_hi[i][t]) : "r"(h_lo), "r"(h_hi));
+                    acc[i][t] = ((uint64_t)((q_hi & ml_hi) | b_hi) << 32) | ((q_lo & ml_lo) | b_lo);
+                }
+        }
+    };
+
+    // Asynchronous fetch of input channels ci0 .. ci0 + ckn - 1.  Activations by bulk copies dealt to the warps (a copy takes its
+    // warp some fifty cycles): the staged rows of a channel are contiguous when rows are uncut, else each row is a copy.  Kernel
+    // words, short pieces at a constant pitch, by 16-byte copies of the threads (what lies behind the last channel keeps old
+    // contents: the accumulators there are never stored).
+    uint32_t *const Bs = smem + p.b_off;
+    const uint32_t bar0 = smem_address(smem + p.bar_off);
+    const int KJ = K * J, nwarps = nthreads >> 5;
+    const uint32_t row_bytes = 4u * (uint32_t)p.pitch;
+    const size_t ap_plane = (size_t)p.ap_rows * p.XBT;
+    const uint32_t *ap_tile = p.ap + (size_t)r0 * p.XBT + seg * p.XO;
+    const int tco4_log2 = 29 - __clz(p.TCO), b_row = tid >> tco4_log2, b_col = 4 * (tid & (p.TCO / 4 - 1));   // TCO / 4 is a power of two
+    const int b_step = nthreads >> tco4_log2, b_rows = co0 + b_col < p.CoP ? 0x7FFFFFFF : 0;
+    const uint32_t *wp_tile = p.wp + (size_t)b_row * p.CoP + co0 + b_col;
+    const float inv_nr = 1.0f / (float)NR;
+    auto fetch = [&](int ci0, int ckn, int stage) {
+        const uint32_t bar = bar0 + 8u * stage;
+        if (tid == 0) mbarrier_arrive_expect(bar, (uint32_t)ckn * NR * row_bytes);
+        const uint32_t a_dst = smem_address(smem + stage * p.a_words);
+        const uint32_t *a_src = ap_tile + ci0 * ap_plane;
+        if (p.NSEG == 1) {
+            for (int c = warp; c < ckn; c += nwarps)
+                if (lane == 0) bulk_copy(a_dst + c * (4 * kPlaneWords), a_src + c * ap_plane, NR * row_bytes, bar);
+        } else {
+            for (int q = lane * nwarps + warp; q < ckn * NR; q += nthreads) {
+                const int c = small_div(q, NR, inv_nr), r = q - c * NR;
+                bulk_copy(a_dst + c * (4 * kPlaneWords) + r * row_bytes, a_src + c * ap_plane + (size_t)r * p.XBT, row_bytes, bar);
+            }
+        }
+        const uint32_t *b_src = wp_tile + (size_t)ci0 * KJ * p.CoP;
+        uint32_t *b_dst = Bs + stage * p.b_words + b_row * kBPitch + b_col;
+        const int rows = min(ckn * KJ, b_rows);
+        for (int k = b_row; k < rows; k += b_step, b_src += (size_t)b_step * p.CoP, b_dst += b_step * kBPitch) cp_async_16(b_dst, b_src);
+        cp_async_commit();
+    };
+    if (tid == 0) {
+        mbarrier_init(bar0, 1);
+        mbarrier_init(bar0 + 8, 1);
+        mbarrier_init_fence();
+    }
+    __syncthreads();
+    grid_dependency_wait();                                    // everything above touched no global memory
+    fetch(0, min(p.CK, p.Ci), 0);
+
+    // one input channel: K rows of J words from the row pointers ap and the kernel words at bp
+    const uint32_t *ap[ROWS], *bp;
+    auto channel = [&]() {
+        if constexpr (KT > 0) {
+            uint32_t a[ROWS][JT];
+#pragma unroll
+            for (int r = 0; r < ROWS; ++r)
+#pragma unroll
+                for (int j = 0; j < JT; ++j) a[r][j] = ap[r][-j];
+#pragma unroll
+            for (int kh = 0; kh < KT; ++kh)
+#pragma unroll
+                for (int j = 0; j < JT; ++j) {
+                    uint32_t b[TN];
+#pragma unroll
+                    for (int t = 0; t < TN; t += 4) {
+                        const uint4 v = *reinterpret_cast<const uint4 *>(bp + (kh * JT + j) * kBPitch + t);
+                        b[t] = v.x; b[t + 1] = v.y; b[t + 2] = v.z; b[t + 3] = v.w;
+                    }
+#pragma unroll
+                    for (int i = 0; i < TM; ++i)
+#pragma unroll
+                        for (int t = 0; t < TN; ++t) packed_mac<SP>(acc[i][t], a[i + kh][j], b[t]);
+                }
+            bp += KT * JT * kBPitch;
+        } else {
+            for (int kh = 0; kh < K; ++kh)
+                for (int j = 0; j < J; ++j, bp += kBPitch) {
+                    uint32_t a[TM], b[TN];
+#pragma unroll
+                    for (int i = 0; i < TM; ++i) a[i] = ap[i][kh * p.pitch - j];
+#pragma unroll
+                    for (int t = 0; t < TN; t += 4) {
+                        const uint4 v = *reinterpret_cast<const uint4 *>(bp + t);
+                        b[t] = v.x; b[t + 1] = v.y; b[t + 2] = v.z; b[t + 3] = v.w;
+                    }
+#pragma unroll
+                    for (int i = 0; i < TM; ++i)
+#pragma unroll
+                        for (int t = 0; t < TN; ++t) packed_mac<SP>(acc[i][t], a[i], b[t]);
+                }
+        }
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r) ap[r] += kPlaneWords;
+    };
+    // a run of input channels between two possible moves: the whole stage, or CF channels of it
+    const int run = HASE ? p.run : p.CK;
+    int moves = 0, runs_left = p.runs_per_move;
+    uint32_t phase = 0;                                        // parity of stage buffer s in bit s
+    int stage = 0;
+    for (int ci0 = 0; ci0 < p.Ci; ci0 += p.CK, stage ^= 1) {
+        const int ckn = min(p.CK, p.Ci - ci0);
+        // this stage has landed (were the wait ever to run out, the sums would be wrong but nothing would hang)
+        mbarrier_wait(bar0 + 8u * stage, (phase >> stage) & 1u);
+        cp_async_wait_all();
+        phase ^= 1u << stage;
+        __syncthreads();                                       // the previous stage is fully consumed
+        if (ci0 + p.CK < p.Ci) fetch(ci0 + p.CK, min(p.CK, p.Ci - ci0 - p.CK), stage ^ 1);
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r) ap[r] = a0 + stage * p.a_words + r * p.pitch;
+        bp = Bs + stage * p.b_words + tn * TN;
+        for (int c = 0; c < ckn; c += run) {
+            const int n = HASE ? min(run, ckn - c) : ckn;
+#pragma unroll 2
+            for (int u = 0; u < n; ++u) channel();
+            if constexpr (HASE) {
+                if (--runs_left == 0 && ci0 + c + n < p.Ci) {  // none is needed after the last channel
+                    move_upper_bits();
+                    ++moves;
+                    runs_left = p.runs_per_move;
+                }
+            }
+        }
+    }
+
+    // ---- words above the N low slots: to the next lane by shuffle, across warps through shared memory
+    uint2 *xch = reinterpret_cast<uint2 *>(smem) + ((warp << tnx_log2) + tn) * (TM * TN);
+    const int lanes_m = 32 >> tnx_log2, lm = lane >> tnx_log2;
+    __syncthreads();
+    if (UP && lm == lanes_m - 1) {
+#pragma unroll
+        for (int i = 0; i < TM; ++i)
+#pragma unroll
+            for (int t = 0; t < TN; ++t)
+                xch[i * TN + t] = make_uint2((uint32_t)(acc[i][t] >> p.SN),
+                                             HASE ? (uint32_t)((((uint64_t)e_hi[HASE ? i : 0][t] << 32) | e_lo[HASE ? i : 0][t]) >> p.SN) : 0u);
+    }
+    __syncthreads();
+    const uint2 *xch_in = xch - p.TNX * (TM * TN);
+    const bool from_smem = lm == 0 && warp > 0;
+    const uint32_t keep = xb == 0 ? 0u : 0xFFFFFFFFu;          // nothing comes in at the left end of a row
+
+    const int x = seg * p.XO + xb - p.halo, w0 = x * N - p.col_off;   // group and its first output column
+    const int h0 = s_img * TM;
+    const int n_rows = min(TM, p.Ho - h0);
+    bool col_ok[N];
+    int32_t base[N];                                           // what is taken off every sum of slot m
+#pragma unroll
+    for (int m = 0; m < N; ++m) {
+        col_ok[m] = pos_ok && xb >= p.halo && x < p.X && w0 + m >= 0 && w0 + m < p.Wo;
+        base[m] = -(moves + 1) * (p.slot_bias[m] + (keep ? p.slot_bias[m + N] : 0));
+    }
+    const int n_ch = min(TN, p.Co - co0 - tn * TN);
+    const uint32_t mask = p.slot_mask;
+
+    // value[m] of accumulator (i, t)
+    auto split = [&](int i, int t, const int32_t (&off)[N], int32_t (&y)[N]) {
+        uint64_t q = acc[i][t];
+        uint32_t q_in = 0, e_in = 0, qf[N], ef[N];
+        uint64_t e = 0;
+        if constexpr (HASE) e = ((uint64_t)e_hi[i][t] << 32) | e_lo[i][t];
+        if constexpr (UP) {
+            q_in = __shfl_up_sync(0xFFFFFFFFu, (uint32_t)(q >> p.SN), p.TNX);
+            if constexpr (HASE) e_in = __shfl_up_sync(0xFFFFFFFFu, (uint32_t)(e >> p.SN), p.TNX);
+            if (from_smem) {
+                const uint2 v = xch_in[i * TN + t];
+                q_in = v.x;
+                if constexpr (HASE) e_in = v.y;
+            }
+            q_in &= keep;
+            if constexpr (HASE) e_in &= keep;
+        }
+        if constexpr (PACKED_ADD && UP) {                   // the words coming in fill at most the low half, and no slot overflows
+            q = (q & 0xFFFFFFFF00000000ull) | (uint32_t)((uint32_t)q + q_in);
+            if constexpr (HASE) e = (e & 0xFFFFFFFF00000000ull) | (uint32_t)((uint32_t)e + e_in);
+        }
+#pragma unroll
+        for (int m = 0; m < N; ++m) {
+            qf[m] = (m == 0 ? (uint32_t)q : (uint32_t)(q >> (p.S * m))) & mask;
+            y[m] = off[m] + (int32_t)qf[m];
+            if constexpr (HASE) {
+                ef[m] = (m == 0 ? (uint32_t)e : (uint32_t)(e >> (p.S * m))) & mask;
+                y[m] += (int32_t)(ef[m] << p.h);
+            }
+            if constexpr (!PACKED_ADD && UP) {
+                if (m < p.up_slots) {
+                    y[m] += (int32_t)((q_in >> (p.S * m)) & mask);
+                    if constexpr (HASE) y[m] += (int32_t)(((e_in >> (p.S * m)) & mask) << p.h);
+                }
+            }
+        }
+    };
+    // base plus, on shifted codes, x_off times the channel's weights at the taps that lie inside the image at column w0 + m
+    auto offsets = [&](int t, int32_t (&off)[N]) {
+#pragma unroll
+        for (int m = 0; m < N; ++m) off[m] = base[m];
+        if (p.corr && t < n_ch) {
+            const int32_t *c = p.corr + co0 + tn * TN + t;
+#pragma unroll
+            for (int m = 0; m < N; ++m)
+                if (col_ok[m]) {
+                    const int k_lo = max(0, p.pad - w0 - m), k_hi = min(K, p.W + p.pad - w0 - m);
+                    off[m] += __ldg(c + k_hi * p.CoP) - __ldg(c + k_lo * p.CoP);
+                }
+        }
+    };
+    const int q_shift = p.shift, q_lo = p.lo, q_hi = p.hi;
+    auto requant = [&](int32_t v) { return max(q_lo, min(q_hi, v >> q_shift)); };
+
+    if (!p.stage_out) {
+        // direct stores; warps whose rows and channels all exist (nearly all) test only the columns
+        const size_t chan = (size_t)p.Ho * p.Wo;
+        const size_t at = (((size_t)(b0 + db) * p.Co + co0 + tn * TN) * p.Ho + h0) * p.Wo + w0;
+        auto finish = [&](auto *dst, auto full_tag) {
+            constexpr bool FULL = decltype(full_tag)::value, REQ = sizeof(*dst) == 1;
+            auto *chan_row = dst + at;
+#pragma unroll
+            for (int t = 0; t < TN; ++t, chan_row += chan) {
+                int32_t off[N], y[N];
+                offsets(t, off);
+                auto *row = chan_row;
+#pragma unroll
+                for (int i = 0; i < TM; ++i, row += p.Wo) {
+                    split(i, t, off, y);
+                    if (FULL || (t < n_ch && i < n_rows)) {
+#pragma unroll
+                        for (int m = 0; m < N; ++m) {
+                            if constexpr (REQ) y[m] = requant(y[m]);
+                            if (col_ok[m]) row[m] = (std::remove_reference_t<decltype(*dst)>)y[m];
+                        }
+                    }
+                }
+            }
+        };
+        const bool full = __all_sync(0xFFFFFFFFu, n_ch >= TN && (n_rows >= TM || !pos_ok));
+        if (p.requant) {
+            if (full) finish((int8_t *)p.out, std::true_type());
+            else finish((int8_t *)p.out, std::false_type());
+        } else {
+            if (full) finish((int32_t *)p.out, std::true_type());
+            else finish((int32_t *)p.out, std::false_type());
+        }
+        return;
+    }
+
+    // ---- requantised codes staged as bytes [channel][row][column]; with a pool the two rows of a pair are reduced first (the
+    // shift and the clamp keep the order, so the maximum is taken before them)
+    int8_t *tile = reinterpret_cast<int8_t *>(smem + p.tile_off);
+    const int rps = p.pool ? TM / 2 : TM;                      // tile rows per strip
+    const int tile_chan = p.TS * rps * p.WTP;
+    const int col0 = seg * p.XO * N;                           // first output column of the segment (segments: col_off == 0)
+    int8_t *tile_at = tile + tn * TN * tile_chan + sl * rps * p.WTP + w0 - col0;
+    auto stage_codes = [&](auto pool_tag) {
+        constexpr bool POOL = decltype(pool_tag)::value;
+#pragma unroll
+        for (int t = 0; t < TN; ++t) {
+            int32_t off[N], y[N], y2[N];
+            offsets(t, off);
+#pragma unroll
+            for (int i = 0; i < TM; i += POOL ? 2 : 1) {
+                split(i, t, off, y);
+                if constexpr (POOL) {
+                    split(i + 1, t, off, y2);
+#pragma unroll
+                    for (int m = 0; m < N; ++m) y[m] = max(y[m], y2[m]);
+                }
+#pragma unroll
+                for (int m = 0; m < N; ++m)
+                    if (col_ok[m]) tile_at[t * tile_chan + (POOL ? i / 2 : i) * p.WTP + m] = (int8_t)requant(y[m]);
+            }
+        }
+    };
+    if (p.pool) stage_codes(std::true_type());
+    else stage_codes(std::false_type());
+    __syncthreads();
+
+    // ---- staged codes leave the CTA in pieces of `vec` bytes along a row, neighbouring columns reduced first with a pool
+    const int sh = p.pool ? 1 : 0, rps_log2 = 31 - __clz(rps);
+    const int Hq = p.Ho >> sh, Wq = p.Wo >> sh;
+    const int wn = (p.NSEG > 1 ? min(p.Wo - col0, p.XO * N) : p.Wo) >> sh;   // output columns of this segment
+    const int ncv = min(p.TCO, p.Co - co0), tr = TSe * rps;
+    const int ppr = p.out_bits < 8 ? ((wn * p.out_bits) >> 3) / p.vec : wn / p.vec;
+    const float inv_ppr = 1.0f / (float)ppr, inv_tr = 1.0f / (float)tr;
+    for (int idx = tid; idx < ncv * tr * ppr; idx += nthreads) {
+        const int rr = small_div(idx, ppr, inv_ppr), piece = idx - rr * ppr;
+        const int cl = small_div(rr, tr, inv_tr), r = rr - cl * tr;
+        const int ts = s0 + (r >> rps_log2), d = fast_div(ts, p.mg_sh);
+        const int hq = (ts - d * p.SH) * rps + (r & (rps - 1));
+        if (hq >= Hq) continue;                                // rows past the image in its last strip
+        const int8_t *src = tile + cl * tile_chan + r * p.WTP;
+        const size_t e0 = (((size_t)(b0 + d) * p.Co + co0 + cl) * Hq + hq) * Wq + (col0 >> sh);   // first code of this segment's row
+        if (p.out_bits < 8) {
+            // dense codes: every output byte gathers 8 / out_bits neighbouring codes (rows and segments start on byte
+            // boundaries, checked on the host)
+            const int ob = p.out_bits, cpb = 8 / ob;
+            const uint32_t cmask = (1u << ob) - 1u;
+            uint8_t *dst = (uint8_t *)p.out + ((e0 * ob) >> 3) + piece * p.vec;
+            uint32_t word = 0;
+            for (int u = 0; u < p.vec * cpb; ++u) {
+                const int col = piece * p.vec * cpb + u;
+                int v = src[p.pool ? 2 * col : col];
+                if (p.pool) {
+                    int v1 = src[2 * col + 1];
+                    if (!p.out_signed) { v &= 0xFF; v1 &= 0xFF; }
+                    v = max(v, v1);
+                }
+                word |= ((uint32_t)v & cmask) << (ob * u);
+            }
+            if (p.vec == 4) *reinterpret_cast<uint32_t *>(dst) = word;
+            else *dst = (uint8_t)word;
+        } else {                                               // one code per byte: staged only for a pool
+            int8_t *dst = (int8_t *)p.out + e0 + piece * p.vec;
+            src += 2 * piece * p.vec;
+            if (p.vec == 8) {
+                const uint4 v = *reinterpret_cast<const uint4 *>(src);
+                *reinterpret_cast<uint2 *>(dst) = p.out_signed ? make_uint2(pool_pairs<true>(v.x, v.y, v.x, v.y), pool_pairs<true>(v.z, v.w, v.z, v.w))
+                                                               : make_uint2(pool_pairs<false>(v.x, v.y, v.x, v.y), pool_pairs<false>(v.z, v.w, v.z, v.w));
+            } else if (p.vec == 4) {
+                const uint2 v = *reinterpret_cast<const uint2 *>(src);
+                *reinterpret_cast<uint32_t *>(dst) = p.out_signed ? pool_pairs<true>(v.x, v.y, v.x, v.y) : pool_pairs<false>(v.x, v.y, v.x, v.y);
+            } else {
+                int a = src[0], b = src[1];
+                if (!p.out_signed) { a &= 0xFF; b &= 0xFF; }
+                *dst = (int8_t)max(a, b);
+            }
+        }
+    }
+}
+
+template <int N, int KT, int JT, int TM, int TN, bool HASE>
+static int launch_strip_tile(const StripLaunch &s, cudaStream_t st) {
+    auto run = [&](auto kern) -> int {
+        if (s.smem_bytes > 48 * 1024)
+            HIKONV_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem_bytes));
+        return launch_dependent(kern, s.grid, dim3(s.threads), s.smem_bytes, st, s.p);
+    };
+    return s.sp ? run(conv2d_strip_kernel<N, KT, JT, TM, TN, true, HASE>) : run(conv2d_strip_kernel<N, KT, JT, TM, TN, false, HASE>);
+}
+
+template <int N, int KT, int JT>
+static int launch_strip(const StripLaunch &s, cudaStream_t st) {
+    if (s.TM == 4 && s.TN == 4) return s.moves ? launch_strip_tile<N, KT, JT, 4, 4, true>(s, st) : launch_strip_tile<N, KT, JT, 4, 4, false>(s, st);
+    if constexpr (KT > 0) {
+        if (s.TM == 2 && s.TN == 8) return s.moves ? launch_strip_tile<N, KT, JT, 2, 8, true>(s, st) : launch_strip_tile<N, KT, JT, 2, 8, false>(s, st);
+        if (s.TM == 2 && s.TN == 4) return s.moves ? launch_strip_tile<N, KT, JT, 2, 4, true>(s, st) : launch_strip_tile<N, KT, JT, 2, 4, false>(s, st);
+        if (s.TM == 4 && s.TN == 8 && !s.moves) return launch_strip_tile<N, KT, JT, 4, 8, false>(s, st);
+    }
+    return HIKONV_ERR_UNSUPPORTED;
+}
+
+}  // namespace hikonv

@@ -55,6 +55,11 @@ int make_layout_byte_slots(int p, int q, int f_signed, int g_signed, int K, hiko
 SplitConsts128 make_split_consts128(const hikonv_layout_t &L, int p, int q, int f_signed, int g_signed, int K);
 SplitConsts make_split_consts(const hikonv_layout_t &L, int p, int q, int f_signed, int g_signed, int K, int M);
 
+// 2-D: input channels that may be accumulated between two moves of upper slot bits (at most M / K; Ci when M covers the layer),
+// or 0 when the layout has no room.  packed_add: the slots above the N low ones are added to the next word's low slots while
+// both accumulators are still packed, so a low slot has to hold its own sum and the one that comes in.
+int move_period(const hikonv_layout_t &L, const SplitConsts &sc, int p, int q, int f_signed, int g_signed, int K, int Ci, bool packed_add);
+
 inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 
 // Words per packed kernel row in the 2-D kernels' shared memory, and the cap on channels per stage that
@@ -65,8 +70,8 @@ inline int stage_channel_cap(int K, int J) {
     return c < 1 ? 1 : (c > 8 ? 8 : c);
 }
 
-// 2-D kernels stage CK input channels at a time and move the upper slot bits to the second
-// accumulator every `fc` stages.  Given the number of channels CF that may be accumulated between two
+// The planner's rule for 2-D layers: the upper slot bits move to the second accumulator every `fc` stages of CK input
+// channels.  Given the number of channels CF that may be accumulated between two
 // such moves, picks CK <= ck_cap and fc with CK * fc <= CF as large as possible (stages of fewer than
 // three channels are avoided when something close is available).  Returns CK * fc.
 inline int pick_chunking(int CF, int Ci, int *CK, int *fc, int ck_cap = 8) {

@@ -480,6 +480,33 @@ SplitConsts make_split_consts(const hikonv_layout_t &L, int p, int q, int fs, in
     return c;
 }
 
+int move_period(const hikonv_layout_t &L, const SplitConsts &sc, int p, int q, int fs, int gs, int K, int Ci, bool packed_add) {
+    const bool moves = L.M < Ci * K;
+    const Range fr = code_range(p, fs ? 1 : 0), gr = code_range(q, gs ? 1 : 0);
+    const long long prods[4] = {fr.lo * gr.lo, fr.lo * gr.hi, fr.hi * gr.lo, fr.hi * gr.hi};
+    const long long pmax = *std::max_element(prods, prods + 4);
+    int T[kMaxSegments];
+    term_counts(L, K, T);
+    const int h = L.carry_bits;
+    const long long low = moves ? (1LL << h) - 1 : 0, room = (1LL << L.S) - 1;
+    for (int cf = moves ? L.M / K : Ci; cf >= 1; --cf) {
+        const long long count = moves ? (Ci + cf - 1) / cf - 1 : 0;  // moves; the second accumulator takes 2^h of them
+        if (moves && count > (1LL << h)) return 0;
+        bool fits = true;
+        for (int m = 0; packed_add && m < L.N && fits; ++m) {
+            long long q_sum = 0, e_sum = 0;                          // largest stored values of the two slots that meet
+            for (int i = m; i < L.segments; i += L.N) {
+                const long long most = low + sc.seg_bias[i] + (long long)cf * K * T[i] * pmax;
+                q_sum += most;
+                e_sum += count * (most >> h);
+            }
+            fits = q_sum <= room && (!moves || e_sum <= room);
+        }
+        if (fits) return cf;
+    }
+    return 0;
+}
+
 }  // namespace hikonv
 
 using namespace hikonv;

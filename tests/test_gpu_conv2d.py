@@ -76,6 +76,24 @@ def test_forced_words_per_block(n):
             _layer(x, w, 1, 4, 4, True, True, hk.ALGO_PACKED32, tune={"N": 4})
 
 
+@pytest.mark.parametrize("K, pad", [(1, 0), (3, 1), (3, 0), (5, 2), (5, 4), (4, 1)])
+def test_strips_of_rows_in_every_tile(K, pad):
+    # two and four output rows per thread, every number of channel lanes, one strip per CTA up to several images, heights that
+    # leave a ragged last strip, rows of one segment and of several, channel counts that are no multiple of the thread tile;
+    # widths with 1 to 4 pixels per word, with and without second accumulators, on shifted codes and not
+    for (B, Ci, H, W, Co) in ((3, 9, 7, 10, 9), (5, 3, 5, 4, 20), (1, 40, 6, 150, 5), (2, 5, 9, 530, 8)):
+        for (p, q, xs, ws) in ((4, 4, True, True), (4, 4, False, True), (8, 8, True, True), (2, 2, False, True), (8, 4, False, True), (5, 5, False, False)):
+            x, w = inputs.conv2d_case(B, Ci, H, W, Co, K, p, q, xs, ws, seed=B + Ci + K + p)
+            ref = direct.conv2d_nchw(x, w, pad)
+            for tile in (0, 1, 2001, 200001, 204003, 401002, 404004, 208008, 1048):
+                try:
+                    got = _layer(x, w, pad, p, q, xs, ws, hk.ALGO_PACKED32, tune={"tile": tile})
+                except hk.HikonvError as err:          # forced shapes that need more threads than a CTA has
+                    assert err.status == hk.ERR_UNSUPPORTED and tile != 0
+                    continue
+                assert_exact(got, ref, "%s K=%d p=%d q=%d tile=%d" % ((B, Ci, H, W, Co), K, p, q, tile))
+
+
 @pytest.mark.parametrize("ci", [4, 7, 20, 64, 130, 256])
 def test_carry_save_schedules(ci):
     # 3x3 layers at N = 3, S = 13 move slot bits to the second accumulator at stage ends (s4 x s4, and any layer
