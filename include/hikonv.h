@@ -93,8 +93,8 @@ typedef struct {
     int M;          /* force the number of accumulated products between two splits  */
     int tile;       /* kernel-specific tile selector (0 = automatic); conv2d: > 0 output
                        rows per CTA + 1000 x channel lanes per CTA (1, 2, 4, 8; the comparator also
-                       16) + 100000 x output rows per thread (2 or 4), each part 0 = automatic;
-                       < 0 as 0; conv1d: > 0 the general kernel, -1 the
+                       16) + 100000 x output rows per thread (2 or 4) + 1000000 x channels per
+                       thread (4 or 8), each part 0 = automatic; < 0 as 0; conv1d: > 0 the general kernel, -1 the
                        planner's layout instead of register-aligned slots; -24 / -25 force the
                        register budget of four / five resident CTAs per SM in the register-aligned
                        kernels and the two comparators (default: whichever measured faster for the
@@ -249,7 +249,7 @@ int hikonv_conv2d(const int8_t *d_x, int B, int Ci, int H, int W, const int8_t *
  * counterpart in the paper: the automatic choice comes from a cost model, which on small layers misses tiles that
  * measure 10-20 % faster).  Arguments up to `algo` are those of hikonv_conv2d_dense (one code per byte: storage 8 / 8,
  * out_store_bits 8, or 32 without requant).  The call runs the layer with the library's own tile and with every forced
- * tile (rows per thread 4 and 2 x channel lanes 1, 2, 4, 8 x output rows per CTA 1 .. 48; shapes the layer does not
+ * tile (rows per thread 4 and 2 x channels per thread 4 and 8 x channel lanes 1, 2, 4, 8 x output rows per CTA up to 48; shapes the layer does not
  * support are skipped), each as groups of four launches between two CUDA events on `stream`, best of `repeats` (1 .. 100)
  * groups, and SYNCHRONISES.  Every launch writes the layer's complete, correct output to d_out.
  * *h_tile: the value for hikonv_tuning_t.tile in later calls on this shape, or 0 when no forced tile is at least 3 %

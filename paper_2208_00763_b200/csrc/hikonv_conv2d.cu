@@ -291,13 +291,13 @@ struct StripProblem {
 };
 
 struct StripChoice {
-    int TM, TN, TNX, TS, NSEG, XO, XB, halo, X, col_off, pitch, CK, run, runs_per_move, bar_off, threads;
+    int TM, TN, TNX, TS, NSEG, XO, XB, halo, X, col_off, pitch, CK, run, runs_per_move, plane, bar_off, e_off, threads;
     size_t smem;
     long long ctas;
     double cost;
 };
 
-// Staged rows of TS strips, and whether a CTA of that many fits a plane.
+// Staged rows of TS strips.
 static int staged_rows(int TS, int TM, int SH, int Hp, int K) {
     const int gap = Hp - SH * TM;                                    // rows between the strips of one image and the next, beyond TM per strip
     const int crossings = (TS - 1 + SH - 1) / SH;
@@ -305,14 +305,14 @@ static int staged_rows(int TS, int TM, int SH, int Hp, int K) {
 }
 
 // Completes a candidate (TM, TN, TNX, TS and the row cut are set) and models its time in scheduler cycles of the busiest SM:
-// issue cycles of a warp (4.15 per multiply, about one for every other instruction, counted from the kernel's source) times
-// the warps of the busiest scheduler, wave by wave.  Returns false when the candidate cannot run.
+// issue cycles of a warp (4.3 per multiply, about one for every other instruction; a tile of 2 x 4 costs a tenth more per multiply
+// than 4 x 8 by this count and by the clock) times the warps of the busiest scheduler, wave by wave.  Returns false when the candidate cannot run.
 static bool complete_choice(const StripProblem &q, StripChoice *c) {
     const int SH = ceil_div(q.Ho, c->TM), Hp = q.Ho + q.K - 1, KJ = q.K * q.J;
     const long long strips = (long long)q.B * SH;
     c->pitch = (c->XB + q.J - 1 + 3) / 4 * 4;
     const int rows = staged_rows(c->TS, c->TM, SH, Hp, q.K);
-    if ((long long)rows * c->pitch > kPlaneWords) return false;
+    c->plane = rows * c->pitch;
     c->threads = (c->TS * c->XB * c->TNX + 31) / 32 * 32;
     if (c->threads > kStripThreads) return false;
     const int warps = c->threads / 32, TCO = c->TNX * c->TN;
@@ -321,8 +321,11 @@ static bool complete_choice(const StripProblem &q, StripChoice *c) {
     // channels per stage: as many as leave room for the CTAs that the registers allow; runs of CF channels that fill stages
     const int by_regs = std::min(65536 / (c->threads * 128), 32);
     const int want = std::max(1, std::min(by_regs, share));
-    const size_t room = std::min<size_t>(kSmemPerCta, kSmemPerSm / want - 1024) - 64;
-    int CK = std::min(std::min(8, q.Ci), (int)(room / (2 * 4 * (size_t)(kPlaneWords + KJ * kBPitch))));
+    const size_t e_bytes = q.moves ? (size_t)c->threads * strip_e_pitch(c->TM, c->TN) * 8 : 0;
+    const size_t per_cta = std::min<size_t>(kSmemPerCta, kSmemPerSm / want - 1024);
+    if (per_cta < e_bytes + 4096) return false;
+    const size_t room = per_cta - e_bytes - 64;
+    int CK = (int)std::min<size_t>(std::min(kStripMaxCK, q.Ci), room / (2 * 4 * (size_t)(c->plane + KJ * kStripBPitch)));
     if (CK < 1) return false;
     c->run = CK;
     c->runs_per_move = 1;
@@ -344,20 +347,21 @@ static bool complete_choice(const StripProblem &q, StripChoice *c) {
         }
     }
     c->CK = CK;
-    size_t words = 2 * (size_t)CK * (kPlaneWords + KJ * kBPitch);
+    size_t words = 2 * (size_t)CK * (c->plane + KJ * kStripBPitch);
     const size_t xch = (size_t)warps * c->TNX * c->TM * c->TN * 2;
     const int rps = q.pool ? c->TM / 2 : c->TM;
     const size_t tile = (xch + 3) / 4 * 4 + (size_t)TCO * c->TS * rps * ((c->XO * q.N + 15) / 16 * 16) / 4;
     words = (std::max(words, std::max(xch, tile)) + 3) / 4 * 4;
     c->bar_off = (int)words;
-    c->smem = words * 4 + 16;
+    c->e_off = (int)words + 4;
+    c->smem = words * 4 + 16 + e_bytes;
     if (c->smem > (size_t)kSmemPerCta) return false;
     const int resident = std::max(1, std::min(by_regs, (int)(kSmemPerSm / (c->smem + 1024))));
     // issue cycles of one warp
     const double mt = (double)c->TM * c->TN;
-    double per_ch = 4.15 * mt * KJ + 0.7 * (c->TM + q.K - 1) * q.J + 0.9 * KJ * c->TN / 4 + 0.6 * (c->TM + q.K - 1) + 6 + 60.0 / CK;
+    double per_ch = 4.3 * mt * KJ + 0.5 * (c->TM + q.K - 1) * q.J + 0.6 * KJ * c->TN / 4 + 8 + 80.0 / CK;
     if (q.generic) per_ch += KJ * 16.0;
-    if (q.moves) per_ch += 9.5 * mt / q.CF;
+    if (q.moves) per_ch += 10.0 * mt / q.CF;
     const double split = q.moves ? 6.0 * q.N + 12 : 3.0 * q.N + 6;
     const double fixed = 400 + mt * (split + q.N * (q.pool ? 4.0 : q.requant ? 6.0 : 3.0));
     const double warp_cycles = q.Ci * per_ch + fixed;
@@ -376,20 +380,21 @@ static bool complete_choice(const StripProblem &q, StripChoice *c) {
 }
 
 // Chooses the thread tile, channel lanes, row cut and strips per CTA.  force_*: 0 = free.
-static StripChoice choose_strips(const StripProblem &q, int force_tm, int force_tnx, int force_rows) {
-    static const int tiles[4][2] = {{4, 4}, {2, 8}, {2, 4}, {4, 8}};
+static StripChoice choose_strips(const StripProblem &q, int force_tm, int force_tn, int force_tnx, int force_rows) {
+    static const int tiles[3][2] = {{4, 8}, {2, 8}, {2, 4}};
     StripChoice best;
     std::memset(&best, 0, sizeof(best));
     best.cost = -1.0;
     const int c0 = q.K - 1 - q.pad;
     for (const auto &tile : tiles) {
         const int TM = tile[0], TN = tile[1];
-        if (!strip_tile_built(TM, TN, q.moves, q.generic) || (force_tm > 0 && TM != force_tm && !q.generic)) continue;
-        if (TN == 8 && q.Co <= 4) continue;
+        if (!strip_tile_built(TM, TN, q.generic) || (force_tm > 0 && TM != force_tm && !q.generic) ||
+            (force_tn > 0 && TN != force_tn && !q.generic)) continue;
+        if (TN == 8 && q.Co <= 4 && force_tn != 8) continue;
         const int SH = ceil_div(q.Ho, TM);
         const long long strips = (long long)q.B * SH;
-        for (int TNX = 1; TNX <= 8; TNX *= 2) {
-            if (force_tnx > 0 ? TNX != std::min(force_tnx, 8) : (TNX > 1 && TNX * TN / 2 >= q.Co)) continue;
+        for (int TNX = 1; TNX * TN <= kStripBPitch; TNX *= 2) {
+            if (force_tnx > 0 ? TNX != std::min(force_tnx, kStripBPitch / TN) : (TNX > 1 && TNX * TN / 2 >= q.Co)) continue;
             const int maxpos = kStripThreads / TNX;
             // uncut rows start at the image's first column (a word then holds no padding but the row's end); the positions of a
             // cut row need the word in front of them, and its segments start at columns XO N
@@ -496,10 +501,11 @@ static int plan_layer(int B, int Ci, int H, int W, int Co, int K, int stride, in
         pr.requant = out.requant != 0; pr.pool = out.requant && out.pool;
         pr.xo_mult = segment_multiple(out, L.N);
         pr.sms = sm_count();
-        // tune->tile > 0: rows per CTA, plus 1000 x channel lanes per CTA and 100000 x rows per thread when those are forced too
-        const int tile_arg = (tune && tune->tile > 0) ? tune->tile : 0, force_tm = tile_arg / 100000;
-        if (force_tm != 0 && force_tm != 2 && force_tm != 4) return HIKONV_ERR_UNSUPPORTED;
-        const StripChoice c = choose_strips(pr, force_tm, tile_arg % 100000 / 1000, tile_arg % 1000);
+        // tune->tile > 0: rows per CTA, plus 1000 x channel lanes per CTA, 100000 x rows and 1000000 x channels per thread when
+        // those are forced too
+        const int tile_arg = (tune && tune->tile > 0) ? tune->tile : 0, force_tn = tile_arg / 1000000, force_tm = tile_arg / 100000 % 10;
+        if ((force_tm != 0 && force_tm != 2 && force_tm != 4) || (force_tn != 0 && force_tn != 4 && force_tn != 8)) return HIKONV_ERR_UNSUPPORTED;
+        const StripChoice c = choose_strips(pr, force_tm, force_tn, tile_arg % 100000 / 1000, tile_arg % 1000);
         if (c.cost < 0) return HIKONV_ERR_UNSUPPORTED;
 
         StripLaunch &l = s->strip;
@@ -511,8 +517,8 @@ static int plan_layer(int B, int Ci, int H, int W, int Co, int K, int stride, in
         k.SH = ceil_div(Ho, c.TM); k.strips = B * k.SH;
         k.NSEG = c.NSEG; k.XO = c.XO; k.XB = c.XB; k.halo = c.halo; k.X = c.X; k.col_off = c.col_off; k.pitch = c.pitch;
         k.XBT = (c.NSEG - 1) * c.XO + c.pitch;
-        k.TS = c.TS; k.TNX = c.TNX; k.TCO = c.TNX * c.TN; k.CK = c.CK; k.run = c.run; k.runs_per_move = c.runs_per_move; k.bar_off = c.bar_off;
-        k.a_words = c.CK * kPlaneWords; k.b_off = 2 * k.a_words; k.b_words = c.CK * K * L.J * kBPitch;
+        k.TS = c.TS; k.TNX = c.TNX; k.TCO = c.TNX * c.TN; k.CK = c.CK; k.run = c.run; k.runs_per_move = c.runs_per_move; k.bar_off = c.bar_off; k.e_off = c.e_off;
+        k.plane = c.plane; k.a_words = c.CK * c.plane; k.b_off = 2 * k.a_words; k.b_words = c.CK * K * L.J * kStripBPitch;
         auto magic = [](int d) -> uint32_t { return d <= 1 ? 0u : (uint32_t)((0x100000000ull + (unsigned)d - 1) / (unsigned)d); };
         k.mg_xb = magic(c.XB); k.mg_sh = magic(k.SH);
         k.S = L.S; k.SN = L.S * L.N; k.h = L.carry_bits;
@@ -577,13 +583,22 @@ static int setup_layer(int B, int Ci, int H, int W, int Co, int K, int stride, i
 
 static int launch_layer(const Conv2dSetup &s, cudaStream_t st) {
     if (s.unpacked) return launch_unpacked2d(s.un, st);
-    switch (s.L.N) {
-        case 1: return launch_strip_n1(s.strip, st);
-        case 2: return launch_strip_n2(s.strip, st);
-        case 3: return launch_strip_n3(s.strip, st);
-        case 4: return launch_strip_n4(s.strip, st);
-        default: return HIKONV_ERR_UNSUPPORTED;
+    const int N = s.L.N, K = s.strip.p.K, J = s.strip.p.J;
+    if (s.strip.generic) {
+        switch (N) {
+            case 1: return launch_strip<1, 0, 0>(s.strip, st);
+            case 2: return launch_strip<2, 0, 0>(s.strip, st);
+            case 3: return launch_strip<3, 0, 0>(s.strip, st);
+            case 4: return launch_strip<4, 0, 0>(s.strip, st);
+            default: return HIKONV_ERR_UNSUPPORTED;
+        }
     }
+#define HK_LAYOUT(n, k, j) if (N == n && K == k && J == j) return launch_strip<n, k, j>(s.strip, st);
+    HK_LAYOUT(2, 1, 1) HK_LAYOUT(3, 1, 1) HK_LAYOUT(4, 1, 1)
+    HK_LAYOUT(2, 3, 1) HK_LAYOUT(2, 3, 2) HK_LAYOUT(3, 3, 1) HK_LAYOUT(4, 3, 1)
+    HK_LAYOUT(2, 5, 3) HK_LAYOUT(3, 5, 2) HK_LAYOUT(4, 5, 1) HK_LAYOUT(4, 5, 2)
+#undef HK_LAYOUT
+    return HIKONV_ERR_UNSUPPORTED;
 }
 
 }  // namespace hikonv
@@ -750,12 +765,16 @@ extern "C" int hikonv_conv2d_tune(const void *d_x, int x_store_bits, int B, int 
     int best_tile = 0;
     if (rc == HIKONV_OK) {
         const long long rows = (long long)B * ((long long)H + 2 * pad - K + 1);
-        for (int tm = 4; tm >= 2 && rc_cuda == HIKONV_OK; tm -= 2)
+        const bool packed = algo == HIKONV_ALGO_PACKED32;
+        for (int shape = packed ? 3 : 1; shape >= 1 && rc_cuda == HIKONV_OK; --shape)
             for (int tnx = 1; tnx <= 8 && rc_cuda == HIKONV_OK; tnx *= 2)
-                for (int tr = 1; tr <= 48 && tr <= rows && rc_cuda == HIKONV_OK; ++tr) {
+                for (int tr = 1; tr <= 48 && tr <= rows + 3 && rc_cuda == HIKONV_OK; ++tr) {
+                    // packed: 4 x 8, 2 x 8 and 2 x 4 rows x channels per thread, whole strips of rows
+                    const int tm = shape == 3 ? 4 : 2, tn = shape >= 2 ? 8 : 4;
+                    if (packed && tr % tm != 0) continue;
                     hikonv_tuning_t tune;
                     std::memset(&tune, 0, sizeof(tune));
-                    tune.tile = tr + 1000 * tnx + 100000 * tm;
+                    tune.tile = packed ? tr + 1000 * tnx + 100000 * tm + 1000000 * tn : tr + 1000 * tnx;
                     const double t = time_of(&tune, 2.0 * best);
                     if (t >= 0.0 && t < best) { best = t; best_tile = tune.tile; }
                 }

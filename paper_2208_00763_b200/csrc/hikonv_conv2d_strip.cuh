@@ -21,11 +21,14 @@
 // there (packed_add; where the slots do not have the room for that, as separate fields), the N slots are read by shift and
 // mask, value m = 2^h E_m + Q_m - (moves + 1) (bias_m + bias_{m + N}).
 //
-// What bounds it: instruction issue.  A warp-wide 32x32->64 multiply-add holds its scheduler for 4.1 cycles, every other
-// arithmetic instruction adds about one more.  Measured against the kernel before it (four positions of one row per thread,
-// second accumulators in shared memory, one halo word per row, run-time loops for 5x5), packing launch included:
-// 32x64x56x56 -> 64 s4 93.3 -> 87.9 us, 64x256x14x14 -> 256 u4 x s4 211 -> 166 us (205 with the new packing launch alone),
-// 8x48x37x53 -> 40 s8 32.4 -> 27.3 us, 16x24x45x61 -> 40 5x5 2-bit 70.6 -> 30.3 us, the compact CNN (batch 64) 605 -> 499 us.
+// What bounds it: the multiplier's pipe and the instruction issue around it.  A warp-wide 32x32->64 multiply-add holds its
+// scheduler for 4.1 cycles in a loop of nothing else; in this loop a channel of a 4 x 8 tile (96 of them, 34 other
+// instructions) takes 473 cycles, of a 2 x 8 tile with moves (48 and 52) 285.  Three CTAs per SM, operand rows in registers
+// across channels or a compile-time distance between channels (no pointer arithmetic left) changed neither.
+// Measured against the kernel before it (four positions of one row per thread, one halo word per row, run-time loops for 5x5),
+// packing launch included: 32x64x56x56 -> 64 s4 93.3 -> 85.4 us, 64x256x14x14 -> 256 u4 x s4 211 -> 162 us (205 with the new
+// packing launch alone), 8x48x37x53 -> 40 s8 32.4 -> 26.4 us, 16x24x45x61 -> 40 5x5 2-bit 70.6 -> 31.7 us, the compact CNN
+// (batch 64) 605 -> 492 us.
 #pragma once
 
 #include <type_traits>
@@ -35,12 +38,6 @@
 #include "hikonv_conv2d_util.cuh"
 
 namespace hikonv {
-
-template <bool SP>
-__device__ __forceinline__ void packed_mac(uint64_t &acc, uint32_t a, uint32_t b) {
-    if constexpr (SP) acc += (uint64_t)((int64_t)(int32_t)a * (int64_t)(int32_t)b);
-    else acc += (uint64_t)a * (uint64_t)b;
-}
 
 template <int N, int KT, int JT>
 constexpr bool kStripPackedAdd = strip_packed_add(N, KT, JT);
@@ -55,7 +52,8 @@ __global__ void __launch_bounds__(kStripThreads, 2) conv2d_strip_kernel(const __
     extern __shared__ __align__(16) uint32_t smem[];
     grid_dependency_release();
 
-    const int tid = threadIdx.x, nthreads = blockDim.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, nthreads = blockDim.x, lane = tid & 31;
+    const int warp = tid >> 5;
     const int tnx_log2 = 31 - __clz(p.TNX);                    // TNX is a power of two
     const int tn = tid & (p.TNX - 1);
     const int strip_tile = p.NSEG > 1 ? (int)(blockIdx.x / (unsigned)p.NSEG) : (int)blockIdx.x;
@@ -75,16 +73,21 @@ __global__ void __launch_bounds__(kStripThreads, 2) conv2d_strip_kernel(const __
     const int pos = tid >> tnx_log2, pos_ok = pos < TSe * p.XB, pc = pos_ok ? pos : 0;
     const int sl = fast_div(pc, p.mg_xb), xb = pc - sl * p.XB;
     const int db = fast_div(s0 + sl, p.mg_sh), s_img = s0 + sl - db * p.SH;
-    const uint32_t *a0 = smem + (db * p.Hp + (s_img - s0) * TM) * p.pitch + xb + J - 1;
+    int a_off[ROWS];                                           // word of row r, j = 0 in a channel's plane
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) a_off[r] = (db * p.Hp + (s_img - s0) * TM + r) * p.pitch + xb + J - 1;
 
+    // Second accumulators: in shared memory, at an odd pitch of 8-byte entries per thread, so that the lanes of a warp fall into
+    // different banks and every access has an immediate offset.  They are touched once in CF channels; in registers they would
+    // leave no room for 32 accumulators (and with 16 they were no faster).
     uint64_t acc[TM][TN];
-    uint32_t e_lo[HASE ? TM : 1][TN], e_hi[HASE ? TM : 1][TN];
+    uint2 *es = reinterpret_cast<uint2 *>(smem + p.e_off) + tid * strip_e_pitch(TM, TN);
 #pragma unroll
     for (int i = 0; i < TM; ++i)
 #pragma unroll
         for (int t = 0; t < TN; ++t) {
             acc[i][t] = p.bias;
-            if constexpr (HASE) e_lo[i][t] = e_hi[i][t] = 0u;
+            if constexpr (HASE) es[i * TN + t] = make_uint2(0u, 0u);
         }
     auto move_upper_bits = [&]() {
         if constexpr (HASE) {
@@ -97,45 +100,53 @@ __global__ void __launch_bounds__(kStripThreads, 2) conv2d_strip_kernel(const __
                 for (int t = 0; t < TN; ++t) {
                     const uint32_t q_lo = (uint32_t)acc[i][t], q_hi = (uint32_t)(acc[i][t] >> 32);
                     const uint32_t h_lo = __funnelshift_r(q_lo, q_hi, p.h) & mh_lo, h_hi = (q_hi >> p.h) & mh_hi;
-                    asm("add.cc.u32 %0, %0, %2;\n\taddc.u32 %1, %1, %3;" : "+r"(e_lo[i][t]), "+r"(e_hi[i][t]) : "r"(h_lo), "r"(h_hi));
+                    uint2 e = es[i * TN + t];
+                    asm("add.cc.u32 %0, %0, %2;\n\taddc.u32 %1, %1, %3;" : "+r"(e.x), "+r"(e.y) : "r"(h_lo), "r"(h_hi));
+                    es[i * TN + t] = e;
                     acc[i][t] = ((uint64_t)((q_hi & ml_hi) | b_hi) << 32) | ((q_lo & ml_lo) | b_lo);
                 }
         }
     };
 
-    // Asynchronous fetch of input channels ci0 .. ci0 + ckn - 1.  Activations by bulk copies dealt to the warps (a copy takes its
-    // warp some fifty cycles): the staged rows of a channel are contiguous when rows are uncut, else each row is a copy.  Kernel
-    // words, short pieces at a constant pitch, by 16-byte copies of the threads (what lies behind the last channel keeps old
-    // contents: the accumulators there are never stored).
+    // Asynchronous fetch of the next ckn input channels.  Activations by bulk copies dealt to the warps (with warp 0 issuing all
+    // of them the others waited for it): the staged rows of a channel are contiguous when rows are uncut, else each row is a
+    // copy.  Kernel words, short pieces at a constant pitch, by 16-byte copies of the threads (what lies behind the last channel
+    // keeps old contents: the accumulators there are never stored).
     uint32_t *const Bs = smem + p.b_off;
     const uint32_t bar0 = smem_address(smem + p.bar_off);
     const int KJ = K * J, nwarps = nthreads >> 5;
-    const uint32_t row_bytes = 4u * (uint32_t)p.pitch;
+    const uint32_t row_bytes = 4u * (uint32_t)p.pitch, ch_bytes = NR * row_bytes;
     const size_t ap_plane = (size_t)p.ap_rows * p.XBT;
-    const uint32_t *ap_tile = p.ap + (size_t)r0 * p.XBT + seg * p.XO;
     const int tco4_log2 = 29 - __clz(p.TCO), b_row = tid >> tco4_log2, b_col = 4 * (tid & (p.TCO / 4 - 1));   // TCO / 4 is a power of two
     const int b_step = nthreads >> tco4_log2, b_rows = co0 + b_col < p.CoP ? 0x7FFFFFFF : 0;
-    const uint32_t *wp_tile = p.wp + (size_t)b_row * p.CoP + co0 + b_col;
-    const float inv_nr = 1.0f / (float)NR;
-    auto fetch = [&](int ci0, int ckn, int stage) {
-        const uint32_t bar = bar0 + 8u * stage;
-        if (tid == 0) mbarrier_arrive_expect(bar, (uint32_t)ckn * NR * row_bytes);
-        const uint32_t a_dst = smem_address(smem + stage * p.a_words);
-        const uint32_t *a_src = ap_tile + ci0 * ap_plane;
+    const uint32_t *a_next = p.ap + (size_t)r0 * p.XBT + seg * p.XO + (p.NSEG == 1 ? warp * ap_plane : 0);   // of the stage to fetch next
+    const uint32_t *b_next = p.wp + (size_t)b_row * p.CoP + co0 + b_col;
+    const size_t a_stage = p.CK * ap_plane, b_stage = (size_t)p.CK * KJ * p.CoP;
+    const uint32_t a_dst0 = smem_address(smem), b_dst0 = smem_address(Bs + b_row * kStripBPitch + b_col);
+    auto fetch = [&](int ckn, int stage) {
+        const uint32_t bar = bar0 + 8u * stage, a_dst = a_dst0 + 4u * stage * p.a_words;
+        if (tid == 0) mbarrier_arrive_expect(bar, ckn * ch_bytes);
         if (p.NSEG == 1) {
-            for (int c = warp; c < ckn; c += nwarps)
-                if (lane == 0) bulk_copy(a_dst + c * (4 * kPlaneWords), a_src + c * ap_plane, NR * row_bytes, bar);
+            if (lane == 0) {
+                if (warp < ckn) bulk_copy(a_dst + 4u * warp * p.plane, a_next, ch_bytes, bar);
+                for (int c = warp + nwarps; c < ckn; c += nwarps)
+                    bulk_copy(a_dst + 4u * c * p.plane, a_next + (size_t)(c - warp) * ap_plane, ch_bytes, bar);
+            }
         } else {
+            const float inv_nr = 1.0f / (float)NR;
             for (int q = lane * nwarps + warp; q < ckn * NR; q += nthreads) {
                 const int c = small_div(q, NR, inv_nr), r = q - c * NR;
-                bulk_copy(a_dst + c * (4 * kPlaneWords) + r * row_bytes, a_src + c * ap_plane + (size_t)r * p.XBT, row_bytes, bar);
+                bulk_copy(a_dst + 4u * c * p.plane + r * row_bytes, a_next + c * ap_plane + (size_t)r * p.XBT, row_bytes, bar);
             }
         }
-        const uint32_t *b_src = wp_tile + (size_t)ci0 * KJ * p.CoP;
-        uint32_t *b_dst = Bs + stage * p.b_words + b_row * kBPitch + b_col;
         const int rows = min(ckn * KJ, b_rows);
-        for (int k = b_row; k < rows; k += b_step, b_src += (size_t)b_step * p.CoP, b_dst += b_step * kBPitch) cp_async_16(b_dst, b_src);
+        const uint32_t b_dst = b_dst0 + 4u * stage * p.b_words;
+        if (b_row < rows) cp_async_16_at(b_dst, b_next);
+        for (int k = b_row + b_step, n = 1; k < rows; k += b_step, ++n)
+            cp_async_16_at(b_dst + n * (4u * kStripBPitch) * b_step, b_next + (size_t)(n * b_step) * p.CoP);
         cp_async_commit();
+        a_next += a_stage;
+        b_next += b_stage;
     };
     if (tid == 0) {
         mbarrier_init(bar0, 1);
@@ -144,17 +155,17 @@ __global__ void __launch_bounds__(kStripThreads, 2) conv2d_strip_kernel(const __
     }
     __syncthreads();
     grid_dependency_wait();                                    // everything above touched no global memory
-    fetch(0, min(p.CK, p.Ci), 0);
+    fetch(min(p.CK, p.Ci), 0);
 
-    // one input channel: K rows of J words from the row pointers ap and the kernel words at bp
-    const uint32_t *ap[ROWS], *bp;
-    auto channel = [&]() {
+    // one input channel: activations from word a_ch of shared memory on, kernel words from word b_ch on (the same for the CTA)
+    const int b_tn = tn * TN;
+    auto channel = [&](int a_ch, int b_ch) {
         if constexpr (KT > 0) {
             uint32_t a[ROWS][JT];
 #pragma unroll
             for (int r = 0; r < ROWS; ++r)
 #pragma unroll
-                for (int j = 0; j < JT; ++j) a[r][j] = ap[r][-j];
+                for (int j = 0; j < JT; ++j) a[r][j] = smem[a_ch + a_off[r] - j];
 #pragma unroll
             for (int kh = 0; kh < KT; ++kh)
 #pragma unroll
@@ -162,55 +173,50 @@ __global__ void __launch_bounds__(kStripThreads, 2) conv2d_strip_kernel(const __
                     uint32_t b[TN];
 #pragma unroll
                     for (int t = 0; t < TN; t += 4) {
-                        const uint4 v = *reinterpret_cast<const uint4 *>(bp + (kh * JT + j) * kBPitch + t);
+                        const uint4 v = *reinterpret_cast<const uint4 *>(smem + b_ch + b_tn + (kh * JT + j) * kStripBPitch + t);
                         b[t] = v.x; b[t + 1] = v.y; b[t + 2] = v.z; b[t + 3] = v.w;
                     }
 #pragma unroll
                     for (int i = 0; i < TM; ++i)
 #pragma unroll
-                        for (int t = 0; t < TN; ++t) packed_mac<SP>(acc[i][t], a[i + kh][j], b[t]);
+                        for (int t = 0; t < TN; ++t) mad_wide<SP>(acc[i][t], a[i + kh][j], b[t]);
                 }
-            bp += KT * JT * kBPitch;
         } else {
             for (int kh = 0; kh < K; ++kh)
-                for (int j = 0; j < J; ++j, bp += kBPitch) {
+                for (int j = 0; j < J; ++j, b_ch += kStripBPitch) {
                     uint32_t a[TM], b[TN];
 #pragma unroll
-                    for (int i = 0; i < TM; ++i) a[i] = ap[i][kh * p.pitch - j];
+                    for (int i = 0; i < TM; ++i) a[i] = smem[a_ch + a_off[i] + kh * p.pitch - j];
 #pragma unroll
                     for (int t = 0; t < TN; t += 4) {
-                        const uint4 v = *reinterpret_cast<const uint4 *>(bp + t);
+                        const uint4 v = *reinterpret_cast<const uint4 *>(smem + b_ch + b_tn + t);
                         b[t] = v.x; b[t + 1] = v.y; b[t + 2] = v.z; b[t + 3] = v.w;
                     }
 #pragma unroll
                     for (int i = 0; i < TM; ++i)
 #pragma unroll
-                        for (int t = 0; t < TN; ++t) packed_mac<SP>(acc[i][t], a[i], b[t]);
+                        for (int t = 0; t < TN; ++t) mad_wide<SP>(acc[i][t], a[i], b[t]);
                 }
         }
-#pragma unroll
-        for (int r = 0; r < ROWS; ++r) ap[r] += kPlaneWords;
     };
     // a run of input channels between two possible moves: the whole stage, or CF channels of it
     const int run = HASE ? p.run : p.CK;
     int moves = 0, runs_left = p.runs_per_move;
-    uint32_t phase = 0;                                        // parity of stage buffer s in bit s
+    uint32_t parity = 0;                                       // of this stage's barrier; both buffers' barriers flip every second stage
     int stage = 0;
     for (int ci0 = 0; ci0 < p.Ci; ci0 += p.CK, stage ^= 1) {
         const int ckn = min(p.CK, p.Ci - ci0);
         // this stage has landed (were the wait ever to run out, the sums would be wrong but nothing would hang)
-        mbarrier_wait(bar0 + 8u * stage, (phase >> stage) & 1u);
+        mbarrier_wait(bar0 + 8u * stage, parity);
         cp_async_wait_all();
-        phase ^= 1u << stage;
+        parity ^= (uint32_t)stage;
         __syncthreads();                                       // the previous stage is fully consumed
-        if (ci0 + p.CK < p.Ci) fetch(ci0 + p.CK, min(p.CK, p.Ci - ci0 - p.CK), stage ^ 1);
-#pragma unroll
-        for (int r = 0; r < ROWS; ++r) ap[r] = a0 + stage * p.a_words + r * p.pitch;
-        bp = Bs + stage * p.b_words + tn * TN;
+        if (ci0 + p.CK < p.Ci) fetch(min(p.CK, p.Ci - ci0 - p.CK), stage ^ 1);
+        int a_ch = stage * p.a_words, b_ch = p.b_off + stage * p.b_words;
         for (int c = 0; c < ckn; c += run) {
             const int n = HASE ? min(run, ckn - c) : ckn;
 #pragma unroll 2
-            for (int u = 0; u < n; ++u) channel();
+            for (int u = 0; u < n; ++u, a_ch += p.plane, b_ch += KJ * kStripBPitch) channel(a_ch, b_ch);
             if constexpr (HASE) {
                 if (--runs_left == 0 && ci0 + c + n < p.Ci) {  // none is needed after the last channel
                     move_upper_bits();
@@ -221,6 +227,10 @@ __global__ void __launch_bounds__(kStripThreads, 2) conv2d_strip_kernel(const __
         }
     }
 
+    auto second = [&](int i, int t) -> uint64_t {
+        const uint2 e = es[i * TN + t];
+        return ((uint64_t)e.y << 32) | e.x;
+    };
     // ---- words above the N low slots: to the next lane by shuffle, across warps through shared memory
     uint2 *xch = reinterpret_cast<uint2 *>(smem) + ((warp << tnx_log2) + tn) * (TM * TN);
     const int lanes_m = 32 >> tnx_log2, lm = lane >> tnx_log2;
@@ -230,8 +240,7 @@ __global__ void __launch_bounds__(kStripThreads, 2) conv2d_strip_kernel(const __
         for (int i = 0; i < TM; ++i)
 #pragma unroll
             for (int t = 0; t < TN; ++t)
-                xch[i * TN + t] = make_uint2((uint32_t)(acc[i][t] >> p.SN),
-                                             HASE ? (uint32_t)((((uint64_t)e_hi[HASE ? i : 0][t] << 32) | e_lo[HASE ? i : 0][t]) >> p.SN) : 0u);
+                xch[i * TN + t] = make_uint2((uint32_t)(acc[i][t] >> p.SN), HASE ? (uint32_t)(second(i, t) >> p.SN) : 0u);
     }
     __syncthreads();
     const uint2 *xch_in = xch - p.TNX * (TM * TN);
@@ -256,7 +265,7 @@ __global__ void __launch_bounds__(kStripThreads, 2) conv2d_strip_kernel(const __
         uint64_t q = acc[i][t];
         uint32_t q_in = 0, e_in = 0, qf[N], ef[N];
         uint64_t e = 0;
-        if constexpr (HASE) e = ((uint64_t)e_hi[i][t] << 32) | e_lo[i][t];
+        if constexpr (HASE) e = second(i, t);
         if constexpr (UP) {
             q_in = __shfl_up_sync(0xFFFFFFFFu, (uint32_t)(q >> p.SN), p.TNX);
             if constexpr (HASE) e_in = __shfl_up_sync(0xFFFFFFFFu, (uint32_t)(e >> p.SN), p.TNX);
@@ -425,23 +434,23 @@ __global__ void __launch_bounds__(kStripThreads, 2) conv2d_strip_kernel(const __
     }
 }
 
-template <int N, int KT, int JT, int TM, int TN, bool HASE>
+template <int N, int KT, int JT, int TM, int TN>
 static int launch_strip_tile(const StripLaunch &s, cudaStream_t st) {
     auto run = [&](auto kern) -> int {
         if (s.smem_bytes > 48 * 1024)
             HIKONV_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem_bytes));
         return launch_dependent(kern, s.grid, dim3(s.threads), s.smem_bytes, st, s.p);
     };
-    return s.sp ? run(conv2d_strip_kernel<N, KT, JT, TM, TN, true, HASE>) : run(conv2d_strip_kernel<N, KT, JT, TM, TN, false, HASE>);
+    if (s.moves) return s.sp ? run(conv2d_strip_kernel<N, KT, JT, TM, TN, true, true>) : run(conv2d_strip_kernel<N, KT, JT, TM, TN, false, true>);
+    return s.sp ? run(conv2d_strip_kernel<N, KT, JT, TM, TN, true, false>) : run(conv2d_strip_kernel<N, KT, JT, TM, TN, false, false>);
 }
 
 template <int N, int KT, int JT>
-static int launch_strip(const StripLaunch &s, cudaStream_t st) {
-    if (s.TM == 4 && s.TN == 4) return s.moves ? launch_strip_tile<N, KT, JT, 4, 4, true>(s, st) : launch_strip_tile<N, KT, JT, 4, 4, false>(s, st);
+int launch_strip(const StripLaunch &s, cudaStream_t st) {
+    if (s.TM == 2 && s.TN == 4) return launch_strip_tile<N, KT, JT, 2, 4>(s, st);
     if constexpr (KT > 0) {
-        if (s.TM == 2 && s.TN == 8) return s.moves ? launch_strip_tile<N, KT, JT, 2, 8, true>(s, st) : launch_strip_tile<N, KT, JT, 2, 8, false>(s, st);
-        if (s.TM == 2 && s.TN == 4) return s.moves ? launch_strip_tile<N, KT, JT, 2, 4, true>(s, st) : launch_strip_tile<N, KT, JT, 2, 4, false>(s, st);
-        if (s.TM == 4 && s.TN == 8 && !s.moves) return launch_strip_tile<N, KT, JT, 4, 8, false>(s, st);
+        if (s.TM == 2 && s.TN == 8) return launch_strip_tile<N, KT, JT, 2, 8>(s, st);
+        if (s.TM == 4 && s.TN == 8) return launch_strip_tile<N, KT, JT, 4, 8>(s, st);
     }
     return HIKONV_ERR_UNSUPPORTED;
 }

@@ -1,5 +1,5 @@
 // Interface between hikonv_conv2d.cu (planning, packing launch, entry points) and the packed layer kernel
-// (hikonv_conv2d_strip.cuh, instantiated per number of pixels in a word by hikonv_conv2d_strip_n*.cu).
+// (hikonv_conv2d_strip.cuh, instantiated per layout by hikonv_conv2d_strip_*.cu: pixels per word, kernel size, words per row).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -9,7 +9,8 @@
 namespace hikonv {
 
 constexpr int kStripThreads = 256;   // most threads of a CTA
-constexpr int kPlaneWords = 1280;    // words between the channels of a staged activation tile (a constant: see the kernel)
+constexpr int kStripBPitch = 32;     // words per packed kernel row in shared memory (TCO or more)
+constexpr int kStripMaxCK = 16;      // most input channels of a stage
 
 struct StripParams {
     const uint32_t *ap;              // packed activations [Ci][B * Hp][XBT]
@@ -23,8 +24,9 @@ struct StripParams {
     int pitch;                       // words per staged activation row (XB + J - 1 rounded up to a multiple of 4)
     int TS, TNX, TCO, CK;            // strips and channel lanes per CTA, channels per CTA, input channels per stage
     int run, runs_per_move;          // input channels between two possible moves (CK or less), such runs between two moves
+    int plane;                       // words between two channels of a staged activation tile
     int a_words, b_off, b_words;     // words per staged activation tile, offset of the first weight tile, words per weight tile
-    int bar_off;                     // word offset of the two mbarriers
+    int bar_off, e_off;              // word offsets of the two mbarriers and of the second accumulators
     uint32_t mg_xb, mg_sh;           // fast_div() multipliers: XB, SH
     // slots: S bits each; every slot starts at bias and moves its bits above the low h to a second accumulator
     int S, SN, h;                    // slot width, S N, h
@@ -50,12 +52,13 @@ struct StripLaunch {
     bool generic;                    // the kernel with run-time loop bounds
 };
 
-// Thread tiles the kernel is built for: 4 x 4, 2 x 8, 2 x 4 rows x channels, and 4 x 8 without second accumulators.
-inline bool strip_tile_built(int TM, int TN, bool moves, bool generic) {
-    if (TM == 4 && TN == 4) return true;
-    if (generic) return false;
-    return (TM == 2 && (TN == 8 || TN == 4)) || (TM == 4 && TN == 8 && !moves);
+// Thread tiles the kernel is built for: 4 x 8, 2 x 8 and 2 x 4 rows x channels (2 x 4 with run-time loop bounds).  4 x 4 was as
+// fast as 2 x 8 on no layer.
+inline bool strip_tile_built(int TM, int TN, bool generic) {
+    return generic ? (TM == 2 && TN == 4) : ((TM == 2 && (TN == 4 || TN == 8)) || (TM == 4 && TN == 8));
 }
+// 8-byte entries of a thread in the second-accumulator area: TM TN and one that keeps the pitch odd.
+__host__ __device__ constexpr int strip_e_pitch(int TM, int TN) { return TM * TN + 1; }
 // Is there a kernel with unrolled loops for (N, K, J), and does it add the upper slots to the next word while packed?
 inline bool strip_unrolled(int N, int K, int J) {
     if (K == 1) return J == 1 && N >= 2 && N <= 4;
@@ -67,9 +70,8 @@ constexpr bool strip_packed_add(int N, int K, int J) {
     return K > 0 && !(J == 1 && K == N + 1) && !(N == 4 && K == 5);
 }
 
-int launch_strip_n1(const StripLaunch &s, cudaStream_t st);
-int launch_strip_n2(const StripLaunch &s, cudaStream_t st);
-int launch_strip_n3(const StripLaunch &s, cudaStream_t st);
-int launch_strip_n4(const StripLaunch &s, cudaStream_t st);
+// Explicitly instantiated, one layout per file: (N, 0, 0) with run-time bounds, (N, K, J) for strip_unrolled ones.
+template <int N, int KT, int JT>
+int launch_strip(const StripLaunch &s, cudaStream_t st);
 
 }  // namespace hikonv

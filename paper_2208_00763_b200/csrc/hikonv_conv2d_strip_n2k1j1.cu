@@ -1,0 +1,8 @@
+// The packed layer kernel for 2 pixels per word, 1x1 kernels, one word per kernel row.
+#include "hikonv_conv2d_strip.cuh"
+
+namespace hikonv {
+
+template int launch_strip<2, 1, 1>(const StripLaunch &s, cudaStream_t st);
+
+}  // namespace hikonv
