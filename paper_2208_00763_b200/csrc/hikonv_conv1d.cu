@@ -10,9 +10,10 @@
 //   splits  y[xN+m] = ((D_x >> S m) & mask) - carry_bias[m],  m < N       (Algorithm 2's shift
 //           and mask; the per-slot bias replaces the sign-borrow increment of Eq. 29)
 // Outputs are staged per warp in shared memory and written with coalesced 16-byte stores.
-// This file holds the argument checks, the layout choice and the general (any N, J, K) kernels; the
+// This file holds the argument checks, the layout choice and the general (any N, J, K) kernels, which run where the layout has
+// no kernel of its own or the caller asks for them; the
 // register-resident kernels of the packed method and of the two comparators are in hikonv_conv1d_tc.cu,
-// the variant on an emulated 64x64 multiplier in hikonv_conv1d_emu64.cu.
+// the kernel for long filters in hikonv_conv1d_long.cu, the variant on an emulated 64x64 multiplier in hikonv_conv1d_emu64.cu.
 #include <cstring>
 
 #include "hikonv_cuda.cuh"
@@ -381,14 +382,17 @@ extern "C" int hikonv_conv1d(const int8_t *d_f, size_t len, const int8_t *d_g, i
     if (L.N > kMaxN1D) return HIKONV_ERR_UNSUPPORTED;
     const SplitConsts sc = make_split_consts(L, p, q, f_signed, g_signed, K, 1);
 
-    if (want_tc && conv1d_packed_tc_available(L.N, L.J)) {
-        const int per_tile = conv1d_tc_outputs_per_tile(L.N);
-        tp.n_tiles = (n_out + per_tile - 1) / per_tile;
-        tp.S = L.S; tp.Kc = L.Kc; tp.hi_shift = L.S * L.N; tp.mask = sc.slot_mask; tp.bias = sc.bias;
+    // register-resident kernels where they are built for the layout; beyond, the kernel for long filters
+    const bool tc = conv1d_packed_tc_available(L.N, L.J);
+    if (want_tc && (tc || conv1d_long_available(L.N))) {
+        tp.S = L.S; tp.Kc = L.Kc; tp.J = L.J; tp.hi_shift = L.S * L.N; tp.mask = sc.slot_mask; tp.bias = sc.bias;
         for (int m = 0; m < kMaxN1D; ++m) {
             tp.seg_shift[m] = m < L.N ? L.S * m : 0;
             tp.carry_bias[m] = m < L.N ? sc.carry_bias[m] : 0;
         }
+        if (!tc) return launch_conv1d_long(tp, L.N, L.signed_prod != 0, f_signed != 0, st);
+        const int per_tile = conv1d_tc_outputs_per_tile(L.N);
+        tp.n_tiles = (n_out + per_tile - 1) / per_tile;
         return launch_conv1d_packed_tc(tp, L.N, L.J, L.signed_prod != 0, f_signed != 0, st);
     }
 

@@ -66,6 +66,38 @@ def test_extreme_codes(signed, algo):
                              "extreme p=%d K=%d signed=%d" % (bits, K, signed))
 
 
+@pytest.mark.parametrize("K", [9, 13, 16, 24, 31, 32])
+def test_long_filters(K):
+    # kernels cut into more chunks than the register-resident kernels take: every width and sign, lengths around a tile of
+    # 256 threads x R blocks, extreme codes, buffers off their alignment, and every block size the kernel is built for
+    rng = np.random.default_rng(600 + K)
+    run = {1: 15, 2: 11, 3: 7, 4: 7, 5: 5, 6: 3, 7: 3, 8: 3}
+    for p in range(1, 9):
+        for fs, gs in ((False, False), (True, True), (False, True), (True, False)):
+            L = hk.conv1d_layout(p, 4, fs, gs, K)
+            per_tile = 256 * run.get(L["N"], 3) * L["N"]
+            g = inputs.uniform_codes(rng, (K,), 4, gs)
+            for n in (K, per_tile - K + 1, per_tile - K + 2, 2 * per_tile + 5):
+                f = inputs.uniform_codes(rng, (n,), p, fs)
+                assert_exact(_run(f, g, p, 4, fs, gs, hk.ALGO_PACKED32), direct.conv1d_full(f, g), "p=%d fs=%d gs=%d n=%d" % (p, fs, gs, n))
+    for f, g in inputs.extreme_1d(6001, K, 4, 4, True, True):
+        assert_exact(_run(f, g, 4, 4, True, True, hk.ALGO_PACKED32), direct.conv1d_full(f, g), "extreme")
+    f, g = inputs.uniform_codes(rng, (9001,), 4, False), inputs.uniform_codes(rng, (K,), 4, True)
+    ref, buf, y = direct.conv1d_full(f, g), torch.zeros(9016, dtype=torch.int8, device="cuda"), torch.zeros(9100, dtype=torch.int32, device="cuda")
+    for off_f, off_y in ((1, 0), (4, 1), (2, 3)):
+        buf[off_f:off_f + 9001] = dev(f)
+        got = hk.conv1d(buf[off_f:off_f + 9001], dev(g), 4, 4, False, True, out=y[off_y:off_y + 9001 + K - 1])
+        assert_exact(got, ref, "offsets %d %d" % (off_f, off_y))
+    for n_forced in range(1, 9):
+        f, g = inputs.uniform_codes(rng, (20011,), 1, False), inputs.uniform_codes(rng, (K,), 1, False)
+        try:
+            got = _run(f, g, 1, 1, False, False, hk.ALGO_PACKED32, {"N": n_forced})
+        except hk.HikonvError as err:                # more chunks than an operand allows
+            assert err.status == hk.ERR_NO_FIT
+            continue
+        assert_exact(got, direct.conv1d_full(f, g), "N=%d" % n_forced)
+
+
 @pytest.mark.parametrize("algo", ALGOS)
 def test_mixed_signedness_and_widths(algo):
     rng = np.random.default_rng(5)
