@@ -27,12 +27,6 @@
 
 namespace hikonv {
 
-__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
-    uint32_t r;
-    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(sel));
-    return r;
-}
-
 // MODE 1 (S = 8): the N = 4 outputs of every block x = 0 .. R-1 from the loaded words.
 template <int J, bool FS, bool SP, int L, int NW>
 __device__ __forceinline__ void compute_s8(const Conv1dBsParams &p, const uint32_t (&Bw)[J], uint64_t init, const uint32_t (&w)[NW],
@@ -54,7 +48,7 @@ __device__ __forceinline__ void compute_s8(const Conv1dBsParams &p, const uint32
             if (SP) D ^= BIAS;
 #pragma unroll
             for (int m = 0; m < 4; ++m)
-                out[4 * x + m] = (int32_t)prmt(D, 0u, SP ? (uint32_t)(m | ((8 | m) * 0x1110)) : (uint32_t)(m | 0x4440));
+                out[4 * x + m] = (int32_t)byte_permute(D, 0u, SP ? (uint32_t)(m | ((8 | m) * 0x1110)) : (uint32_t)(m | 0x4440));
         }
         carry = (uint32_t)(Q >> 32);
     }
@@ -75,10 +69,10 @@ __device__ __forceinline__ void compute_n2(int S, uint32_t mask3, int32_t half3,
     for (int x = -J; x < R; ++x) {
         const int pos = FRONT + 2 * x;
         if constexpr (MODE == 2) {
-            A[x + J] = prmt(s[pos / 4], 0u, pos % 4 == 0 ? 0x4140u : 0x4342u);
+            A[x + J] = byte_permute(s[pos / 4], 0u, pos % 4 == 0 ? 0x4140u : 0x4342u);
         } else {
-            const uint32_t c0 = prmt(s[pos / 4], 0u, pos % 4 == 0 ? 0x4440u : 0x4442u);
-            const uint32_t c1 = prmt(s[pos / 4], 0u, pos % 4 == 0 ? 0x4441u : 0x4443u);
+            const uint32_t c0 = byte_permute(s[pos / 4], 0u, pos % 4 == 0 ? 0x4440u : 0x4442u);
+            const uint32_t c1 = byte_permute(s[pos / 4], 0u, pos % 4 == 0 ? 0x4441u : 0x4443u);
             A[x + J] = c0 + (c1 << S);
         }
     }
@@ -92,8 +86,8 @@ __device__ __forceinline__ void compute_n2(int S, uint32_t mask3, int32_t half3,
             if (x >= 0) {
                 uint32_t D = (uint32_t)Q + carry;
                 if (SP) D ^= BIAS;
-                out[2 * x] = (int32_t)prmt(D, 0u, SP ? 0x9910u : 0x4410u);
-                out[2 * x + 1] = (int32_t)prmt(D, 0u, SP ? 0xBB32u : 0x4432u);
+                out[2 * x] = (int32_t)byte_permute(D, 0u, SP ? 0x9910u : 0x4410u);
+                out[2 * x + 1] = (int32_t)byte_permute(D, 0u, SP ? 0xBB32u : 0x4432u);
             }
             carry = (uint32_t)(Q >> 32);
         }

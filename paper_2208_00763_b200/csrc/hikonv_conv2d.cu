@@ -13,6 +13,7 @@
 
 #include "hikonv_cuda.cuh"
 #include "hikonv_conv2d_output.h"
+#include "hikonv_conv2d_small.h"
 #include "hikonv_conv2d_strip.h"
 #include "hikonv_conv2d_unpacked.h"
 #include "hikonv_conv2d_util.cuh"
@@ -130,14 +131,6 @@ struct ActPackDivs {
     Div32 per_plane, b, xq;    // pieces per (ci, b) plane, images, 16-byte pieces per packed row
 };
 
-// Byte mask of the bytes of word i (bytes 4 i .. 4 i + 3) whose index lies in [first, last).
-__device__ __forceinline__ uint32_t byte_range_mask(int i, int first, int last) {
-    const int lo = max(first - 4 * i, 0), n = max(last - 4 * i - lo, 0);
-    uint32_t m;
-    asm("bmsk.clamp.b32 %0, %1, %2;" : "=r"(m) : "r"(8 * lo), "r"(8 * n));      // 8 n bits from bit 8 lo on, clamped to the word
-    return m;
-}
-
 template <bool XS, int N>
 __global__ void __launch_bounds__(256) pack_operands_kernel(const int8_t *__restrict__ x, int B, int Ci, int H, int W, int Hp,
                                                             int pad, int col_first, int S, int XBT,
@@ -168,31 +161,7 @@ __global__ void __launch_bounds__(256) pack_operands_kernel(const int8_t *__rest
     if ((row_in || wq.x_off != 0) && col0 + 4 * N > 0 && col0 < W) {
         const size_t row_e = (((size_t)b * Ci + ci) * H + (row_in ? hi : 0)) * W;   // first code of the input row
         if (x_bits == 8) {
-            const int8_t *src = x + row_e + col0;                    // not dereferenced outside the row
-            const int off = (int)((uintptr_t)src & 3);
-            const uint32_t *al = reinterpret_cast<const uint32_t *>(src - off);
-            // aligned word i holds the codes of columns col0 - off + 4 i .. + 3: loaded when one of them is in the row
-            uint32_t v[N + 1];
-#pragma unroll
-            for (int i = 0; i <= N; ++i) {
-                const int c = col0 - off + 4 * i;
-                v[i] = (row_in && c + 3 >= 0 && c < W) ? __ldg(al + i) : 0u;
-            }
-            const uint32_t off4 = (uint32_t)wq.x_off * 0x01010101u;
-#pragma unroll
-            for (int i = 0; i < N; ++i) {
-                v[i] = __funnelshift_r(v[i], v[i + 1], 8 * off);
-                if (wq.x_off != 0) v[i] = __vsub4(v[i], off4);
-                v[i] &= byte_range_mask(i, -col0, W - col0);
-            }
-            const uint32_t step = 1u << S;
-#pragma unroll
-            for (int w = 0; w < 4; ++w) {
-                uint32_t a = extract_code<XS>(v[(w * N + N - 1) / 4], (w * N + N - 1) % 4);
-#pragma unroll
-                for (int n = N - 2; n >= 0; --n) a = a * step + extract_code<XS>(v[(w * N + n) / 4], (w * N + n) % 4);
-                word[w] = a;
-            }
+            pack_row_words<N>(x + row_e, W, col0, row_in, (uint32_t)wq.x_off * 0x01010101u, XS, S, word);
         } else {
 #pragma unroll
             for (int w = 0; w < 4; ++w)
@@ -263,6 +232,8 @@ __global__ void __launch_bounds__(256) maxpool2x2_kernel(const int8_t *__restric
 struct Conv2dSetup {
     hikonv_layout_t L;
     bool unpacked;
+    bool one_launch;      // the kernel for small layers, which packs its operands itself
+    SmallLaunch small;
     StripLaunch strip;    // the packed kernel, or
     UnpackedLaunch un;    // the comparator
     // packed operands in the workspace: weights [Ci K J][CoP], x_off corrections [K + 1][CoP], activations [Ci][B Hp][XBT]
@@ -432,6 +403,61 @@ static StripChoice choose_strips(const StripProblem &q, int force_tm, int force_
     return best;
 }
 
+// The one-launch kernel for small layers: its tile and cut of the input channels, and the modelled cycles of the call.
+struct SmallChoice {
+    int TNX, TS, ks_log2, Cz, rows, XB, pitch, threads;
+    size_t words;
+    long long ctas;
+    double cost;
+};
+
+static SmallChoice choose_small(const StripProblem &q) {
+    SmallChoice best;
+    std::memset(&best, 0, sizeof(best));
+    best.cost = -1.0;
+    constexpr int TM = kSmallTM, TN = kSmallTN;
+    const int SH = ceil_div(q.Ho, TM), Hp = q.Ho + q.K - 1, KJ = q.K * q.J;
+    const long long strips = (long long)q.B * SH;
+    SmallChoice c;
+    c.XB = ceil_div(q.Wo + q.K - 1 - q.pad, q.N);
+    c.pitch = (c.XB + q.J - 1 + 3) / 4 * 4;
+    // not worth looking at beyond a few million multiplies per SM
+    if ((double)strips * c.XB * q.Co * q.Ci * KJ * TM > 3.0e6 * q.sms) return best;
+    for (c.TNX = 1; c.TNX <= 8; c.TNX *= 2) {
+        const int TCO = c.TNX * TN;
+        if (c.TNX > 1 && TCO / 2 >= q.Co) break;
+        for (c.TS = 1; c.TS * c.XB * c.TNX <= kStripThreads && c.TS <= strips; ++c.TS) {
+            c.threads = (c.TS * c.XB * c.TNX + 31) / 32 * 32;
+            c.rows = staged_rows(c.TS, TM, SH, Hp, q.K);
+            const int warps = c.threads / 32, per_sched = ceil_div(warps, 4);
+            const long long tiles = (strips + c.TS - 1) / c.TS * ceil_div(q.Co, TCO);
+            for (c.ks_log2 = 0; c.ks_log2 <= (q.pool ? 2 : 3); ++c.ks_log2) {
+                const int ks = 1 << c.ks_log2;
+                if (ks > q.Ci) break;
+                c.Cz = ceil_div(q.Ci, ks);
+                c.ctas = tiles * ks;
+                const double a_items = (double)c.Cz * c.rows * (c.pitch / 4), b_items = (double)c.Cz * KJ * TCO;
+                if (a_items >= 65536.0) continue;
+                const size_t stage = (size_t)c.Cz * ((size_t)c.rows * c.pitch + KJ * kStripBPitch);
+                const size_t xch = (size_t)warps * c.TNX * TM * TN * 2, red = ks > 1 ? (size_t)c.threads * TM * TN * q.N : 0;
+                const size_t tile = q.pool ? (size_t)TCO * c.TS * ((c.XB * q.N + 15) / 16 * 16) / 4 : 0;
+                c.words = (std::max(stage, xch + red + tile) + 3) / 4 * 4;
+                if (c.words * 4 > (size_t)(kSmemPerCta - 1024)) continue;
+                const int resident = std::max(1, std::min(std::min(65536 / (c.threads * 128), (int)(kSmemPerSm / (c.words * 4 + 1024))), 32));
+                const long long share = (c.ctas + q.sms - 1) / q.sms;
+                const double waves = std::ceil((double)share / resident), at_once = (double)std::min<long long>(share, resident) * per_sched;
+                const double mul = 4.3 * TM * TN * KJ;
+                const double pack = (std::ceil(a_items / c.threads) * 75 + std::ceil(b_items / c.threads) * (25 + 8 * q.K)) * at_once + 1800;
+                const double mults = c.Cz * std::max(at_once * (mul + 30 + (q.moves ? 80.0 / q.CF : 0)), mul + 120 + (q.moves ? 200.0 / q.CF : 0));
+                const double split = at_once * TM * TN * 14 * q.N + 500 + (ks > 1 ? 2000 + 60.0 * ks : 0);
+                c.cost = 4000 + waves * (pack + mults + split);
+                if (best.cost < 0 || c.cost < best.cost) best = c;
+            }
+        }
+    }
+    return best;
+}
+
 static int plan_layer(int B, int Ci, int H, int W, int Co, int K, int stride, int pad, int p, int q, int xs, int ws,
                       const OutputSpec &out, int algo, const hikonv_tuning_t *tune, Conv2dSetup *s) {
     if (B < 1 || Ci < 1 || H < 1 || W < 1 || Co < 1 || K < 1 || K > kMaxK) return HIKONV_ERR_INVALID_ARG;
@@ -452,6 +478,7 @@ static int plan_layer(int B, int Ci, int H, int W, int Co, int K, int stride, in
     s->CoP = (Co + 3) / 4 * 4;
     s->Hp = Ho + K - 1;
     s->x_off = 0;
+    s->one_launch = false;
     hikonv_layout_t &L = s->L;
     if (s->unpacked) {
         std::memset(&L, 0, sizeof(L));
@@ -542,6 +569,43 @@ static int plan_layer(int B, int Ci, int H, int W, int Co, int K, int stride, in
         l.smem_bytes = c.smem;
         const long long share = (c.ctas + pr.sms - 1) / pr.sms;
         if (share <= 4) l.smem_bytes = std::max(c.smem, (size_t)(kSmemPerSm / (share + 1) - 1024 + 256));
+
+        // one launch instead of two, where it is modelled to be faster (tune->tile == -1: never, -2: always)
+        const bool force_small = tune && tune->tile == -2;
+        if (!pr.generic && s->x_off == 0 && out.byte_inputs && out.out_bits == 8 && tile_arg == 0 && !(tune && tune->tile == -1)) {
+            const SmallChoice sm = choose_small(pr);
+            // both models brought to measured times on 59 layers (3 to 122 channels, 1 to 64 images, every layout): they leave out
+            // latencies of a few thousand cycles, and the packing launch takes 2.3 us and 12 us per million 16-byte pieces.  The
+            // one launch measured faster below about 10 us (10x20x64, one image: 7.4 against 16.8 us; 16 images: 14.6 against
+            // 15.4; 64 images: 23.4 against 18.1)
+            const double two = 4500 + 1.3 * c.cost + 0.024 * Ci * B * s->Hp * (k.XBT / 4);
+            const double one = sm.cost + 0.9 * std::max(0.0, sm.cost - 9800);
+            if (sm.cost >= 0 && (one < two || force_small)) {
+                s->one_launch = true;
+                SmallLaunch &ml = s->small;
+                SmallParams &mp = ml.p;
+                std::memset(&mp, 0, sizeof(mp));
+                mp.s = k;
+                StripParams &ms = mp.s;
+                ms.SH = ceil_div(Ho, kSmallTM); ms.strips = B * ms.SH;
+                ms.NSEG = 1; ms.XO = ms.XB = ms.X = sm.XB; ms.halo = 0; ms.col_off = K - 1 - pad; ms.pitch = sm.pitch;
+                ms.TS = sm.TS; ms.TNX = sm.TNX; ms.TCO = sm.TNX * kSmallTN;
+                ms.plane = sm.rows * sm.pitch; ms.b_off = sm.Cz * ms.plane;
+                ms.mg_xb = magic(sm.XB); ms.mg_sh = magic(ms.SH);
+                ms.WTP = (sm.XB * L.N + 15) / 16 * 16;
+                mp.B = B; mp.H = H; mp.x_signed = xs; mp.w_signed = ws; mp.Kc = L.Kc;
+                mp.Cz = sm.Cz; mp.CF = pr.moves ? pr.CF : Ci + 1; mp.ks_log2 = sm.ks_log2; mp.rows = sm.rows;
+                mp.col_first = -(L.J - 1) * L.N;
+                mp.mg_hp = magic(s->Hp); mp.mg_xq = magic(sm.pitch / 4); mp.mg_rows = magic(sm.rows);
+                mp.red_off = sm.threads / 32 * sm.TNX * kSmallTM * kSmallTN * 2;
+                ms.tile_off = mp.red_off + (sm.ks_log2 > 0 ? sm.threads * kSmallTM * kSmallTN * L.N : 0);
+                ml.threads = sm.threads; ml.sp = L.signed_prod != 0;
+                ml.smem_bytes = sm.words * 4;
+                ml.grid = dim3((unsigned)((ms.strips + sm.TS - 1) / sm.TS), (unsigned)ceil_div(Co, ms.TCO), 1u << sm.ks_log2);
+                const long long even = (sm.ctas + pr.sms - 1) / pr.sms;          // spread evenly, as above
+                if (even <= 4 && sm.ks_log2 == 0) ml.smem_bytes = std::max(ml.smem_bytes, (size_t)(kSmemPerSm / (even + 1) - 1024 + 256));
+            }
+        }
         s->XBT = k.XBT;
         s->col_first = c.halo ? K - 1 - pad - L.J * L.N : -(L.J - 1) * L.N;
         s->positions = (double)B * Ho * c.NSEG * c.XB;
@@ -566,7 +630,7 @@ static int setup_layer(int B, int Ci, int H, int W, int Co, int K, int stride, i
     static thread_local Kept kept[kKept];
     const int key[26] = {B, Ci, H, W, Co, K, stride, pad, p, q, xs, ws, out.requant, out.shift, out.lo, out.hi, out.pool, out.out_bits,
                          (int)((uintptr_t)out.d_out % 16), algo, tune ? tune->N : 0, tune ? tune->S : 0, tune ? tune->M : 0,
-                         tune ? tune->tile : 0, sm_count(), 0};
+                         tune ? tune->tile : 0, sm_count(), out.byte_inputs};
     uint32_t hash = 2166136261u;                                     // FNV-1a over the words of the key
     for (int v : key) hash = (hash ^ (uint32_t)v) * 16777619u;
     Kept &k = kept[(hash ^ (hash >> 15)) % kKept];
@@ -628,7 +692,7 @@ static int conv2d_run(const void *d_x, int x_bits, int B, int Ci, int H, int W, 
                       const hikonv_tuning_t *tune, void *stream) {
     if (!d_x || !d_w || !d_out) return HIKONV_ERR_INVALID_ARG;
     Conv2dSetup s;
-    const OutputSpec out = {requant, shift, lo, hi, pool, out_bits, d_out};
+    const OutputSpec out = {requant, shift, lo, hi, pool, out_bits, d_out, x_bits == 8 && w_bits == 8};
     int rc = setup_layer(B, Ci, H, W, Co, K, stride, pad, p, q, x_signed ? 1 : 0, w_signed ? 1 : 0, out, algo, tune, &s);
     if (rc != HIKONV_OK) return rc;
     if (!requant && ((uintptr_t)d_out % 4) != 0) return HIKONV_ERR_INVALID_ARG;
@@ -645,6 +709,10 @@ static int conv2d_run(const void *d_x, int x_bits, int B, int Ci, int H, int W, 
     } else {
         s.strip.p.wp = d_wp; s.strip.p.ap = d_ap; s.strip.p.out = d_out;
         s.strip.p.corr = s.x_off ? d_corr : nullptr;
+    }
+    if (s.one_launch) {
+        s.small.p.x = (const int8_t *)d_x; s.small.p.w = (const int8_t *)d_w; s.small.p.s.out = d_out;
+        return launch_small(s.small, s.L.N, st);
     }
     // a2: reversed kernel rows packed per (ci, kh, chunk); a3: activation rows packed per block; one launch
     {
@@ -913,7 +981,7 @@ extern "C" int hikonv_conv2d_layout(int B, int Ci, int H, int W, int Co, int K, 
                                     int w_signed, const hikonv_tuning_t *tune, hikonv_layout_t *out, int *x_shift) {
     if (!out) return HIKONV_ERR_INVALID_ARG;
     Conv2dSetup s;
-    const OutputSpec sums = {0, 0, 0, 0, 0, 8, nullptr};
+    const OutputSpec sums = {0, 0, 0, 0, 0, 8, nullptr, 0};
     const int rc = setup_layer(B, Ci, H, W, Co, K, 1, pad, p, q, x_signed ? 1 : 0, w_signed ? 1 : 0, sums, HIKONV_ALGO_PACKED32, tune, &s);
     if (rc != HIKONV_OK) return rc;
     *out = s.L;
@@ -924,7 +992,7 @@ extern "C" int hikonv_conv2d_layout(int B, int Ci, int H, int W, int Co, int K, 
 extern "C" double hikonv_conv2d_multiplies(int B, int Ci, int H, int W, int Co, int K, int pad, int p, int q, int x_signed,
                                            int w_signed, int algo, const hikonv_tuning_t *tune) {
     Conv2dSetup s;
-    const OutputSpec sums = {0, 0, 0, 0, 0, 8, nullptr};
+    const OutputSpec sums = {0, 0, 0, 0, 0, 8, nullptr, 0};
     if (setup_layer(B, Ci, H, W, Co, K, 1, pad, p, q, x_signed ? 1 : 0, w_signed ? 1 : 0, sums, algo, tune, &s) != HIKONV_OK) return 0.0;
     // one multiply per position, channel pair and (kh, j): halo positions included, idle threads not
     return s.positions * (double)Co * Ci * K * s.L.J;

@@ -437,9 +437,8 @@ __global__ void __launch_bounds__(kStripThreads, 2) conv2d_strip_kernel(const __
 template <int N, int KT, int JT, int TM, int TN>
 static int launch_strip_tile(const StripLaunch &s, cudaStream_t st) {
     auto run = [&](auto kern) -> int {
-        if (s.smem_bytes > 48 * 1024)
-            HIKONV_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem_bytes));
-        return launch_dependent(kern, s.grid, dim3(s.threads), s.smem_bytes, st, s.p);
+        return with_dynamic_smem(reinterpret_cast<const void *>(kern), s.smem_bytes,
+                                 [&] { return launch_dependent(kern, s.grid, dim3(s.threads), s.smem_bytes, st, s.p); });
     };
     if (s.moves) return s.sp ? run(conv2d_strip_kernel<N, KT, JT, TM, TN, true, true>) : run(conv2d_strip_kernel<N, KT, JT, TM, TN, false, true>);
     return s.sp ? run(conv2d_strip_kernel<N, KT, JT, TM, TN, true, false>) : run(conv2d_strip_kernel<N, KT, JT, TM, TN, false, false>);

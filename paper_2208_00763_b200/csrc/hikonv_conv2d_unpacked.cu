@@ -393,9 +393,8 @@ int setup_unpacked(int B, int Ci, int H, int W, int Co, int K, int pad, const Ou
 template <int KT, int PITCH>
 static int launch_pitch(const UnpackedLaunch &u, cudaStream_t st) {
     auto kern = conv2d_unpacked_kernel<KT, PITCH>;
-    if (u.smem_bytes > 48 * 1024)
-        HIKONV_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)u.smem_bytes));
-    return launch_dependent(kern, u.grid, dim3(u.threads), u.smem_bytes, st, u.p);
+    return with_dynamic_smem(reinterpret_cast<const void *>(kern), u.smem_bytes,
+                             [&] { return launch_dependent(kern, u.grid, dim3(u.threads), u.smem_bytes, st, u.p); });
 }
 
 template <int KT>

@@ -5,6 +5,8 @@
 
 #include <cstdint>
 
+#include "hikonv_cuda.cuh"
+
 namespace hikonv {
 
 // n / d for 0 <= n < 2^22 and d > 0 with inv_d = 1.0f / d: the float quotient is off by at most one.
@@ -42,6 +44,49 @@ __host__ inline Div32 make_div32(uint32_t d) {
 __device__ __forceinline__ uint32_t div32(uint32_t n, const Div32 &d) {
     const uint32_t t = __umulhi(d.m, n);
     return (t + ((n - t) >> d.s1)) >> d.s2;
+}
+
+// Byte mask of the bytes of word i (bytes 4 i .. 4 i + 3) whose index lies in [first, last).
+__device__ __forceinline__ uint32_t byte_range_mask(int i, int first, int last) {
+    const int lo = max(first - 4 * i, 0), n = max(last - 4 * i - lo, 0);
+    uint32_t m;
+    asm("bmsk.clamp.b32 %0, %1, %2;" : "=r"(m) : "r"(8 * lo), "r"(8 * n));      // 8 n bits from bit 8 lo on, clamped to the word
+    return m;
+}
+
+// Four packed words (Eq. 5) of N codes each, from column col0 on, of an image row of W one-byte codes: zero outside the row, and
+// everywhere when row_in is false (the row is then not read).  off4: a byte repeated four times that is taken from every
+// code inside the columns of the image (in rows that are not read too), is_signed: the codes, after that, are signed.
+// The codes start at any byte: the N + 1 aligned words around them are loaded (those that hold a code of the row), shifted into
+// place, blanked outside the row with one mask per word, and packed by byte permute and Horner's rule.
+template <int N>
+__device__ __forceinline__ void pack_row_words(const int8_t *row, int W, int col0, bool row_in, uint32_t off4, bool is_signed, int S,
+                                               uint32_t (&word)[4]) {
+    const int8_t *src = row + col0;                              // not dereferenced outside the row
+    const int off = (int)((uintptr_t)src & 3);
+    const uint32_t *al = reinterpret_cast<const uint32_t *>(src - off);
+    uint32_t v[N + 1];
+#pragma unroll
+    for (int i = 0; i <= N; ++i) {
+        const int c = col0 - off + 4 * i;                        // aligned word i holds the codes of columns c .. c + 3
+        v[i] = (row_in && c + 3 >= 0 && c < W) ? __ldg(al + i) : 0u;
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        v[i] = __funnelshift_r(v[i], v[i + 1], 8 * off);
+        if (off4 != 0) v[i] = __vsub4(v[i], off4);
+        v[i] &= byte_range_mask(i, -col0, W - col0);
+    }
+    const uint32_t step = 1u << S, ext = is_signed ? 0x8880u : 0x4440u, rep = is_signed ? 0x1111u : 1u;
+    // permute selector of byte b, sign- or zero-extended (see extract_code)
+    auto code = [&](int e) { return byte_permute(v[e / 4], 0u, ext + (uint32_t)(e % 4) * rep); };
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+        uint32_t a = code(w * N + N - 1);
+#pragma unroll
+        for (int n = N - 2; n >= 0; --n) a = a * step + code(w * N + n);
+        word[w] = a;
+    }
 }
 
 // Maxima of neighbouring bytes of two rows of eight bytes: four bytes.

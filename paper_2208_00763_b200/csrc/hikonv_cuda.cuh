@@ -55,6 +55,32 @@ inline int launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 block, si
     return cudaLaunchKernelEx(&cfg, kernel, args...) == cudaSuccess ? HIKONV_OK : HIKONV_ERR_CUDA;
 }
 
+// Runs `launch` (which returns a hikonv status) for a kernel that needs `bytes` of dynamic shared memory.  Beyond 48 KB the
+// kernel's limit has to be raised, once per device; every thread remembers for which kernels it has seen that done.  A launch
+// that fails all the same (the device may have been reset in between) is tried once more with the limit raised again.
+template <typename Launch>
+inline int with_dynamic_smem(const void *kernel, size_t bytes, Launch launch) {
+    constexpr size_t kPlain = 48 * 1024;
+    constexpr int kMost = 227 * 1024, kSlots = 256;
+    struct Raised {
+        const void *kernel;
+        int dev;
+    };
+    static thread_local Raised raised[kSlots];
+    if (bytes <= kPlain) return launch();
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return HIKONV_ERR_CUDA;
+    Raised &r = raised[(((uintptr_t)kernel >> 4) ^ (uintptr_t)dev) % kSlots];
+    const bool known = r.kernel == kernel && r.dev == dev;
+    if (!known && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost) != cudaSuccess) return HIKONV_ERR_CUDA;
+    r.kernel = kernel;
+    r.dev = dev;
+    const int rc = launch();
+    if (rc == HIKONV_OK || !known) return rc;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost) != cudaSuccess) return HIKONV_ERR_CUDA;
+    return launch();
+}
+
 // The 32x32->64 product of two packed words (Eq. 9).  The multiply is given as inline PTX (mul.wide) and the
 // 64-bit add is left to the compiler, which fuses the pair into one wide multiply-add.  Two other spellings were
 // tried and dropped after counting instructions per opcode in the profiler: mad.wide as inline PTX came out as a
@@ -95,6 +121,13 @@ __device__ __forceinline__ int32_t code_value(int8_t b) {
 template <bool SIGNED>
 __device__ __forceinline__ int32_t load_code(const int8_t *p) {
     return code_value<SIGNED>(__ldg(p));
+}
+
+// prmt with a selector known at run time (__byte_perm ignores the bit that replicates a byte's sign).
+__device__ __forceinline__ uint32_t byte_permute(uint32_t a, uint32_t b, uint32_t sel) {
+    uint32_t r;
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(sel));
+    return r;
 }
 
 // Byte `b` (0..3) of w as a 32-bit value, sign- or zero-extended: one prmt.

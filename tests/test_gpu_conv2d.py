@@ -94,6 +94,29 @@ def test_strips_of_rows_in_every_tile(K, pad):
                 assert_exact(got, ref, "%s K=%d p=%d q=%d tile=%d" % ((B, Ci, H, W, Co), K, p, q, tile))
 
 
+@pytest.mark.parametrize("K, pad", [(1, 0), (3, 1), (3, 0), (3, 2), (5, 2)])
+def test_small_layers_in_one_launch(K, pad):
+    # tile = -2: operands packed by the layer kernel, input channels shared by the CTAs of a cluster; channel counts that cut
+    # unevenly or leave the last CTAs none, strips of several images, ragged last strips, sums, codes and pooled codes, against
+    # the two-launch form (tile = -1) and the oracle
+    for (B, Ci, H, W, Co) in ((1, 64, 10, 20, 64), (3, 5, 7, 9, 6), (5, 11, 6, 6, 33), (1, 3, 8, 150, 7), (2, 33, 4, 4, 4), (1, 1, 5, 5, 1)):
+        for (p, q, xs, ws) in ((4, 4, True, True), (4, 4, False, True), (8, 8, True, True), (2, 2, False, False), (8, 4, False, True), (5, 5, False, False)):
+            x, w = inputs.conv2d_case(B, Ci, H, W, Co, K, p, q, xs, ws, seed=50 + B + Ci + K + p)
+            ref = direct.conv2d_nchw(x, w, pad)
+            d_x, d_w = dev(x), dev(w)
+            for rq in (None, (p, 0, 15), (p, -8, 7)):
+                want = direct.requant(ref, *rq) if rq else ref
+                for tile in (-1, -2):
+                    got = hk.conv2d(d_x, d_w, pad, p, q, xs, ws, requant=rq, tune={"tile": tile})
+                    assert_exact(got, want, "%s K=%d p=%d q=%d %s tile=%d" % ((B, Ci, H, W, Co), K, p, q, rq, tile))
+                if rq and ref.shape[2] % 2 == 0 and ref.shape[3] % 2 == 0:
+                    got = hk.conv2d_dense(d_x.reshape(-1), x.shape, 8, d_w.reshape(-1), w.shape, 8, pad, p, q, xs, ws, requant=rq, pool=True,
+                                          tune={"tile": -2})
+                    assert_exact(got, direct.maxpool2x2(want), "pool %s K=%d p=%d q=%d %s" % ((B, Ci, H, W, Co), K, p, q, rq))
+    for x, w in inputs.extreme_2d(1, 70, 6, 10, 8, K, 4, 4, True, True):
+        assert_exact(_layer(x, w, pad, 4, 4, True, True, hk.ALGO_PACKED32, tune={"tile": -2}), direct.conv2d_nchw(x, w, pad), "extreme")
+
+
 @pytest.mark.parametrize("ci", [4, 7, 20, 64, 130, 256])
 def test_carry_save_schedules(ci):
     # 3x3 layers at N = 3, S = 13 move slot bits to the second accumulator at stage ends (s4 x s4, and any layer
