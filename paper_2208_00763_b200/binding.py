@@ -2,6 +2,10 @@
 
 PyTorch is used for device memory and streams; every arithmetic step runs in the CUDA
 library.  Loading fails loudly when the library has not been built: there is no fallback.
+
+The calls of every step (``conv1d``, ``conv1d_dense``, ``pack``, ``conv2d``, ``conv2d_dense`` without tuning record and
+explicit stream) go through the extension module ``_fast`` first, which makes the same checks on the tensors natively and
+returns None where anything is amiss; the Python code below then raises the error.
 """
 from __future__ import annotations
 
@@ -41,6 +45,7 @@ class TuningT(ctypes.Structure):
 
 
 _lib = None
+_fast = None          # the extension module, its entry points bound to the library's
 
 _vp, _sz, _i, _d = ctypes.c_void_p, ctypes.c_size_t, ctypes.c_int, ctypes.c_double
 
@@ -76,13 +81,17 @@ _SIGNATURES = {
 }
 
 
+_FAST_ENTRY_POINTS = ("hikonv_conv1d", "hikonv_conv1d_dense", "hikonv_pack", "hikonv_conv2d", "hikonv_conv2d_dense",
+                      "hikonv_conv2d_workspace_bytes")
+
+
 def exported_names():
     return sorted(_SIGNATURES)
 
 
 def lib():
     """The loaded CUDA library.  Raises if it has not been built (no CPU fallback exists)."""
-    global _lib
+    global _lib, _fast
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise RuntimeError(
@@ -93,8 +102,20 @@ def lib():
             fn = getattr(handle, name)
             fn.restype = res
             fn.argtypes = args
-        _lib = handle
+        try:
+            from . import _fast as ext
+        except ImportError as err:
+            raise RuntimeError("the binding's extension module is missing or does not load (%s): run "
+                               "`python -m paper_2208_00763_b200.build` first" % err) from err
+        for name in _FAST_ENTRY_POINTS:
+            ext.bind(name, ctypes.cast(getattr(handle, name), ctypes.c_void_p).value)
+        _lib, _fast = handle, ext
     return _lib
+
+
+def _load_fast():
+    lib()
+    return _fast
 
 
 def status_string(status: int) -> str:
@@ -192,6 +213,10 @@ def conv2d_layout(B, Ci, H, W, Co, K, pad, p, q, x_signed, w_signed, tune=None) 
 # ------------------------------------------------------------------ device entry points
 
 def pack(d_in: torch.Tensor, bits: int, is_signed: bool, S: int, N: int, word_bits: int = 32, stream=None) -> torch.Tensor:
+    if stream is None:
+        done = (_fast or _load_fast()).pack(d_in, bits, is_signed, S, N, word_bits)
+        if done is not None:
+            return done
     n = d_in.numel()
     n_words = (n + N - 1) // N
     out = torch.empty(n_words, dtype=torch.int32 if word_bits == 32 else torch.int64, device=d_in.device)
@@ -214,6 +239,10 @@ def check_range(d_in: torch.Tensor, bits: int, is_signed: bool, stream=None) -> 
 
 def conv1d(d_f: torch.Tensor, d_g: torch.Tensor, p: int, q: int, f_signed: bool, g_signed: bool,
            algo: int = ALGO_PACKED32, tune=None, out: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
+    if tune is None and stream is None:
+        done = (_fast or _load_fast()).conv1d(d_f, d_g, p, q, f_signed, g_signed, algo, out)
+        if done is not None:
+            return done
     n, K = d_f.numel(), d_g.numel()
     if out is None:
         out = torch.empty(n + K - 1, dtype=torch.int32, device=d_f.device)
@@ -226,6 +255,10 @@ def conv1d(d_f: torch.Tensor, d_g: torch.Tensor, p: int, q: int, f_signed: bool,
 def conv1d_dense(d_f_dense: torch.Tensor, n: int, d_g: torch.Tensor, p: int, q: int, f_signed: bool, g_signed: bool,
                  tune=None, out: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """`d_f_dense`: uint8 tensor holding `n` codes of p bits, 8 / p per byte."""
+    if tune is None and stream is None:
+        done = (_fast or _load_fast()).conv1d_dense(d_f_dense, n, d_g, p, q, f_signed, g_signed, out)
+        if done is not None:
+            return done
     K = d_g.numel()
     if d_f_dense.dtype != torch.uint8 or not d_f_dense.is_cuda or not d_f_dense.is_contiguous():
         raise ValueError("d_f_dense must be a contiguous CUDA uint8 tensor")
@@ -260,6 +293,10 @@ def conv2d(d_x: torch.Tensor, d_w: torch.Tensor, pad: int, p: int, q: int, x_sig
            requant: Optional[tuple] = None, algo: int = ALGO_PACKED32, tune=None, workspace: Optional[torch.Tensor] = None,
            out: Optional[torch.Tensor] = None, stride: int = 1, stream=None) -> torch.Tensor:
     """requant = (shift, lo, hi) selects int8 output, None the exact int32 sums."""
+    if tune is None and stream is None:
+        done = (_fast or _load_fast()).conv2d(d_x, d_w, pad, p, q, x_signed, w_signed, requant, algo, workspace, out, stride)
+        if done is not None:
+            return done
     B, Ci, H, W = d_x.shape
     Co, Ci2, K, K2 = d_w.shape
     if Ci != Ci2 or K != K2:
@@ -299,6 +336,11 @@ def conv2d_dense(d_x: torch.Tensor, x_shape, x_store_bits: int, d_w: torch.Tenso
     tensors holding the codes of ``x_shape`` = (B, Ci, H, W) / ``w_shape`` = (Co, Ci, K, K).  Returns int32
     [B, Co, Ho, Wo] without ``requant``; with it a flat uint8 tensor of the (optionally pooled) output codes,
     ``out_store_bits`` per code (8: shaped [B, Co, Ho', Wo'] int8)."""
+    if tune is None and stream is None and _tuner_repeats is None:
+        done = (_fast or _load_fast()).conv2d_dense(d_x, x_shape, x_store_bits, d_w, w_shape, w_store_bits, pad, p, q, x_signed, w_signed,
+                                                    requant, out_store_bits, pool, algo, workspace, out, stride)
+        if done is not None:
+            return done
     B, Ci, H, W = x_shape
     Co, Ci2, K, K2 = w_shape
     if Ci != Ci2 or K != K2:
