@@ -94,7 +94,8 @@ typedef struct {
     int tile;       /* kernel-specific tile selector (0 = automatic); conv2d: > 0 output
                        rows per CTA + 1000 x channel lanes per CTA (1, 2, 4, 8; the comparator also
                        16) + 100000 x output rows per thread (2 or 4) + 1000000 x channels per
-                       thread (4 or 8), each part 0 = automatic; -1 packs the operands in a launch of
+                       thread (4 or 8) + 10000000 x thread groups per tile (1, 2 or 4: they share the input
+                       channels), each part 0 = automatic; -1 packs the operands in a launch of
                        its own, -2 in the layer's launch where that is built (small layers); conv1d: > 0 the general kernel, -1 the
                        planner's layout instead of register-aligned slots; -24 / -25 force the
                        register budget of four / five resident CTAs per SM in the register-aligned

@@ -255,6 +255,7 @@ constexpr int kSmemPerCta = 227 * 1024;
 struct StripProblem {
     int B, Ci, Co, Ho, Wo, N, K, J, pad;
     int CF, max_moves;          // input channels between two moves, moves the second accumulator takes
+    int split_moves[kStripMaxGroups + 1];   // most moves that so many groups sharing the input channels may make together (0: their sums may not be added)
     bool moves, generic;
     bool requant, pool;
     int xo_mult;
@@ -262,7 +263,7 @@ struct StripProblem {
 };
 
 struct StripChoice {
-    int TM, TN, TNX, TS, NSEG, XO, XB, halo, X, col_off, pitch, CK, run, runs_per_move, plane, bar_off, e_off, threads;
+    int TM, TN, TNX, KS, TS, NSEG, XO, XB, halo, X, col_off, pitch, CK, run, runs_per_move, plane, bar_off, e_off, threads;
     size_t smem;
     long long ctas;
     double cost;
@@ -284,7 +285,7 @@ static bool complete_choice(const StripProblem &q, StripChoice *c) {
     c->pitch = (c->XB + q.J - 1 + 3) / 4 * 4;
     const int rows = staged_rows(c->TS, c->TM, SH, Hp, q.K);
     c->plane = rows * c->pitch;
-    c->threads = (c->TS * c->XB * c->TNX + 31) / 32 * 32;
+    c->threads = (c->TS * c->XB * c->TNX + 31) / 32 * 32 * c->KS;
     if (c->threads > kStripThreads) return false;
     const int warps = c->threads / 32, TCO = c->TNX * c->TN;
     c->ctas = (strips + c->TS - 1) / c->TS * c->NSEG * ceil_div(q.Co, TCO);
@@ -296,7 +297,9 @@ static bool complete_choice(const StripProblem &q, StripChoice *c) {
     const size_t per_cta = std::min<size_t>(kSmemPerCta, kSmemPerSm / want - 1024);
     if (per_cta < e_bytes + 4096) return false;
     const size_t room = per_cta - e_bytes - 64;
-    int CK = (int)std::min<size_t>(std::min(kStripMaxCK, q.Ci), room / (2 * 4 * (size_t)(c->plane + KJ * kStripBPitch)));
+    // CK: channels of a stage and group
+    const int Cg = ceil_div(q.Ci, c->KS);
+    int CK = (int)std::min<size_t>(std::min(std::min(kStripMaxCK, 32 / c->KS), Cg), room / (2 * 4 * (size_t)c->KS * (c->plane + KJ * kStripBPitch)));
     if (CK < 1) return false;
     c->run = CK;
     c->runs_per_move = 1;
@@ -316,13 +319,17 @@ static bool complete_choice(const StripProblem &q, StripChoice *c) {
             c->runs_per_move = q.CF / CK;
             c->run = CK;
         }
+        // each of several groups also makes a move after its last channel, and their second accumulators are added
+        if (c->KS > 1 && c->KS * ceil_div(Cg, c->run * c->runs_per_move) > q.split_moves[c->KS]) return false;
     }
+    const double warp_ci = Cg;                                       // input channels that a warp goes through
+    CK *= c->KS;
     c->CK = CK;
     size_t words = 2 * (size_t)CK * (c->plane + KJ * kStripBPitch);
-    const size_t xch = (size_t)warps * c->TNX * c->TM * c->TN * 2;
+    const size_t xch = (size_t)warps * c->TNX * c->TM * c->TN / c->KS * 2, sums = c->KS > 1 ? (size_t)c->threads * c->TM * c->TN * 2 : 0;
     const int rps = q.pool ? c->TM / 2 : c->TM;
     const size_t tile = (xch + 3) / 4 * 4 + (size_t)TCO * c->TS * rps * ((c->XO * q.N + 15) / 16 * 16) / 4;
-    words = (std::max(words, std::max(xch, tile)) + 3) / 4 * 4;
+    words = (std::max(words, std::max(xch + sums, tile)) + 3) / 4 * 4;
     c->bar_off = (int)words;
     c->e_off = (int)words + 4;
     c->smem = words * 4 + 16 + e_bytes;
@@ -330,14 +337,19 @@ static bool complete_choice(const StripProblem &q, StripChoice *c) {
     const int resident = std::max(1, std::min(by_regs, (int)(kSmemPerSm / (c->smem + 1024))));
     // issue cycles of one warp
     const double mt = (double)c->TM * c->TN;
-    double per_ch = 4.3 * mt * KJ + 0.5 * (c->TM + q.K - 1) * q.J + 0.6 * KJ * c->TN / 4 + 8 + 80.0 / CK;
+    double per_ch = 4.3 * mt * KJ + 0.5 * (c->TM + q.K - 1) * q.J + 0.6 * KJ * c->TN / 4 + 8 + 80.0 * c->KS / CK;
     if (q.generic) per_ch += KJ * 16.0;
     if (q.moves) per_ch += 10.0 * mt / q.CF;
     const double split = q.moves ? 6.0 * q.N + 12 : 3.0 * q.N + 6;
-    const double fixed = 400 + mt * (split + q.N * (q.pool ? 4.0 : q.requant ? 6.0 : 3.0));
-    const double warp_cycles = q.Ci * per_ch + fixed;
+    double fixed = 400 + mt / c->KS * (split + q.N * (q.pool ? 4.0 : q.requant ? 6.0 : 3.0));
+    if (c->KS > 1) fixed += 100 + mt * (q.moves ? 18.0 : 6.0);
+    const double warp_cycles = warp_ci * per_ch + fixed;
     // n resident CTAs of this size on an SM
-    auto cycles_of = [&](double n) { return std::max(n * ceil_div(warps, 4), 1.5) * warp_cycles + 1500 + 250.0 * q.Ci / CK; };
+    // (few warps hide less of each other's latencies: two per scheduler took a sixth longer than eight, by the clock over 17 layers)
+    auto cycles_of = [&](double n) {
+        const double per_scheduler = n * ceil_div(warps, 4);
+        return std::max(per_scheduler, 1.5) * (1.0 + 0.3 / per_scheduler) * warp_cycles + 1500 + 250.0 * q.Ci / CK;
+    };
     const double slots = (double)resident * q.sms, waves = c->ctas / slots;
     double cycles;
     if (waves <= 1.0) cycles = cycles_of(share);
@@ -350,15 +362,17 @@ static bool complete_choice(const StripProblem &q, StripChoice *c) {
     return true;
 }
 
-// Chooses the thread tile, channel lanes, row cut and strips per CTA.  force_*: 0 = free.
-static StripChoice choose_strips(const StripProblem &q, int force_tm, int force_tn, int force_tnx, int force_rows) {
-    static const int tiles[3][2] = {{4, 8}, {2, 8}, {2, 4}};
+// Chooses the thread tile, thread groups, channel lanes, row cut and strips per CTA.  force_*: 0 = free.
+static StripChoice choose_strips(const StripProblem &q, int force_tm, int force_tn, int force_ks, int force_tnx, int force_rows) {
+    static const int tiles[6][3] = {{4, 8, 1}, {2, 8, 1}, {2, 4, 1}, {2, 8, 2}, {2, 4, 2}, {2, 4, 4}};
     StripChoice best;
     std::memset(&best, 0, sizeof(best));
     best.cost = -1.0;
     const int c0 = q.K - 1 - q.pad;
     for (const auto &tile : tiles) {
-        const int TM = tile[0], TN = tile[1];
+        const int TM = tile[0], TN = tile[1], KS = tile[2];
+        if (KS > 1 && (!strip_split_built(TM, TN, KS, q.generic) || q.Ci < 2 * KS || (q.moves && q.split_moves[KS] == 0))) continue;
+        if (force_ks > 0 && KS != force_ks && !q.generic) continue;
         if (!strip_tile_built(TM, TN, q.generic) || (force_tm > 0 && TM != force_tm && !q.generic) ||
             (force_tn > 0 && TN != force_tn && !q.generic)) continue;
         if (TN == 8 && q.Co <= 4 && force_tn != 8) continue;
@@ -366,13 +380,13 @@ static StripChoice choose_strips(const StripProblem &q, int force_tm, int force_
         const long long strips = (long long)q.B * SH;
         for (int TNX = 1; TNX * TN <= kStripBPitch; TNX *= 2) {
             if (force_tnx > 0 ? TNX != std::min(force_tnx, kStripBPitch / TN) : (TNX > 1 && TNX * TN / 2 >= q.Co)) continue;
-            const int maxpos = kStripThreads / TNX;
+            const int maxpos = kStripThreads / (TNX * KS);
             // uncut rows start at the image's first column (a word then holds no padding but the row's end); the positions of a
             // cut row need the word in front of them, and its segments start at columns XO N
             int tried = 0;
             for (int cut = 1; cut <= 4096 && tried < 3; ++cut) {
                 StripChoice c;
-                c.TM = TM; c.TN = TN; c.TNX = TNX;
+                c.TM = TM; c.TN = TN; c.TNX = TNX; c.KS = KS;
                 if (cut == 1) {
                     c.NSEG = 1; c.halo = 0; c.col_off = c0;
                     c.X = c.XO = c.XB = ceil_div(q.Wo + c0, q.N);
@@ -525,20 +539,23 @@ static int plan_layer(int B, int Ci, int H, int W, int Co, int K, int stride, in
             pr.CF = move_period(L, sc, p, q, xs, ws, K, Ci, false);
         }
         if (pr.CF == 0) return HIKONV_ERR_NO_FIT;                    // not even one channel's kernel rows between two moves
+        for (int ks = 0; ks <= kStripMaxGroups; ++ks)
+            pr.split_moves[ks] = pr.moves && !pr.generic && ks > 1 ? most_split_moves(L, sc, p, q, xs, ws, K, pr.CF, ks, strip_packed_add(L.N, K, L.J)) : 0;
         pr.requant = out.requant != 0; pr.pool = out.requant && out.pool;
         pr.xo_mult = segment_multiple(out, L.N);
         pr.sms = sm_count();
         // tune->tile > 0: rows per CTA, plus 1000 x channel lanes per CTA, 100000 x rows and 1000000 x channels per thread when
         // those are forced too
-        const int tile_arg = (tune && tune->tile > 0) ? tune->tile : 0, force_tn = tile_arg / 1000000, force_tm = tile_arg / 100000 % 10;
-        if ((force_tm != 0 && force_tm != 2 && force_tm != 4) || (force_tn != 0 && force_tn != 4 && force_tn != 8)) return HIKONV_ERR_UNSUPPORTED;
-        const StripChoice c = choose_strips(pr, force_tm, force_tn, tile_arg % 100000 / 1000, tile_arg % 1000);
+        const int tile_arg = (tune && tune->tile > 0) ? tune->tile : 0, force_ks = tile_arg / 10000000, force_tn = tile_arg / 1000000 % 10, force_tm = tile_arg / 100000 % 10;
+        if ((force_tm != 0 && force_tm != 2 && force_tm != 4) || (force_tn != 0 && force_tn != 4 && force_tn != 8) ||
+            force_ks == 3 || force_ks > 4) return HIKONV_ERR_UNSUPPORTED;
+        const StripChoice c = choose_strips(pr, force_tm, force_tn, force_ks, tile_arg % 100000 / 1000, tile_arg % 1000);
         if (c.cost < 0) return HIKONV_ERR_UNSUPPORTED;
 
         StripLaunch &l = s->strip;
         StripParams &k = l.p;
         std::memset(&k, 0, sizeof(k));
-        l.TM = c.TM; l.TN = c.TN; l.sp = L.signed_prod != 0; l.moves = pr.moves; l.generic = pr.generic; l.threads = c.threads;
+        l.TM = c.TM; l.TN = c.TN; l.KS = c.KS; l.sp = L.signed_prod != 0; l.moves = pr.moves; l.generic = pr.generic; l.threads = c.threads;
         k.Ci = Ci; k.Co = Co; k.CoP = s->CoP; k.K = K; k.J = L.J; k.Ho = Ho; k.Wo = Wo; k.W = W; k.pad = pad;
         k.Hp = s->Hp; k.ap_rows = B * s->Hp;
         k.SH = ceil_div(Ho, c.TM); k.strips = B * k.SH;
@@ -557,7 +574,7 @@ static int plan_layer(int B, int Ci, int H, int W, int Co, int K, int stride, in
         rc = output_staging(out, Ho, Wo, c.NSEG, c.XO * L.N, &k.stage_out, &k.vec);
         if (rc != HIKONV_OK) return rc;
         k.WTP = (c.XO * L.N + 15) / 16 * 16;
-        k.tile_off = (c.threads / 32 * c.TNX * c.TM * c.TN * 2 + 3) / 4 * 4;
+        k.tile_off = (c.threads / 32 * c.TNX * c.TM * c.TN / c.KS * 2 + 3) / 4 * 4;
         const long long gx = ((long long)k.strips + c.TS - 1) / c.TS * c.NSEG;
         const int gy = ceil_div(Co, k.TCO);
         if (gx > 0x7FFFFFFFLL || gy > 65535) return HIKONV_ERR_UNSUPPORTED;
@@ -574,12 +591,13 @@ static int plan_layer(int B, int Ci, int H, int W, int Co, int K, int stride, in
         const bool force_small = tune && tune->tile == -2;
         if (!pr.generic && s->x_off == 0 && out.byte_inputs && out.out_bits == 8 && tile_arg == 0 && !(tune && tune->tile == -1)) {
             const SmallChoice sm = choose_small(pr);
-            // both models brought to measured times on 59 layers (3 to 122 channels, 1 to 64 images, every layout): they leave out
-            // latencies of a few thousand cycles, and the packing launch takes 2.3 us and 12 us per million 16-byte pieces.  The
-            // one launch measured faster below about 10 us (10x20x64, one image: 7.4 against 16.8 us; 16 images: 14.6 against
-            // 15.4; 64 images: 23.4 against 18.1)
-            const double two = 4500 + 1.3 * c.cost + 0.024 * Ci * B * s->Hp * (k.XBT / 4);
-            const double one = sm.cost + 0.9 * std::max(0.0, sm.cost - 9800);
+            // both models brought to measured times on 66 layers (3 to 200 channels, 1 to 32 images, every layout; 8 and 16 % rms):
+            // they leave out latencies of a few thousand cycles, and the packing launch takes 2.3 us and 13 us per million 16-byte
+            // pieces.  Over those layers the calls took 700 us together, 719 us always in two launches, 696 us with the faster of
+            // the two each time.  One launch is the faster one for little work (2x195x33x28 -> 9, 8 bits: 12.5 against 14.1 us;
+            // 5x5x7x46 -> 183: 4.4 against 5.9), two from about 15 us on (9x23x16x18 -> 151, 5x5: 24.0 against 13.9)
+            const double two = 4300 + 1.1 * c.cost + 0.025 * Ci * B * s->Hp * (k.XBT / 4);
+            const double one = 2.4 * sm.cost - 11200 - 0.8 * std::max(0.0, sm.cost - 9800);
             if (sm.cost >= 0 && (one < two || force_small)) {
                 s->one_launch = true;
                 SmallLaunch &ml = s->small;

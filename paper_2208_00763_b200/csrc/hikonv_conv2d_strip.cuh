@@ -10,8 +10,14 @@
 // group in front of a lane's is in the lane before it, whatever the row of the strip.
 //
 // A CTA computes TS consecutive strips (of one or several images) of one row segment times TCO channels.  Packed activation
-// rows and kernel rows are streamed in stages of CK input channels with asynchronous copies into double-buffered shared memory.  The distance between two channels of a stage is a constant (kPlaneWords), so that the unrolled channel
-// loop needs no address arithmetic whatever the width of the rows.
+// rows and kernel rows are streamed in stages of CK input channels with asynchronous copies into double-buffered shared memory.
+//
+// Thread groups.  A layer of few strips leaves schedulers with one or two warps, which cannot hide each other's latencies, or SMs
+// with nothing.  There KS groups of threads work on one tile, each on its share of a stage's input channels; the packed sums (and
+// second accumulators) are added in shared memory, and every group splits and stores TN / KS of the channels.  Each group has the
+// prologue and the moves to itself, so this is for layers that lack warps, by the cost model's estimate: 32 images 128x7x7 -> 256
+// 30.9 -> 23.9 us, 1x175x15x62 -> 57 5x5 104 -> 35 us (four groups), 4x128x28x28 -> 128 31.3 -> 24.3 us; but 56x56x64 (four
+// warps per scheduler without) 86.6 -> 100 us.
 //
 // Split.  Every slot starts at a bias that makes its running sum non-negative, so slots never borrow from each other (this
 // replaces the sign-borrow increment of Eq. 29).  After CF input channels a slot could overflow; the bits of every slot above
@@ -27,8 +33,8 @@
 // across channels or a compile-time distance between channels (no pointer arithmetic left) changed neither.
 // Measured against the kernel before it (four positions of one row per thread, one halo word per row, run-time loops for 5x5),
 // packing launch included: 32x64x56x56 -> 64 s4 93.3 -> 85.4 us, 64x256x14x14 -> 256 u4 x s4 211 -> 162 us (205 with the new
-// packing launch alone), 8x48x37x53 -> 40 s8 32.4 -> 26.4 us, 16x24x45x61 -> 40 5x5 2-bit 70.6 -> 31.7 us, the compact CNN
-// (batch 64) 605 -> 492 us.
+// packing launch alone), 8x48x37x53 -> 40 s8 32.4 -> 26.4 us, 16x24x45x61 -> 40 5x5 2-bit 70.6 -> 30.0 us, the compact CNN
+// (batch 64) 605 -> 484 us.
 #pragma once
 
 #include <type_traits>
@@ -43,8 +49,9 @@ template <int N, int KT, int JT>
 constexpr bool kStripPackedAdd = strip_packed_add(N, KT, JT);
 
 // N: pixels per word; KT, JT: kernel size and words per kernel row (0: run-time bounds); TM x TN: rows x channels per thread;
-// SP: signed product; HASE: with second accumulators.
-template <int N, int KT, int JT, int TM, int TN, bool SP, bool HASE>
+// SP: signed product; HASE: with second accumulators; KS: thread
+// groups that share the input channels of a tile.
+template <int N, int KT, int JT, int TM, int TN, bool SP, bool HASE, int KS>
 __global__ void __launch_bounds__(kStripThreads, 2) conv2d_strip_kernel(const __grid_constant__ StripParams p) {
     constexpr bool PACKED_ADD = kStripPackedAdd<N, KT, JT>;
     constexpr bool UP = N > 1 && KT != 1;                       // some products have slots above the N low ones
@@ -54,8 +61,10 @@ __global__ void __launch_bounds__(kStripThreads, 2) conv2d_strip_kernel(const __
 
     const int tid = threadIdx.x, nthreads = blockDim.x, lane = tid & 31;
     const int warp = tid >> 5;
+    const int group_threads = nthreads / KS, group = KS > 1 ? warp / ((nthreads / KS) >> 5) : 0, gtid = tid - group * group_threads;
+    constexpr int TE = TN / KS;                                // channels that a thread finishes: TE group ..
     const int tnx_log2 = 31 - __clz(p.TNX);                    // TNX is a power of two
-    const int tn = tid & (p.TNX - 1);
+    const int tn = gtid & (p.TNX - 1);
     const int strip_tile = p.NSEG > 1 ? (int)(blockIdx.x / (unsigned)p.NSEG) : (int)blockIdx.x;
     const int seg = (int)blockIdx.x - strip_tile * p.NSEG;
     const int g0 = strip_tile * p.TS;                          // first strip
@@ -70,7 +79,7 @@ __global__ void __launch_bounds__(kStripThreads, 2) conv2d_strip_kernel(const __
     const int NR = min(dbl * p.Hp + (tl - dbl * p.SH) * TM - s0 * TM + TM + K - 1, p.ap_rows - r0);
 
     // this thread's strip and group (an idle thread works on position 0; its results are dropped)
-    const int pos = tid >> tnx_log2, pos_ok = pos < TSe * p.XB, pc = pos_ok ? pos : 0;
+    const int pos = gtid >> tnx_log2, pos_ok = pos < TSe * p.XB, pc = pos_ok ? pos : 0;
     const int sl = fast_div(pc, p.mg_xb), xb = pc - sl * p.XB;
     const int db = fast_div(s0 + sl, p.mg_sh), s_img = s0 + sl - db * p.SH;
     int a_off[ROWS];                                           // word of row r, j = 0 in a channel's plane
@@ -206,6 +215,8 @@ __global__ void __launch_bounds__(kStripThreads, 2) conv2d_strip_kernel(const __
     int stage = 0;
     for (int ci0 = 0; ci0 < p.Ci; ci0 += p.CK, stage ^= 1) {
         const int ckn = min(p.CK, p.Ci - ci0);
+        // the groups' shares of a stage (the last ones' may be shorter; moves happen at the same places in all)
+        const int share = (ckn + KS - 1) / KS, own = min(ckn - group * share, share);
         // this stage has landed (were the wait ever to run out, the sums would be wrong but nothing would hang)
         mbarrier_wait(bar0 + 8u * stage, parity);
         cp_async_wait_all();
@@ -213,12 +224,16 @@ __global__ void __launch_bounds__(kStripThreads, 2) conv2d_strip_kernel(const __
         __syncthreads();                                       // the previous stage is fully consumed
         if (ci0 + p.CK < p.Ci) fetch(min(p.CK, p.Ci - ci0 - p.CK), stage ^ 1);
         int a_ch = stage * p.a_words, b_ch = p.b_off + stage * p.b_words;
-        for (int c = 0; c < ckn; c += run) {
-            const int n = HASE ? min(run, ckn - c) : ckn;
+        if constexpr (KS > 1) {
+            a_ch += group * share * p.plane;
+            b_ch += group * share * KJ * kStripBPitch;
+        }
+        for (int c = 0; c < share; c += run) {
+            const int n = HASE ? min(run, own - c) : own;
 #pragma unroll 2
             for (int u = 0; u < n; ++u, a_ch += p.plane, b_ch += KJ * kStripBPitch) channel(a_ch, b_ch);
             if constexpr (HASE) {
-                if (--runs_left == 0 && ci0 + c + n < p.Ci) {  // none is needed after the last channel
+                if (--runs_left == 0 && (c + run < share || ci0 + p.CK < p.Ci)) {  // none is needed after the last channel
                     move_upper_bits();
                     ++moves;
                     runs_left = p.runs_per_move;
@@ -227,24 +242,66 @@ __global__ void __launch_bounds__(kStripThreads, 2) conv2d_strip_kernel(const __
         }
     }
 
+    // ---- several groups: each finishes a share of a tile's channels, summed through shared memory.  Of the KS biases in a sum all
+    // but one are taken off; the bits above the low h have all moved before, so no slot overflows
+    uint2 *const xch0 = reinterpret_cast<uint2 *>(smem);
+    uint64_t fin[TM][TE];
+    __syncthreads();
+    if constexpr (KS > 1) {
+        if constexpr (HASE) {
+            move_upper_bits();
+            ++moves;
+        }
+        uint2 *const sums = xch0 + (nthreads >> 5) * p.TNX * (TM * TE);
+#pragma unroll
+        for (int i = 0; i < TM; ++i)
+#pragma unroll
+            for (int t = 0; t < TN; ++t) sums[(i * TN + t) * nthreads + tid] = make_uint2((uint32_t)acc[i][t], (uint32_t)(acc[i][t] >> 32));
+        __syncthreads();
+        const uint2 *from = sums + group * TE * nthreads + gtid;
+#pragma unroll
+        for (int i = 0; i < TM; ++i)
+#pragma unroll
+            for (int t = 0; t < TE; ++t) {
+                uint64_t v = (uint64_t)(1 - KS) * p.bias;
+#pragma unroll
+                for (int k = 0; k < KS; ++k) {
+                    const uint2 part = from[(i * TN + t) * nthreads + k * group_threads];
+                    v += ((uint64_t)part.y << 32) | part.x;
+                }
+                fin[i][t] = v;
+            }
+    } else {
+#pragma unroll
+        for (int i = 0; i < TM; ++i)
+#pragma unroll
+            for (int t = 0; t < TE; ++t) fin[i][t] = acc[i][t];
+    }
+    const int ch0 = tn * TN + group * TE;                      // first of this thread's finished channels
+    const uint2 *const es0 = reinterpret_cast<uint2 *>(smem + p.e_off) + gtid * strip_e_pitch(TM, TN) + group * TE;
     auto second = [&](int i, int t) -> uint64_t {
-        const uint2 e = es[i * TN + t];
-        return ((uint64_t)e.y << 32) | e.x;
+        const uint2 e = es0[i * TN + t];
+        uint64_t v = ((uint64_t)e.y << 32) | e.x;
+#pragma unroll
+        for (int k = 1; k < KS; ++k) {
+            const uint2 f = es0[k * group_threads * strip_e_pitch(TM, TN) + i * TN + t];
+            v += ((uint64_t)f.y << 32) | f.x;
+        }
+        return v;
     };
     // ---- words above the N low slots: to the next lane by shuffle, across warps through shared memory
-    uint2 *xch = reinterpret_cast<uint2 *>(smem) + ((warp << tnx_log2) + tn) * (TM * TN);
+    uint2 *xch = xch0 + ((warp << tnx_log2) + tn) * (TM * TE);
     const int lanes_m = 32 >> tnx_log2, lm = lane >> tnx_log2;
-    __syncthreads();
     if (UP && lm == lanes_m - 1) {
 #pragma unroll
         for (int i = 0; i < TM; ++i)
 #pragma unroll
-            for (int t = 0; t < TN; ++t)
-                xch[i * TN + t] = make_uint2((uint32_t)(acc[i][t] >> p.SN), HASE ? (uint32_t)(second(i, t) >> p.SN) : 0u);
+            for (int t = 0; t < TE; ++t)
+                xch[i * TE + t] = make_uint2((uint32_t)(fin[i][t] >> p.SN), HASE ? (uint32_t)(second(i, t) >> p.SN) : 0u);
     }
     __syncthreads();
-    const uint2 *xch_in = xch - p.TNX * (TM * TN);
-    const bool from_smem = lm == 0 && warp > 0;
+    const uint2 *xch_in = xch - p.TNX * (TM * TE);
+    const bool from_smem = lm == 0 && gtid >= 32;
     const uint32_t keep = xb == 0 ? 0u : 0xFFFFFFFFu;          // nothing comes in at the left end of a row
 
     const int x = seg * p.XO + xb - p.halo, w0 = x * N - p.col_off;   // group and its first output column
@@ -255,14 +312,14 @@ __global__ void __launch_bounds__(kStripThreads, 2) conv2d_strip_kernel(const __
 #pragma unroll
     for (int m = 0; m < N; ++m) {
         col_ok[m] = pos_ok && xb >= p.halo && x < p.X && w0 + m >= 0 && w0 + m < p.Wo;
-        base[m] = -(moves + 1) * (p.slot_bias[m] + (keep ? p.slot_bias[m + N] : 0));
+        base[m] = -(KS * moves + 1) * (p.slot_bias[m] + (keep ? p.slot_bias[m + N] : 0));
     }
-    const int n_ch = min(TN, p.Co - co0 - tn * TN);
+    const int n_ch = min(TE, p.Co - co0 - ch0);
     const uint32_t mask = p.slot_mask;
 
     // value[m] of accumulator (i, t)
     auto split = [&](int i, int t, const int32_t (&off)[N], int32_t (&y)[N]) {
-        uint64_t q = acc[i][t];
+        uint64_t q = fin[i][t];
         uint32_t q_in = 0, e_in = 0, qf[N], ef[N];
         uint64_t e = 0;
         if constexpr (HASE) e = second(i, t);
@@ -270,7 +327,7 @@ __global__ void __launch_bounds__(kStripThreads, 2) conv2d_strip_kernel(const __
             q_in = __shfl_up_sync(0xFFFFFFFFu, (uint32_t)(q >> p.SN), p.TNX);
             if constexpr (HASE) e_in = __shfl_up_sync(0xFFFFFFFFu, (uint32_t)(e >> p.SN), p.TNX);
             if (from_smem) {
-                const uint2 v = xch_in[i * TN + t];
+                const uint2 v = xch_in[i * TE + t];
                 q_in = v.x;
                 if constexpr (HASE) e_in = v.y;
             }
@@ -302,7 +359,7 @@ __global__ void __launch_bounds__(kStripThreads, 2) conv2d_strip_kernel(const __
 #pragma unroll
         for (int m = 0; m < N; ++m) off[m] = base[m];
         if (p.corr && t < n_ch) {
-            const int32_t *c = p.corr + co0 + tn * TN + t;
+            const int32_t *c = p.corr + co0 + ch0 + t;
 #pragma unroll
             for (int m = 0; m < N; ++m)
                 if (col_ok[m]) {
@@ -317,12 +374,12 @@ __global__ void __launch_bounds__(kStripThreads, 2) conv2d_strip_kernel(const __
     if (!p.stage_out) {
         // direct stores; warps whose rows and channels all exist (nearly all) test only the columns
         const size_t chan = (size_t)p.Ho * p.Wo;
-        const size_t at = (((size_t)(b0 + db) * p.Co + co0 + tn * TN) * p.Ho + h0) * p.Wo + w0;
+        const size_t at = (((size_t)(b0 + db) * p.Co + co0 + ch0) * p.Ho + h0) * p.Wo + w0;
         auto finish = [&](auto *dst, auto full_tag) {
             constexpr bool FULL = decltype(full_tag)::value, REQ = sizeof(*dst) == 1;
             auto *chan_row = dst + at;
 #pragma unroll
-            for (int t = 0; t < TN; ++t, chan_row += chan) {
+            for (int t = 0; t < TE; ++t, chan_row += chan) {
                 int32_t off[N], y[N];
                 offsets(t, off);
                 auto *row = chan_row;
@@ -339,7 +396,7 @@ __global__ void __launch_bounds__(kStripThreads, 2) conv2d_strip_kernel(const __
                 }
             }
         };
-        const bool full = __all_sync(0xFFFFFFFFu, n_ch >= TN && (n_rows >= TM || !pos_ok));
+        const bool full = __all_sync(0xFFFFFFFFu, n_ch >= TE && (n_rows >= TM || !pos_ok));
         if (p.requant) {
             if (full) finish((int8_t *)p.out, std::true_type());
             else finish((int8_t *)p.out, std::false_type());
@@ -356,11 +413,11 @@ __global__ void __launch_bounds__(kStripThreads, 2) conv2d_strip_kernel(const __
     const int rps = p.pool ? TM / 2 : TM;                      // tile rows per strip
     const int tile_chan = p.TS * rps * p.WTP;
     const int col0 = seg * p.XO * N;                           // first output column of the segment (segments: col_off == 0)
-    int8_t *tile_at = tile + tn * TN * tile_chan + sl * rps * p.WTP + w0 - col0;
+    int8_t *tile_at = tile + ch0 * tile_chan + sl * rps * p.WTP + w0 - col0;
     auto stage_codes = [&](auto pool_tag) {
         constexpr bool POOL = decltype(pool_tag)::value;
 #pragma unroll
-        for (int t = 0; t < TN; ++t) {
+        for (int t = 0; t < TE; ++t) {
             int32_t off[N], y[N], y2[N];
             offsets(t, off);
 #pragma unroll
@@ -434,18 +491,24 @@ __global__ void __launch_bounds__(kStripThreads, 2) conv2d_strip_kernel(const __
     }
 }
 
-template <int N, int KT, int JT, int TM, int TN>
+template <int N, int KT, int JT, int TM, int TN, int KS = 1>
 static int launch_strip_tile(const StripLaunch &s, cudaStream_t st) {
     auto run = [&](auto kern) -> int {
         return with_dynamic_smem(reinterpret_cast<const void *>(kern), s.smem_bytes,
                                  [&] { return launch_dependent(kern, s.grid, dim3(s.threads), s.smem_bytes, st, s.p); });
     };
-    if (s.moves) return s.sp ? run(conv2d_strip_kernel<N, KT, JT, TM, TN, true, true>) : run(conv2d_strip_kernel<N, KT, JT, TM, TN, false, true>);
-    return s.sp ? run(conv2d_strip_kernel<N, KT, JT, TM, TN, true, false>) : run(conv2d_strip_kernel<N, KT, JT, TM, TN, false, false>);
+    if (s.moves) return s.sp ? run(conv2d_strip_kernel<N, KT, JT, TM, TN, true, true, KS>) : run(conv2d_strip_kernel<N, KT, JT, TM, TN, false, true, KS>);
+    return s.sp ? run(conv2d_strip_kernel<N, KT, JT, TM, TN, true, false, KS>) : run(conv2d_strip_kernel<N, KT, JT, TM, TN, false, false, KS>);
 }
 
 template <int N, int KT, int JT>
 int launch_strip(const StripLaunch &s, cudaStream_t st) {
+    if constexpr (KT > 0) {
+        if (s.TM == 2 && s.TN == 4 && s.KS == 2) return launch_strip_tile<N, KT, JT, 2, 4, 2>(s, st);
+        if (s.TM == 2 && s.TN == 8 && s.KS == 2) return launch_strip_tile<N, KT, JT, 2, 8, 2>(s, st);
+        if (s.TM == 2 && s.TN == 4 && s.KS == 4) return launch_strip_tile<N, KT, JT, 2, 4, 4>(s, st);
+    }
+    if (s.KS != 1) return HIKONV_ERR_UNSUPPORTED;
     if (s.TM == 2 && s.TN == 4) return launch_strip_tile<N, KT, JT, 2, 4>(s, st);
     if constexpr (KT > 0) {
         if (s.TM == 2 && s.TN == 8) return launch_strip_tile<N, KT, JT, 2, 8>(s, st);

@@ -10,7 +10,8 @@ namespace hikonv {
 
 constexpr int kStripThreads = 256;   // most threads of a CTA
 constexpr int kStripBPitch = 32;     // words per packed kernel row in shared memory (TCO or more)
-constexpr int kStripMaxCK = 16;      // most input channels of a stage
+constexpr int kStripMaxCK = 16;      // most input channels of a stage and thread group
+constexpr int kStripMaxGroups = 4;   // most thread groups that share the input channels of a tile
 
 struct StripParams {
     const uint32_t *ap;              // packed activations [Ci][B * Hp][XBT]
@@ -46,7 +47,7 @@ struct StripLaunch {
     dim3 grid;
     int threads;
     size_t smem_bytes;
-    int TM, TN;                      // output rows and channels per thread
+    int TM, TN, KS;                  // output rows and channels per thread, thread groups that share the input channels
     bool sp;                         // signed product
     bool moves;                      // the layer needs the second accumulator
     bool generic;                    // the kernel with run-time loop bounds
@@ -57,6 +58,8 @@ struct StripLaunch {
 inline bool strip_tile_built(int TM, int TN, bool generic) {
     return generic ? (TM == 2 && TN == 4) : ((TM == 2 && (TN == 4 || TN == 8)) || (TM == 4 && TN == 8));
 }
+// Tiles that are also built with two or four thread groups, which share the input channels.
+inline bool strip_split_built(int TM, int TN, int KS, bool generic) { return !generic && TM == 2 && (KS == 2 || (KS == 4 && TN == 4)); }
 // 8-byte entries of a thread in the second-accumulator area: TM TN and one that keeps the pitch odd.
 __host__ __device__ constexpr int strip_e_pitch(int TM, int TN) { return TM * TN + 1; }
 // Is there a kernel with unrolled loops for (N, K, J), and does it add the upper slots to the next word while packed?

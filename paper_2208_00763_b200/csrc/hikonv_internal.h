@@ -59,6 +59,9 @@ SplitConsts make_split_consts(const hikonv_layout_t &L, int p, int q, int f_sign
 // or 0 when the layout has no room.  packed_add: the slots above the N low ones are added to the next word's low slots while
 // both accumulators are still packed, so a low slot has to hold its own sum and the one that comes in.
 int move_period(const hikonv_layout_t &L, const SplitConsts &sc, int p, int q, int f_signed, int g_signed, int K, int Ci, bool packed_add);
+// 2-D, layers with moves whose input channels up to `groups` groups of threads share: the most moves they may make together (one
+// after a group's last channel included) with cf channels between two, or 0 when the groups' sums may not be added while packed.
+int most_split_moves(const hikonv_layout_t &L, const SplitConsts &sc, int p, int q, int f_signed, int g_signed, int K, int cf, int groups, bool packed_add);
 
 inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 

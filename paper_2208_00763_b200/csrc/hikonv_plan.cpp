@@ -507,6 +507,29 @@ int move_period(const hikonv_layout_t &L, const SplitConsts &sc, int p, int q, i
     return 0;
 }
 
+int most_split_moves(const hikonv_layout_t &L, const SplitConsts &sc, int p, int q, int fs, int gs, int K, int cf, int groups, bool packed_add) {
+    const Range fr = code_range(p, fs ? 1 : 0), gr = code_range(q, gs ? 1 : 0);
+    const long long prods[4] = {fr.lo * gr.lo, fr.lo * gr.hi, fr.hi * gr.lo, fr.hi * gr.hi};
+    const long long pmax = *std::max_element(prods, prods + 4);
+    int T[kMaxSegments];
+    term_counts(L, K, T);
+    const int h = L.carry_bits;
+    const long long low = (1LL << h) - 1;
+    long long moves = 1LL << h;
+    for (int m = 0; m < L.segments; ++m) {
+        // after the last moves a slot of the sum holds its bias and the low bits of all groups; with the upper slots added, of both slots
+        const long long room = (1LL << (m == L.segments - 1 ? L.top_bits : L.S)) - 1;
+        long long q_sum = 0, e_one = 0;
+        for (int i = m; i < L.segments; i += packed_add ? L.N : L.segments) {
+            q_sum += sc.seg_bias[i] + groups * low;
+            e_one += (low + sc.seg_bias[i] + (long long)cf * K * T[i] * pmax) >> h;
+        }
+        if (q_sum > room) return 0;
+        if (e_one > 0) moves = std::min(moves, room / e_one);
+    }
+    return (int)moves;
+}
+
 }  // namespace hikonv
 
 using namespace hikonv;

@@ -94,6 +94,40 @@ def test_strips_of_rows_in_every_tile(K, pad):
                 assert_exact(got, ref, "%s K=%d p=%d q=%d tile=%d" % ((B, Ci, H, W, Co), K, p, q, tile))
 
 
+@pytest.mark.parametrize("K, pad", [(1, 0), (3, 1), (5, 2), (5, 4)])
+def test_input_channels_shared_by_thread_groups(K, pad):
+    # two and four thread groups per tile: channel counts that leave the last groups short or idle in the last stage, few and many
+    # moves of the second accumulators, ragged strips, several images and row segments, sums and pooled codes, largest sums
+    taken = 0
+    for (B, Ci, H, W, Co) in ((3, 9, 8, 10, 9), (1, 41, 6, 150, 5), (2, 70, 10, 20, 20), (5, 17, 6, 4, 33), (1, 130, 4, 8, 8)):
+        for (p, q, xs, ws) in ((4, 4, True, True), (4, 4, False, True), (8, 8, True, True), (2, 2, False, True), (8, 4, False, True), (6, 6, False, False)):
+            x, w = inputs.conv2d_case(B, Ci, H, W, Co, K, p, q, xs, ws, seed=60 + B + Ci + K + p)
+            ref = direct.conv2d_nchw(x, w, pad)
+            d_x, d_w = dev(x), dev(w)
+            for tile in (20000000, 24202002, 28201000, 40000000, 44202000):
+                what = "%s K=%d p=%d q=%d tile=%d" % ((B, Ci, H, W, Co), K, p, q, tile)
+                try:
+                    assert_exact(hk.conv2d(d_x, d_w, pad, p, q, xs, ws, tune={"tile": tile}), ref, what)
+                except hk.HikonvError as err:          # layouts without such a kernel or without room for the groups' sums
+                    assert err.status == hk.ERR_UNSUPPORTED
+                    continue
+                taken += 1
+                if ref.shape[2] % 2 == 0 and ref.shape[3] % 2 == 0:
+                    got = hk.conv2d_dense(d_x.reshape(-1), x.shape, 8, d_w.reshape(-1), w.shape, 8, pad, p, q, xs, ws, requant=(p, 0, 15), pool=True,
+                                          tune={"tile": tile})
+                    assert_exact(got, direct.maxpool2x2(direct.requant(ref, p, 0, 15)), "pool " + what)
+    assert taken >= 40
+    for bits, signed in ((4, True), (4, False), (8, True)):
+        for x, w in inputs.extreme_2d(1, 70, 6, 10, 8, K, bits, bits, signed, True):
+            for tile in (20000000, 40000000):
+                try:
+                    got = _layer(x, w, pad, bits, bits, signed, True, hk.ALGO_PACKED32, tune={"tile": tile})
+                except hk.HikonvError as err:
+                    assert err.status == hk.ERR_UNSUPPORTED
+                    continue
+                assert_exact(got, direct.conv2d_nchw(x, w, pad), "extreme bits=%d tile=%d" % (bits, tile))
+
+
 @pytest.mark.parametrize("K, pad", [(1, 0), (3, 1), (3, 0), (3, 2), (5, 2)])
 def test_small_layers_in_one_launch(K, pad):
     # tile = -2: operands packed by the layer kernel, input channels shared by the CTAs of a cluster; channel counts that cut
