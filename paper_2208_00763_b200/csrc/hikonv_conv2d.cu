@@ -76,6 +76,7 @@ __device__ __forceinline__ void pack_weight_words(const WeightPackParams &q, int
 
 // corr[k][co] = x_off * sum_{ci, kh, kw < k} W[co][ci][kh][kw], k = 0 .. K: one CTA per output channel, so that the few loads
 // of a thread are all in flight together (one warp per channel, a load at a time, was the longest part of the launch).
+template <int CTAS>
 __device__ __forceinline__ void sum_channel_weights(const WeightPackParams &q, int co, int tid) {
     __shared__ int32_t s_part[8][4];
     const int rows = q.Ci * q.K;
@@ -84,7 +85,7 @@ __device__ __forceinline__ void sum_channel_weights(const WeightPackParams &q, i
     for (int k0 = 0; k0 < q.K; k0 += 4) {
         int32_t sum[4] = {0, 0, 0, 0};
         if (co < q.Co) {
-#pragma unroll 4
+#pragma unroll(CTAS == 3 ? 4 : 1)
             for (int r = tid; r < rows; r += 256) {
                 const size_t e = ((size_t)co * rows + r) * q.K + k0;
 #pragma unroll
@@ -131,8 +132,13 @@ struct ActPackDivs {
     Div32 per_plane, b, xq;    // pieces per (ci, b) plane, images, 16-byte pieces per packed row
 };
 
-template <bool XS, int N>
-__global__ void __launch_bounds__(256) pack_operands_kernel(const int8_t *__restrict__ x, int B, int Ci, int H, int W, int Hp,
+// CTAS: CTAs that fit an SM by their registers.  The loads of a thread come in one group and all of a CTA's together, so a large
+// launch wants as many warps as an SM holds: with three CTAs (80 registers) the first layer of the compact CNN (4984 CTAs) took
+// 17.2 us, with eight 10.7 (32 images of 64x56x56: 11.4 and 7.6).  A launch of few CTAs starts while the kernel before it still
+// runs, and with eight they pile up on the SMs that are free first: 24x45x61 and 48x37x53 layers took 31.1 and 27.2 us a call
+// instead of 29.8 and 26.3.
+template <bool XS, int N, int CTAS>
+__global__ void __launch_bounds__(256, CTAS) pack_operands_kernel(const int8_t *__restrict__ x, int B, int Ci, int H, int W, int Hp,
                                                             int pad, int col_first, int S, int XBT,
                                                             uint32_t *__restrict__ ap, int weight_blocks, const WeightPackParams wq,
                                                             int x_bits, const ActPackDivs dv, unsigned act_items) {
@@ -141,7 +147,7 @@ __global__ void __launch_bounds__(256) pack_operands_kernel(const int8_t *__rest
     // the first CTAs sum the channels' weights (the longest serial work of the launch) and pack the kernel rows
     if ((int)blockIdx.x < weight_blocks) {
         const int cb = weight_blocks - wq.w_blocks;                  // CTAs that sum weights (0 unless x_off != 0)
-        if ((int)blockIdx.x < cb) sum_channel_weights(wq, (int)blockIdx.x, (int)threadIdx.x);
+        if ((int)blockIdx.x < cb) sum_channel_weights<CTAS>(wq, (int)blockIdx.x, (int)threadIdx.x);
         else pack_weight_words(wq, ((int)blockIdx.x - cb) * 8 + ((int)threadIdx.x >> 5), (int)threadIdx.x & 31);
         return;
     }
@@ -751,9 +757,13 @@ static int conv2d_run(const void *d_x, int x_bits, int B, int Ci, int H, int W, 
         dv.per_plane = make_div32((uint32_t)(s.Hp * (s.XBT / 4)));
         dv.b = make_div32((uint32_t)B);
         dv.xq = make_div32((uint32_t)(s.XBT / 4));
-#define HK_PACK(XSIGN, NN)                                                                                                 \
-    rc = launch_dependent(pack_operands_kernel<XSIGN, NN>, dim3(grid), dim3(256), 0, st, (const int8_t *)d_x, B, Ci, H, W, s.Hp, \
-                          pad, s.col_first, s.L.S, s.XBT, d_ap, (int)(w_blocks + corr_blocks), wq, x_bits, dv, (unsigned)act_items)
+        // (10 CTAs per SM are faster in the first way, 3 in the second)
+        const bool many = grid > 6u * (unsigned)sm_count();
+        auto pack = [&](auto kern) {
+            return launch_dependent(kern, dim3(grid), dim3(256), 0, st, (const int8_t *)d_x, B, Ci, H, W, s.Hp, pad, s.col_first, s.L.S,
+                                    s.XBT, d_ap, (int)(w_blocks + corr_blocks), wq, x_bits, dv, (unsigned)act_items);
+        };
+#define HK_PACK(XSIGN, NN) rc = many ? pack(pack_operands_kernel<XSIGN, NN, 8>) : pack(pack_operands_kernel<XSIGN, NN, 3>)
         switch (s.L.N * 2 + (x_signed || s.x_off ? 1 : 0)) {
             case 2: HK_PACK(false, 1); break;
             case 3: HK_PACK(true, 1); break;

@@ -32,9 +32,9 @@
 // instructions) takes 473 cycles, of a 2 x 8 tile with moves (48 and 52) 285.  Three CTAs per SM, operand rows in registers
 // across channels or a compile-time distance between channels (no pointer arithmetic left) changed neither.
 // Measured against the kernel before it (four positions of one row per thread, one halo word per row, run-time loops for 5x5),
-// packing launch included: 32x64x56x56 -> 64 s4 93.3 -> 85.4 us, 64x256x14x14 -> 256 u4 x s4 211 -> 162 us (205 with the new
-// packing launch alone), 8x48x37x53 -> 40 s8 32.4 -> 26.4 us, 16x24x45x61 -> 40 5x5 2-bit 70.6 -> 30.0 us, the compact CNN
-// (batch 64) 605 -> 484 us.
+// packing launch included: 32x64x56x56 -> 64 s4 93.3 -> 84.6 us, 64x256x14x14 -> 256 u4 x s4 211 -> 160 us (205 with the new
+// packing launch alone), 8x48x37x53 -> 40 s8 32.4 -> 26.3 us, 16x24x45x61 -> 40 5x5 2-bit 70.6 -> 30.0 us, the compact CNN
+// (batch 64) 605 -> 475 us.
 #pragma once
 
 #include <type_traits>

@@ -128,6 +128,15 @@ def test_input_channels_shared_by_thread_groups(K, pad):
                 assert_exact(got, direct.conv2d_nchw(x, w, pad), "extreme bits=%d tile=%d" % (bits, tile))
 
 
+@pytest.mark.parametrize("p, q, xs, ws", [(4, 4, True, True), (4, 4, False, True), (8, 8, True, True), (8, 4, False, True), (2, 2, False, False)])
+def test_packing_launch_of_many_blocks(p, q, xs, ws):
+    # more than six blocks per SM pack the activations (layers below that run the packing kernel with fewer per SM): odd row width
+    # and alignment, shifted codes from 128 channels on, one channel per block and several
+    for (B, Ci, H, W, Co, K, pad) in ((9, 130, 61, 61, 3, 1, 0), (4, 31, 160, 321, 2, 3, 1)):
+        x, w = inputs.conv2d_case(B, Ci, H, W, Co, K, p, q, xs, ws, seed=90 + p)
+        assert_exact(_layer(x, w, pad, p, q, xs, ws, hk.ALGO_PACKED32), direct.conv2d_nchw(x, w, pad), "%s p=%d q=%d" % ((B, Ci, H, W), p, q))
+
+
 @pytest.mark.parametrize("K, pad", [(1, 0), (3, 1), (3, 0), (3, 2), (5, 2)])
 def test_small_layers_in_one_launch(K, pad):
     # tile = -2: operands packed by the layer kernel, input channels shared by the CTAs of a cluster; channel counts that cut
