@@ -53,7 +53,7 @@ NCU_TRAFFIC = {
 
 
 # Warp instructions one launch of the packed layer kernel executes (smsp__inst_executed.sum of the captures behind
-# profiles/conv2d_kernel_c3.txt and _c4.txt), for the issue model of the 2-D rooflines; void when the source changes.
+# profiles/conv2d_strip_kernel_c3.txt and _c4.txt), for the issue model of the 2-D rooflines; void when the source changes.
 NCU_INSTRUCTIONS = {
     "c3": {"sha256": "dd5f48402620b0de3ccab755f40e1210a87800596c3d25131297b506941b6beb", "warp_instructions": 41575448.0},
     "c4": {"sha256": "dd5f48402620b0de3ccab755f40e1210a87800596c3d25131297b506941b6beb", "warp_instructions": 87595968.0},
@@ -581,7 +581,7 @@ def run_layer_main(args, torch, np, ranks, hk, inputs, network, dev, world, rank
     }
     if muls is not None:
         line["roofline"] = alu_roofline(muls, ms, imad_peak, args.algo, args.workload)
-        line["roofline"]["kernel"] = "conv2d_kernel" + (" (nine layer launches, multiplies summed)" if args.workload == "c5" else "")
+        line["roofline"]["kernel"] = "conv2d_strip_kernel" + (" (nine layer launches, multiplies summed)" if args.workload == "c5" else "")
     if rank == 0:
         print(json.dumps(line), flush=True)
     ranks.shutdown()
@@ -604,7 +604,7 @@ def alu_roofline(muls: float, ms: float, imad_peak: dict, key: str, workload: st
     # instruction of the layer kernel (counted under ncu); the sum over the device's schedulers is the time the layer
     # kernel cannot go below with this instruction mix, to be read against the step (which also holds the packing launch).
     rec, issue = NCU_INSTRUCTIONS.get(workload or ""), imad_peak.get("issue")
-    if key == "packed" and rec and issue and rec["sha256"] == _source_hash("hikonv_conv2d.cu"):
+    if key == "packed" and rec and issue and rec["sha256"] == _source_hash("hikonv_conv2d_strip.cuh"):
         mads = muls / 32.0
         others = rec["warp_instructions"] - mads
         cycles = issue["cycles_per_wide_multiply_add"] * mads + issue["cycles_added_per_other_instruction"] * others
