@@ -40,23 +40,23 @@ TABLE_REPEATS = 7                    # timed repeats per cell of the per-case ta
 
 # dram__bytes_read.sum + dram__bytes_write.sum per launch from the last ncu capture of the kernel: six
 # consecutive launches of the p=q=4, K=3 signed case at 2^24 rotating over three input and three output
-# buffers, caches not flushed between launches (steady state): 12.5-13.4 MB read, 62.9-66.1 MB written
+# buffers, caches not flushed between launches (steady state): 13.1-13.7 MB read, 63.1-66.2 MB written
 # (the 8-bit K=7 case: 79.9 MB in all).  (With the caches flushed before each launch the same kernel shows
 # 16.8 MB read and 8-9 MB written: most of a launch's output is then still in the 126 MB L2 when its
 # counters stop.)  The SHA-256 values are those of the kernel sources at capture time; a changed source voids
 # the figure.
 NCU_TRAFFIC = {
-    "conv1d_bs": {"sha256": "36e8f9ed30e2667834955a0cfb06cb0462a71beae17cbcfc024e007a0ee74fd9",
-                  "sha256_run": "322f9167bd95031f2841bdd2e540d4bd24431054ad2d45e0ce1474457f5564c2",
-                  "bytes_per_output": (13.08e6 + 65.07e6) / 16777218.0},
+    "conv1d_bs": {"sha256": "5655bc948411944c895bc88fbc1ce61e93428afcd63aa7d4740d6c3f16a0914b",
+                  "sha256_run": "b59f92e42efa632279f0ce0a71b93fe1bf792a1fa715e00ef8575d0a99e2e512",
+                  "bytes_per_output": (13.37e6 + 65.20e6) / 16777218.0},
 }
 
 
 # Warp instructions one launch of the packed layer kernel executes (smsp__inst_executed.sum of the captures behind
 # profiles/conv2d_strip_kernel_c3.txt and _c4.txt), for the issue model of the 2-D rooflines; void when the source changes.
 NCU_INSTRUCTIONS = {
-    "c3": {"sha256": "dd5f48402620b0de3ccab755f40e1210a87800596c3d25131297b506941b6beb", "warp_instructions": 41575448.0},
-    "c4": {"sha256": "dd5f48402620b0de3ccab755f40e1210a87800596c3d25131297b506941b6beb", "warp_instructions": 87595968.0},
+    "c3": {"sha256": "f49f0bd00385c1ffeffe5b882f52dc2b78c9a828c16bd6084420e0526e7da9ff", "warp_instructions": 34620336.0},
+    "c4": {"sha256": "f49f0bd00385c1ffeffe5b882f52dc2b78c9a828c16bd6084420e0526e7da9ff", "warp_instructions": 64448064.0},
 }
 
 
@@ -543,7 +543,7 @@ def run_layer_main(args, torch, np, ranks, hk, inputs, network, dev, world, rank
 
         def step():
             net.forward(d_x, algo=algo)
-        launches_per_step = 2 * 9       # nine layers of two launches (packing + layer; the four pools run inside their layers)
+        launches_per_step = 2 * 9       # nine layers of two launches (packing + layer; the four pools run inside their layers; none runs in one launch)
         name = ("c5: compact 4-bit CNN, batch %d, 3x160x320, 8 conv3x3 + 4 pools + 1x1 head; tiles %s: %s"
                 % (x.shape[0], {"tune": "timed once at set-up", "auto": "the library's own"}.get(args.c5_tiles, "given"),
                    [t["tile"] if t else None for t in tiles]))
