@@ -47,7 +47,7 @@ TABLE_REPEATS = 7                    # timed repeats per cell of the per-case ta
 # the figure.
 NCU_TRAFFIC = {
     "conv1d_bs": {"sha256": "5655bc948411944c895bc88fbc1ce61e93428afcd63aa7d4740d6c3f16a0914b",
-                  "sha256_run": "b59f92e42efa632279f0ce0a71b93fe1bf792a1fa715e00ef8575d0a99e2e512",
+                  "sha256_run": "ff003dacc21c948f04a6b5e0ee717c8420ab96ffc1c03d52a54906dad43f8413",
                   "bytes_per_output": (13.37e6 + 65.20e6) / 16777218.0},
 }
 
