@@ -55,8 +55,8 @@ NCU_TRAFFIC = {
 # Warp instructions one launch of the packed layer kernel executes (smsp__inst_executed.sum of the captures behind
 # profiles/conv2d_strip_kernel_c3.txt and _c4.txt), for the issue model of the 2-D rooflines; void when the source changes.
 NCU_INSTRUCTIONS = {
-    "c3": {"sha256": "f49f0bd00385c1ffeffe5b882f52dc2b78c9a828c16bd6084420e0526e7da9ff", "warp_instructions": 34620336.0},
-    "c4": {"sha256": "f49f0bd00385c1ffeffe5b882f52dc2b78c9a828c16bd6084420e0526e7da9ff", "warp_instructions": 64448064.0},
+    "c3": {"sha256": "ab2d80e5c86d7fc3753e0f7e7e1d1d5262fe17f15767e58466568c621eb0dc10", "warp_instructions": 34620336.0},
+    "c4": {"sha256": "ab2d80e5c86d7fc3753e0f7e7e1d1d5262fe17f15767e58466568c621eb0dc10", "warp_instructions": 64448064.0},
 }
 
 

@@ -337,6 +337,13 @@ int hikonv_conv2d_static_scratch(const int8_t *d_x, int B, int Ci, int H, int W,
                                  int requant, int shift, int lo, int hi, int algo, const hikonv_tuning_t *tune,
                                  void *stream);
 
+/*
+ * hikonv_conv2d_wait_timeouts - threads of 2-D layer kernels on the current device whose wait for their own operand copies ran
+ * out (a limit far above any copy's time) since the last call; 0 unless the device is at fault, and the layers since then
+ * are not to be trusted otherwise.  A debug aid; synchronises the device and clears the count.
+ */
+int hikonv_conv2d_wait_timeouts(unsigned int *h_count);
+
 /* Device scratch needed by hikonv_conv2d_host: x, w, out and the kernel workspace. */
 size_t hikonv_conv2d_host_workspace_bytes(int B, int Ci, int H, int W, int Co, int K, int pad, int requant);
 

@@ -67,6 +67,7 @@ _SIGNATURES = {
     "hikonv_conv2d_tune": (_i, [_vp, _i, _i, _i, _i, _i, _vp, _i, _i, _i, _i, _i, _i, _i, _i, _i, _vp, _i, _i, _i, _i, _i, _i, _vp, _sz,
                                 _i, _i, ctypes.POINTER(_i), ctypes.POINTER(_d), ctypes.POINTER(_d), _vp]),
     "hikonv_conv2d_workspace_bytes": (_sz, [_i] * 7),
+    "hikonv_conv2d_wait_timeouts": (_i, [_vp]),
     "hikonv_conv2d_static_scratch": (_i, [_vp, _i, _i, _i, _i, _vp, _i, _i, _i, _i, _i, _i, _i, _i, _vp, _i, _i, _i, _i, _i,
                                           ctypes.POINTER(TuningT), _vp]),
     "hikonv_conv2d_host_workspace_bytes": (_sz, [_i] * 8),
@@ -235,6 +236,13 @@ def check_range(d_in: torch.Tensor, bits: int, is_signed: bool, stream=None) -> 
         _check(rc, "hikonv_check_range")
     assert (rc == ERR_RANGE) == (found.value > 0)
     return int(found.value)
+
+
+def conv2d_wait_timeouts() -> int:
+    """Waits of 2-D layer kernels on the current device that ran out since the last call (0 on a healthy device).  Synchronises."""
+    count = ctypes.c_uint(0)
+    _check(lib().hikonv_conv2d_wait_timeouts(ctypes.byref(count)), "hikonv_conv2d_wait_timeouts")
+    return int(count.value)
 
 
 def conv1d(d_f: torch.Tensor, d_g: torch.Tensor, p: int, q: int, f_signed: bool, g_signed: bool,

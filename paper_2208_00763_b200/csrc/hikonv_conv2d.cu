@@ -781,6 +781,22 @@ static int conv2d_run(const void *d_x, int x_bits, int B, int Ci, int H, int W, 
     return launch_layer(s, st);
 }
 
+extern "C" int hikonv_conv2d_wait_timeouts(unsigned int *h_count) {
+    if (!h_count) return HIKONV_ERR_INVALID_ARG;
+    static int (*const counters[])(unsigned int *) = {
+        strip_wait_timeouts<1, 0, 0>, strip_wait_timeouts<2, 1, 1>, strip_wait_timeouts<3, 1, 1>, strip_wait_timeouts<4, 1, 1>,
+        strip_wait_timeouts<2, 3, 1>, strip_wait_timeouts<2, 3, 2>, strip_wait_timeouts<3, 3, 1>, strip_wait_timeouts<4, 3, 1>,
+        strip_wait_timeouts<2, 5, 3>, strip_wait_timeouts<3, 5, 2>, strip_wait_timeouts<4, 5, 1>, strip_wait_timeouts<4, 5, 2>};
+    *h_count = 0;
+    for (auto counter : counters) {
+        unsigned int n = 0;
+        const int rc = counter(&n);
+        if (rc != HIKONV_OK) return rc;
+        *h_count += n;
+    }
+    return HIKONV_OK;
+}
+
 extern "C" int hikonv_conv2d(const int8_t *d_x, int B, int Ci, int H, int W, const int8_t *d_w, int Co, int K, int stride,
                              int pad, int p, int q, int x_signed, int w_signed, void *d_out, int requant, int shift, int lo,
                              int hi, void *d_workspace, size_t workspace_bytes, int algo, const hikonv_tuning_t *tune,

@@ -45,6 +45,9 @@
 
 namespace hikonv {
 
+// Threads of this file's kernels whose wait for a stage ran out (one counter per file; read and cleared by strip_wait_timeouts).
+static __device__ unsigned int strip_timeouts;
+
 template <int N, int KT, int JT>
 constexpr bool kStripPackedAdd = strip_packed_add(N, KT, JT);
 
@@ -217,8 +220,9 @@ __global__ void __launch_bounds__(kStripThreads, 2) conv2d_strip_kernel(const __
         const int ckn = min(p.CK, p.Ci - ci0);
         // the groups' shares of a stage (the last ones' may be shorter; moves happen at the same places in all)
         const int share = (ckn + KS - 1) / KS, own = min(ckn - group * share, share);
-        // this stage has landed (were the wait ever to run out, the sums would be wrong but nothing would hang)
-        mbarrier_wait(bar0 + 8u * stage, parity);
+        // this stage has landed (were the wait ever to run out, the sums would be wrong, and counted as such, but nothing would hang;
+        // later stages and the other buffer are still waited for, with the same limit)
+        if (!mbarrier_wait(bar0 + 8u * stage, parity)) atomicAdd(&strip_timeouts, 1u);
         cp_async_wait_all();
         parity ^= (uint32_t)stage;
         __syncthreads();                                       // the previous stage is fully consumed
@@ -499,6 +503,14 @@ static int launch_strip_tile(const StripLaunch &s, cudaStream_t st) {
     };
     if (s.moves) return s.sp ? run(conv2d_strip_kernel<N, KT, JT, TM, TN, true, true, KS>) : run(conv2d_strip_kernel<N, KT, JT, TM, TN, false, true, KS>);
     return s.sp ? run(conv2d_strip_kernel<N, KT, JT, TM, TN, true, false, KS>) : run(conv2d_strip_kernel<N, KT, JT, TM, TN, false, false, KS>);
+}
+
+template <int N, int KT, int JT>
+int strip_wait_timeouts(unsigned int *h_count) {
+    const unsigned int zero = 0;
+    if (cudaMemcpyFromSymbol(h_count, strip_timeouts, sizeof(zero)) != cudaSuccess) return HIKONV_ERR_CUDA;
+    if (*h_count != 0 && cudaMemcpyToSymbol(strip_timeouts, &zero, sizeof(zero)) != cudaSuccess) return HIKONV_ERR_CUDA;
+    return HIKONV_OK;
 }
 
 template <int N, int KT, int JT>

@@ -4,6 +4,7 @@
 namespace hikonv {
 
 template int launch_strip<1, 0, 0>(const StripLaunch &s, cudaStream_t st);
+template int strip_wait_timeouts<1, 0, 0>(unsigned int *h_count);
 template int launch_strip<2, 0, 0>(const StripLaunch &s, cudaStream_t st);
 template int launch_strip<3, 0, 0>(const StripLaunch &s, cudaStream_t st);
 template int launch_strip<4, 0, 0>(const StripLaunch &s, cudaStream_t st);

@@ -4,5 +4,6 @@
 namespace hikonv {
 
 template int launch_strip<2, 3, 2>(const StripLaunch &s, cudaStream_t st);
+template int strip_wait_timeouts<2, 3, 2>(unsigned int *h_count);
 
 }  // namespace hikonv

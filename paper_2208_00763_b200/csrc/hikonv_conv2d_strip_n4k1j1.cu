@@ -4,5 +4,6 @@
 namespace hikonv {
 
 template int launch_strip<4, 1, 1>(const StripLaunch &s, cudaStream_t st);
+template int strip_wait_timeouts<4, 1, 1>(unsigned int *h_count);
 
 }  // namespace hikonv

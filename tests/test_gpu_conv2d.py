@@ -135,6 +135,7 @@ def test_packing_launch_of_many_blocks(p, q, xs, ws):
     for (B, Ci, H, W, Co, K, pad) in ((9, 130, 61, 61, 3, 1, 0), (4, 31, 160, 321, 2, 3, 1)):
         x, w = inputs.conv2d_case(B, Ci, H, W, Co, K, p, q, xs, ws, seed=90 + p)
         assert_exact(_layer(x, w, pad, p, q, xs, ws, hk.ALGO_PACKED32), direct.conv2d_nchw(x, w, pad), "%s p=%d q=%d" % ((B, Ci, H, W), p, q))
+    assert hk.conv2d_wait_timeouts() == 0
 
 
 @pytest.mark.parametrize("K, pad", [(1, 0), (3, 1), (3, 0), (3, 2), (5, 2)])
