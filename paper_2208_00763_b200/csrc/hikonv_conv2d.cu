@@ -576,7 +576,8 @@ static int plan_layer(int B, int Ci, int H, int W, int Co, int K, int stride, in
         for (int m = 0; m < 8; ++m) k.slot_bias[m] = m < L.segments ? sc.seg_bias[m] : 0;
         k.up_slots = L.segments - L.N;
         k.requant = out.requant ? 1 : 0; k.shift = out.shift; k.lo = out.lo; k.hi = out.hi;
-        k.pool = pr.pool ? 1 : 0; k.out_bits = out.out_bits; k.out_signed = out.lo < 0 ? 1 : 0;
+        k.pool = !pr.pool ? 0 : out.lo < 0 && out.hi > 127 ? 2 : 1;   // 2: the bytes of codes above 127 are negative
+        k.out_bits = out.out_bits; k.out_signed = out.lo < 0 ? 1 : 0;
         rc = output_staging(out, Ho, Wo, c.NSEG, c.XO * L.N, &k.stage_out, &k.vec);
         if (rc != HIKONV_OK) return rc;
         k.WTP = (c.XO * L.N + 15) / 16 * 16;

@@ -230,8 +230,12 @@ __global__ void __launch_bounds__(kStripThreads, 2) conv2d_small_kernel(const __
         for (int t = 0; t < TN; ++t)
             if (((2 * t) >> share_log2) == rank) {
 #pragma unroll
-                for (int m = 0; m < N; ++m)
-                    if (col_ok[m]) tile[(tn * TN + t) * tile_chan + sl * p.WTP + w0 + m] = (int8_t)requant(max(y[0][t][m], y[1][t][m]));
+                for (int m = 0; m < N; ++m) {
+                    // (codes from below 0 to above 127: the maximum of the bytes, as they are stored)
+                    const int32_t v = p.pool == 2 ? max((int32_t)(int8_t)requant(y[0][t][m]), (int32_t)(int8_t)requant(y[1][t][m]))
+                                                  : requant(max(y[0][t][m], y[1][t][m]));
+                    if (col_ok[m]) tile[(tn * TN + t) * tile_chan + sl * p.WTP + w0 + m] = (int8_t)v;
+                }
             }
         __syncthreads();
         const int nt_log2 = share_log2 - 1;                    // channels of a thread that this CTA finishes

@@ -412,14 +412,15 @@ __global__ void __launch_bounds__(kStripThreads, 2) conv2d_strip_kernel(const __
     }
 
     // ---- requantised codes staged as bytes [channel][row][column]; with a pool the two rows of a pair are reduced first (the
-    // shift and the clamp keep the order, so the maximum is taken before them)
+    // shift and the clamp keep the order, so the maximum is taken before them; only a clamp range that reaches from below 0 to
+    // above 127 does not, because the codes above 127 are negative bytes: pool == 2, the maximum of the bytes)
     int8_t *tile = reinterpret_cast<int8_t *>(smem + p.tile_off);
     const int rps = p.pool ? TM / 2 : TM;                      // tile rows per strip
     const int tile_chan = p.TS * rps * p.WTP;
     const int col0 = seg * p.XO * N;                           // first output column of the segment (segments: col_off == 0)
     int8_t *tile_at = tile + ch0 * tile_chan + sl * rps * p.WTP + w0 - col0;
     auto stage_codes = [&](auto pool_tag) {
-        constexpr bool POOL = decltype(pool_tag)::value;
+        constexpr int POOL = decltype(pool_tag)::value;
 #pragma unroll
         for (int t = 0; t < TE; ++t) {
             int32_t off[N], y[N], y2[N];
@@ -430,16 +431,18 @@ __global__ void __launch_bounds__(kStripThreads, 2) conv2d_strip_kernel(const __
                 if constexpr (POOL) {
                     split(i + 1, t, off, y2);
 #pragma unroll
-                    for (int m = 0; m < N; ++m) y[m] = max(y[m], y2[m]);
+                    for (int m = 0; m < N; ++m)
+                        y[m] = POOL == 2 ? max((int32_t)(int8_t)requant(y[m]), (int32_t)(int8_t)requant(y2[m])) : max(y[m], y2[m]);
                 }
 #pragma unroll
                 for (int m = 0; m < N; ++m)
-                    if (col_ok[m]) tile_at[t * tile_chan + (POOL ? i / 2 : i) * p.WTP + m] = (int8_t)requant(y[m]);
+                    if (col_ok[m]) tile_at[t * tile_chan + (POOL ? i / 2 : i) * p.WTP + m] = (int8_t)(POOL == 2 ? y[m] : requant(y[m]));
             }
         }
     };
-    if (p.pool) stage_codes(std::true_type());
-    else stage_codes(std::false_type());
+    if (p.pool == 1) stage_codes(std::integral_constant<int, 1>());
+    else if (p.pool) stage_codes(std::integral_constant<int, 2>());
+    else stage_codes(std::integral_constant<int, 0>());
     __syncthreads();
 
     // ---- staged codes leave the CTA in pieces of `vec` bytes along a row, neighbouring columns reduced first with a pool

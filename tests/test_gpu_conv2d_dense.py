@@ -7,7 +7,7 @@ import torch
 from oracle import direct
 from paper_2208_00763_b200 import binding as hk
 from paper_2208_00763_b200 import inputs
-from gpu_util import assert_exact
+from gpu_util import assert_exact, dev
 
 pytestmark = pytest.mark.gpu
 
@@ -127,3 +127,20 @@ def test_refusals():
     x3, w3 = inputs.conv2d_case(1, 4, 6, 8, 4, 3, 3, 3, False, False, seed=2)
     with pytest.raises(hk.HikonvError):      # 3-bit codes straddle bytes: no dense format
         hk.conv2d_dense(_store(x3, 3, 8), x3.shape, 3, _store(w3, 3, 8), w3.shape, 8, 1, 3, 3, False, False)
+
+
+@pytest.mark.parametrize("K, pad, tile", [(3, 1, 0), (3, 1, -1), (1, 0, -2), (5, 2, -1), (7, 3, 0), (3, 1, 20000000)])
+def test_pool_of_codes_whose_bytes_wrap(K, pad, tile):
+    # a clamp range from below 0 to above 127: codes above 127 are stored as negative bytes, and the fused pool takes the maximum
+    # of the stored bytes (as the layer followed by maxpool2x2_i8 does), rows of a window included
+    for (B, Ci, H, W, Co) in ((2, 9, 8, 12, 6), (1, 40, 6, 70, 9)):
+        x, w = inputs.conv2d_case(B, Ci, H, W, Co, K, 4, 4, True, True, seed=400 + K + Ci)
+        acc = direct.conv2d_nchw(x, w, pad)
+        for (shift, lo, hi) in ((0, -128, 255), (0, -8, 200), (1, -1, 128)):
+            codes = direct.requant(acc, shift, lo, hi).astype(np.int64)
+            want = direct.maxpool2x2((codes + 128) % 256 - 128)
+            assert (codes < 0).any() and ((codes > 127).any() or shift > 0)
+            for algo in (hk.ALGO_PACKED32, hk.ALGO_UNPACKED_IMAD):
+                got = hk.conv2d_dense(dev(x).reshape(-1), x.shape, 8, dev(w).reshape(-1), w.shape, 8, pad, 4, 4, True, True,
+                                      requant=(shift, lo, hi), pool=True, algo=algo, tune={"tile": tile if algo == hk.ALGO_PACKED32 else 0})
+                assert_exact(got, want, "%s K=%d %s tile=%d algo=%d" % ((B, Ci, H, W, Co), K, (shift, lo, hi), tile, algo))
