@@ -31,7 +31,7 @@ struct WeightPackParams {
     int w_blocks;              // CTAs that pack kernel rows, one word per thread; the CTAs before them sum the weights of a channel each (x_off != 0)
     Div32 d_cg, d_j;           // divisions by the number of groups of eight channels and by J
     int x_off;                 // offset taken from every activation code (0: none)
-    int32_t *corr;             // corr[k][co] = x_off * sum of channel co's weights over ci, kh and kw < k; K + 1 rows of CoP entries
+    int32_t *corr;             // corr[k][co] = x_off * sum of channel co's weights over ci, kh and kw <= k; K rows of CoP entries
 };
 
 // Code number e of a tensor stored densely with `bits` (1, 2, 4 or 8) bits per code: code e occupies bits
@@ -74,14 +74,13 @@ __device__ __forceinline__ void pack_weight_words(const WeightPackParams &q, int
     q.wp[(size_t)rj * q.CoP + co] = word;
 }
 
-// corr[k][co] = x_off * sum_{ci, kh, kw < k} W[co][ci][kh][kw], k = 0 .. K: one CTA per output channel, so that the few loads
+// corr[k][co] = x_off * sum_{ci, kh, kw <= k} W[co][ci][kh][kw], k < K: one CTA per output channel, so that the few loads
 // of a thread are all in flight together (one warp per channel, a load at a time, was the longest part of the launch).
 template <int CTAS>
 __device__ __forceinline__ void sum_channel_weights(const WeightPackParams &q, int co, int tid) {
     __shared__ int32_t s_part[8][4];
     const int rows = q.Ci * q.K;
     int32_t run = 0;                                                 // thread 0: the sum over the taps done
-    if (tid == 0) q.corr[co] = 0;
     for (int k0 = 0; k0 < q.K; k0 += 4) {
         int32_t sum[4] = {0, 0, 0, 0};
         if (co < q.Co) {
@@ -109,7 +108,7 @@ __device__ __forceinline__ void sum_channel_weights(const WeightPackParams &q, i
         if (tid == 0) {
             for (int k = 0; k < 4 && k0 + k < q.K; ++k) {
                 for (int w = 0; w < 8; ++w) run += s_part[w][k];
-                q.corr[(size_t)(k0 + k + 1) * q.CoP + co] = run * q.x_off;
+                q.corr[(size_t)(k0 + k) * q.CoP + co] = run * q.x_off;
             }
         }
         __syncthreads();
@@ -242,7 +241,7 @@ struct Conv2dSetup {
     SmallLaunch small;
     StripLaunch strip;    // the packed kernel, or
     UnpackedLaunch un;    // the comparator
-    // packed operands in the workspace: weights [Ci K J][CoP], x_off corrections [K + 1][CoP], activations [Ci][B Hp][XBT]
+    // packed operands in the workspace: weights [Ci K J][CoP], x_off corrections [K][CoP], activations [Ci][B Hp][XBT]
     int CoP, Hp, XBT, col_first, x_off;
     size_t corr_off, wp_bytes, ap_words;
     double positions;     // words multiplied per (ci, kh, j) and output channel
@@ -524,7 +523,8 @@ static int plan_layer(int B, int Ci, int H, int W, int Co, int K, int stride, in
             // about thirteen, shared by the N pixels of a word; the shifted codes are taken for a gain of 7 % or more,
             // always when they put more pixels into a word, else under the depth conditions above
             auto cycles = [&](const hikonv_layout_t &l) { return (l.J * 4.1 + 13.0 / std::min(l.M, Ci * K)) / l.N; };
-            if (make_layout(p, q, 1, ws, K, 2, Ci * K, Wo, tune, &Ls) == HIKONV_OK && cycles(Ls) <= 0.93 * cycles(L) &&
+            // (not with one tap per word, which only a forced layout has: the corrections would not fit the workspace)
+            if (make_layout(p, q, 1, ws, K, 2, Ci * K, Wo, tune, &Ls) == HIKONV_OK && (K == 1 || Ls.J < K) && cycles(Ls) <= 0.93 * cycles(L) &&
                 (Ls.N > L.N || (L.M < Ci * K && (Ci >= 128 || (Ci >= 32 && !small_layer))))) {
                 L = Ls;
                 xs = 1;
@@ -636,7 +636,7 @@ static int plan_layer(int B, int Ci, int H, int W, int Co, int K, int stride, in
         s->positions = (double)B * Ho * c.NSEG * c.XB;
     }
     s->corr_off = align_up((size_t)Ci * K * L.J * s->CoP * sizeof(uint32_t), 256);
-    s->wp_bytes = s->corr_off + (s->x_off ? align_up((size_t)(K + 1) * s->CoP * sizeof(int32_t), 256) : 0);
+    s->wp_bytes = s->corr_off + (s->x_off ? align_up((size_t)K * s->CoP * sizeof(int32_t), 256) : 0);
     s->ap_words = (size_t)Ci * B * s->Hp * s->XBT;
     if (s->ap_words >= 0x7FFFFFFFull || (size_t)Ci * K * L.J * s->CoP >= 0x7FFFFFFFull) return HIKONV_ERR_UNSUPPORTED;
     return HIKONV_OK;
@@ -698,8 +698,10 @@ extern "C" size_t hikonv_conv2d_workspace_bytes(int B, int Ci, int H, int W, int
     if (B < 1 || Ci < 1 || H < 1 || W < 1 || Co < 1 || K < 1 || pad < 0) return 0;
     const long long Ho = (long long)H + 2 * pad - K + 1, Wo = (long long)W + 2 * pad - K + 1;
     if (Ho < 1 || Wo < 1) return 0;
-    // packed kernel rows: at most K words per (ci, kh) row (one tap per word in the comparator), Co rounded up to 4
-    // (plus one int32 per channel: the correction of layers that run unsigned activations as signed ones)
+    // packed kernel rows: at most K words per (ci, kh) row (one tap per word in the comparator), Co rounded up to 4, plus one
+    // int32 per channel.  The K rows of corrections of layers that run unsigned activations as signed ones fit into this:
+    // with K == 1 they are that one row, and with two or more taps per word (plan_layer sees to it) the packed kernel rows leave
+    // Ci K (K - J) >= K - 1 rows free
     const size_t weights = align_up((size_t)Ci * K * K * ((Co + 3) / 4 * 4) * sizeof(uint32_t), 256) +
                            align_up((size_t)((Co + 3) / 4 * 4) * sizeof(int32_t), 256);
     // packed activation rows: at most one word per output pixel plus K halo words per row (the comparator's

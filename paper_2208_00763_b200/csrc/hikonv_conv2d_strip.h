@@ -38,7 +38,7 @@ struct StripParams {
     // output
     int requant, shift, lo, hi;
     int stage_out, pool, out_bits, out_signed, vec, WTP, tile_off;   // pool: 0, 1, or 2 where the stored bytes do not keep the order of the codes
-    const int32_t *corr;             // x_off * (sum of a channel's weights over the taps 0 .. k - 1), [K + 1][CoP]; null when x_off == 0
+    const int32_t *corr;             // x_off * (sum of a channel's weights over the taps 0 .. k), [K][CoP]; null when x_off == 0
     int W, pad;
 };
 

@@ -4,6 +4,8 @@ printed numbers; argument validation returns status codes without touching a GPU
 import ctypes
 import os
 import re
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -353,3 +355,37 @@ def test_tuner_refuses_bad_arguments_before_touching_the_device():
     assert hk.lib().hikonv_conv2d_tune(*args, 0, ctypes.byref(tile), None, None, None) == hk.ERR_INVALID_ARG
     assert hk.lib().hikonv_conv2d_tune(*args, 101, ctypes.byref(tile), None, None, None) == hk.ERR_INVALID_ARG
     assert tile.value == -1
+
+
+_WORKSPACE_PROBE = '''
+import ctypes, random, sys
+from paper_2208_00763_b200 import binding as hk
+lib = hk.lib()
+shapes = [(1, 16, 1, 1, 512, 1, 0), (1, 12, 1, 1, 241, 1, 0), (1, 4, 6, 6, 482, 1, 0), (1, 3, 13, 3, 779, 1, 0), (1, 64, 1, 1, 1280, 1, 0),
+          (1, 1, 1, 1, 4, 1, 0), (1, 130, 1, 1, 2000, 3, 1), (1, 1, 1, 1, 999, 5, 4)]
+r = random.Random(7)
+for _ in range(3000):
+    K = r.choice([1, 1, 1, 2, 3, 5, 7, 16])
+    shapes.append((r.choice([1, 1, 2]), r.choice([1, 2, 3, 16, 40, 130]), r.randint(1, 9), r.randint(1, 40), r.choice([1, 3, 16, 241, 512, 1500]), K, r.randrange(K)))
+allowed = {hk.OK, hk.ERR_CUDA, hk.ERR_UNSUPPORTED, hk.ERR_INVALID_ARG, hk.ERR_NO_FIT}
+planned = 0
+for B, Ci, H, W, Co, K, pad in shapes:
+    n = lib.hikonv_conv2d_workspace_bytes(B, Ci, H, W, Co, K, pad)
+    if n == 0:
+        continue
+    p, q = r.randint(1, 8), r.randint(1, 8)
+    for p, q, force in ((p, q, 0), (p, q, r.randint(1, 4)), (4, 4, 0), (5, 5, 0), (6, 6, 0)):
+        tune = ctypes.byref(hk.TuningT(N=force)) if force else None
+        for xs, ws, algo in ((0, 1, 0), (0, 1, 1), (1, 1, 0)):
+            st = lib.hikonv_conv2d(4096, B, Ci, H, W, 8192, Co, K, 1, pad, p, q, xs, ws, 16384, 0, 0, 0, 0, 65536, n, algo, tune, None)
+            assert st in allowed, (st, (B, Ci, H, W, Co, K, pad), p, q, xs, ws, algo, force)
+            planned += st == hk.ERR_CUDA
+assert planned > 10000, planned
+'''
+
+
+def test_layers_accept_a_workspace_of_the_queried_size():
+    # the sizes are compared before anything is launched; in a process that sees no device, so that nothing is
+    out = subprocess.run([sys.executable, "-c", _WORKSPACE_PROBE], cwd=ROOT, env=dict(os.environ, CUDA_VISIBLE_DEVICES=""),
+                         capture_output=True, text=True, timeout=600)
+    assert out.returncode == 0, out.stderr[-2000:]

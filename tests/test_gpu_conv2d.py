@@ -192,6 +192,13 @@ def test_deep_unsigned_layers_on_shifted_codes(p):
         assert_exact(_layer(x, w, 1, p, 4, False, True, hk.ALGO_PACKED32), direct.conv2d_nchw(x, w, 1), "extreme p=%d" % p)
 
 
+def test_wide_pointwise_layers_in_the_queried_workspace():
+    # one pixel or a small map to many channels on shifted codes: the correction table shares the workspace with the packed rows
+    for (B, Ci, H, W, Co, p) in ((1, 64, 1, 1, 1280, 4), (1, 16, 1, 1, 512, 5), (1, 3, 13, 3, 779, 6), (2, 130, 2, 3, 301, 4)):
+        x, w = inputs.conv2d_case(B, Ci, H, W, Co, 1, p, p, False, True, seed=Co)
+        assert_exact(_layer(x, w, 0, p, p, False, True, hk.ALGO_PACKED32), direct.conv2d_nchw(x, w, 0), "%s p=%d" % ((B, Ci, H, W, Co), p))
+
+
 @pytest.mark.parametrize("algo", ALGOS)
 def test_extreme_codes(algo):
     for (p, q, xs, ws) in ((4, 4, True, True), (4, 4, False, True), (8, 4, False, True), (8, 8, True, True), (1, 1, True, True)):
