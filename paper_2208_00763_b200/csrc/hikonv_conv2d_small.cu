@@ -18,8 +18,10 @@
 
 namespace hikonv {
 
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// Not the .aligned forms: those want all threads of a warp at the instruction together, and the code in front of both barriers has
+// branches that the threads of a warp take apart (the words from another warp, the stores).
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 __device__ __forceinline__ int32_t load_cluster(uint32_t smem_addr, uint32_t rank) {
     uint32_t remote;
     int32_t v;
