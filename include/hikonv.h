@@ -339,10 +339,14 @@ int hikonv_conv2d_static_scratch(const int8_t *d_x, int B, int Ci, int H, int W,
 
 /*
  * hikonv_conv2d_wait_timeouts - threads of 2-D layer kernels on the current device whose wait for their own operand copies ran
- * out (a limit far above any copy's time) since the last call; 0 unless the device is at fault, and the layers since then
- * are not to be trusted otherwise.  A debug aid; synchronises the device and clears the count.
+ * out (after a second, far above any copy's time) since the last call of any thread; 0 unless the device is at fault.  A CTA
+ * whose wait ran out leaves its part of the output unwritten; the layer call has returned HIKONV_OK by then, so a caller that
+ * wants to know asks here.  Synchronises the device, all its streams.
+ * hikonv_conv2d_wait_check - a debug aid for the above: enqueues one thread that waits `cycles` (at most 2e9) of the GPU's clock for a
+ * barrier that nothing completes, gives up and is counted like a layer's wait.
  */
 int hikonv_conv2d_wait_timeouts(unsigned int *h_count);
+int hikonv_conv2d_wait_check(long long cycles, void *stream);
 
 /* Device scratch needed by hikonv_conv2d_host: x, w, out and the kernel workspace. */
 size_t hikonv_conv2d_host_workspace_bytes(int B, int Ci, int H, int W, int Co, int K, int pad, int requant);

@@ -68,6 +68,7 @@ _SIGNATURES = {
                                 _i, _i, ctypes.POINTER(_i), ctypes.POINTER(_d), ctypes.POINTER(_d), _vp]),
     "hikonv_conv2d_workspace_bytes": (_sz, [_i] * 7),
     "hikonv_conv2d_wait_timeouts": (_i, [_vp]),
+    "hikonv_conv2d_wait_check": (_i, [ctypes.c_longlong, _vp]),
     "hikonv_conv2d_static_scratch": (_i, [_vp, _i, _i, _i, _i, _vp, _i, _i, _i, _i, _i, _i, _i, _i, _vp, _i, _i, _i, _i, _i,
                                           ctypes.POINTER(TuningT), _vp]),
     "hikonv_conv2d_host_workspace_bytes": (_sz, [_i] * 8),
@@ -243,6 +244,11 @@ def conv2d_wait_timeouts() -> int:
     count = ctypes.c_uint(0)
     _check(lib().hikonv_conv2d_wait_timeouts(ctypes.byref(count)), "hikonv_conv2d_wait_timeouts")
     return int(count.value)
+
+
+def conv2d_wait_check(cycles: int, stream=None) -> None:
+    """One thread waits `cycles` for a barrier that nothing completes, gives up and is counted."""
+    _check(lib().hikonv_conv2d_wait_check(int(cycles), _stream(stream)), "hikonv_conv2d_wait_check")
 
 
 def conv1d(d_f: torch.Tensor, d_g: torch.Tensor, p: int, q: int, f_signed: bool, g_signed: bool,

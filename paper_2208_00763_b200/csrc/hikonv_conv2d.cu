@@ -791,14 +791,29 @@ extern "C" int hikonv_conv2d_wait_timeouts(unsigned int *h_count) {
         strip_wait_timeouts<1, 0, 0>, strip_wait_timeouts<2, 1, 1>, strip_wait_timeouts<3, 1, 1>, strip_wait_timeouts<4, 1, 1>,
         strip_wait_timeouts<2, 3, 1>, strip_wait_timeouts<2, 3, 2>, strip_wait_timeouts<3, 3, 1>, strip_wait_timeouts<4, 3, 1>,
         strip_wait_timeouts<2, 5, 3>, strip_wait_timeouts<3, 5, 2>, strip_wait_timeouts<4, 5, 1>, strip_wait_timeouts<4, 5, 2>};
+    constexpr int kDevices = 64;
+    static std::mutex mutex;
+    static unsigned int told[kDevices];                              // what earlier calls have reported
     *h_count = 0;
+    int dev = 0;
+    // all streams, the non-blocking ones too; the counters only grow, so none that comes in meanwhile is lost
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices || cudaDeviceSynchronize() != cudaSuccess) return HIKONV_ERR_CUDA;
+    std::lock_guard<std::mutex> lock(mutex);
+    unsigned int total = 0;
     for (auto counter : counters) {
         unsigned int n = 0;
         const int rc = counter(&n);
         if (rc != HIKONV_OK) return rc;
-        *h_count += n;
+        total += n;
     }
+    *h_count = total - told[dev];
+    told[dev] = total;
     return HIKONV_OK;
+}
+
+extern "C" int hikonv_conv2d_wait_check(long long cycles, void *stream) {
+    if (cycles < 0 || cycles > kWaitCycles) return HIKONV_ERR_INVALID_ARG;
+    return launch_wait_check(cycles, (cudaStream_t)stream);
 }
 
 extern "C" int hikonv_conv2d(const int8_t *d_x, int B, int Ci, int H, int W, const int8_t *d_w, int Co, int K, int stride,

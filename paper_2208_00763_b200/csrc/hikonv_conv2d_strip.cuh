@@ -45,7 +45,7 @@
 
 namespace hikonv {
 
-// Threads of this file's kernels whose wait for a stage ran out (one counter per file; read and cleared by strip_wait_timeouts).
+// Threads of this file's kernels whose wait for a stage ran out (one counter per file, which only grows).
 static __device__ unsigned int strip_timeouts;
 
 template <int N, int KT, int JT>
@@ -220,12 +220,16 @@ __global__ void __launch_bounds__(kStripThreads, 2) conv2d_strip_kernel(const __
         const int ckn = min(p.CK, p.Ci - ci0);
         // the groups' shares of a stage (the last ones' may be shorter; moves happen at the same places in all)
         const int share = (ckn + KS - 1) / KS, own = min(ckn - group * share, share);
-        // this stage has landed (were the wait ever to run out, the sums would be wrong, and counted as such, but nothing would hang;
-        // later stages and the other buffer are still waited for, with the same limit)
-        if (!mbarrier_wait(bar0 + 8u * stage, parity)) atomicAdd(&strip_timeouts, 1u);
+        // this stage has landed, and the previous one is fully consumed.  Were a wait ever to run out, the CTA would count it, wait
+        // for its copies once more (those of this stage are all that can be in flight) and leave its outputs unwritten
+        const bool landed = mbarrier_wait(bar0 + 8u * stage, parity);
         cp_async_wait_all();
+        if (__syncthreads_or(!landed)) {
+            if (!landed) atomicAdd(&strip_timeouts, 1u);
+            mbarrier_wait(bar0 + 8u * stage, parity);
+            return;
+        }
         parity ^= (uint32_t)stage;
-        __syncthreads();                                       // the previous stage is fully consumed
         if (ci0 + p.CK < p.Ci) fetch(min(p.CK, p.Ci - ci0 - p.CK), stage ^ 1);
         int a_ch = stage * p.a_words, b_ch = p.b_off + stage * p.b_words;
         if constexpr (KS > 1) {
@@ -510,10 +514,7 @@ static int launch_strip_tile(const StripLaunch &s, cudaStream_t st) {
 
 template <int N, int KT, int JT>
 int strip_wait_timeouts(unsigned int *h_count) {
-    const unsigned int zero = 0;
-    if (cudaMemcpyFromSymbol(h_count, strip_timeouts, sizeof(zero)) != cudaSuccess) return HIKONV_ERR_CUDA;
-    if (*h_count != 0 && cudaMemcpyToSymbol(strip_timeouts, &zero, sizeof(zero)) != cudaSuccess) return HIKONV_ERR_CUDA;
-    return HIKONV_OK;
+    return cudaMemcpyFromSymbol(h_count, strip_timeouts, sizeof(*h_count)) == cudaSuccess ? HIKONV_OK : HIKONV_ERR_CUDA;
 }
 
 template <int N, int KT, int JT>

@@ -76,9 +76,11 @@ constexpr bool strip_packed_add(int N, int K, int J) {
 // Explicitly instantiated, one layout per file: (N, 0, 0) with run-time bounds, (N, K, J) for strip_unrolled ones.
 template <int N, int KT, int JT>
 int launch_strip(const StripLaunch &s, cudaStream_t st);
-// Threads of the layout's kernels whose bounded wait for a stage of operands ran out since the last call (the generic kernels share
-// the counter of N = 1).  Synchronises.
+// Threads of the layout's kernels on the current device whose bounded wait for a stage of operands ran out (the generic kernels
+// share the counter of N = 1).  Reads a device variable: the caller synchronises.
 template <int N, int KT, int JT>
 int strip_wait_timeouts(unsigned int *h_count);
+// Launches one thread that waits `cycles` for a barrier of its own which nothing completes and counts that wait with the generic kernels'.
+int launch_wait_check(long long cycles, cudaStream_t st);
 
 }  // namespace hikonv

@@ -168,17 +168,23 @@ __device__ __forceinline__ void bulk_copy(uint32_t smem_dst, const void *gmem_sr
                  "r"(bytes), "r"(bar)
                  : "memory");
 }
-// Waits for the phase of this parity to complete, with a limit far above any copy's time (a quarter of a million polls, some
-// milliseconds at least).  Returns false when it ran out.
-__device__ __forceinline__ bool mbarrier_wait(uint32_t bar, uint32_t parity) {
-    for (int i = 0; i < (1 << 18); ++i) {
-        uint32_t done;
-        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                     : "=r"(done)
-                     : "r"(bar), "r"(parity)
-                     : "memory");
-        if (done) return true;
-    }
+__device__ __forceinline__ bool mbarrier_try_wait(uint32_t bar, uint32_t parity) {
+    uint32_t done;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(done)
+                 : "r"(bar), "r"(parity)
+                 : "memory");
+    return done != 0;
+}
+// Waits for the phase of this parity to complete, for so many cycles at most (the default, one second, is far above any copy's
+// time).  Returns false when they ran out.
+constexpr long long kWaitCycles = 2000000000ll;
+__device__ __forceinline__ bool mbarrier_wait(uint32_t bar, uint32_t parity, long long cycles = kWaitCycles) {
+    if (mbarrier_try_wait(bar, parity)) return true;
+    const long long start = clock64();
+    do {
+        if (mbarrier_try_wait(bar, parity)) return true;
+    } while (clock64() - start < cycles);
     return false;
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }

@@ -192,6 +192,20 @@ def test_deep_unsigned_layers_on_shifted_codes(p):
         assert_exact(_layer(x, w, 1, p, 4, False, True, hk.ALGO_PACKED32), direct.conv2d_nchw(x, w, 1), "extreme p=%d" % p)
 
 
+def test_waits_that_run_out_are_counted():
+    # one thread waits a millisecond for a barrier that nothing completes, on a stream that does not wait for the default one
+    hk.conv2d_wait_timeouts()
+    side = torch.cuda.Stream()
+    for n in (1, 2):
+        for _ in range(n):
+            hk.conv2d_wait_check(2000000, stream=side)
+        assert hk.conv2d_wait_timeouts() == n
+        assert hk.conv2d_wait_timeouts() == 0
+    with pytest.raises(hk.HikonvError) as err:
+        hk.conv2d_wait_check(1 << 40)
+    assert err.value.status == hk.ERR_INVALID_ARG
+
+
 def test_wide_pointwise_layers_in_the_queried_workspace():
     # one pixel or a small map to many channels on shifted codes: the correction table shares the workspace with the packed rows
     for (B, Ci, H, W, Co, p) in ((1, 64, 1, 1, 1280, 4), (1, 16, 1, 1, 512, 5), (1, 3, 13, 3, 779, 6), (2, 130, 2, 3, 301, 4)):
