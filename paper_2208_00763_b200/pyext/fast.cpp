@@ -4,6 +4,8 @@
 // Every function takes the wrapper's arguments and returns the output tensor, or None when anything is not as the fast path
 // expects it (a wrong type, layout, device or size, an argument out of range, a status other than OK): the wrapper then goes
 // its own way, which raises the error.  Nothing is decided here that the wrapper would decide differently.
+// As under ctypes, the library's calls run without the interpreter lock: a launch blocks while its stream's queue is full, and what
+// empties the queue may be a Python callback.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
@@ -110,6 +112,16 @@ PyObject *result(PyObject *given, const at::Tensor &made) {
     return THPVariable_Wrap(made);
 }
 
+// Calls into the library with the interpreter lock released.
+template <typename F>
+int unlocked(F call) {
+    int status;
+    Py_BEGIN_ALLOW_THREADS
+    status = call();
+    Py_END_ALLOW_THREADS
+    return status;
+}
+
 template <typename F>
 PyObject *guarded(F f) {
     try {
@@ -134,9 +146,11 @@ PyObject *conv1d(PyObject *, PyObject *const *a, Py_ssize_t n) {
         if (!given) made = empty({n_out}, at::kInt, *f);
         const at::Tensor &y = given ? *given : made;
         if (!output_ok(y, n_out, false, *f)) return nullptr;
-        if (g_conv1d((const int8_t *)f->data_ptr(), (size_t)len, (const int8_t *)g->data_ptr(), (int)g->numel(), p, q, fs, gs,
-                     (int32_t *)y.data_ptr(), algo, nullptr, current_stream()) != HIKONV_OK)
-            return nullptr;
+        const int8_t *f_ptr = (const int8_t *)f->data_ptr(), *g_ptr = (const int8_t *)g->data_ptr();
+        const int K = (int)g->numel();
+        int32_t *y_ptr = (int32_t *)y.data_ptr();
+        void *st = current_stream();
+        if (unlocked([&] { return g_conv1d(f_ptr, (size_t)len, g_ptr, K, p, q, fs, gs, y_ptr, algo, nullptr, st); }) != HIKONV_OK) return nullptr;
         return result(a[7], made);
     });
 }
@@ -157,9 +171,12 @@ PyObject *conv1d_dense(PyObject *, PyObject *const *a, Py_ssize_t n) {
         if (!given) made = empty({n_out}, at::kInt, *f);
         const at::Tensor &y = given ? *given : made;
         if (!output_ok(y, n_out, false, *f)) return nullptr;
-        if (g_conv1d_dense((const uint8_t *)f->data_ptr(), (size_t)len, (const int8_t *)g->data_ptr(), (int)g->numel(), p, q, fs, gs,
-                           (int32_t *)y.data_ptr(), nullptr, current_stream()) != HIKONV_OK)
-            return nullptr;
+        const uint8_t *f_ptr = (const uint8_t *)f->data_ptr();
+        const int8_t *g_ptr = (const int8_t *)g->data_ptr();
+        const int K = (int)g->numel();
+        int32_t *y_ptr = (int32_t *)y.data_ptr();
+        void *st = current_stream();
+        if (unlocked([&] { return g_conv1d_dense(f_ptr, (size_t)len, g_ptr, K, p, q, fs, gs, y_ptr, nullptr, st); }) != HIKONV_OK) return nullptr;
         return result(a[7], made);
     });
 }
@@ -173,8 +190,9 @@ PyObject *pack(PyObject *, PyObject *const *a, Py_ssize_t n) {
         if (!in.ok || !codes(x) || N < 1 || (word_bits != 32 && word_bits != 64)) return nullptr;
         const int64_t count = x->numel();
         const at::Tensor words = empty({(count + N - 1) / N}, word_bits == 32 ? at::kInt : at::kLong, *x);
-        if (g_pack((const int8_t *)x->data_ptr(), (size_t)count, bits, is_signed, S, N, word_bits, words.data_ptr(), current_stream()) != HIKONV_OK)
-            return nullptr;
+        const int8_t *x_ptr = (const int8_t *)x->data_ptr();
+        void *words_ptr = words.data_ptr(), *st = current_stream();
+        if (unlocked([&] { return g_pack(x_ptr, (size_t)count, bits, is_signed, S, N, word_bits, words_ptr, st); }) != HIKONV_OK) return nullptr;
         return THPVariable_Wrap(words);
     });
 }
@@ -227,10 +245,13 @@ PyObject *conv2d(PyObject *, PyObject *const *a, Py_ssize_t n) {
         if (!given) made = empty({l.B, l.Co, l.Ho(), l.Wo()}, rq ? at::kChar : at::kInt, *x);
         const at::Tensor &y = given ? *given : made;
         if (!output_ok(y, l.B * l.Co * l.Ho() * l.Wo(), rq, *x)) return nullptr;
-        if (g_conv2d((const int8_t *)x->data_ptr(), (int)l.B, (int)l.Ci, (int)l.H, (int)l.W, (const int8_t *)w->data_ptr(), (int)l.Co, (int)l.K,
-                     stride, l.pad, p, q, xs, ws, y.data_ptr(), rq ? 1 : 0, shift, lo, hi, space_ptr, space_bytes, algo, nullptr,
-                     current_stream()) != HIKONV_OK)
-            return nullptr;
+        const int8_t *x_ptr = (const int8_t *)x->data_ptr(), *w_ptr = (const int8_t *)w->data_ptr();
+        void *y_ptr = y.data_ptr(), *st = current_stream();
+        const int status = unlocked([&] {
+            return g_conv2d(x_ptr, (int)l.B, (int)l.Ci, (int)l.H, (int)l.W, w_ptr, (int)l.Co, (int)l.K, stride, l.pad, p, q, xs, ws, y_ptr,
+                            rq ? 1 : 0, shift, lo, hi, space_ptr, space_bytes, algo, nullptr, st);
+        });
+        if (status != HIKONV_OK) return nullptr;
         return result(a[10], made);
     });
 }
@@ -272,10 +293,13 @@ PyObject *conv2d_dense(PyObject *, PyObject *const *a, Py_ssize_t n) {
                  : out_bits == 8 ? empty({l.B, l.Co, Hq, Wq}, at::kChar, *x) : empty({n_out}, at::kByte, *x);
         const at::Tensor &y = given ? *given : made;
         if (!output_ok(y, n_out, rq, *x)) return nullptr;
-        if (g_conv2d_dense(x->data_ptr(), x_bits, (int)l.B, (int)l.Ci, (int)l.H, (int)l.W, w->data_ptr(), w_bits, (int)l.Co, (int)l.K, stride,
-                           l.pad, p, q, xs, ws, y.data_ptr(), rq ? out_bits : 32, rq ? 1 : 0, shift, lo, hi, pool, space_ptr, space_bytes,
-                           algo, nullptr, current_stream()) != HIKONV_OK)
-            return nullptr;
+        const void *x_ptr = x->data_ptr(), *w_ptr = w->data_ptr();
+        void *y_ptr = y.data_ptr(), *st = current_stream();
+        const int status = unlocked([&] {
+            return g_conv2d_dense(x_ptr, x_bits, (int)l.B, (int)l.Ci, (int)l.H, (int)l.W, w_ptr, w_bits, (int)l.Co, (int)l.K, stride, l.pad, p, q,
+                                  xs, ws, y_ptr, rq ? out_bits : 32, rq ? 1 : 0, shift, lo, hi, pool, space_ptr, space_bytes, algo, nullptr, st);
+        });
+        if (status != HIKONV_OK) return nullptr;
         return result(a[16], made);
     });
 }

@@ -1,4 +1,9 @@
 """The binding's native fast path against its Python path (taken when a stream is given), and what neither may accept."""
+import ctypes
+import subprocess
+import threading
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -85,3 +90,39 @@ def test_errors_are_those_of_the_python_path():
     assert err.value.status == hk.ERR_UNSUPPORTED
     with pytest.raises(ValueError):
         hk.conv2d_dense(x.reshape(-1), (1, 4, 6, 7), 8, w.reshape(-1), w.shape, 8, 1, 4, 4, True, True)
+
+
+def test_other_threads_run_during_a_library_call(tmp_path):
+    # the native path bound to a stand-in that sleeps: a second Python thread must get on meanwhile
+    src, so = tmp_path / "slow.c", tmp_path / "slow.so"
+    src.write_text("#include <time.h>\nint slow(void) { struct timespec t = {0, 300000000}; nanosleep(&t, 0); return 0; }\n")
+    subprocess.run(["gcc", "-shared", "-fPIC", "-o", str(so), str(src)], check=True)
+    slow = ctypes.cast(ctypes.CDLL(str(so)).slow, ctypes.c_void_p).value
+    f, g = torch.zeros(64, dtype=torch.int8, device="cuda"), torch.zeros(3, dtype=torch.int8, device="cuda")
+    x, w = torch.zeros((1, 4, 6, 6), dtype=torch.int8, device="cuda"), torch.zeros((2, 4, 3, 3), dtype=torch.int8, device="cuda")
+    calls = {"hikonv_conv1d": lambda: hk.conv1d(f, g, 4, 4, False, False),
+             "hikonv_conv1d_dense": lambda: hk.conv1d_dense(f.view(torch.uint8), 64, g, 4, 4, False, False),
+             "hikonv_pack": lambda: hk.pack(f, 4, False, 10, 3),
+             "hikonv_conv2d": lambda: hk.conv2d(x, w, 1, 4, 4, True, True),
+             "hikonv_conv2d_dense": lambda: hk.conv2d_dense(x.reshape(-1), x.shape, 8, w.reshape(-1), w.shape, 8, 1, 4, 4, True, True)}
+    for name, call in calls.items():
+        call()
+        hk._fast.bind(name, slow)
+        try:
+            done, ticks = threading.Event(), []
+
+            def tick():
+                while not done.is_set():
+                    ticks.append(time.monotonic())
+                    time.sleep(0.01)
+
+            other = threading.Thread(target=tick)
+            other.start()
+            t0 = time.monotonic()
+            call()
+            t1 = time.monotonic()
+            done.set()
+            other.join()
+        finally:
+            hk._fast.bind(name, ctypes.cast(getattr(hk.lib(), name), ctypes.c_void_p).value)
+        assert t1 - t0 > 0.25 and sum(t0 + 0.05 < t < t1 - 0.05 for t in ticks) >= 3, name
