@@ -55,20 +55,21 @@ __device__ __forceinline__ uint32_t byte_range_mask(int i, int first, int last) 
 }
 
 // Four packed words (Eq. 5) of N codes each, from column col0 on, of an image row of W one-byte codes: zero outside the row, and
-// everywhere when row_in is false (the row is then not read).  off4: a byte repeated four times that is taken from every
-// code inside the columns of the image (in rows that are not read too), is_signed: the codes, after that, are signed.
+// everywhere when row_in is false (the row is then not read).  The row starts at code `row` of the tensor x of `codes` codes.
+// off4: a byte repeated four times that is taken from every code inside the columns of the image (in rows that are not read too),
+// is_signed: the codes, after that, are signed.
 // The codes start at any byte: the N + 1 aligned words around them are loaded (those that hold a code of the row), shifted into
-// place, blanked outside the row with one mask per word, and packed by byte permute and Horner's rule.
-// [x, x_end): the tensor the row belongs to.  Where one of those words reaches outside it (the first codes of an unaligned tensor,
-// the last ones of one whose size is not a multiple of four) the codes are loaded byte by byte.
+// place, blanked outside the row with one mask per word, and packed by byte permute and Horner's rule.  Where one of those words
+// reaches outside the tensor (the first codes of an unaligned tensor, the last ones of one whose size is not a multiple of four)
+// the codes are loaded byte by byte.
 template <int N>
-__device__ __forceinline__ void pack_row_words(const int8_t *row, const int8_t *x, const int8_t *x_end, int W, int col0, bool row_in, uint32_t off4,
-                                               bool is_signed, int S, uint32_t (&word)[4]) {
-    const int8_t *src = row + col0;                              // not dereferenced outside the row
-    const int off = (int)((uintptr_t)src & 3);
-    const uint32_t *al = reinterpret_cast<const uint32_t *>(src - off);
+__device__ __forceinline__ void pack_row_words(const int8_t *x, int row, int codes, int W, int col0, bool row_in, uint32_t off4, bool is_signed,
+                                               int S, uint32_t (&word)[4]) {
+    const int off = ((int)(uintptr_t)x + row + col0) & 3;        // of the first code in its aligned word
+    const int first = row + col0 - off;                          // code at the start of that word (not in the tensor, where col0 < 0)
     uint32_t v[N + 1];
-    if (!row_in || (src - off >= x && src - off + 4 * (N + 1) <= x_end)) {
+    if (!row_in || (first >= 0 && first <= codes - 4 * (N + 1))) {
+        const uint32_t *al = reinterpret_cast<const uint32_t *>(x + first);
 #pragma unroll
         for (int i = 0; i <= N; ++i) {
             const int c = col0 - off + 4 * i;                    // aligned word i holds the codes of columns c .. c + 3
@@ -78,10 +79,10 @@ __device__ __forceinline__ void pack_row_words(const int8_t *row, const int8_t *
 #pragma unroll
         for (int i = 0; i <= N; ++i) {
             v[i] = 0u;
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
+#pragma unroll 1
+            for (int b = 3; b >= 0; --b) {                       // (a loop: few threads come here, and the launch has registers for few)
                 const int c = col0 - off + 4 * i + b;
-                if (c >= 0 && c < W) v[i] |= (uint32_t)(uint8_t)__ldg(row + c) << (8 * b);
+                v[i] = v[i] << 8 | (c >= 0 && c < W ? (uint32_t)(uint8_t)__ldg(x + row + c) : 0u);
             }
         }
     }

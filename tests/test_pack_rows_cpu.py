@@ -59,7 +59,7 @@ template <int N> void sweep(int W, int rows, int shift, bool is_signed, int off,
             for (int col0 = -2 * N; col0 < W; col0 += (rand() % 3) + 1) {
                 if (col0 + 4 * N <= 0) continue;
                 uint32_t word[4];
-                pack_row_words<N>(x + r * W, x, x + n, W, col0, in != 0, (uint32_t)off * 0x01010101u, is_signed || off != 0, S, word);
+                pack_row_words<N>(x, r * W, n, W, col0, in != 0, (uint32_t)off * 0x01010101u, is_signed || off != 0, S, word);
                 for (int w = 0; w < 4; ++w, ++g_words) {
                     uint32_t want = 0;
                     for (int k = 0; k < N; ++k) {
