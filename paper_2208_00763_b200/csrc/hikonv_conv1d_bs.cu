@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(kThreadsTc, MINB) conv1d_bs_kernel(const Conv1
         for (int k = 0; k < N; ++k) {
             const int idx = j * N + k;
             if (idx < p.K) {
-                const int8_t raw = __ldg(p.g + idx);
+                const int8_t raw = load_ordered(p.g + idx);
                 const int32_t v = p.g_signed ? (int32_t)raw : (int32_t)(uint8_t)raw;
                 b += (uint32_t)v << (S * k);
             }
@@ -163,10 +163,10 @@ static int launch_bs_sign(const Conv1dBsParams &p, bool fs, bool sp, cudaStream_
 }
 
 int launch_conv1d_bs(const Conv1dBsParams &p, int mode, int J, bool fs, bool sp, int variant, cudaStream_t st) {
-    // Measured over the 48 sweep cases at 2^24 codes: kernels with one or two kernel words per block fit the
-    // register budget of five resident CTAs per SM and stream 2-3 % faster with them; with three or four words
-    // that budget spills, and four CTAs are faster.
-    const bool five = variant == 25 || (variant != 24 && (mode == 1 || J <= 2));
+    // Measured over the 48 sweep cases at 2^24 codes: the register budget of five resident CTAs per SM streams faster than
+    // that of four in every one of them, by 0.1 to 0.7 of 15.5 us (three and four kernel words spill a few bytes with it: 15.0
+    // instead of 15.6 us for 8-bit codes and seven taps).
+    const bool five = variant != 24;
 #define HK_BS(m, j)                                                                          \
     if (mode == m && J == j) {                                                               \
         if (five) return launch_bs_sign<m, j, 24, 5>(p, fs, sp, st);                        \

@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(kLongThreads, N == 3 ? 6 : 3) conv1d_long_kern
         for (int k = 0; k < p.Kc; ++k) {
             const int idx = tid * p.Kc + k;
             if (idx < p.K) {
-                const int8_t raw = __ldg(p.g + idx);
+                const int8_t raw = load_ordered(p.g + idx);
                 b += (uint32_t)(p.g_signed ? (int32_t)raw : (int32_t)(uint8_t)raw) << (p.S * k);
             }
         }
@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(kLongThreads, N == 3 ? 6 : 3) conv1d_long_kern
         if (p.aligned && e0 >= 0 && e0 + 4 * N <= p.len) {
             const uint32_t *src = reinterpret_cast<const uint32_t *>(p.f + e0);
 #pragma unroll
-            for (int i = 0; i < N; ++i) w[i] = __ldg(src + i);
+            for (int i = 0; i < N; ++i) w[i] = load_ordered(src + i);
         } else {
 #pragma unroll
             for (int i = 0; i < N; ++i) {
@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(kLongThreads, N == 3 ? 6 : 3) conv1d_long_kern
 #pragma unroll
                 for (int b = 0; b < 4; ++b) {
                     const long long e = e0 + 4 * i + b;
-                    if (e >= 0 && e < p.len) v |= (uint32_t)(uint8_t)__ldg(p.f + e) << (8 * b);   // Eq. 2: zero outside
+                    if (e >= 0 && e < p.len) v |= (uint32_t)(uint8_t)load_ordered(p.f + e) << (8 * b);   // Eq. 2: zero outside
                 }
                 w[i] = v;
             }

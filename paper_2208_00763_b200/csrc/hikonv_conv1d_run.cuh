@@ -20,7 +20,7 @@ __device__ __forceinline__ void load_words(const int8_t *f, long long len, long 
     if (fast) {
         const uint32_t *src = reinterpret_cast<const uint32_t *>(f + e0) - HW;
 #pragma unroll
-        for (int i = 0; i < NWORDS; ++i) w[i] = __ldg(src + i);
+        for (int i = 0; i < NWORDS; ++i) w[i] = load_ordered(src + i);
     } else {
 #pragma unroll
         for (int i = 0; i < NWORDS; ++i) {
@@ -28,7 +28,7 @@ __device__ __forceinline__ void load_words(const int8_t *f, long long len, long 
 #pragma unroll
             for (int b = 0; b < 4; ++b) {
                 const long long idx = e0 + 4 * (i - HW) + b;
-                if (idx >= 0 && idx < len) v |= (uint32_t)(uint8_t)__ldg(f + idx) << (8 * b);   // Eq. 2: zero outside
+                if (idx >= 0 && idx < len) v |= (uint32_t)(uint8_t)load_ordered(f + idx) << (8 * b);   // Eq. 2: zero outside
             }
             w[i] = v;
         }
@@ -101,7 +101,7 @@ __device__ __forceinline__ void walk_tiles(const int8_t *f, int32_t *y, long lon
         if (fast) {
             const uint32_t *src = f_lane + (size_t)tt * (8 * L);
 #pragma unroll
-            for (int i = 0; i < NW; ++i) dst[i] = __ldg(src + i);
+            for (int i = 0; i < NW; ++i) dst[i] = load_ordered(src + i);
         } else {
             load_words<NW, HW>(f, len, (long long)tt * (32 * L) + lane * L, false, dst);
         }

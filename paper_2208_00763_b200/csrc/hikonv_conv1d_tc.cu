@@ -50,7 +50,7 @@ __device__ __forceinline__ void load_dense(const int8_t *f, long long len, long 
         const uint32_t *src = reinterpret_cast<const uint32_t *>(f) + w0;
         uint32_t w[NV + 1];
 #pragma unroll
-        for (int i = 0; i < NV + 1; ++i) w[i] = __ldg(src + i);
+        for (int i = 0; i < NV + 1; ++i) w[i] = load_ordered(src + i);
 #pragma unroll
         for (int i = 0; i < NV; ++i) v[i] = __funnelshift_r(w[i], w[i + 1], boff);
     } else {
@@ -60,7 +60,7 @@ __device__ __forceinline__ void load_dense(const int8_t *f, long long len, long 
         for (int k = 0; k < NE; ++k) {
             const long long e = e_first + k;
             if (e >= 0 && e < len) {
-                const uint32_t byte = (uint8_t)__ldg(f + (e * P) / 8);
+                const uint32_t byte = (uint8_t)load_ordered(f + (e * P) / 8);
                 v[k / EPW] |= ((byte >> (int)((e * P) % 8)) & ((1u << P) - 1u)) << ((k % EPW) * P);
             }
         }
@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(kThreadsTc, ((N >= 9 && P == 0) ? 3 : 4)) conv
         for (int k = 0; k < p.Kc; ++k) {
             const int idx = j * p.Kc + k;
             if (idx < p.K) {
-                const int8_t raw = __ldg(p.g + idx);
+                const int8_t raw = load_ordered(p.g + idx);
                 const int32_t v = p.g_signed ? (int32_t)raw : (int32_t)(uint8_t)raw;
                 b += (uint32_t)v << (S * k);
             }
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(kThreadsTc, MINB) conv1d_unpacked_tc_kernel(co
     int32_t gk[K];
 #pragma unroll
     for (int k = 0; k < K; ++k) {
-        const int8_t raw = __ldg(p.g + k);
+        const int8_t raw = load_ordered(p.g + k);
         gk[k] = p.g_signed ? (int32_t)raw : (int32_t)(uint8_t)raw;
     }
     walk_tiles<L, HW>(p.f, p.y, p.len, p.n_out, (unsigned)p.n_tiles, p.fast_after_first, s_stage[threadIdx.x >> 5],
@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(kThreadsTc, MINB) conv1d_dp4a_tc_kernel(const 
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int k = 4 * t + 3 - j;
-            if (k < p.K) v |= (uint32_t)(uint8_t)__ldg(p.g + k) << (8 * j);
+            if (k < p.K) v |= (uint32_t)(uint8_t)load_ordered(p.g + k) << (8 * j);
         }
         gw[t] = v;
     }

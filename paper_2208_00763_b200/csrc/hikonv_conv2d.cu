@@ -39,7 +39,7 @@ struct WeightPackParams {
 // features kept compressed in memory and unpacked as they are read).
 __device__ __forceinline__ int32_t load_dense_code(const int8_t *base, size_t e, int bits, bool is_signed) {
     const size_t bit = e * (size_t)bits;
-    const uint32_t byte = (uint8_t)__ldg(base + (bit >> 3));
+    const uint32_t byte = (uint8_t)load_ordered(base + (bit >> 3));
     const uint32_t v = (byte >> (int)(bit & 7)) & ((1u << bits) - 1u);
     const uint32_t sb = 1u << (bits - 1);
     return is_signed ? (int32_t)((v ^ sb) - sb) : (int32_t)v;
@@ -62,7 +62,7 @@ __device__ __forceinline__ void pack_weight_words(const WeightPackParams &q, int
             if (g_idx < q.K) {
                 int32_t v;
                 if (q.w_bits == 8) {
-                    const int8_t raw = __ldg(q.w + row_e + (q.K - 1 - g_idx));
+                    const int8_t raw = load_ordered(q.w + row_e + (q.K - 1 - g_idx));
                     v = q.w_signed ? (int32_t)raw : (int32_t)(uint8_t)raw;
                 } else {
                     v = load_dense_code(q.w, row_e + (q.K - 1 - g_idx), q.w_bits, q.w_signed != 0);
@@ -91,7 +91,7 @@ __device__ __forceinline__ void sum_channel_weights(const WeightPackParams &q, i
                 for (int k = 0; k < 4; ++k)
                     if (k0 + k < q.K) {
                         if (q.w_bits == 8) {
-                            const int8_t raw = __ldg(q.w + e + k);
+                            const int8_t raw = load_ordered(q.w + e + k);
                             sum[k] += q.w_signed ? (int32_t)raw : (int32_t)(uint8_t)raw;
                         } else {
                             sum[k] += load_dense_code(q.w, e + k, q.w_bits, q.w_signed != 0);
@@ -137,7 +137,7 @@ struct ActPackDivs {
 // runs, and with eight they pile up on the SMs that are free first: 24x45x61 and 48x37x53 layers took 31.1 and 27.2 us a call
 // instead of 29.8 and 26.3.
 template <bool XS, int N, int CTAS>
-__global__ void __launch_bounds__(256, CTAS) pack_operands_kernel(const int8_t *__restrict__ x, int codes, int B, int Ci, int H,
+__global__ void __launch_bounds__(256, CTAS) pack_operands_kernel(const int8_t *x, int codes, int B, int Ci, int H,
                                                             int W, int Hp, int pad, int col_first, int S, int XBT,
                                                             uint32_t *__restrict__ ap, int weight_blocks, const WeightPackParams wq,
                                                             int x_bits, const ActPackDivs dv, unsigned act_items) {
@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(256, CTAS) pack_operands_kernel(const int8_t *
 // 16-byte loads, one 8-byte store), per-byte maxima; needs W % VEC == 0 and VEC-byte aligned input,
 // VEC/2-byte aligned output.
 template <bool SIGNED, int VEC>
-__global__ void __launch_bounds__(256) maxpool2x2_vec_kernel(const int8_t *__restrict__ in, long long items, int H, int W,
+__global__ void __launch_bounds__(256) maxpool2x2_vec_kernel(const int8_t *in, long long items, int H, int W,
                                                              int8_t *__restrict__ out) {
     grid_dependency_release();
     grid_dependency_wait();
@@ -200,12 +200,12 @@ __global__ void __launch_bounds__(256) maxpool2x2_vec_kernel(const int8_t *__res
         const int8_t *src = in + (c * H + 2 * ho) * (long long)W + VEC * wv;
         int8_t *dst = out + (c * Ho + ho) * (long long)(W / 2) + (VEC / 2) * wv;
         if constexpr (VEC == 16) {
-            const uint4 r0 = __ldg(reinterpret_cast<const uint4 *>(src));
-            const uint4 r1 = __ldg(reinterpret_cast<const uint4 *>(src + W));
+            const uint4 r0 = load_ordered(reinterpret_cast<const uint4 *>(src));
+            const uint4 r1 = load_ordered(reinterpret_cast<const uint4 *>(src + W));
             *reinterpret_cast<uint2 *>(dst) = make_uint2(pool_pairs<SIGNED>(r0.x, r0.y, r1.x, r1.y), pool_pairs<SIGNED>(r0.z, r0.w, r1.z, r1.w));
         } else {
-            const uint2 r0 = __ldg(reinterpret_cast<const uint2 *>(src));
-            const uint2 r1 = __ldg(reinterpret_cast<const uint2 *>(src + W));
+            const uint2 r0 = load_ordered(reinterpret_cast<const uint2 *>(src));
+            const uint2 r1 = load_ordered(reinterpret_cast<const uint2 *>(src + W));
             *reinterpret_cast<uint32_t *>(dst) = pool_pairs<SIGNED>(r0.x, r0.y, r1.x, r1.y);
         }
     }

@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(kStripThreads, 2) conv2d_small_kernel(const __
             const int8_t *src = q.w + ((size_t)(co0 + c) * p.Ci * KT + c0 * KT + row) * KT;
             int8_t code[KT];
 #pragma unroll
-            for (int k = 0; k < KT; ++k) code[k] = __ldg(src + k);
+            for (int k = 0; k < KT; ++k) code[k] = load_ordered(src + k);
 #pragma unroll
             for (int g = 0; g < KT; ++g) {                     // tap g of the reversed row belongs to chunk g / Kc
                 const int32_t v = q.w_signed ? (int32_t)code[KT - 1 - g] : (int32_t)(uint8_t)code[KT - 1 - g];

@@ -372,7 +372,7 @@ __global__ void __launch_bounds__(kStripThreads, 2) conv2d_strip_kernel(const __
             for (int m = 0; m < N; ++m)
                 if (col_ok[m]) {
                     const int k_lo = max(0, p.pad - w0 - m), k_hi = min(K, p.W + p.pad - w0 - m);
-                    off[m] += __ldg(c + (k_hi - 1) * p.CoP) - (k_lo > 0 ? __ldg(c + (k_lo - 1) * p.CoP) : 0);   // k_hi >= K - pad > 0
+                    off[m] += load_ordered(c + (k_hi - 1) * p.CoP) - (k_lo > 0 ? load_ordered(c + (k_lo - 1) * p.CoP) : 0);   // k_hi >= K - pad > 0
                 }
         }
     };

@@ -73,7 +73,7 @@ __device__ __forceinline__ void pack_row_words(const int8_t *x, int row, int cod
 #pragma unroll
         for (int i = 0; i <= N; ++i) {
             const int c = col0 - off + 4 * i;                    // aligned word i holds the codes of columns c .. c + 3
-            v[i] = (row_in && c + 3 >= 0 && c < W) ? __ldg(al + i) : 0u;
+            v[i] = (row_in && c + 3 >= 0 && c < W) ? load_ordered(al + i) : 0u;
         }
     } else {
 #pragma unroll
@@ -82,7 +82,7 @@ __device__ __forceinline__ void pack_row_words(const int8_t *x, int row, int cod
 #pragma unroll 1
             for (int b = 3; b >= 0; --b) {                       // (a loop: few threads come here, and the launch has registers for few)
                 const int c = col0 - off + 4 * i + b;
-                v[i] = v[i] << 8 | (c >= 0 && c < W ? (uint32_t)(uint8_t)__ldg(x + row + c) : 0u);
+                v[i] = v[i] << 8 | (c >= 0 && c < W ? (uint32_t)(uint8_t)load_ordered(x + row + c) : 0u);
             }
         }
     }

@@ -37,6 +37,12 @@ inline int launch_plain(void (*kernel)(Params...), dim3 grid, dim3 block, size_t
 // visible).  grid_dependency_release() lets the NEXT kernel of the stream be scheduled early; it takes
 // effect once every CTA of this grid has called it or exited.  Every CTA of every such kernel waits, so
 // completion of a kernel still implies completion of all kernels before it.
+// What a kernel reads that is launched this way may be written by the kernel before while it already runs, so it is not constant
+// over the kernel's lifetime: ordinary loads, which stay behind the wait, and not the read-only path (__ldg, const __restrict__).
+template <typename T>
+__device__ __forceinline__ T load_ordered(const T *p) {
+    return *p;
+}
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dependency_release() { asm volatile("griddepcontrol.launch_dependents;"); }
 
@@ -120,7 +126,7 @@ __device__ __forceinline__ int32_t code_value(int8_t b) {
 
 template <bool SIGNED>
 __device__ __forceinline__ int32_t load_code(const int8_t *p) {
-    return code_value<SIGNED>(__ldg(p));
+    return code_value<SIGNED>(load_ordered(p));
 }
 
 // prmt with a selector known at run time (__byte_perm ignores the bit that replicates a byte's sign).

@@ -13,7 +13,7 @@ constexpr int kMaxPackN = 12;
 // pieces.  The last, partial group is packed code by code by the thread it falls to.  2^24 4-bit codes, three per 32-bit
 // word: 15.9 -> 8.2 us on the device (39 MB, 4.8 TB/s), 20.5 -> 10.7 us a call among others.
 template <bool SIGNED, typename WORD, int N>
-__global__ void __launch_bounds__(256) pack_groups_kernel(const int8_t *__restrict__ in, size_t n, int S, WORD *__restrict__ words,
+__global__ void __launch_bounds__(256) pack_groups_kernel(const int8_t *in, size_t n, int S, WORD *__restrict__ words,
                                                           size_t n_words) {
     grid_dependency_release();
     grid_dependency_wait();
@@ -27,18 +27,18 @@ __global__ void __launch_bounds__(256) pack_groups_kernel(const int8_t *__restri
         if constexpr (N % 4 == 0) {
 #pragma unroll
             for (int i = 0; i < N; i += 4) {
-                const uint4 v = __ldg(reinterpret_cast<const uint4 *>(src) + i / 4);
+                const uint4 v = load_ordered(reinterpret_cast<const uint4 *>(src) + i / 4);
                 w[i] = v.x; w[i + 1] = v.y; w[i + 2] = v.z; w[i + 3] = v.w;
             }
         } else if constexpr (N % 2 == 0) {
 #pragma unroll
             for (int i = 0; i < N; i += 2) {
-                const uint2 v = __ldg(reinterpret_cast<const uint2 *>(src) + i / 2);
+                const uint2 v = load_ordered(reinterpret_cast<const uint2 *>(src) + i / 2);
                 w[i] = v.x; w[i + 1] = v.y;
             }
         } else {
 #pragma unroll
-            for (int i = 0; i < N; ++i) w[i] = __ldg(reinterpret_cast<const uint32_t *>(src) + i);
+            for (int i = 0; i < N; ++i) w[i] = load_ordered(reinterpret_cast<const uint32_t *>(src) + i);
         }
         const uint32_t step = sizeof(WORD) == 4 && S < 32 ? 1u << S : 0u;      // S >= 32 only with N == 1
 #pragma unroll
