@@ -137,7 +137,7 @@ struct ActPackDivs {
 // runs, and with eight they pile up on the SMs that are free first: 24x45x61 and 48x37x53 layers took 31.1 and 27.2 us a call
 // instead of 29.8 and 26.3.
 template <bool XS, int N, int CTAS>
-__global__ void __launch_bounds__(256, CTAS) pack_operands_kernel(const int8_t *x, int codes, int B, int Ci, int H,
+__global__ void __launch_bounds__(256, CTAS) pack_operands_kernel(const int8_t *x, int ragged, int B, int Ci, int H,
                                                             int W, int Hp, int pad, int col_first, int S, int XBT,
                                                             uint32_t *__restrict__ ap, int weight_blocks, const WeightPackParams wq,
                                                             int x_bits, const ActPackDivs dv, unsigned act_items) {
@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(256, CTAS) pack_operands_kernel(const int8_t *
     if ((row_in || wq.x_off != 0) && col0 + 4 * N > 0 && col0 < W) {
         const int row_e = ((b * Ci + ci) * H + (row_in ? hi : 0)) * W;   // first code of the input row (below 2^31)
         if (x_bits == 8) {
-            pack_row_words<N>(x, row_e, codes, W, col0, row_in, (uint32_t)wq.x_off * 0x01010101u, XS, S, word);
+            pack_row_words<N>(x, row_e, ragged, W, col0, row_in, (uint32_t)wq.x_off * 0x01010101u, XS, S, word);
         } else {
 #pragma unroll
             for (int w = 0; w < 4; ++w)
@@ -737,9 +737,9 @@ static int conv2d_run(const void *d_x, int x_bits, int B, int Ci, int H, int W, 
         s.strip.p.wp = d_wp; s.strip.p.ap = d_ap; s.strip.p.out = d_out;
         s.strip.p.corr = s.x_off ? d_corr : nullptr;
     }
-    const int codes = (int)((long long)B * Ci * H * W);                // below 2^31 (plan_layer)
+    const int ragged = ragged_codes(d_x, (int)((long long)B * Ci * H * W));        // (fewer than 2^31 codes: plan_layer)
     if (s.one_launch) {
-        s.small.p.x = (const int8_t *)d_x; s.small.p.codes = codes; s.small.p.w = (const int8_t *)d_w; s.small.p.s.out = d_out;
+        s.small.p.x = (const int8_t *)d_x; s.small.p.ragged = ragged; s.small.p.w = (const int8_t *)d_w; s.small.p.s.out = d_out;
         return launch_small(s.small, s.L.N, st);
     }
     // a2: reversed kernel rows packed per (ci, kh, chunk); a3: activation rows packed per block; one launch
@@ -764,7 +764,7 @@ static int conv2d_run(const void *d_x, int x_bits, int B, int Ci, int H, int W, 
         // (10 CTAs per SM are faster in the first way, 3 in the second)
         const bool many = grid > 6u * (unsigned)sm_count();
         auto pack = [&](auto kern) {
-            return launch_dependent(kern, dim3(grid), dim3(256), 0, st, (const int8_t *)d_x, codes, B, Ci, H, W, s.Hp, pad, s.col_first, s.L.S,
+            return launch_dependent(kern, dim3(grid), dim3(256), 0, st, (const int8_t *)d_x, ragged, B, Ci, H, W, s.Hp, pad, s.col_first, s.L.S,
                                     s.XBT, d_ap, (int)(w_blocks + corr_blocks), wq, x_bits, dv, (unsigned)act_items);
         };
 #define HK_PACK(XSIGN, NN) rc = many ? pack(pack_operands_kernel<XSIGN, NN, 8>) : pack(pack_operands_kernel<XSIGN, NN, 3>)

@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(kStripThreads, 2) conv2d_small_kernel(const __
         const int col0 = q.col_first + 4 * w4 * N;
         const bool row_in = b < q.B && h >= 0 && h < q.H;
         if (row_in && col0 + 4 * N > 0 && col0 < p.W)
-            pack_row_words<N>(q.x, ((b * p.Ci + c0 + c) * q.H + h) * p.W, q.codes, p.W, col0, true, 0u, q.x_signed != 0, p.S, word);
+            pack_row_words<N>(q.x, ((b * p.Ci + c0 + c) * q.H + h) * p.W, q.ragged, p.W, col0, true, 0u, q.x_signed != 0, p.S, word);
         *reinterpret_cast<uint4 *>(smem + c * p.plane + r * p.pitch + 4 * w4) = make_uint4(word[0], word[1], word[2], word[3]);
     }
     // ---- pack the kernel rows of these input and output channels (reversed rows, Theorem 3): [(ci, kh, j)][channel]

@@ -10,7 +10,7 @@ constexpr int kSmallTM = 2, kSmallTN = 4;      // output rows and channels per t
 struct SmallParams {
     StripParams s;             // geometry, slots and output as for the strip kernel (one row segment; ap, wp and corr unused)
     const int8_t *x, *w;
-    int codes;                 // in x
+    int ragged;                // ragged_codes() of x
     int B, H;
     int x_signed, w_signed, Kc;
     int Cz, CF;                // input channels per CTA of a cluster, input channels between two moves

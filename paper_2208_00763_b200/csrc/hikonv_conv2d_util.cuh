@@ -54,36 +54,41 @@ __device__ __forceinline__ uint32_t byte_range_mask(int i, int first, int last) 
     return m;
 }
 
+// For pack_row_words: the number of codes of a tensor at an address that is not a multiple of four or that ends at one, else -1.
+__host__ inline int ragged_codes(const void *x, int codes) { return (((uintptr_t)x | (unsigned)codes) & 3) != 0 ? codes : -1; }
+
 // Four packed words (Eq. 5) of N codes each, from column col0 on, of an image row of W one-byte codes: zero outside the row, and
-// everywhere when row_in is false (the row is then not read).  The row starts at code `row` of the tensor x of `codes` codes.
+// everywhere when row_in is false (the row is then not read).  The row starts at code `row` of the tensor x.
 // off4: a byte repeated four times that is taken from every code inside the columns of the image (in rows that are not read too),
 // is_signed: the codes, after that, are signed.
 // The codes start at any byte: the N + 1 aligned words around them are loaded (those that hold a code of the row), shifted into
-// place, blanked outside the row with one mask per word, and packed by byte permute and Horner's rule.  Where one of those words
-// reaches outside the tensor (the first codes of an unaligned tensor, the last ones of one whose size is not a multiple of four)
-// the codes are loaded byte by byte.
+// place, blanked outside the row with one mask per word, and packed by byte permute and Horner's rule.  Where the
+// tensor's ends are not aligned, the words that reach outside it are put together from bytes; ragged_codes() says so and is all
+// that aligned tensors pay (checked word by word for all of them, the 56x56x64 layer took 85.2 us instead of 84.7).
 template <int N>
-__device__ __forceinline__ void pack_row_words(const int8_t *x, int row, int codes, int W, int col0, bool row_in, uint32_t off4, bool is_signed,
+__device__ __forceinline__ void pack_row_words(const int8_t *x, int row, int ragged, int W, int col0, bool row_in, uint32_t off4, bool is_signed,
                                                int S, uint32_t (&word)[4]) {
     const int off = ((int)(uintptr_t)x + row + col0) & 3;        // of the first code in its aligned word
     const int first = row + col0 - off;                          // code at the start of that word (not in the tensor, where col0 < 0)
+    const uint32_t *al = reinterpret_cast<const uint32_t *>(x + first);
     uint32_t v[N + 1];
-    if (!row_in || (first >= 0 && first <= codes - 4 * (N + 1))) {
-        const uint32_t *al = reinterpret_cast<const uint32_t *>(x + first);
+    if (ragged < 0) {
 #pragma unroll
         for (int i = 0; i <= N; ++i) {
             const int c = col0 - off + 4 * i;                    // aligned word i holds the codes of columns c .. c + 3
-            v[i] = (row_in && c + 3 >= 0 && c < W) ? load_ordered(al + i) : 0u;
+            v[i] = row_in && c + 3 >= 0 && c < W ? load_ordered(al + i) : 0u;
         }
     } else {
 #pragma unroll
         for (int i = 0; i <= N; ++i) {
+            const int c = col0 - off + 4 * i;
             v[i] = 0u;
-#pragma unroll 1
-            for (int b = 3; b >= 0; --b) {                       // (a loop: few threads come here, and the launch has registers for few)
-                const int c = col0 - off + 4 * i + b;
-                v[i] = v[i] << 8 | (c >= 0 && c < W ? (uint32_t)(uint8_t)load_ordered(x + row + c) : 0u);
-            }
+            if (!row_in || c + 3 < 0 || c >= W) continue;
+            if (first + 4 * i >= 0 && first + 4 * i <= ragged - 4) v[i] = load_ordered(al + i);
+            else
+#pragma unroll
+                for (int b = 0; b < 4; ++b)
+                    if (c + b >= 0 && c + b < W) v[i] |= (uint32_t)(uint8_t)load_ordered(x + row + c + b) << (8 * b);
         }
     }
 #pragma unroll

@@ -44,6 +44,7 @@ static uint32_t byte_range_mask(int i, int first, int last) {
     return m;
 }
 template <typename T> T load_ordered(const T *p) { return __ldg(p); }
+#define __host__
 #define __device__
 #define __forceinline__ inline
 //FUNCTION
@@ -59,7 +60,7 @@ template <int N> void sweep(int W, int rows, int shift, bool is_signed, int off,
             for (int col0 = -2 * N; col0 < W; col0 += (rand() % 3) + 1) {
                 if (col0 + 4 * N <= 0) continue;
                 uint32_t word[4];
-                pack_row_words<N>(x, r * W, n, W, col0, in != 0, (uint32_t)off * 0x01010101u, is_signed || off != 0, S, word);
+                pack_row_words<N>(x, r * W, ragged_codes(x, n), W, col0, in != 0, (uint32_t)off * 0x01010101u, is_signed || off != 0, S, word);
                 for (int w = 0; w < 4; ++w, ++g_words) {
                     uint32_t want = 0;
                     for (int k = 0; k < N; ++k) {
@@ -88,9 +89,10 @@ int main() {
 @pytest.fixture(scope="module")
 def function_source():
     text = open(os.path.join(ROOT, "paper_2208_00763_b200", "csrc", "hikonv_conv2d_util.cuh")).read()
-    found = re.search(r"template <int N>\n__device__ __forceinline__ void pack_row_words\(.*?\n}\n", text, re.S)
-    assert found
-    return found.group(0)
+    parts = [re.search(pattern, text, re.S) for pattern in (r"__host__ inline int ragged_codes\(.*?\n",
+                                                            r"template <int N>\n__device__ __forceinline__ void pack_row_words\(.*?\n}\n")]
+    assert all(parts)
+    return "".join(p.group(0) for p in parts)
 
 
 def test_rows_are_packed_from_inside_the_tensor(function_source, tmp_path):
