@@ -503,6 +503,7 @@ int move_period(const hikonv_layout_t &L, const SplitConsts &sc, int p, int q, i
             fits = q_sum <= room && (!moves || e_sum <= room);
         }
         if (fits) return cf;
+        if (!moves) return 0;                                        // without moves the kernels sum all channels
     }
     return 0;
 }
