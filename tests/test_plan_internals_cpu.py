@@ -6,6 +6,7 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 DRIVER = r"""
 #include <cstdio>
+#include <initializer_list>
 #include "hikonv_internal.h"
 using namespace hikonv;
 // Layers whose layout needs no moves, with slots made narrower than the planner's: either all channels fit, or the answer is 0.
