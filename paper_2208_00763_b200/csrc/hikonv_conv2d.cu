@@ -284,7 +284,8 @@ static int staged_rows(int TS, int TM, int SH, int Hp, int K) {
 // Completes a candidate (TM, TN, TNX, TS and the row cut are set) and models its time in scheduler cycles of the busiest SM:
 // issue cycles of a warp (4.3 per multiply, about one for every other instruction; a tile of 2 x 4 costs a tenth more per multiply
 // than 4 x 8 by this count and by the clock) times the warps of the busiest scheduler, wave by wave.  Returns false when the candidate cannot run.
-static bool complete_choice(const StripProblem &q, StripChoice *c) {
+// most_resident: the CTAs of an SM that share its memory, at most.
+static bool complete_choice(const StripProblem &q, StripChoice *c, int most_resident = 32) {
     const int SH = ceil_div(q.Ho, c->TM), Hp = q.Ho + q.K - 1, KJ = q.K * q.J;
     const long long strips = (long long)q.B * SH;
     c->pitch = (c->XB + q.J - 1 + 3) / 4 * 4;
@@ -296,7 +297,7 @@ static bool complete_choice(const StripProblem &q, StripChoice *c) {
     c->ctas = (strips + c->TS - 1) / c->TS * c->NSEG * ceil_div(q.Co, TCO);
     const int share = (int)std::min<long long>(1000000, (c->ctas + q.sms - 1) / q.sms);
     // channels per stage: as many as leave room for the CTAs that the registers allow; runs of CF channels that fill stages
-    const int by_regs = std::min(65536 / (c->threads * 128), 32);
+    const int by_regs = std::min(65536 / (c->threads * 128), most_resident);
     const int want = std::max(1, std::min(by_regs, share));
     const size_t e_bytes = q.moves ? (size_t)c->threads * strip_e_pitch(c->TM, c->TN) * 8 : 0;
     const size_t per_cta = std::min<size_t>(kSmemPerCta, kSmemPerSm / want - 1024);
@@ -380,7 +381,7 @@ static StripChoice choose_strips(const StripProblem &q, int force_tm, int force_
         if (force_ks > 0 && KS != force_ks && !q.generic) continue;
         if (!strip_tile_built(TM, TN, q.generic) || (force_tm > 0 && TM != force_tm && !q.generic) ||
             (force_tn > 0 && TN != force_tn && !q.generic)) continue;
-        if (TN == 8 && q.Co <= 4 && force_tn != 8) continue;
+        if (TN == 8 && q.Co <= 4 && force_tn != 8 && force_tm != 4) continue;      // (four rows are built with eight channels only)
         const int SH = ceil_div(q.Ho, TM);
         const long long strips = (long long)q.B * SH;
         for (int TNX = 1; TNX * TN <= kStripBPitch; TNX *= 2) {
@@ -410,11 +411,15 @@ static StripChoice choose_strips(const StripProblem &q, int force_tm, int force_
                 if (cut > 1 && c.XO < 24 && best.cost >= 0) break;     // narrow segments only where nothing else fits
                 ++tried;
                 const int ts_hi = (int)std::max<long long>(1, std::min<long long>(maxpos / c.XB, strips));
-                const int ts_forced = force_rows > 0 ? std::min(ceil_div(force_rows, TM), ts_hi) : 0;
-                for (int TS = ts_forced > 0 ? ts_forced : 1; TS <= (ts_forced > 0 ? ts_forced : ts_hi); ++TS) {
+                // a forced height stands for itself, or for the greatest below it that fits
+                const bool forced = force_rows > 0;
+                for (int TS = forced ? std::min(ceil_div(force_rows, TM), ts_hi) : 1; TS >= 1 && TS <= ts_hi; TS += forced ? -1 : 1) {
                     c.TS = TS;
-                    if (!complete_choice(q, &c)) continue;
+                    bool fits = complete_choice(q, &c);
+                    for (int resident = 16; forced && !fits && resident >= 1; resident /= 2) fits = complete_choice(q, &c, resident);
+                    if (!fits) continue;
                     if (best.cost < 0 || c.cost < best.cost * (1.0 - 1e-9)) best = c;
+                    if (forced) break;
                 }
             }
         }

@@ -389,3 +389,12 @@ def test_layers_accept_a_workspace_of_the_queried_size():
     out = subprocess.run([sys.executable, "-c", _WORKSPACE_PROBE], cwd=ROOT, env=dict(os.environ, CUDA_VISIBLE_DEVICES=""),
                          capture_output=True, text=True, timeout=600)
     assert out.returncode == 0, out.stderr[-2000:]
+
+
+def test_forced_tiles_never_refuse_a_layer():
+    # heights that do not fit the shared memory of a wide kernel, four rows per thread with few output channels
+    for (B, Ci, H, W, Co, K, pad, p, q) in ((8, 5, 700, 20, 9, 17, 5, 2, 1), (64, 128, 700, 2, 4, 16, 9, 4, 3), (32, 5, 5, 14, 100, 16, 9, 3, 3),
+                                            (1, 16, 8, 57, 4, 3, 1, 4, 4), (2, 3, 57, 57, 3, 5, 2, 6, 6), (1, 2, 3, 320, 4, 1, 0, 2, 2), (1, 9, 6, 6, 1, 7, 3, 3, 3)):
+        want = hk.conv2d_layout(B, Ci, H, W, Co, K, pad, p, q, True, True)
+        for tile in (1, 3, 22, 48, 1001, 1009, 2003, 8000, 16000, 200000, 202010, 400000, 400006, 401001, 401040, 404048, 4000000, 8000000, 8400000, -1, -2):
+            assert hk.conv2d_layout(B, Ci, H, W, Co, K, pad, p, q, True, True, tune={"tile": tile}) == want, tile
