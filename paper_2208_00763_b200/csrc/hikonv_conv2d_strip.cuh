@@ -526,10 +526,8 @@ int launch_strip(const StripLaunch &s, cudaStream_t st) {
     }
     if (s.KS != 1) return HIKONV_ERR_UNSUPPORTED;
     if (s.TM == 2 && s.TN == 4) return launch_strip_tile<N, KT, JT, 2, 4>(s, st);
-    if constexpr (KT > 0) {
-        if (s.TM == 2 && s.TN == 8) return launch_strip_tile<N, KT, JT, 2, 8>(s, st);
-        if (s.TM == 4 && s.TN == 8) return launch_strip_tile<N, KT, JT, 4, 8>(s, st);
-    }
+    if (s.TM == 2 && s.TN == 8) return launch_strip_tile<N, KT, JT, 2, 8>(s, st);
+    if (s.TM == 4 && s.TN == 8) return launch_strip_tile<N, KT, JT, 4, 8>(s, st);
     return HIKONV_ERR_UNSUPPORTED;
 }
 

@@ -53,11 +53,8 @@ struct StripLaunch {
     bool generic;                    // the kernel with run-time loop bounds
 };
 
-// Thread tiles the kernel is built for: 4 x 8, 2 x 8 and 2 x 4 rows x channels (2 x 4 with run-time loop bounds).  4 x 4 was as
-// fast as 2 x 8 on no layer.
-inline bool strip_tile_built(int TM, int TN, bool generic) {
-    return generic ? (TM == 2 && TN == 4) : ((TM == 2 && (TN == 4 || TN == 8)) || (TM == 4 && TN == 8));
-}
+// Thread tiles the kernel is built for: 4 x 8, 2 x 8 and 2 x 4 rows x channels.  4 x 4 was as fast as 2 x 8 on no layer.
+inline bool strip_tile_built(int TM, int TN) { return (TM == 2 && (TN == 4 || TN == 8)) || (TM == 4 && TN == 8); }
 // Tiles that are also built with two or four thread groups, which share the input channels.
 inline bool strip_split_built(int TM, int TN, int KS, bool generic) { return !generic && TM == 2 && (KS == 2 || (KS == 4 && TN == 4)); }
 // 8-byte entries of a thread in the second-accumulator area: TM TN and one that keeps the pitch odd.

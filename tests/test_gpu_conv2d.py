@@ -192,6 +192,30 @@ def test_deep_unsigned_layers_on_shifted_codes(p):
         assert_exact(_layer(x, w, 1, p, 4, False, True, hk.ALGO_PACKED32), direct.conv2d_nchw(x, w, 1), "extreme p=%d" % p)
 
 
+@pytest.mark.parametrize("K, pad", [(2, 0), (4, 1), (6, 2), (7, 3), (9, 4), (16, 7), (33, 16)])
+def test_kernel_sizes_without_unrolled_loops(K, pad):
+    # run-time loop bounds: every thread tile (2 x 4, 2 x 8 and 4 x 8 rows x channels, ragged strips and channels), both signs, pixels
+    # per word from four to one, sums and pooled codes; wide kernels on small maps
+    for (B, Ci, H, W, Co) in ((2, 5, 10, 12, 9), (1, 17, 6, 40, 20)):
+        if H + 2 * pad < K or W + 2 * pad < K:
+            continue
+        widths = ((4, 4, True, True), (1, 1, False, False), (2, 2, False, True), (8, 8, True, True)) if K < 33 else ((1, 1, False, False),)
+        for (p, q, xs, ws) in widths:                          # (33 taps fit the multiplier at one bit only)
+            x, w = inputs.conv2d_case(B, Ci, H, W, Co, K, p, q, xs, ws, seed=80 + K + Ci + p)
+            ref = direct.conv2d_nchw(x, w, pad)
+            d_x, d_w = dev(x), dev(w)
+            for tile in (0, 4200000, 8202000, 8402004):
+                what = "%s K=%d p=%d tile=%d" % ((B, Ci, H, W, Co), K, p, tile)
+                assert_exact(hk.conv2d(d_x, d_w, pad, p, q, xs, ws, tune={"tile": tile}), ref, what)
+                if ref.shape[2] % 2 == 0 and ref.shape[3] % 2 == 0:
+                    got = hk.conv2d_dense(d_x.reshape(-1), x.shape, 8, d_w.reshape(-1), w.shape, 8, pad, p, q, xs, ws, requant=(p, -8, 7), pool=True,
+                                          tune={"tile": tile})
+                    assert_exact(got, direct.maxpool2x2(direct.requant(ref, p, -8, 7)), "pool " + what)
+    bits, signed = (4, True) if K < 33 else (1, False)
+    for x, w in inputs.extreme_2d(1, 9, K, K + 3, 6, K, bits, bits, signed, signed):
+        assert_exact(_layer(x, w, pad, bits, bits, signed, signed, hk.ALGO_PACKED32, tune={"tile": 8400000}), direct.conv2d_nchw(x, w, pad), "extreme")
+
+
 def test_waits_that_run_out_are_counted():
     # one thread waits a millisecond for a barrier that nothing completes, on a stream that does not wait for the default one
     hk.conv2d_wait_timeouts()
