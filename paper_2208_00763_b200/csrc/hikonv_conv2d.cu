@@ -367,6 +367,11 @@ static bool complete_choice(const StripProblem &q, StripChoice *c, int most_resi
     // With run-time bounds the tile of 2 x 8 is the fastest oftener than this count says, in small CTAs above all (by the clock over 24
     // layers of 2x2 to 9x9 kernels the choice is 1.8 % off the best tile, 3 % without these two).
     if (q.generic) cycles *= (c->TM == 4 ? 1.1 : 1.0) * (waves > 1.0 ? 1.0 + 0.1 * (1.0 / resident - 0.5) : 1.0);
+    // Where CTAs follow one another, more and smaller ones on an SM cover each other's barriers: at costs within half a per cent, four
+    // CTAs of 128 threads took 5 to 6 % less than two of 256 (32x64x56x56 -> 64 at 8 bits unsigned 241.6 -> 229.6 us, signed 228.0 ->
+    // 220.5; 16x24x56x61 -> 256 6 x 4 bits 141.6 -> 126.4).  Enough to decide between tiles of equal cost: with more of it the 4-bit
+    // 56x56 layer took 91 us instead of 84.
+    if (waves > 1.0 && !q.generic) cycles *= 1.0 + 0.03 * (1.0 / resident - 0.5);
     c->cost = cycles;
     return true;
 }
