@@ -277,6 +277,15 @@ int hikonv_conv2d_layout(int B, int Ci, int H, int W, int Co, int K, int pad, in
                          int w_signed, const hikonv_tuning_t *tune, hikonv_layout_t *out, int *x_shift);
 
 /*
+ * hikonv_conv2d_launches - how many kernels a layer on tensors of one code per byte runs in (host only): *launches is 2, or 1 for the
+ * small layers whose operands are packed by the layer kernel itself; *cluster (may be NULL) is then the number of CTAs that
+ * share a tile's input channels (1, 2, 4 or 8), else 0.  requant and pool as for hikonv_conv2d_dense; other arguments and
+ * errors as for hikonv_conv2d_layout.
+ */
+int hikonv_conv2d_launches(int B, int Ci, int H, int W, int Co, int K, int pad, int p, int q, int x_signed, int w_signed,
+                           int requant, int pool, const hikonv_tuning_t *tune, int *launches, int *cluster);
+
+/*
  * hikonv_conv2d_dense - hikonv_conv2d on tensors stored without their unused bits (Section V-B, single convolver
  * architecture: the weights sit in memory in compressed form, and the section notes that features can be kept
  * that way at run time too), with the layer's requantised output written in the same compressed form and,

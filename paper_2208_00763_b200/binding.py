@@ -67,6 +67,7 @@ _SIGNATURES = {
     "hikonv_conv2d_tune": (_i, [_vp, _i, _i, _i, _i, _i, _vp, _i, _i, _i, _i, _i, _i, _i, _i, _i, _vp, _i, _i, _i, _i, _i, _i, _vp, _sz,
                                 _i, _i, ctypes.POINTER(_i), ctypes.POINTER(_d), ctypes.POINTER(_d), _vp]),
     "hikonv_conv2d_workspace_bytes": (_sz, [_i] * 7),
+    "hikonv_conv2d_launches": (_i, [_i] * 13 + [ctypes.POINTER(TuningT), ctypes.POINTER(_i), ctypes.POINTER(_i)]),
     "hikonv_conv2d_wait_timeouts": (_i, [_vp]),
     "hikonv_conv2d_wait_check": (_i, [ctypes.c_longlong, _vp]),
     "hikonv_conv2d_static_scratch": (_i, [_vp, _i, _i, _i, _i, _vp, _i, _i, _i, _i, _i, _i, _i, _i, _vp, _i, _i, _i, _i, _i,
@@ -210,6 +211,14 @@ def conv2d_layout(B, Ci, H, W, Co, K, pad, p, q, x_signed, w_signed, tune=None) 
     d = {n: getattr(out, n) for n, _ in LayoutT._fields_}
     d["x_shift"] = shift.value
     return d
+
+
+def conv2d_launches(B, Ci, H, W, Co, K, pad, p, q, x_signed, w_signed, requant=False, pool=False, tune=None) -> tuple:
+    """(kernels a layer runs in, CTAs that share a tile's input channels in a single one or 0)."""
+    launches, cluster = ctypes.c_int(0), ctypes.c_int(0)
+    _check(lib().hikonv_conv2d_launches(B, Ci, H, W, Co, K, pad, p, q, int(x_signed), int(w_signed), int(bool(requant)), int(pool),
+                                        _tune(tune), ctypes.byref(launches), ctypes.byref(cluster)), "hikonv_conv2d_launches")
+    return launches.value, cluster.value
 
 
 # ------------------------------------------------------------------ device entry points

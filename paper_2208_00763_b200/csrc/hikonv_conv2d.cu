@@ -1065,6 +1065,18 @@ extern "C" int hikonv_conv2d_layout(int B, int Ci, int H, int W, int Co, int K, 
     return HIKONV_OK;
 }
 
+extern "C" int hikonv_conv2d_launches(int B, int Ci, int H, int W, int Co, int K, int pad, int p, int q, int x_signed, int w_signed,
+                                      int requant, int pool, const hikonv_tuning_t *tune, int *launches, int *cluster) {
+    if (!launches) return HIKONV_ERR_INVALID_ARG;
+    Conv2dSetup s;
+    const OutputSpec out = {requant ? 1 : 0, 0, 0, 0, pool ? 1 : 0, 8, nullptr, 1};
+    const int rc = setup_layer(B, Ci, H, W, Co, K, 1, pad, p, q, x_signed ? 1 : 0, w_signed ? 1 : 0, out, HIKONV_ALGO_PACKED32, tune, &s);
+    if (rc != HIKONV_OK) return rc;
+    *launches = s.one_launch ? 1 : 2;
+    if (cluster) *cluster = s.one_launch ? (int)s.small.grid.z : 0;
+    return HIKONV_OK;
+}
+
 extern "C" double hikonv_conv2d_multiplies(int B, int Ci, int H, int W, int Co, int K, int pad, int p, int q, int x_signed,
                                            int w_signed, int algo, const hikonv_tuning_t *tune) {
     Conv2dSetup s;

@@ -85,13 +85,9 @@ def test_strips_of_rows_in_every_tile(K, pad):
         for (p, q, xs, ws) in ((4, 4, True, True), (4, 4, False, True), (8, 8, True, True), (2, 2, False, True), (8, 4, False, True), (5, 5, False, False)):
             x, w = inputs.conv2d_case(B, Ci, H, W, Co, K, p, q, xs, ws, seed=B + Ci + K + p)
             ref = direct.conv2d_nchw(x, w, pad)
-            for tile in (0, 1, 2001, 200001, 204003, 401002, 404004, 208008, 1048):
-                try:
-                    got = _layer(x, w, pad, p, q, xs, ws, hk.ALGO_PACKED32, tune={"tile": tile})
-                except hk.HikonvError as err:          # forced shapes that need more threads than a CTA has
-                    assert err.status == hk.ERR_UNSUPPORTED and tile != 0
-                    continue
-                assert_exact(got, ref, "%s K=%d p=%d q=%d tile=%d" % ((B, Ci, H, W, Co), K, p, q, tile))
+            for tile in (0, 1, 2001, 200001, 204003, 401002, 404004, 208008, 1048):       # none is refused
+                assert_exact(_layer(x, w, pad, p, q, xs, ws, hk.ALGO_PACKED32, tune={"tile": tile}), ref,
+                             "%s K=%d p=%d q=%d tile=%d" % ((B, Ci, H, W, Co), K, p, q, tile))
 
 
 @pytest.mark.parametrize("K, pad", [(1, 0), (3, 1), (5, 2), (5, 4)])
@@ -143,6 +139,8 @@ def test_small_layers_in_one_launch(K, pad):
     # tile = -2: operands packed by the layer kernel, input channels shared by the CTAs of a cluster; channel counts that cut
     # unevenly or leave the last CTAs none, strips of several images, ragged last strips, sums, codes and pooled codes, against
     # the two-launch form (tile = -1) and the oracle
+    form = lambda B, Ci, H, W, Co, p, q, xs, ws, tile, **kw: hk.conv2d_launches(B, Ci, H, W, Co, K, pad, p, q, xs, ws, tune={"tile": tile}, **kw)
+    single, pooled, clusters = 0, 0, set()
     for (B, Ci, H, W, Co) in ((1, 64, 10, 20, 64), (3, 5, 7, 9, 6), (5, 11, 6, 6, 33), (1, 3, 8, 150, 7), (2, 33, 4, 4, 4), (1, 1, 5, 5, 1)):
         for (p, q, xs, ws) in ((4, 4, True, True), (4, 4, False, True), (8, 8, True, True), (2, 2, False, False), (8, 4, False, True), (5, 5, False, False)):
             x, w = inputs.conv2d_case(B, Ci, H, W, Co, K, p, q, xs, ws, seed=50 + B + Ci + K + p)
@@ -150,6 +148,10 @@ def test_small_layers_in_one_launch(K, pad):
             d_x, d_w = dev(x), dev(w)
             for rq in (None, (p, 0, 15), (p, -8, 7)):
                 want = direct.requant(ref, *rq) if rq else ref
+                assert form(B, Ci, H, W, Co, p, q, xs, ws, -1, requant=rq)[0] == 2
+                launches, cluster = form(B, Ci, H, W, Co, p, q, xs, ws, -2, requant=rq)
+                single += launches == 1
+                clusters.add(cluster)
                 for tile in (-1, -2):
                     got = hk.conv2d(d_x, d_w, pad, p, q, xs, ws, requant=rq, tune={"tile": tile})
                     assert_exact(got, want, "%s K=%d p=%d q=%d %s tile=%d" % ((B, Ci, H, W, Co), K, p, q, rq, tile))
@@ -157,8 +159,20 @@ def test_small_layers_in_one_launch(K, pad):
                     got = hk.conv2d_dense(d_x.reshape(-1), x.shape, 8, d_w.reshape(-1), w.shape, 8, pad, p, q, xs, ws, requant=rq, pool=True,
                                           tune={"tile": -2})
                     assert_exact(got, direct.maxpool2x2(want), "pool %s K=%d p=%d q=%d %s" % ((B, Ci, H, W, Co), K, p, q, rq))
+                    pooled += form(B, Ci, H, W, Co, p, q, xs, ws, -2, requant=rq, pool=True)[0] == 1
+    assert single >= 100 and pooled >= 40 and clusters >= {1, 8}, (single, pooled, clusters)     # (it falls back where it is not built)
     for x, w in inputs.extreme_2d(1, 70, 6, 10, 8, K, 4, 4, True, True):
         assert_exact(_layer(x, w, pad, 4, 4, True, True, hk.ALGO_PACKED32, tune={"tile": -2}), direct.conv2d_nchw(x, w, pad), "extreme")
+
+
+@pytest.mark.parametrize("layer, K, pad, bits, cluster", [
+    ((4, 3, 9, 9, 33), 3, 1, 8, 1), ((2, 24, 40, 24, 90), 3, 1, 8, 2), ((2, 9, 17, 36, 73), 5, 2, 8, 2), ((8, 33, 34, 19, 35), 1, 0, 8, 2),
+    ((1, 6, 40, 40, 16), 5, 2, 4, 4), ((2, 24, 20, 20, 32), 3, 1, 2, 8)])
+def test_every_cluster_size_of_the_one_launch_kernel(layer, K, pad, bits, cluster):
+    B, Ci, H, W, Co = layer
+    assert hk.conv2d_launches(B, Ci, H, W, Co, K, pad, bits, bits, True, True, tune={"tile": -2}) == (1, cluster)
+    x, w = inputs.conv2d_case(B, Ci, H, W, Co, K, bits, bits, True, True, seed=60 + Ci)
+    assert_exact(_layer(x, w, pad, bits, bits, True, True, hk.ALGO_PACKED32, tune={"tile": -2}), direct.conv2d_nchw(x, w, pad), "%s" % (layer,))
 
 
 @pytest.mark.parametrize("ci", [4, 7, 20, 64, 130, 256])
