@@ -9,8 +9,9 @@ A "step" is one pass of the whole hot path over the 1-D bitwidth sweep: 48 full 
 16 MiB input and writing its own 64 MiB int32 output, so a step streams about 3.9 GB and nothing
 is served from L2.  The metric is effective multiply-accumulates of the plain definition per
 second.  The line also carries the roofline of the dominant kernel, the same path timed end to
-end from pinned host buffers, the oracle timed on the host cores, and (unless --no-extra) the
-2-D layer and full-network workloads with the one-product-per-multiply comparator beside them.
+end from pinned host buffers, the oracle timed on the host cores, and (unless --no-extra) a summary of the
+2-D layer and full-network workloads with the one-product-per-multiply comparator beside them; the tables
+behind that summary go to the file named by --extra-out, so that the line stays short.
 """
 from __future__ import annotations
 
@@ -43,11 +44,10 @@ TABLE_REPEATS = 7                    # timed repeats per cell of the per-case ta
 # buffers, caches not flushed between launches (steady state): 13.1-13.7 MB read, 63.1-66.2 MB written
 # (the 8-bit K=7 case: 79.9 MB in all).  (With the caches flushed before each launch the same kernel shows
 # 16.8 MB read and 8-9 MB written: most of a launch's output is then still in the 126 MB L2 when its
-# counters stop.)  The SHA-256 values are those of the kernel sources at capture time; a changed source voids
-# the figure.
+# counters stop.)  The SHA-256 values are those of the kernel sources, the headers they are compiled from among them, at capture
+# time; a changed source voids the figure.
 NCU_TRAFFIC = {
     "conv1d_bs": {"sha256": "5655bc948411944c895bc88fbc1ce61e93428afcd63aa7d4740d6c3f16a0914b",
-                  "sha256_run": "ff003dacc21c948f04a6b5e0ee717c8420ab96ffc1c03d52a54906dad43f8413",
                   "bytes_per_output": (13.37e6 + 65.20e6) / 16777218.0},
 }
 
@@ -60,9 +60,16 @@ NCU_INSTRUCTIONS = {
 }
 
 
-def _source_hash(name: str) -> str:
-    with open(os.path.join(ROOT, "paper_2208_00763_b200", "csrc", name), "rb") as fh:
-        return hashlib.sha256(fh.read()).hexdigest()
+BS_SOURCES = ("hikonv_conv1d_bs.cu", "hikonv_conv1d_run.cuh", "hikonv_conv1d_tc.h", "hikonv_cuda.cuh")
+STRIP_SOURCES = ("hikonv_conv2d_strip.cuh", "hikonv_conv2d_strip.h", "hikonv_conv2d_util.cuh", "hikonv_cuda.cuh")
+
+
+def _source_hash(names) -> str:
+    h = hashlib.sha256()
+    for name in names:
+        with open(os.path.join(ROOT, "paper_2208_00763_b200", "csrc", name), "rb") as fh:
+            h.update(fh.read())
+    return h.hexdigest()
 
 
 def measured_peaks():
@@ -372,8 +379,7 @@ def run_ours(args):
     achieved_gbs = bytes_per_launch / avg_launch_s / 1e9
     traffic = None
     rec = NCU_TRAFFIC.get("conv1d_bs")
-    if args.algo == "packed" and rec and rec.get("sha256") == _source_hash("hikonv_conv1d_bs.cu") and \
-            rec.get("sha256_run") == _source_hash("hikonv_conv1d_run.cuh"):
+    if args.algo == "packed" and rec and rec.get("sha256") == _source_hash(BS_SOURCES):
         traffic = rec["bytes_per_output"] * outputs_per_step / launches_per_step
     roofline = {"bound": "hbm", "achieved": achieved_gbs, "peak": hbm_peak_gbs, "unit": "GB/s",
                 "frac": achieved_gbs / hbm_peak_gbs, "traffic": traffic, "peak_kind": "of " + peak_kind,
@@ -477,7 +483,9 @@ def run_ours(args):
             torch.cuda.empty_cache()
             extra.update(layer_workloads(torch, np, hk, inputs, network, dev, imad_peak))
             extra["peaks"] = peaks
-            line["extra"] = extra
+            line["extra"] = summary_of(extra)
+            if rank == 0:
+                line["extra"]["file"] = write_extra(args.extra_out, extra)
         line["cpu_baseline"] = cpu_baseline(1 << 22)
 
     if rank == 0:
@@ -588,6 +596,30 @@ def run_layer_main(args, torch, np, ranks, hk, inputs, network, dev, world, rank
     return 0
 
 
+def summary_of(extra: dict) -> dict:
+    """What the line says of the workloads beside the sweep: milliseconds, packed against comparator, share of the measured
+    multiply rate."""
+    out = {"c2_unpacked_ms": extra["c2_unpacked"]["ms_per_step"],
+           "c2_cases_packed_faster_tied_slower": [len(extra["c2_packed_vs_unpacked"][k]) for k in
+                                                  ("cases_packed_faster", "cases_tied_within_spread", "cases_packed_not_faster")]}
+    for name in ("c3", "c4", "c5"):
+        out[name] = {"packed_ms": extra[name]["packed"]["ms"], "unpacked_ms": extra[name]["unpacked"]["ms"],
+                     "frac": extra[name]["packed"]["roofline"]["frac"]}
+    out["c3_shape_ms_by_bits"] = {p: round(row["packed_ms"], 4) for p, row in extra["c3_shape_by_bitwidth"].items()}
+    return out
+
+
+def write_extra(path: str, extra: dict):
+    """Writes the tables to `path`; its name for the line, or None where it cannot be written (the line is printed all the same)."""
+    try:
+        os.makedirs(os.path.dirname(os.path.abspath(path)), exist_ok=True)
+        with open(path, "w") as fh:
+            json.dump(extra, fh, indent=1)
+    except OSError:
+        return None
+    return os.path.relpath(path, ROOT)
+
+
 def alu_roofline(muls: float, ms: float, imad_peak: dict, key: str, workload: str = None) -> dict:
     """Multiplies executed per second against the rate of that multiply: `peak` is the rate the library's own
     register-only kernel reached on this GPU (hikonv_pipe_rate) when it was measured, `frac_of_derived` divides by
@@ -604,7 +636,7 @@ def alu_roofline(muls: float, ms: float, imad_peak: dict, key: str, workload: st
     # instruction of the layer kernel (counted under ncu); the sum over the device's schedulers is the time the layer
     # kernel cannot go below with this instruction mix, to be read against the step (which also holds the packing launch).
     rec, issue = NCU_INSTRUCTIONS.get(workload or ""), imad_peak.get("issue")
-    if key == "packed" and rec and issue and rec["sha256"] == _source_hash("hikonv_conv2d_strip.cuh"):
+    if key == "packed" and rec and issue and rec["sha256"] == _source_hash(STRIP_SOURCES):
         mads = muls / 32.0
         others = rec["warp_instructions"] - mads
         cycles = issue["cycles_per_wide_multiply_add"] * mads + issue["cycles_added_per_other_instruction"] * others
@@ -805,6 +837,8 @@ def main():
     ap.add_argument("--warmup", type=int, default=3)
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
     ap.add_argument("--no-extra", action="store_true", help="skip the comparator, per-case and 2-D workloads")
+    ap.add_argument("--extra-out", default=os.path.join(ROOT, "build", "bench_extra.json"),
+                    help="file for the tables of the comparator, per-case and 2-D workloads")
     ap.add_argument("--e2e-steps", type=int, default=2)
     ap.add_argument("--length", type=int, default=1 << 24, help="signal length of the sweep (benchmark value: 2^24)")
     ap.add_argument("--workload", default="c2", choices=["c2", "c3", "c4", "c5"],

@@ -250,9 +250,9 @@ int hikonv_conv2d(const int8_t *d_x, int B, int Ci, int H, int W, const int8_t *
  * hikonv_conv2d_tune - times the tile shapes of one layer on the device and returns the fastest (a set-up aid with no
  * counterpart in the paper: the automatic choice comes from a cost model, which on small layers misses tiles that
  * measure 10-20 % faster).  Arguments up to `algo` are those of hikonv_conv2d_dense (one code per byte: storage 8 / 8,
- * out_store_bits 8, or 32 without requant).  The call runs the layer with the library's own tile and with every forced
- * tile (rows per thread 4 and 2 x channels per thread 4 and 8 x channel lanes 1, 2, 4, 8 x output rows per CTA up to 48; shapes the layer does not
- * support are skipped), each as groups of four launches between two CUDA events on `stream`, best of `repeats` (1 .. 100)
+ * out_store_bits 8, or 32 without requant).  The call runs the layer with the library's own choice and with every forced
+ * tile of one thread group in two launches (4 x 8, 2 x 8 and 2 x 4 rows x channels per thread x channel lanes 1, 2, 4, 8 x output
+ * rows per CTA up to 48; several thread groups and the one-launch form are left to the library's choice), each as groups of four launches between two CUDA events on `stream`, best of `repeats` (1 .. 100)
  * groups, and SYNCHRONISES.  Every launch writes the layer's complete, correct output to d_out.
  * *h_tile: the value for hikonv_tuning_t.tile in later calls on this shape, or 0 when no forced tile is at least 3 %
  * faster than the automatic one.  *h_us / *h_default_us (may be NULL): microseconds per launch of the winner and of

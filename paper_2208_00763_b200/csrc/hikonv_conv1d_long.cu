@@ -8,7 +8,7 @@
 // registers, across threads through shared memory; the outputs leave through shared memory in 16-byte pieces.
 // What bounds it: instruction issue (4 R wide multiplies and about R + 8 other instructions per four chunks), near the memory
 // floor for the shortest filters that come here.  The kernel it replaces for them (one block per lane, a shuffle and a shared
-// load per multiply, byte loads) took 18.7 us a call for 4.2 M codes and 31 taps (u4 x s4, N = 3, eleven chunks); this one 7.1.
+// load per multiply, byte loads) took 18.6 us a call for 4.2 M codes and 31 taps (u4 x s4, N = 3, eleven chunks); this one 6.9.
 #include "hikonv_conv1d_run.cuh"
 
 namespace hikonv {
@@ -19,8 +19,8 @@ constexpr int kLongJ = (kMaxJ + 3) / 4 * 4;                    // chunks, rounde
 __host__ __device__ constexpr int long_run(int N) { return N == 1 ? 15 : N == 2 ? 11 : N <= 4 ? 7 : N == 5 ? 5 : 3; }
 
 // Resident CTAs: a signal of a few million codes is about one wave of them, with a tail of a few per cent at five CTAs per SM
-// and none at six, which N = 3 reaches without spilling (4.2 M codes, 12 / 16 / 31 taps: 6.3 / 7.0 / 7.7 -> 5.5 / 6.3 / 7.3 us on
-// the device; the other block sizes lost 2 to 20 % at five or six).
+// and none at six, which N = 3 reaches without spilling (4.2 M codes, 12 / 16 / 31 taps: 6.3 / 7.0 / 7.7 -> 5.5 / 6.3 / 7.3 us for
+// a launch by itself; the other block sizes lost 2 to 20 % at five or six).
 template <int N, bool SP, bool FS>
 __global__ void __launch_bounds__(kLongThreads, N == 3 ? 6 : 3) conv1d_long_kernel(const Conv1dTcParams p) {
     constexpr int R = long_run(N), TILE = kLongThreads * R, FRONT = kLongJ;   // blocks per tile; packed words in front of it

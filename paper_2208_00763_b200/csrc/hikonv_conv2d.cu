@@ -232,8 +232,6 @@ __global__ void __launch_bounds__(256) maxpool2x2_kernel(const int8_t *__restric
 
 // ------------------------------------------------------------------ host side
 
-// ------------------------------------------------------------------ host side
-
 struct Conv2dSetup {
     hikonv_layout_t L;
     bool unpacked;
@@ -774,7 +772,7 @@ static int conv2d_run(const void *d_x, int x_bits, int B, int Ci, int H, int W, 
         dv.per_plane = make_div32((uint32_t)(s.Hp * (s.XBT / 4)));
         dv.b = make_div32((uint32_t)B);
         dv.xq = make_div32((uint32_t)(s.XBT / 4));
-        // (10 CTAs per SM are faster in the first way, 3 in the second)
+        // eight CTAs per SM where the launch has enough of them, three where it is small (see the kernel)
         const bool many = grid > 6u * (unsigned)sm_count();
         auto pack = [&](auto kern) {
             return launch_dependent(kern, dim3(grid), dim3(256), 0, st, (const int8_t *)d_x, ragged, B, Ci, H, W, s.Hp, pad, s.col_first, s.L.S,
@@ -855,7 +853,7 @@ extern "C" int hikonv_conv2d_dense(const void *d_x, int x_store_bits, int B, int
                       requant ? out_store_bits : 8, requant, shift, lo, hi, pool, d_workspace, workspace_bytes, algo, tune, stream);
 }
 
-// Times the layer with the library's own tile and with every forced tile shape (positions per thread x channel lanes x
+// Times the layer with the library's own choice and with every tile of one thread group (rows x channels per thread x channel lanes x
 // rows per CTA), `batch` launches between two events, best of `repeats`; the result of every launch is the layer's output.
 extern "C" int hikonv_conv2d_tune(const void *d_x, int x_store_bits, int B, int Ci, int H, int W, const void *d_w,
                                   int w_store_bits, int Co, int K, int stride, int pad, int p, int q, int x_signed,

@@ -73,10 +73,10 @@ inline int stage_channel_cap(int K, int J) {
     return c < 1 ? 1 : (c > 8 ? 8 : c);
 }
 
-// The planner's rule for 2-D layers: the upper slot bits move to the second accumulator every `fc` stages of CK input
-// channels.  Given the number of channels CF that may be accumulated between two
-// such moves, picks CK <= ck_cap and fc with CK * fc <= CF as large as possible (stages of fewer than
-// three channels are avoided when something close is available).  Returns CK * fc.
+// How the planner rounds the products M between two moves of a 2-D layer: to what fc stages of CK input channels hold.  Given the
+// number of channels CF that may be accumulated, picks CK <= ck_cap and fc with CK * fc <= CF as large as possible (stages of
+// fewer than three channels are avoided when something close is available).  Returns CK * fc.  The layer kernel has longer stages
+// and moves after any number of channels (move_period()), so the rounding is stricter than it needs.
 inline int pick_chunking(int CF, int Ci, int *CK, int *fc, int ck_cap = 8) {
     if (CF >= Ci) {
         *CK = Ci < ck_cap ? Ci : ck_cap;

@@ -11,7 +11,7 @@ constexpr int kMaxPackN = 12;
 // words of codes whatever N is, so a thread loads those (16 or 8 bytes at a time where N allows), takes each code out
 // with one byte permute, adds it by Horner's rule (one multiply-add per code for 32-bit words) and writes 16-byte
 // pieces.  The last, partial group is packed code by code by the thread it falls to.  2^24 4-bit codes, three per 32-bit
-// word: 15.9 -> 8.2 us on the device (39 MB, 4.8 TB/s), 20.5 -> 10.7 us a call among others.
+// word: 20.5 -> 7.0 us a call among others (39 MB, 5.6 TB/s).
 template <bool SIGNED, typename WORD, int N>
 __global__ void __launch_bounds__(256) pack_groups_kernel(const int8_t *in, size_t n, int S, WORD *__restrict__ words,
                                                           size_t n_words) {

@@ -151,7 +151,7 @@ static bool check_candidate(int p, int q, int fs, int gs, int K, int N, int S, b
                 if (fits_cs(mid, h)) a = mid; else b = mid - 1;
             }
             if (a < carry_save_total) {
-                // the kernel moves bits at channel-stage borders: whole channels, in the staging it can realise
+                // whole channels, in groups of short stages (stricter than the layer kernel asks for, see pick_chunking)
                 const int Ci = (int)(carry_save_total / K);
                 if (a < K) continue;
                 int ck, fc;
