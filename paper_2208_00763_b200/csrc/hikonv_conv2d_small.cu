@@ -7,9 +7,10 @@
 // finishing the rows and channels that fall to it.  Tile, products, moves, overlap-add and slots are those of the strip
 // kernel (hikonv_conv2d_strip.cuh) with 2 x 4 rows x channels per thread.
 // The packing is repeated by every CTA that reads a row, and a cluster's sums cross the network between SMs, so larger layers
-// are faster on two launches: plan_layer compares the modelled times.  Device time of one against two launches: 64 -> 64 channels
-// on one 10x20 map 7.4 / 16.8 us, on 64 of them 23.4 / 18.1; 119 -> 37 channels 5x5 8-bit on two 18x17 maps 17.7 / 68.2; the
-// compact CNN on one image 82 / 124 us (seven of its nine layers run here), 128 / 145 us a call among others, bound by the host.
+// are faster on two launches: plan_layer compares the modelled times.  Time of one against two launches, one call after the
+// other in a graph: 5 -> 183 channels on five 7x46 maps 3.7 / 4.2 us, 64 -> 36 channels 1x1 on one 10x20 map 5.0 / 6.9, 64 -> 64
+// channels 3x3 on one 10x20 map 6.65 / 6.67, on 64 of them 22.5 / 16.3; 119 -> 37 channels 5x5 8-bit on two 18x17 maps 22.2 / 20.6.
+// (The layers of the compact CNN run in two launches for one image, too.)
 #include <type_traits>
 
 #include "hikonv_cuda.cuh"
