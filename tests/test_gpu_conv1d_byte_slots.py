@@ -117,3 +117,24 @@ def test_unaligned_pointers(bits):
             assert_exact(y, ref, "offset %d" % shift)
             torch.cuda.synchronize()
             assert int(big_y[shift - 1]) == -7 and int(big_y[shift + 20004]) == -7     # nothing written outside
+
+
+@pytest.mark.parametrize("bits, K, signed", [(3, 7, False), (4, 5, True), (4, 7, False), (8, 5, True), (8, 7, False), (4, 3, True)])
+def test_both_register_budgets_on_a_stream_and_in_a_graph(bits, K, signed):
+    # the register budgets of four and five CTAs per SM, of which the latter is the default for every number of kernel words, on a
+    # stream (dependent launches) and in a graph (ordinary ones), on signals of many tiles and of less than one
+    L = hk.conv1d_layout(bits, bits, signed, signed, K)
+    for n in (300, 700001):
+        f, g = inputs.conv1d_case(n, K, bits, bits, signed, signed, seed=900 + bits + K)
+        ref = direct.conv1d_full(f, g)
+        d_f, d_g = dev(f), dev(g)
+        for tune in (None, {"tile": -24}, {"tile": -25}):
+            assert_exact(hk.conv1d(d_f, d_g, bits, bits, signed, signed, tune=tune), ref, "stream %s J=%d" % (tune, L["J"]))
+            out = torch.empty(ref.size, dtype=torch.int32, device="cuda")
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph):
+                hk.conv1d(d_f, d_g, bits, bits, signed, signed, tune=tune, out=out)
+            out.fill_(-1)
+            graph.replay()
+            assert_exact(out, ref, "graph %s J=%d" % (tune, L["J"]))
+            del graph
