@@ -278,7 +278,8 @@ int hikonv_conv2d_layout(int B, int Ci, int H, int W, int Co, int K, int pad, in
 
 /*
  * hikonv_conv2d_launches - how many kernels a layer on tensors of one code per byte runs in (host only): *launches is 2, or 1 for the
- * small layers whose operands are packed by the layer kernel itself; *cluster (may be NULL) is then the number of CTAs that
+ * layers whose operands are packed by the layer kernel itself (small ones, and pooled ones of few input channels and wide codes, whose
+ * words hold the weights of three filters: hikonv_conv2d_layout and hikonv_conv2d_multiplies describe the two-launch form); *cluster (may be NULL) is then the number of CTAs that
  * share a tile's input channels (1, 2, 4 or 8), else 0.  requant and pool as for hikonv_conv2d_dense; other arguments and
  * errors as for hikonv_conv2d_layout.
  */

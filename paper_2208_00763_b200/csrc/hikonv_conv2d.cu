@@ -12,6 +12,7 @@
 #include <mutex>
 
 #include "hikonv_cuda.cuh"
+#include "hikonv_conv2d_filters.h"
 #include "hikonv_conv2d_output.h"
 #include "hikonv_conv2d_small.h"
 #include "hikonv_conv2d_strip.h"
@@ -237,6 +238,8 @@ struct Conv2dSetup {
     bool unpacked;
     bool one_launch;      // the kernel for small layers, which packs its operands itself
     SmallLaunch small;
+    bool filters;         // the kernel whose words hold the weights of several filters
+    FiltersLaunch filt;
     StripLaunch strip;    // the packed kernel, or
     UnpackedLaunch un;    // the comparator
     // packed operands in the workspace: weights [Ci K J][CoP], x_off corrections [K][CoP], activations [Ci][B Hp][XBT]
@@ -488,6 +491,85 @@ static SmallChoice choose_small(const StripProblem &q) {
     return best;
 }
 
+constexpr int kFiltersMaxCi = 6, kFiltersMinCo = 16;    // see plan_layer
+constexpr double kFiltersMinOutputs = 1.0e6;
+
+// The kernel whose words hold the weights of several filters: its tile and the modelled cycles of the call.
+struct FiltersChoice {
+    int NW, groups, TQ, NSEG, TS, pos_warps, CK, rows, PW, threads;
+    size_t smem;
+    long long tiles, gx, gy;
+    double cost;
+};
+
+static FiltersChoice choose_filters(const StripProblem &q) {
+    FiltersChoice best;
+    std::memset(&best, 0, sizeof(best));
+    best.cost = -1.0;
+    constexpr int K = kFiltersK, KK = K * K, NS = kFiltersSlots;
+    const int SH = ceil_div(q.Ho, 2), QT = ceil_div(q.Wo, 2), Hp = q.Ho + K - 1;
+    FiltersChoice c;
+    const long long strips = (long long)q.B * SH;
+    const int words = ceil_div(q.Co, NS);
+    static const int word_tiles[3] = {6, 4, 2};
+    for (int NW : word_tiles)
+        for (c.groups = 1; c.groups <= 8 && (c.groups == 1 || (c.groups - 1) * NW < words); c.groups *= 2) {
+            c.NW = NW;
+            const int warps_max = kFiltersThreads / 32 / c.groups, WT = NW * c.groups;
+            const size_t word_bytes = 8 * (size_t)q.Ci * KK * WT;
+            c.gy = ceil_div(words, WT);
+            int last_tq = 0;
+            for (int cut = 1; cut <= ceil_div(QT, 32); ++cut) {
+                // whole rows, or segments of whole warps of pixel pairs
+                c.NSEG = cut;
+                c.TQ = ceil_div(QT, cut);
+                if (cut > 1) {
+                    c.TQ = (c.TQ + 31) / 32 * 32;
+                    c.NSEG = ceil_div(QT, c.TQ);
+                }
+                if (c.TQ == last_tq) continue;
+                last_tq = c.TQ;
+                if (c.TQ > warps_max * 32) continue;
+                const int ts_hi = (int)std::max<long long>(1, std::min<long long>(warps_max * 32 / c.TQ, strips));
+                for (c.TS = 1; c.TS <= ts_hi; ++c.TS) {
+                    c.pos_warps = ceil_div(c.TS * c.TQ, 32);
+                    c.threads = c.pos_warps * 32 * c.groups;
+                    c.rows = staged_rows(c.TS, 2, SH, Hp, K);
+                    c.PW = (2 * c.TQ + K - 1 + 3) / 4 * 4;
+                    c.tiles = (strips + c.TS - 1) / c.TS * c.NSEG;
+                    const int by_regs = std::min(filters_resident(NW) * (kFiltersThreads / c.threads), 8);
+                    const size_t plane = 8 * (size_t)c.rows * c.PW;
+                    const double items = (double)c.rows * (c.PW / 4) / c.threads;      // rows of four codes that a thread stages per channel
+                    for (int want = 1; want <= by_regs; ++want) {
+                        if (want > 1 && c.tiles * c.gy <= (long long)(want - 1) * q.sms) break;
+                        c.gx = std::max<long long>(1, std::min<long long>(c.tiles, (long long)want * q.sms / c.gy));
+                        const long long per_cta = (c.tiles + c.gx - 1) / c.gx;
+                        c.gx = (c.tiles + per_cta - 1) / per_cta;
+                        const double resident = std::max(1.0, std::min((double)want, std::ceil((double)(c.gx * c.gy) / q.sms)));
+                        const double rounds = std::ceil((double)(c.gx * c.gy) / (resident * q.sms));
+                        const size_t room = std::min<size_t>(kSmemPerCta, kSmemPerSm / want - 1024);
+                        for (int part = 1; part <= 8; part *= 2) {
+                            const int CK = ceil_div(q.Ci, part);
+                            const size_t smem = word_bytes + 2 * CK * plane;
+                            if (smem > room) continue;
+                            // issue cycles of a warp for one tile, and what its own latencies leave it at least
+                            const double n = resident * ceil_div(c.threads / 32, 4);
+                            const double products = q.Ci * KK * 4.0 * NW * 2.1, rest = q.Ci * (40.0 + items * 45.0) + 150 + 4.0 * NW * NS * 8.0;
+                            const double alone = q.Ci * (KK * std::max(4.0 * NW * 2.1, 18.0) + 150 + std::max(0.0, items - 2.0) * 150) + 600;
+                            const double steps = (double)per_cta * ceil_div(q.Ci, CK);
+                            c.cost = 1500 + std::ceil((double)q.Ci * KK * WT / (4.0 * c.threads)) * (500 + 150 * n) + std::ceil(CK * items / 2.0) * (400 + 100 * n) +
+                                     rounds * (per_cta * std::max(n * (products + 0.6 * rest), alone) + steps * 150);
+                            c.CK = CK;
+                            c.smem = smem;
+                            if (best.cost < 0 || c.cost < best.cost * (1.0 - 1e-9)) best = c;
+                        }
+                    }
+                }
+            }
+        }
+    return best;
+}
+
 static int plan_layer(int B, int Ci, int H, int W, int Co, int K, int stride, int pad, int p, int q, int xs, int ws,
                       const OutputSpec &out, int algo, const hikonv_tuning_t *tune, Conv2dSetup *s) {
     if (B < 1 || Ci < 1 || H < 1 || W < 1 || Co < 1 || K < 1 || K > kMaxK) return HIKONV_ERR_INVALID_ARG;
@@ -505,10 +587,12 @@ static int plan_layer(int B, int Ci, int H, int W, int Co, int K, int stride, in
     if ((double)Ci * K * K * max_code >= 1073741824.0) return HIKONV_ERR_UNSUPPORTED;
 
     s->unpacked = (algo == HIKONV_ALGO_UNPACKED_IMAD);
+    const int own_xs = xs;                                       // (layers on shifted codes change xs)
     s->CoP = (Co + 3) / 4 * 4;
     s->Hp = Ho + K - 1;
     s->x_off = 0;
     s->one_launch = false;
+    s->filters = false;
     hikonv_layout_t &L = s->L;
     if (s->unpacked) {
         std::memset(&L, 0, sizeof(L));
@@ -642,6 +726,47 @@ static int plan_layer(int B, int Ci, int H, int W, int Co, int K, int stride, in
                 if (even <= 4 && sm.ks_log2 == 0) ml.smem_bytes = std::max(ml.smem_bytes, (size_t)(kSmemPerSm / (even + 1) - 1024 + 256));
             }
         }
+        // Words of several filters (tune->tile == -3: wherever the layer fits them): the slots hold the sums of the whole layer.  They are
+        // the faster ones for pooled layers of few input channels whose words of pixels hold three products at best (N = 2, two words
+        // per kernel row): the pool is then a thread's own pixels.  As graphs, two launches / this kernel: 3 -> 16 channels u8 x s4 on
+        // 160x320 maps, 1 / 2 / 4 / 16 / 64 images 7.0 / 9.7 / 12.5 / 34.5 / 123.7 against 6.9 / 8.1 / 9.7 / 29.8 / 81.9 us, sixteen
+        // 48x48 maps 5.4 / 5.8 (0.6 million sums: the line lies at a million); 3 -> 32 and 3 -> 64 on sixteen 160x320 maps 63.7 / 48.6 and
+        // 119 / 79.9; 6 -> 32 at 6 bits 95.2 / 77.9; 3 -> 8 (three of four words used) 19.7 / 21.9.  Without a pool the other form's stores
+        // are direct: 3 -> 32 on 64 112x112 maps 55.7 / 79.4, four 160x320 maps 11.1 / 11.2.
+        const bool own_layout = tune && (tune->N || tune->S || tune->M || tune->tile);
+        const bool force_filters = tune && tune->tile == -3 && !tune->N && !tune->S && !tune->M;
+        if (K == kFiltersK && out.byte_inputs && out.out_bits == 8 && (!own_layout || force_filters)) {
+            const double x_lo = own_xs ? -(double)(1 << (p - 1)) : 0.0, x_hi = own_xs ? (1 << (p - 1)) - 1 : (1 << p) - 1;
+            const double w_lo = ws ? -(double)(1 << (q - 1)) : 0.0, w_hi = ws ? (1 << (q - 1)) - 1 : (1 << q) - 1;
+            const double least = std::min(0.0, std::min(x_lo * w_hi, x_hi * w_lo));
+            const double most = std::max(0.0, std::max(x_lo * w_lo, x_hi * w_hi));
+            const bool fits = Ci * 9.0 * (most - least) < (double)(1 << kFiltersSlotBits);
+            const bool gains = out.pool && Ci <= kFiltersMaxCi && Co >= kFiltersMinCo && L.N <= 2 && L.J >= 2 && (double)B * Ho * Wo * Co >= kFiltersMinOutputs;
+            FiltersChoice fc;
+            fc.cost = -1.0;
+            if (fits && (gains || force_filters)) fc = choose_filters(pr);
+            if (fc.cost >= 0 && fc.gy <= 65535 && fc.tiles <= 0x3FFFFFFF) {
+                FiltersLaunch &fl = s->filt;
+                FiltersParams &f = fl.p;
+                std::memset(&f, 0, sizeof(f));
+                f.B = B; f.Ci = Ci; f.H = H; f.W = W; f.Co = Co; f.pad = pad; f.Ho = Ho; f.Wo = Wo; f.Hp = s->Hp;
+                f.SH = ceil_div(Ho, 2); f.strips = B * f.SH; f.tiles = (int)fc.tiles;
+                f.NSEG = fc.NSEG; f.TQ = fc.TQ; f.TS = fc.TS; f.pos_warps = fc.pos_warps; f.groups = fc.groups;
+                f.WT = fc.NW * fc.groups; f.CK = fc.CK; f.rows = fc.rows; f.PW = fc.PW; f.plane = fc.rows * fc.PW;
+                f.mg_tq = magic(fc.TQ); f.mg_sh = magic(f.SH); f.mg_hp = magic(f.Hp);
+                f.x_signed = own_xs; f.w_signed = ws;
+                f.slot_bias = (int)(-least * Ci * 9.0);
+                for (int i = 0; i < kFiltersSlots; ++i) f.bias = f.bias * (double)(1 << kFiltersSlotBits) + f.slot_bias;
+                f.requant = k.requant; f.shift = out.shift; f.lo = out.lo; f.hi = out.hi; f.pool = k.pool;
+                f.pair_stores = Wo % 2 == 0 && (uintptr_t)out.d_out % (out.requant ? 2 : 8) == 0 ? 1 : 0;
+                fl.NW = fc.NW; fl.threads = fc.threads; fl.smem_bytes = fc.smem;
+                fl.grid = dim3((unsigned)fc.gx, (unsigned)fc.gy, 1);
+                const long long even = (fc.gx * fc.gy + pr.sms - 1) / pr.sms;    // spread evenly, as above
+                if (even <= 4) fl.smem_bytes = std::max(fl.smem_bytes, (size_t)(kSmemPerSm / (even + 1) - 1024 + 256));
+                s->filters = true;
+                s->one_launch = false;
+            }
+        }
         s->XBT = k.XBT;
         s->col_first = c.halo ? K - 1 - pad - L.J * L.N : -(L.J - 1) * L.N;
         s->positions = (double)B * Ho * c.NSEG * c.XB;
@@ -749,6 +874,10 @@ static int conv2d_run(const void *d_x, int x_bits, int B, int Ci, int H, int W, 
         s.strip.p.corr = s.x_off ? d_corr : nullptr;
     }
     const int ragged = ragged_codes(d_x, (int)((long long)B * Ci * H * W));        // (fewer than 2^31 codes: plan_layer)
+    if (s.filters) {
+        s.filt.p.x = (const int8_t *)d_x; s.filt.p.ragged = ragged; s.filt.p.w = (const int8_t *)d_w; s.filt.p.out = d_out;
+        return launch_filters(s.filt, st);
+    }
     if (s.one_launch) {
         s.small.p.x = (const int8_t *)d_x; s.small.p.ragged = ragged; s.small.p.w = (const int8_t *)d_w; s.small.p.s.out = d_out;
         return launch_small(s.small, s.L.N, st);
@@ -1070,8 +1199,8 @@ extern "C" int hikonv_conv2d_launches(int B, int Ci, int H, int W, int Co, int K
     const OutputSpec out = {requant ? 1 : 0, 0, 0, 0, pool ? 1 : 0, 8, nullptr, 1};
     const int rc = setup_layer(B, Ci, H, W, Co, K, 1, pad, p, q, x_signed ? 1 : 0, w_signed ? 1 : 0, out, HIKONV_ALGO_PACKED32, tune, &s);
     if (rc != HIKONV_OK) return rc;
-    *launches = s.one_launch ? 1 : 2;
-    if (cluster) *cluster = s.one_launch ? (int)s.small.grid.z : 0;
+    *launches = s.one_launch || s.filters ? 1 : 2;
+    if (cluster) *cluster = s.filters ? 1 : s.one_launch ? (int)s.small.grid.z : 0;
     return HIKONV_OK;
 }
 
