@@ -13,7 +13,11 @@
 
 namespace hikonv {
 
-constexpr int kLongThreads = 256;
+// Threads of a CTA.  At two codes per word half of 256, with twice the CTAs per SM: the same warps, but a barrier holds up four of them and
+// the phases of more CTAs (load and pack, multiply, store) lie beside each other: 4.2 M 8-bit codes, 24 taps 8.9 -> 8.06 us a call.  At
+// three codes it changed nothing (31 taps 6.93 / 6.93), at four and more it cost 5 % (20 taps at 2 bits 5.15 -> 5.4).
+__host__ __device__ constexpr int long_threads(int N) { return N == 2 ? 128 : 256; }
+__host__ __device__ constexpr int long_resident(int N) { return N == 3 || N == 2 ? 6 : 3; }
 constexpr int kLongJ = (kMaxJ + 3) / 4 * 4;                    // chunks, rounded up to whole groups of four
 // Blocks per thread: odd, and at most 28 outputs.
 __host__ __device__ constexpr int long_run(int N) { return N == 1 ? 15 : N == 2 ? 11 : N <= 4 ? 7 : N == 5 ? 5 : 3; }
@@ -22,8 +26,8 @@ __host__ __device__ constexpr int long_run(int N) { return N == 1 ? 15 : N == 2 
 // and none at six, which N = 3 reaches without spilling (4.2 M codes, 12 / 16 / 31 taps: 6.3 / 7.0 / 7.7 -> 5.5 / 6.3 / 7.3 us for
 // a launch by itself; the other block sizes lost 2 to 20 % at five or six).
 template <int N, bool SP, bool FS>
-__global__ void __launch_bounds__(kLongThreads, N == 3 ? 6 : 3) conv1d_long_kernel(const Conv1dTcParams p) {
-    constexpr int R = long_run(N), TILE = kLongThreads * R, FRONT = kLongJ;   // blocks per tile; packed words in front of it
+__global__ void __launch_bounds__(long_threads(N), long_resident(N)) conv1d_long_kernel(const Conv1dTcParams p) {
+    constexpr int kLongThreads = long_threads(N), R = long_run(N), TILE = kLongThreads * R, FRONT = kLongJ;   // blocks per tile; packed words in front of it
     static_assert(TILE % 4 == 0 && FRONT % 4 == 0 && FRONT > kMaxJ - 1, "groups of four words");
     __shared__ __align__(16) uint32_t s_A[FRONT + TILE];
     __shared__ __align__(16) uint32_t s_B[kLongJ];
@@ -123,10 +127,10 @@ __global__ void __launch_bounds__(kLongThreads, N == 3 ? 6 : 3) conv1d_long_kern
 
 template <int N>
 static int launch_long_n(const Conv1dTcParams &p, bool sp, bool fs, cudaStream_t st) {
-    const long long per_tile = (long long)kLongThreads * long_run(N) * N;
+    const long long per_tile = (long long)long_threads(N) * long_run(N) * N;
     const long long tiles = (p.n_out + per_tile - 1) / per_tile;
     if (tiles > 0x7FFFFFFFLL) return HIKONV_ERR_UNSUPPORTED;
-    const dim3 grid((unsigned)tiles), block(kLongThreads);
+    const dim3 grid((unsigned)tiles), block(long_threads(N));
     if (!sp) return launch_dependent(conv1d_long_kernel<N, false, false>, grid, block, 0, st, p);
     if (fs) return launch_dependent(conv1d_long_kernel<N, true, true>, grid, block, 0, st, p);
     return launch_dependent(conv1d_long_kernel<N, true, false>, grid, block, 0, st, p);
