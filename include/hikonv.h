@@ -236,6 +236,7 @@ int hikonv_conv1d_host(const int8_t *h_f, size_t len, const int8_t *h_g, int K, 
  * d_workspace: hikonv_conv2d_workspace_bytes(...) bytes of device memory, 256-byte aligned; the call
  * overwrites it and needs nothing from it afterwards.  The unpacked comparator uses the same workspace for
  * int32 copies of the weights and codes.
+ * d_out may share memory with d_x or d_w (the layer then never runs in one launch), not with d_workspace.
  * stride must be 1 and 0 <= pad < K.  Limits (HIKONV_ERR_UNSUPPORTED beyond them): Ho < 60000; B Ci H W and B Ho
  * below 2^31; (images a tile of rows can touch + 1) x Co x Ho x Wo below 2^32 (output offsets inside a CTA are 32-bit).
  * Layers with unsigned activations and signed weights may run on activation codes shifted by 2^(p-1) where that

@@ -847,6 +847,19 @@ extern "C" size_t hikonv_conv2d_workspace_bytes(int B, int Ci, int H, int W, int
     return weights + align_up(acts, 256);
 }
 
+// Do the outputs of a layer on one code per byte (int32 sums or one code per byte) share memory with its inputs?  The forms in one
+// launch read the inputs while CTAs that are done write outputs; in two launches the packing launch has read all of them before.
+static bool writes_inputs(const void *d_x, const void *d_w, const void *d_out, int B, int Ci, int H, int W, int Co, int K, int pad, int requant, int pool) {
+    if (B < 1 || Ci < 1 || H < 1 || W < 1 || Co < 1 || K < 1 || pad < 0) return false;                 // (refused by plan_layer)
+    const double Ho = std::max(0.0, (double)H + 2.0 * pad - K + 1), Wo = std::max(0.0, (double)W + 2.0 * pad - K + 1);
+    const double out_bytes = requant ? (double)B * Co * Ho * Wo / (pool ? 4 : 1) : 4.0 * B * Co * Ho * Wo;
+    auto shares = [&](const void *d_in, double bytes) {
+        const double apart = (double)(intptr_t)((uintptr_t)d_in - (uintptr_t)d_out);                     // sizes are below 2^53 or refused
+        return apart < out_bytes && -apart < bytes;
+    };
+    return shares(d_x, (double)B * Ci * H * W) || shares(d_w, (double)Co * Ci * K * K);
+}
+
 // One layer: packing launch, then the layer kernel.  x_bits / w_bits: storage of activations and weights (8 = one code
 // per byte, else dense); out_bits and pool describe the requantised output (see OutputSpec).
 static int conv2d_run(const void *d_x, int x_bits, int B, int Ci, int H, int W, const void *d_w, int w_bits, int Co, int K,
@@ -855,7 +868,8 @@ static int conv2d_run(const void *d_x, int x_bits, int B, int Ci, int H, int W, 
                       const hikonv_tuning_t *tune, void *stream) {
     if (!d_x || !d_w || !d_out) return HIKONV_ERR_INVALID_ARG;
     Conv2dSetup s;
-    const OutputSpec out = {requant, shift, lo, hi, pool, out_bits, d_out, x_bits == 8 && w_bits == 8};
+    const OutputSpec out = {requant, shift, lo, hi, pool, out_bits, d_out,
+                            x_bits == 8 && w_bits == 8 && !writes_inputs(d_x, d_w, d_out, B, Ci, H, W, Co, K, pad, requant, pool)};
     int rc = setup_layer(B, Ci, H, W, Co, K, stride, pad, p, q, x_signed ? 1 : 0, w_signed ? 1 : 0, out, algo, tune, &s);
     if (rc != HIKONV_OK) return rc;
     if (!requant && ((uintptr_t)d_out % 4) != 0) return HIKONV_ERR_INVALID_ARG;

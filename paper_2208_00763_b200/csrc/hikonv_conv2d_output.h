@@ -12,7 +12,8 @@ struct OutputSpec {
     int pool;                  // 2x2 maximum after requantisation
     int out_bits;              // requantised codes: 8 (one per byte) or 1 / 2 / 4 (dense)
     const void *d_out;         // its alignment decides the width of the stores
-    int byte_inputs;           // activations and weights are stored one code per byte (not what a layer writes, but what decides how it may run)
+    int byte_inputs;           // activations and weights are stored one code per byte, in memory that the outputs do not share: the layer
+                               // kernel may read them itself (not what a layer writes, but what decides how it may run)
 };
 
 // Output staging of a layer whose row segments hold `seg_cols` output columns: nothing for plain results, which are stored
