@@ -887,9 +887,9 @@ static int conv2d_run(const void *d_x, int x_bits, int B, int Ci, int H, int W, 
         s.strip.p.wp = d_wp; s.strip.p.ap = d_ap; s.strip.p.out = d_out;
         s.strip.p.corr = s.x_off ? d_corr : nullptr;
     }
-    const int ragged = ragged_codes(d_x, (int)((long long)B * Ci * H * W));        // (fewer than 2^31 codes: plan_layer)
+    const int codes = (int)((long long)B * Ci * H * W), ragged = ragged_codes(d_x, codes);        // (fewer than 2^31 codes: plan_layer)
     if (s.filters) {
-        s.filt.p.x = (const int8_t *)d_x; s.filt.p.ragged = ragged; s.filt.p.w = (const int8_t *)d_w; s.filt.p.out = d_out;
+        s.filt.p.x = (const int8_t *)d_x; s.filt.p.codes = codes; s.filt.p.w = (const int8_t *)d_w; s.filt.p.out = d_out;
         return launch_filters(s.filt, st);
     }
     if (s.one_launch) {

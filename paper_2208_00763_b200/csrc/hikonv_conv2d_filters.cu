@@ -30,7 +30,8 @@ constexpr int kWords = 4;                // kernel words of a thread whose codes
 // 2^52 + byte b of v.
 __device__ __forceinline__ double byte_as_double(uint32_t v, int b) { return __hiloint2double(0x43300000, (int)extract_code<false>(v, b)); }
 
-template <int NW>
+// RAGGED: the input begins at any byte, or ends at any (an instantiation of its own: the branch for it cost aligned inputs 2 %).
+template <int NW, bool RAGGED>
 __global__ void __launch_bounds__(kFiltersThreads, filters_resident(NW)) conv2d_filters_kernel(const __grid_constant__ FiltersParams p) {
     constexpr int NS = kFiltersSlots, S = kFiltersSlotBits, KT = kFiltersK, KK = KT * KT, AC = KT + 1;   // AC: columns of a row that a thread's pixels read
     extern __shared__ __align__(16) double smem_d[];
@@ -77,23 +78,8 @@ __global__ void __launch_bounds__(kFiltersThreads, filters_resident(NW)) conv2d_
             if (n_row >= n_rows) continue;
             f_at[u] = n_c * p.plane + n_r * p.PW + 4 * a_col;
             const int d = fast_div(n_h0 + n_r, p.mg_hp), b = n_b0 + d, h = n_h0 + n_r - d * p.Hp - p.pad;
-            if (b < p.B && h >= 0 && h < p.H) {
-                const int8_t *src = p.x + ((b * p.Ci + n_ci0 + n_c) * hw + h * p.W + n_col0);    // (fewer than 2^31 codes)
-                if (p.ragged < 0) {
-                    // the aligned words around the four codes that hold codes of the row
-                    const uint32_t off = (uint32_t)(uintptr_t)src & 3u;
-                    const uint32_t *al = reinterpret_cast<const uint32_t *>(src - off);
-                    const int first = n_col0 - (int)off;
-                    f_off[u] = off;
-                    if (first + 3 >= 0 && first < p.W) f_lo[u] = load_ordered(al);
-                    if (off != 0u && first + 7 >= 0 && first + 4 < p.W) f_hi[u] = load_ordered(al + 1);
-                } else {
-                    // a tensor with unaligned ends: code by code
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        if (n_col0 + k >= 0 && n_col0 + k < p.W) f_lo[u] |= (uint32_t)(uint8_t)load_ordered(src + k) << (8 * k);
-                }
-            }
+            if (b < p.B && h >= 0 && h < p.H)
+                load_row_codes<RAGGED>(p.x, (b * p.Ci + n_ci0 + n_c) * hw + h * p.W, p.codes, p.W, n_col0, f_lo[u], f_hi[u], f_off[u]);   // (fewer than 2^31 codes)
             n_row += a_step;
             n_c += a_step_c;
             n_r += a_step_r;
@@ -292,9 +278,11 @@ __global__ void __launch_bounds__(kFiltersThreads, filters_resident(NW)) conv2d_
 
 template <int NW>
 static int launch_filters_as(const FiltersLaunch &l, cudaStream_t st) {
-    auto kern = conv2d_filters_kernel<NW>;
-    return with_dynamic_smem(reinterpret_cast<const void *>(kern), l.smem_bytes,
-                             [&] { return launch_dependent(kern, l.grid, dim3(l.threads), l.smem_bytes, st, l.p); });
+    auto launch = [&](auto kern) {
+        return with_dynamic_smem(reinterpret_cast<const void *>(kern), l.smem_bytes,
+                                 [&] { return launch_dependent(kern, l.grid, dim3(l.threads), l.smem_bytes, st, l.p); });
+    };
+    return (((uintptr_t)l.p.x | (unsigned)l.p.codes) & 3) != 0 ? launch(conv2d_filters_kernel<NW, true>) : launch(conv2d_filters_kernel<NW, false>);
 }
 
 int launch_filters(const FiltersLaunch &l, cudaStream_t st) {

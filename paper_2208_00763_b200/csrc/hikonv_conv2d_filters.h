@@ -15,7 +15,7 @@ constexpr int kFiltersSlotBits = 17;     // bits of a slot: three of them in the
 struct FiltersParams {
     const int8_t *x, *w;
     void *out;
-    int ragged;                          // ragged_codes() of x
+    int codes;                           // of x, all of them
     int B, Ci, H, W, Co, pad, Ho, Wo;
     int Hp;                              // padded rows per image
     int SH, strips;                      // pairs of output rows per image, in the layer
