@@ -530,6 +530,10 @@ static FiltersChoice choose_filters(const StripProblem &q) {
                 if (c.TQ == last_tq) continue;
                 last_tq = c.TQ;
                 if (c.TQ > warps_max * 32) continue;
+                // issue cycles of a warp for one tile's products, and the least that is beside them
+                const double products = q.Ci * KK * 4.0 * NW * 2.1, outside = q.Ci * 40.0 + 150 + 4.0 * NW * NS * 8.0;
+                auto hopeless = [&](double cycles) { return best.cost >= 0 && 1500 + cycles * (1.0 - 1e-9) >= best.cost; };
+                if (hopeless((double)(strips * c.NSEG * c.TQ * c.groups * c.gy) / (128.0 * q.sms) * (products + 0.6 * outside))) continue;
                 const int ts_hi = (int)std::max<long long>(1, std::min<long long>(warps_max * 32 / c.TQ, strips));
                 for (c.TS = 1; c.TS <= ts_hi; ++c.TS) {
                     c.pos_warps = ceil_div(c.TS * c.TQ, 32);
@@ -540,6 +544,15 @@ static FiltersChoice choose_filters(const StripProblem &q) {
                     const int by_regs = std::min(filters_resident(NW) * (kFiltersThreads / c.threads), 8);
                     const size_t plane = 8 * (size_t)c.rows * c.PW;
                     const double items = (double)c.rows * (c.PW / 4) / c.threads;      // rows of four codes that a thread stages per channel
+                    // all of it, and what a warp's own latencies leave a tile at least
+                    const double rest = outside + q.Ci * items * 45.0;
+                    const double alone = q.Ci * (KK * std::max(4.0 * NW * 2.1, 18.0) + 150 + std::max(0.0, items - 2.0) * 150) + 600;
+                    const int per_sched = ceil_div(c.threads / 32, 4);
+                    // what comes before the first tile, with n warps on a scheduler: packing the kernel words, fetching the first step's CK channels
+                    const double word_rounds = std::ceil((double)q.Ci * KK * WT / (4.0 * c.threads));
+                    auto before = [&](double n, int CK) { return word_rounds * (500 + 150 * n) + std::ceil(CK * items / 2.0) * (400 + 100 * n); };
+                    const double share = (double)(c.tiles * c.gy) / q.sms;
+                    if (hopeless(before(per_sched, 1) + std::max(share * per_sched * (products + 0.6 * rest), alone))) continue;
                     for (int want = 1; want <= by_regs; ++want) {
                         if (want > 1 && c.tiles * c.gy <= (long long)(want - 1) * q.sms) break;
                         c.gx = std::max<long long>(1, std::min<long long>(c.tiles, (long long)want * q.sms / c.gy));
@@ -547,18 +560,15 @@ static FiltersChoice choose_filters(const StripProblem &q) {
                         c.gx = (c.tiles + per_cta - 1) / per_cta;
                         const double resident = std::max(1.0, std::min((double)want, std::ceil((double)(c.gx * c.gy) / q.sms)));
                         const double rounds = std::ceil((double)(c.gx * c.gy) / (resident * q.sms));
+                        const double n = resident * per_sched, tiles_alone = per_cta * std::max(n * (products + 0.6 * rest), alone);
+                        if (hopeless(before(n, 1) + rounds * tiles_alone)) continue;
                         const size_t room = std::min<size_t>(kSmemPerCta, kSmemPerSm / want - 1024);
-                        for (int part = 1; part <= 8; part *= 2) {
-                            const int CK = ceil_div(q.Ci, part);
+                        for (int part = 1, CK = 0; part <= 8; part *= 2) {
+                            if (CK == ceil_div(q.Ci, part)) continue;
+                            CK = ceil_div(q.Ci, part);
                             const size_t smem = word_bytes + 2 * CK * plane;
                             if (smem > room) continue;
-                            // issue cycles of a warp for one tile, and what its own latencies leave it at least
-                            const double n = resident * ceil_div(c.threads / 32, 4);
-                            const double products = q.Ci * KK * 4.0 * NW * 2.1, rest = q.Ci * (40.0 + items * 45.0) + 150 + 4.0 * NW * NS * 8.0;
-                            const double alone = q.Ci * (KK * std::max(4.0 * NW * 2.1, 18.0) + 150 + std::max(0.0, items - 2.0) * 150) + 600;
-                            const double steps = (double)per_cta * ceil_div(q.Ci, CK);
-                            c.cost = 1500 + std::ceil((double)q.Ci * KK * WT / (4.0 * c.threads)) * (500 + 150 * n) + std::ceil(CK * items / 2.0) * (400 + 100 * n) +
-                                     rounds * (per_cta * std::max(n * (products + 0.6 * rest), alone) + steps * 150);
+                            c.cost = 1500 + before(n, CK) + rounds * (tiles_alone + (double)per_cta * ceil_div(q.Ci, CK) * 150);
                             c.CK = CK;
                             c.smem = smem;
                             if (best.cost < 0 || c.cost < best.cost * (1.0 - 1e-9)) best = c;
@@ -689,43 +699,6 @@ static int plan_layer(int B, int Ci, int H, int W, int Co, int K, int stride, in
         const long long share = (c.ctas + pr.sms - 1) / pr.sms;
         if (share <= 4) l.smem_bytes = std::max(c.smem, (size_t)(kSmemPerSm / (share + 1) - 1024 + 256));
 
-        // one launch instead of two, where it is modelled to be faster (tune->tile == -1: never, -2: always)
-        const bool force_small = tune && tune->tile == -2;
-        if (!pr.generic && s->x_off == 0 && out.byte_inputs && out.out_bits == 8 && tile_arg == 0 && !(tune && tune->tile == -1)) {
-            const SmallChoice sm = choose_small(pr);
-            // both models brought to measured times on 66 layers (3 to 200 channels, 1 to 32 images, every layout; 8 and 16 % rms):
-            // they leave out latencies of a few thousand cycles, and the packing launch takes 2.3 us and 13 us per million 16-byte
-            // pieces.  Over those layers the calls took 700 us together, 719 us always in two launches, 696 us with the faster of
-            // the two each time.  One launch is the faster one for little work (2x195x33x28 -> 9, 8 bits: 12.5 against 14.1 us;
-            // 5x5x7x46 -> 183: 4.4 against 5.9), two from about 15 us on (9x23x16x18 -> 151, 5x5: 24.0 against 13.9)
-            const double two = 4300 + 1.1 * c.cost + 0.025 * Ci * B * s->Hp * (k.XBT / 4);
-            const double one = 2.4 * sm.cost - 11200 - 0.8 * std::max(0.0, sm.cost - 9800);
-            if (sm.cost >= 0 && (one < two || force_small)) {
-                s->one_launch = true;
-                SmallLaunch &ml = s->small;
-                SmallParams &mp = ml.p;
-                std::memset(&mp, 0, sizeof(mp));
-                mp.s = k;
-                StripParams &ms = mp.s;
-                ms.SH = ceil_div(Ho, kSmallTM); ms.strips = B * ms.SH;
-                ms.NSEG = 1; ms.XO = ms.XB = ms.X = sm.XB; ms.halo = 0; ms.col_off = K - 1 - pad; ms.pitch = sm.pitch;
-                ms.TS = sm.TS; ms.TNX = sm.TNX; ms.TCO = sm.TNX * kSmallTN;
-                ms.plane = sm.rows * sm.pitch; ms.b_off = sm.Cz * ms.plane;
-                ms.mg_xb = magic(sm.XB); ms.mg_sh = magic(ms.SH);
-                ms.WTP = (sm.XB * L.N + 15) / 16 * 16;
-                mp.B = B; mp.H = H; mp.x_signed = xs; mp.w_signed = ws; mp.Kc = L.Kc;
-                mp.Cz = sm.Cz; mp.CF = pr.moves ? pr.CF : Ci + 1; mp.ks_log2 = sm.ks_log2; mp.rows = sm.rows;
-                mp.col_first = -(L.J - 1) * L.N;
-                mp.mg_hp = magic(s->Hp); mp.mg_xq = magic(sm.pitch / 4); mp.mg_rows = magic(sm.rows);
-                mp.red_off = sm.threads / 32 * sm.TNX * kSmallTM * kSmallTN * 2;
-                ms.tile_off = mp.red_off + (sm.ks_log2 > 0 ? sm.threads * kSmallTM * kSmallTN * L.N : 0);
-                ml.threads = sm.threads; ml.sp = L.signed_prod != 0;
-                ml.smem_bytes = sm.words * 4;
-                ml.grid = dim3((unsigned)((ms.strips + sm.TS - 1) / sm.TS), (unsigned)ceil_div(Co, ms.TCO), 1u << sm.ks_log2);
-                const long long even = (sm.ctas + pr.sms - 1) / pr.sms;          // spread evenly, as above
-                if (even <= 4 && sm.ks_log2 == 0) ml.smem_bytes = std::max(ml.smem_bytes, (size_t)(kSmemPerSm / (even + 1) - 1024 + 256));
-            }
-        }
         // Words of several filters (tune->tile == -3: wherever the layer fits them): the slots hold the sums of the whole layer.  They are
         // the faster ones for pooled layers of few input channels whose words of pixels hold three products at best (N = 2, two words
         // per kernel row): the pool is then a thread's own pixels.  As graphs, two launches / this kernel: 3 -> 16 channels u8 x s4 on
@@ -764,7 +737,43 @@ static int plan_layer(int B, int Ci, int H, int W, int Co, int K, int stride, in
                 const long long even = (fc.gx * fc.gy + pr.sms - 1) / pr.sms;    // spread evenly, as above
                 if (even <= 4) fl.smem_bytes = std::max(fl.smem_bytes, (size_t)(kSmemPerSm / (even + 1) - 1024 + 256));
                 s->filters = true;
-                s->one_launch = false;
+            }
+        }
+        // one launch instead of two, where it is modelled to be faster (tune->tile == -1: never, -2: always)
+        const bool force_small = tune && tune->tile == -2;
+        if (!s->filters && !pr.generic && s->x_off == 0 && out.byte_inputs && out.out_bits == 8 && tile_arg == 0 && !(tune && tune->tile == -1)) {
+            const SmallChoice sm = choose_small(pr);
+            // both models brought to measured times on 66 layers (3 to 200 channels, 1 to 32 images, every layout; 8 and 16 % rms):
+            // they leave out latencies of a few thousand cycles, and the packing launch takes 2.3 us and 13 us per million 16-byte
+            // pieces.  Over those layers the calls took 700 us together, 719 us always in two launches, 696 us with the faster of
+            // the two each time.  One launch is the faster one for little work (2x195x33x28 -> 9, 8 bits: 12.5 against 14.1 us;
+            // 5x5x7x46 -> 183: 4.4 against 5.9), two from about 15 us on (9x23x16x18 -> 151, 5x5: 24.0 against 13.9)
+            const double two = 4300 + 1.1 * c.cost + 0.025 * Ci * B * s->Hp * (k.XBT / 4);
+            const double one = 2.4 * sm.cost - 11200 - 0.8 * std::max(0.0, sm.cost - 9800);
+            if (sm.cost >= 0 && (one < two || force_small)) {
+                s->one_launch = true;
+                SmallLaunch &ml = s->small;
+                SmallParams &mp = ml.p;
+                std::memset(&mp, 0, sizeof(mp));
+                mp.s = k;
+                StripParams &ms = mp.s;
+                ms.SH = ceil_div(Ho, kSmallTM); ms.strips = B * ms.SH;
+                ms.NSEG = 1; ms.XO = ms.XB = ms.X = sm.XB; ms.halo = 0; ms.col_off = K - 1 - pad; ms.pitch = sm.pitch;
+                ms.TS = sm.TS; ms.TNX = sm.TNX; ms.TCO = sm.TNX * kSmallTN;
+                ms.plane = sm.rows * sm.pitch; ms.b_off = sm.Cz * ms.plane;
+                ms.mg_xb = magic(sm.XB); ms.mg_sh = magic(ms.SH);
+                ms.WTP = (sm.XB * L.N + 15) / 16 * 16;
+                mp.B = B; mp.H = H; mp.x_signed = xs; mp.w_signed = ws; mp.Kc = L.Kc;
+                mp.Cz = sm.Cz; mp.CF = pr.moves ? pr.CF : Ci + 1; mp.ks_log2 = sm.ks_log2; mp.rows = sm.rows;
+                mp.col_first = -(L.J - 1) * L.N;
+                mp.mg_hp = magic(s->Hp); mp.mg_xq = magic(sm.pitch / 4); mp.mg_rows = magic(sm.rows);
+                mp.red_off = sm.threads / 32 * sm.TNX * kSmallTM * kSmallTN * 2;
+                ms.tile_off = mp.red_off + (sm.ks_log2 > 0 ? sm.threads * kSmallTM * kSmallTN * L.N : 0);
+                ml.threads = sm.threads; ml.sp = L.signed_prod != 0;
+                ml.smem_bytes = sm.words * 4;
+                ml.grid = dim3((unsigned)((ms.strips + sm.TS - 1) / sm.TS), (unsigned)ceil_div(Co, ms.TCO), 1u << sm.ks_log2);
+                const long long even = (sm.ctas + pr.sms - 1) / pr.sms;          // spread evenly, as above
+                if (even <= 4 && sm.ks_log2 == 0) ml.smem_bytes = std::max(ml.smem_bytes, (size_t)(kSmemPerSm / (even + 1) - 1024 + 256));
             }
         }
         s->XBT = k.XBT;
@@ -779,7 +788,7 @@ static int plan_layer(int B, int Ci, int H, int W, int Co, int K, int stride, in
 }
 
 // plan_layer is a function of its arguments, the SM count and the alignment of the output address, and takes longer than the
-// two launches of a layer (tile choice: 20 to 100 us): every thread keeps the last few plans.  No pointer is kept with them.
+// two launches of a layer (tile choice: 60 us on average, up to 140): every thread keeps the last few plans.  No pointer is kept with them.
 static int setup_layer(int B, int Ci, int H, int W, int Co, int K, int stride, int pad, int p, int q, int xs, int ws,
                        const OutputSpec &out, int algo, const hikonv_tuning_t *tune, Conv2dSetup *s) {
     struct Kept {
