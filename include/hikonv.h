@@ -96,7 +96,12 @@ typedef struct {
                        16) + 100000 x output rows per thread (2 or 4) + 1000000 x channels per
                        thread (4 or 8) + 10000000 x thread groups per tile (1, 2 or 4: they share the input
                        channels), each part 0 = automatic; -1 packs the operands in a launch of
-                       its own, -2 in the layer's launch where that is built (small layers); conv1d: > 0 the general kernel, -1 the
+                       its own, -2 in the layer's launch where that is built (small layers), -3 multiplies
+                       words of the weights of three filters where the layer fits them (one code per
+                       byte, 3x3, sums within 17 bits, no forced N, S, M), and -(3 + 10 x words per
+                       thread (2, 4, 6) + 100 x groups of words (1, 2, 4, 8) + 1000 x input channels per step +
+                       100000 x most CTAs that share the tiles) forces parts of that tile; where -2, -3 or the
+                       parts do not fit, the choice is automatic; conv1d: > 0 the general kernel, -1 the
                        planner's layout instead of register-aligned slots; -24 / -25 force the
                        register budget of four / five resident CTAs per SM in the register-aligned
                        kernels and the two comparators (default: whichever measured faster for the
@@ -231,11 +236,12 @@ int hikonv_conv1d_host(const int8_t *h_f, size_t len, const int8_t *h_g, int K, 
  *   requant != 0: d_out is int8, clamp(sum >> shift, lo, hi) with an arithmetic (floor) shift,
  *                 0 <= shift <= 31, -128 <= lo <= hi <= 255 (values above 127 are stored as the
  *                 byte of the unsigned code).
- * Two kernels run on `stream`: the reversed kernel rows (g = W[co][ci][kh][K-1:0], Theorem 3) and the
- * activation rows are packed (Eq. 5) into d_workspace, then the layer kernel streams the packed words.
- * d_workspace: hikonv_conv2d_workspace_bytes(...) bytes of device memory, 256-byte aligned; the call
- * overwrites it and needs nothing from it afterwards.  The unpacked comparator uses the same workspace for
- * int32 copies of the weights and codes.
+ * Runs on `stream` in one of four forms (hikonv_conv2d_form).  Two launches: the reversed kernel rows (g = W[co][ci][kh][K-1:0], Theorem 3)
+ * and the activation rows are packed (Eq. 5) into d_workspace, then the layer kernel streams the packed words; the unpacked comparator
+ * keeps int32 copies of weights and codes there instead.  One launch: small layers whose kernel packs the same words itself, and pooled
+ * layers of few input channels and wide codes, whose kernel multiplies by words of the weights of three filters.
+ * d_workspace: hikonv_conv2d_workspace_bytes(...) bytes of device memory, 256-byte aligned, in every form; the call may
+ * overwrite it and needs nothing from it afterwards.
  * d_out may share memory with d_x or d_w (the layer then never runs in one launch), not with d_workspace.
  * stride must be 1 and 0 <= pad < K.  Limits (HIKONV_ERR_UNSUPPORTED beyond them): Ho < 60000; B Ci H W and B Ho
  * below 2^31; (images a tile of rows can touch + 1) x Co x Ho x Wo below 2^32 (output offsets inside a CTA are 32-bit).
@@ -280,12 +286,37 @@ int hikonv_conv2d_layout(int B, int Ci, int H, int W, int Co, int K, int pad, in
 /*
  * hikonv_conv2d_launches - how many kernels a layer on tensors of one code per byte runs in (host only): *launches is 2, or 1 for the
  * layers whose operands are packed by the layer kernel itself (small ones, and pooled ones of few input channels and wide codes, whose
- * words hold the weights of three filters: hikonv_conv2d_layout and hikonv_conv2d_multiplies describe the two-launch form); *cluster (may be NULL) is then the number of CTAs that
- * share a tile's input channels (1, 2, 4 or 8), else 0.  requant and pool as for hikonv_conv2d_dense; other arguments and
- * errors as for hikonv_conv2d_layout.
+ * words hold the weights of three filters); *cluster (may be NULL) is then the number of CTAs that share a tile's input channels (1, 2, 4
+ * or 8), else 0.  hikonv_conv2d_form tells the forms apart.  requant and pool as for hikonv_conv2d_dense; other arguments and errors
+ * as for hikonv_conv2d_layout.
  */
 int hikonv_conv2d_launches(int B, int Ci, int H, int W, int Co, int K, int pad, int p, int q, int x_signed, int w_signed,
                            int requant, int pool, const hikonv_tuning_t *tune, int *launches, int *cluster);
+
+/*
+ * hikonv_conv2d_form - the form a layer on tensors of one code per byte runs in, its tile and the multiplies it executes (host only).
+ * Arguments as for hikonv_conv2d_launches, algo as for hikonv_conv2d.  Layers whose outputs share memory with their inputs never run in
+ * one launch, whatever is said here.  hikonv_conv2d_layout and hikonv_conv2d_multiplies describe the layer in two launches.
+ */
+typedef enum {
+    HIKONV_FORM_TWO_LAUNCHES = 0, /* operands are packed into the workspace, words of pixels and taps           */
+    HIKONV_FORM_ONE_LAUNCH = 1,   /* the same words, packed by the layer kernel (small layers)                  */
+    HIKONV_FORM_FILTERS = 2,      /* one launch, words of the weights of three filters, double-precision unit   */
+    HIKONV_FORM_UNPACKED = 3      /* the unpacked comparator, two launches                                      */
+} hikonv_conv2d_form_kind;
+
+typedef struct {
+    int form;                 /* hikonv_conv2d_form_kind                                                        */
+    int launches;
+    int cluster;              /* HIKONV_FORM_ONE_LAUNCH: CTAs that share a tile's input channels                */
+    int words, groups, step_channels; /* HIKONV_FORM_FILTERS: words per thread, groups of words and input channels per step, ... */
+    int ctas, tiles, segments;        /* ... CTAs that share the tiles, tiles, segments of a row                  */
+    double multiplies;        /* 32-bit multiplies (32x32->64; the comparator: 32x32->32); halo positions included, idle threads not */
+    double double_multiplies; /* double-precision multiply-adds of HIKONV_FORM_FILTERS                          */
+} hikonv_conv2d_form_t;
+
+int hikonv_conv2d_form(int B, int Ci, int H, int W, int Co, int K, int pad, int p, int q, int x_signed, int w_signed,
+                       int requant, int pool, int algo, const hikonv_tuning_t *tune, hikonv_conv2d_form_t *form);
 
 /*
  * hikonv_conv2d_dense - hikonv_conv2d on tensors stored without their unused bits (Section V-B, single convolver

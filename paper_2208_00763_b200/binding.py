@@ -21,6 +21,7 @@ LIB_PATH = os.path.join(_HERE, "libhikonv.so")
 OK, ERR_INVALID_ARG, ERR_UNSUPPORTED, ERR_NO_FIT, ERR_WORKSPACE, ERR_CUDA, ERR_TOO_LARGE, ERR_RANGE = range(8)
 STATIC_SCRATCH_BYTES = 4 << 20
 ALGO_PACKED32, ALGO_PACKED64EMU, ALGO_UNPACKED_IMAD, ALGO_DP4A = 0, 1, 2, 3
+FORM_TWO_LAUNCHES, FORM_ONE_LAUNCH, FORM_FILTERS, FORM_UNPACKED = 0, 1, 2, 3
 GB_SINGLE, GB_1D, GB_DNN = 0, 1, 2
 PIPE_KINDS = {"mad_wide_u32": 0, "mad_wide_s32": 1, "mad_lo_s32": 2, "logic": 3, "shift": 4, "prmt": 5,
               "mad_wide_with_logic": 6}
@@ -42,6 +43,11 @@ class LayoutT(ctypes.Structure):
 
 class TuningT(ctypes.Structure):
     _fields_ = [(n, ctypes.c_int) for n in ("N", "S", "M", "tile")]
+
+
+class Conv2dFormT(ctypes.Structure):
+    _fields_ = ([(n, ctypes.c_int) for n in ("form", "launches", "cluster", "words", "groups", "step_channels", "ctas", "tiles", "segments")]
+                + [(n, ctypes.c_double) for n in ("multiplies", "double_multiplies")])
 
 
 _lib = None
@@ -68,6 +74,7 @@ _SIGNATURES = {
                                 _i, _i, ctypes.POINTER(_i), ctypes.POINTER(_d), ctypes.POINTER(_d), _vp]),
     "hikonv_conv2d_workspace_bytes": (_sz, [_i] * 7),
     "hikonv_conv2d_launches": (_i, [_i] * 13 + [ctypes.POINTER(TuningT), ctypes.POINTER(_i), ctypes.POINTER(_i)]),
+    "hikonv_conv2d_form": (_i, [_i] * 14 + [ctypes.POINTER(TuningT), ctypes.POINTER(Conv2dFormT)]),
     "hikonv_conv2d_wait_timeouts": (_i, [_vp]),
     "hikonv_conv2d_wait_check": (_i, [ctypes.c_longlong, _vp]),
     "hikonv_conv2d_static_scratch": (_i, [_vp, _i, _i, _i, _i, _vp, _i, _i, _i, _i, _i, _i, _i, _i, _vp, _i, _i, _i, _i, _i,
@@ -219,6 +226,14 @@ def conv2d_launches(B, Ci, H, W, Co, K, pad, p, q, x_signed, w_signed, requant=F
     _check(lib().hikonv_conv2d_launches(B, Ci, H, W, Co, K, pad, p, q, int(x_signed), int(w_signed), int(bool(requant)), int(pool),
                                         _tune(tune), ctypes.byref(launches), ctypes.byref(cluster)), "hikonv_conv2d_launches")
     return launches.value, cluster.value
+
+
+def conv2d_form(B, Ci, H, W, Co, K, pad, p, q, x_signed, w_signed, requant=False, pool=False, algo=ALGO_PACKED32, tune=None) -> dict:
+    """The form a layer on one code per byte runs in (``FORM_*``), its launches, its tile and the multiplies it executes."""
+    out = Conv2dFormT()
+    _check(lib().hikonv_conv2d_form(B, Ci, H, W, Co, K, pad, p, q, int(x_signed), int(w_signed), int(bool(requant)), int(pool), algo,
+                                    _tune(tune), ctypes.byref(out)), "hikonv_conv2d_form")
+    return {n: getattr(out, n) for n, _ in Conv2dFormT._fields_}
 
 
 # ------------------------------------------------------------------ device entry points

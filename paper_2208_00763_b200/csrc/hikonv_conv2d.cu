@@ -245,7 +245,8 @@ struct Conv2dSetup {
     // packed operands in the workspace: weights [Ci K J][CoP], x_off corrections [K][CoP], activations [Ci][B Hp][XBT]
     int CoP, Hp, XBT, col_first, x_off;
     size_t corr_off, wp_bytes, ap_words;
-    double positions;     // words multiplied per (ci, kh, j) and output channel
+    double positions;     // words multiplied per (ci, kh, j) and output channel, in two launches
+    int small_blocks;     // words per row in the one-launch kernel
 };
 
 static int sm_count() {
@@ -502,7 +503,12 @@ struct FiltersChoice {
     double cost;
 };
 
-static FiltersChoice choose_filters(const StripProblem &q) {
+// What tune->tile forces of it: words per thread, groups of words, input channels per step, most CTAs that share the tiles (0: free).
+struct FiltersForced {
+    int NW, groups, CK, ctas;
+};
+
+static FiltersChoice choose_filters(const StripProblem &q, const FiltersForced &force) {
     FiltersChoice best;
     std::memset(&best, 0, sizeof(best));
     best.cost = -1.0;
@@ -514,6 +520,7 @@ static FiltersChoice choose_filters(const StripProblem &q) {
     static const int word_tiles[3] = {6, 4, 2};
     for (int NW : word_tiles)
         for (c.groups = 1; c.groups <= 8 && (c.groups == 1 || (c.groups - 1) * NW < words); c.groups *= 2) {
+            if ((force.NW > 0 && NW != force.NW) || (force.groups > 0 && c.groups != force.groups)) continue;
             c.NW = NW;
             const int warps_max = kFiltersThreads / 32 / c.groups, WT = NW * c.groups;
             const size_t word_bytes = 8 * (size_t)q.Ci * KK * WT;
@@ -556,6 +563,7 @@ static FiltersChoice choose_filters(const StripProblem &q) {
                     for (int want = 1; want <= by_regs; ++want) {
                         if (want > 1 && c.tiles * c.gy <= (long long)(want - 1) * q.sms) break;
                         c.gx = std::max<long long>(1, std::min<long long>(c.tiles, (long long)want * q.sms / c.gy));
+                        if (force.ctas > 0) c.gx = std::min<long long>(c.gx, force.ctas);
                         const long long per_cta = (c.tiles + c.gx - 1) / c.gx;
                         c.gx = (c.tiles + per_cta - 1) / per_cta;
                         const double resident = std::max(1.0, std::min((double)want, std::ceil((double)(c.gx * c.gy) / q.sms)));
@@ -564,8 +572,9 @@ static FiltersChoice choose_filters(const StripProblem &q) {
                         if (hopeless(before(n, 1) + rounds * tiles_alone)) continue;
                         const size_t room = std::min<size_t>(kSmemPerCta, kSmemPerSm / want - 1024);
                         for (int part = 1, CK = 0; part <= 8; part *= 2) {
-                            if (CK == ceil_div(q.Ci, part)) continue;
-                            CK = ceil_div(q.Ci, part);
+                            const int divided = force.CK > 0 ? std::min(force.CK, q.Ci) : ceil_div(q.Ci, part);
+                            if (CK == divided) continue;
+                            CK = divided;
                             const size_t smem = word_bytes + 2 * CK * plane;
                             if (smem > room) continue;
                             c.cost = 1500 + before(n, CK) + rounds * (tiles_alone + (double)per_cta * ceil_div(q.Ci, CK) * 150);
@@ -699,7 +708,7 @@ static int plan_layer(int B, int Ci, int H, int W, int Co, int K, int stride, in
         const long long share = (c.ctas + pr.sms - 1) / pr.sms;
         if (share <= 4) l.smem_bytes = std::max(c.smem, (size_t)(kSmemPerSm / (share + 1) - 1024 + 256));
 
-        // Words of several filters (tune->tile == -3: wherever the layer fits them): the slots hold the sums of the whole layer.  They are
+        // Words of several filters (tune->tile == -3: wherever the layer fits them, and more digits in front force parts of its tile): the slots hold the sums of the whole layer.  They are
         // the faster ones for pooled layers of few input channels whose words of pixels hold three products at best (N = 2, two words
         // per kernel row): the pool is then a thread's own pixels.  As graphs, two launches / this kernel: 3 -> 16 channels u8 x s4 on
         // 160x320 maps, 1 / 2 / 4 / 16 / 64 images 7.0 / 9.7 / 12.5 / 34.5 / 123.7 against 6.9 / 8.1 / 9.7 / 29.8 / 81.9 us, sixteen
@@ -707,7 +716,7 @@ static int plan_layer(int B, int Ci, int H, int W, int Co, int K, int stride, in
         // 119 / 79.9; 6 -> 32 at 6 bits 95.2 / 77.9; 3 -> 8 (three of four words used) 19.7 / 21.9.  Without a pool the other form's stores
         // are direct: 3 -> 32 on 64 112x112 maps 55.7 / 79.4, four 160x320 maps 11.1 / 11.2.
         const bool own_layout = tune && (tune->N || tune->S || tune->M || tune->tile);
-        const bool force_filters = tune && tune->tile == -3 && !tune->N && !tune->S && !tune->M;
+        const bool force_filters = tune && tune->tile <= -3 && tune->tile % 10 == -3 && !tune->N && !tune->S && !tune->M;
         if (K == kFiltersK && out.byte_inputs && out.out_bits == 8 && (!own_layout || force_filters)) {
             const double x_lo = own_xs ? -(double)(1 << (p - 1)) : 0.0, x_hi = own_xs ? (1 << (p - 1)) - 1 : (1 << p) - 1;
             const double w_lo = ws ? -(double)(1 << (q - 1)) : 0.0, w_hi = ws ? (1 << (q - 1)) - 1 : (1 << q) - 1;
@@ -717,7 +726,8 @@ static int plan_layer(int B, int Ci, int H, int W, int Co, int K, int stride, in
             const bool gains = out.pool && Ci <= kFiltersMaxCi && Co >= kFiltersMinCo && L.N <= 2 && L.J >= 2 && (double)B * Ho * Wo * Co >= kFiltersMinOutputs;
             FiltersChoice fc;
             fc.cost = -1.0;
-            if (fits && (gains || force_filters)) fc = choose_filters(pr);
+            const int digits = force_filters ? -tune->tile : 0;
+            if (fits && (gains || force_filters)) fc = choose_filters(pr, {digits / 10 % 10, digits / 100 % 10, digits / 1000 % 100, digits / 100000});
             if (fc.cost >= 0 && fc.gy <= 65535 && fc.tiles <= 0x3FFFFFFF) {
                 FiltersLaunch &fl = s->filt;
                 FiltersParams &f = fl.p;
@@ -752,6 +762,7 @@ static int plan_layer(int B, int Ci, int H, int W, int Co, int K, int stride, in
             const double one = 2.4 * sm.cost - 11200 - 0.8 * std::max(0.0, sm.cost - 9800);
             if (sm.cost >= 0 && (one < two || force_small)) {
                 s->one_launch = true;
+                s->small_blocks = sm.XB;
                 SmallLaunch &ml = s->small;
                 SmallParams &mp = ml.p;
                 std::memset(&mp, 0, sizeof(mp));
@@ -1224,6 +1235,31 @@ extern "C" int hikonv_conv2d_launches(int B, int Ci, int H, int W, int Co, int K
     if (rc != HIKONV_OK) return rc;
     *launches = s.one_launch || s.filters ? 1 : 2;
     if (cluster) *cluster = s.filters ? 1 : s.one_launch ? (int)s.small.grid.z : 0;
+    return HIKONV_OK;
+}
+
+extern "C" int hikonv_conv2d_form(int B, int Ci, int H, int W, int Co, int K, int pad, int p, int q, int x_signed, int w_signed, int requant,
+                                  int pool, int algo, const hikonv_tuning_t *tune, hikonv_conv2d_form_t *form) {
+    if (!form) return HIKONV_ERR_INVALID_ARG;
+    Conv2dSetup s;
+    const OutputSpec out = {requant ? 1 : 0, 0, 0, 0, pool ? 1 : 0, 8, nullptr, 1};
+    const int rc = setup_layer(B, Ci, H, W, Co, K, 1, pad, p, q, x_signed ? 1 : 0, w_signed ? 1 : 0, out, algo, tune, &s);
+    if (rc != HIKONV_OK) return rc;
+    std::memset(form, 0, sizeof(*form));
+    const double rows = (double)B * (H + 2 * pad - K + 1), row = W + 2 * pad - K + 1, pairs = (double)Ci * K;    // (input channel, kernel row) pairs
+    if (!s.unpacked && s.filters) {
+        const FiltersParams &f = s.filt.p;
+        form->form = HIKONV_FORM_FILTERS;
+        form->launches = 1;
+        form->words = s.filt.NW; form->groups = f.groups; form->step_channels = f.CK;
+        form->ctas = (int)s.filt.grid.x; form->tiles = f.tiles; form->segments = f.NSEG;
+        form->double_multiplies = rows * row * ceil_div(Co, kFiltersSlots) * pairs * K;
+        return HIKONV_OK;
+    }
+    form->form = s.unpacked ? HIKONV_FORM_UNPACKED : s.one_launch ? HIKONV_FORM_ONE_LAUNCH : HIKONV_FORM_TWO_LAUNCHES;
+    form->launches = form->form == HIKONV_FORM_ONE_LAUNCH ? 1 : 2;
+    form->cluster = form->form == HIKONV_FORM_ONE_LAUNCH ? (int)s.small.grid.z : 0;
+    form->multiplies = (form->form == HIKONV_FORM_ONE_LAUNCH ? rows * s.small_blocks : s.positions) * Co * pairs * s.L.J;
     return HIKONV_OK;
 }
 

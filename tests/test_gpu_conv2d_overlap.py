@@ -24,6 +24,8 @@ def test_outputs_over_inputs(layer, p, q, xs, pool, tile):
         codes = direct.maxpool2x2(codes)
     n_x, n_w, n_out = x.size, w.size, codes.size
     tune = {"tile": tile} if tile else None
+    form = hk.conv2d_form(B, Ci, H, W, Co, 3, 1, p, q, xs, True, requant=True, pool=pool, tune=tune)["form"]     # where nothing overlaps
+    assert form == {(3, 0): hk.FORM_FILTERS, (3, -3): hk.FORM_FILTERS, (24, -2): hk.FORM_ONE_LAUNCH}.get((Ci, tile), form)
     # where the output begins relative to the activations (half-way through, at their last piece, in front of them), or over the weights
     for at_x, at_w, at_out in ((0, None, 0), (0, None, n_x // 512 * 256), (0, None, (n_x - 1) // 256 * 256), (n_out // 512 * 256, None, 0), (None, 0, 0)):
         buf = torch.zeros(max(n_x, n_w) + 2 * n_out, dtype=torch.int8, device="cuda")
