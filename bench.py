@@ -37,6 +37,7 @@ HBM_FALLBACK_GBS = 6650.0            # earlier pool measurement, used only when 
 # the packed kernels on 32.
 IMAD32_PER_CLK_PER_SM = 64
 IMAD_WIDE_PER_CLK_PER_SM = 32
+FMA64_PER_CLK_PER_SM = 64            # double-precision multiply-adds (the kernel on words of three filters)
 TABLE_REPEATS = 7                    # timed repeats per cell of the per-case table (median and max - min are reported)
 
 # dram__bytes_read.sum + dram__bytes_write.sum per launch from the last ncu capture of the kernel: six
@@ -284,6 +285,7 @@ def run_ours(args):
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
     # multiply-adds per second by kind of multiply
     imad_peak = {"packed": sms * IMAD_WIDE_PER_CLK_PER_SM * sm_max_mhz * 1e6,
+                 "double": sms * FMA64_PER_CLK_PER_SM * sm_max_mhz * 1e6,
                  "unpacked": sms * IMAD32_PER_CLK_PER_SM * sm_max_mhz * 1e6}
 
     def barrier():
@@ -293,11 +295,11 @@ def run_ours(args):
     def max_over_ranks(ms: float) -> float:
         return ranks.max_over_ranks(ms, dev)
 
-    # measured integer-pipe rates (register-only kernels of the library), the denominators of the "alu" rooflines
+    # measured pipe rates (register-only kernels of the library), the denominators of the "alu" rooflines
     peaks = None
     if rank == 0:
         peaks = {}
-        for kind in ("mad_wide_u32", "mad_wide_s32", "mad_lo_s32", "logic", "shift", "prmt", "mad_wide_with_logic"):
+        for kind in ("mad_wide_u32", "mad_wide_s32", "mad_lo_s32", "logic", "shift", "prmt", "mad_wide_with_logic", "fma_f64"):
             r = hk.pipe_rate(kind, iters=2048, device=dev)
             peaks[kind] = {"T_per_s": r["ops_per_second"] / 1e12, "lanes_per_clk_per_sm_at_max_clock": r["lanes_per_clock_per_sm"]}
         peaks["derived"] = {"mad_wide_T_per_s": imad_peak["packed"] / 1e12, "mad_lo_T_per_s": imad_peak["unpacked"] / 1e12,
@@ -310,6 +312,7 @@ def run_ours(args):
                                 "cycles_added_per_other_instruction": 2.0 * (128.0 / mixed - 128.0 / pure)}
         imad_peak["issue"] = dict(peaks["issue_model"], schedulers=4 * sms, clock_hz=sm_max_mhz * 1e6)
         imad_peak["packed_measured"] = max(peaks["mad_wide_u32"]["T_per_s"], peaks["mad_wide_s32"]["T_per_s"]) * 1e12
+        imad_peak["double_measured"] = peaks["fma_f64"]["T_per_s"] * 1e12
         imad_peak["unpacked_measured"] = peaks["mad_lo_s32"]["T_per_s"] * 1e12
 
     # ---- the sweep: every rank runs the whole sweep on its own data (weak scaling, no exchange)
@@ -494,6 +497,38 @@ def run_ours(args):
     return 0
 
 
+def layer_forms(hk, shape, algo):
+    """The form of one layer workload (``hk.conv2d_form``)."""
+    return [hk.conv2d_form(shape["B"], shape["Ci"], shape["H"], shape["W"], shape["Co"], shape["K"], shape["pad"], shape["p"], shape["q"],
+                           shape["x_signed"], shape["w_signed"], requant=bool(shape["requant"]), algo=algo)]
+
+
+def network_forms(hk, layers, head_w, batch, H, W, algo, tiles):
+    """The forms of the network's nine layers, as ``CompactCnn.forward`` calls them (pools inside their layers), and its multiply-adds."""
+    forms, macs = [], 0.0
+    for L, tile in zip(layers, tiles):
+        Co, Ci, K, _ = L["w"].shape
+        macs += float(batch) * Co * H * W * Ci * K * K
+        forms.append(hk.conv2d_form(batch, Ci, H, W, Co, K, L["pad"], L["p"], L["q"], L["x_signed"], L["w_signed"], requant=True,
+                                    pool=bool(L["pool"]), algo=algo, tune=tile))
+        if L["pool"]:
+            H, W = H // 2, W // 2
+    Co, Ci = head_w.shape[:2]
+    macs += float(batch) * Co * H * W * Ci
+    forms.append(hk.conv2d_form(batch, Ci, H, W, Co, 1, 0, 4, 4, False, True, algo=algo))
+    return forms, macs, (H, W)
+
+
+def kernels_of(hk, forms):
+    """Names of the layer kernels of these forms, with how many layers run each."""
+    names = {hk.FORM_TWO_LAUNCHES: "conv2d_strip_kernel", hk.FORM_ONE_LAUNCH: "conv2d_small_kernel",
+             hk.FORM_FILTERS: "conv2d_filters_kernel", hk.FORM_UNPACKED: "conv2d_unpacked_kernel"}
+    found = [names[f["form"]] for f in forms]
+    if len(found) == 1:
+        return found[0]
+    return ", ".join("%d x %s" % (found.count(n), n) for n in sorted(set(found), key=found.index)) + " (multiplies summed)"
+
+
 def run_layer_main(args, torch, np, ranks, hk, inputs, network, dev, world, rank, local_rank, barrier, max_over_ranks, imad_peak):
     """Main line for --workload c3/c4/c5: a step is one layer (or one network pass) on this rank's batch,
     timed with one event pair per step and an L2 flush (256 MB memset) before each step."""
@@ -517,13 +552,11 @@ def run_layer_main(args, torch, np, ranks, hk, inputs, network, dev, world, rank
         Wo = shape["W"] + 2 * shape["pad"] - shape["K"] + 1
         o = torch.empty((shape["B"], shape["Co"], Ho, Wo), dtype=torch.int8 if rq else torch.int32, device=dev)
         macs = float(shape["B"]) * shape["Co"] * Ho * Wo * shape["Ci"] * shape["K"] ** 2
-        muls = hk.conv2d_multiplies(shape["B"], shape["Ci"], shape["H"], shape["W"], shape["Co"], shape["K"], shape["pad"],
-                                    shape["p"], shape["q"], shape["x_signed"], shape["w_signed"], algo)
+        forms = layer_forms(hk, shape, algo)
 
         def step():
             hk.conv2d(d_x, d_w, shape["pad"], shape["p"], shape["q"], shape["x_signed"], shape["w_signed"], requant=rq,
                       algo=algo, workspace=ws, out=o)
-        launches_per_step = 2           # one packing launch, one layer launch
         name = "%s: 2-D layer %dx%dx%dx%d -> %d channels, %dx%d, pad %d, p=%d q=%d" % (
             args.workload, shape["B"], shape["Ci"], shape["H"], shape["W"], shape["Co"], shape["K"], shape["K"], shape["pad"],
             shape["p"], shape["q"])
@@ -538,26 +571,17 @@ def run_layer_main(args, torch, np, ranks, hk, inputs, network, dev, world, rank
         else:                                               # "auto": the library's own tiles; else tile values found earlier, one per layer
             tiles = [None] * len(layers) if args.c5_tiles == "auto" else [{"tile": int(t)} if int(t) else None for t in args.c5_tiles.split(",")]
             net.set_tiles(d_x.shape, tiles, algo=algo)
-        macs, muls = 0.0, 0.0
-        H, W = x.shape[2], x.shape[3]
-        for L, tile in zip(layers, tiles):
-            Co, Ci, K, _ = L["w"].shape
-            macs += float(x.shape[0]) * Co * H * W * Ci * K * K
-            muls += hk.conv2d_multiplies(x.shape[0], Ci, H, W, Co, K, L["pad"], L["p"], L["q"], L["x_signed"], L["w_signed"], algo, tile)
-            if L["pool"]:
-                H, W = H // 2, W // 2
-        macs += float(x.shape[0]) * head_w.shape[0] * H * W * head_w.shape[1]
-        muls += hk.conv2d_multiplies(x.shape[0], head_w.shape[1], H, W, head_w.shape[0], 1, 0, 4, 4, False, True, algo)
+        forms, macs, (H, W) = network_forms(hk, layers, head_w, x.shape[0], x.shape[2], x.shape[3], algo, tiles)
 
         def step():
             net.forward(d_x, algo=algo)
-        launches_per_step = 2 * 9       # nine layers of two launches (packing + layer; the four pools run inside their layers; none runs in one launch)
         name = ("c5: compact 4-bit CNN, batch %d, 3x160x320, 8 conv3x3 + 4 pools + 1x1 head; tiles %s: %s"
                 % (x.shape[0], {"tune": "timed once at set-up", "auto": "the library's own"}.get(args.c5_tiles, "given"),
                    [t["tile"] if t else None for t in tiles]))
         h2d = d_x.numel()
         d2h = x.shape[0] * 36 * H * W * 4
 
+    launches_per_step = sum(f["launches"] for f in forms)
     for _ in range(max(args.warmup, 3)):
         step()
     sampler = ClockSampler(local_rank)
@@ -587,9 +611,8 @@ def run_layer_main(args, torch, np, ranks, hk, inputs, network, dev, world, rank
         "config": {"workload": name, "algo": args.algo, "l2": "flushed before every step (256 MB memset outside the timed events)"},
         "gpu_launches": args.steps * launches_per_step, "clocks": clocks,
     }
-    if muls is not None:
-        line["roofline"] = alu_roofline(muls, ms, imad_peak, args.algo, args.workload)
-        line["roofline"]["kernel"] = "conv2d_strip_kernel" + (" (nine layer launches, multiplies summed)" if args.workload == "c5" else "")
+    line["roofline"] = alu_roofline(forms, ms, imad_peak, args.algo, args.workload)
+    line["roofline"]["kernel"] = kernels_of(hk, forms)
     if rank == 0:
         print(json.dumps(line), flush=True)
     ranks.shutdown()
@@ -620,18 +643,25 @@ def write_extra(path: str, extra: dict):
     return os.path.relpath(path, ROOT)
 
 
-def alu_roofline(muls: float, ms: float, imad_peak: dict, key: str, workload: str = None) -> dict:
-    """Multiplies executed per second against the rate of that multiply: `peak` is the rate the library's own
-    register-only kernel reached on this GPU (hikonv_pipe_rate) when it was measured, `frac_of_derived` divides by
-    SMs x lanes per clock x maximum SM clock instead.  The step also holds the packing kernel of the layer."""
-    achieved = muls / (ms * 1e-3)
-    derived = imad_peak[key]
-    measured = imad_peak.get(key + "_measured")
+def alu_roofline(forms: list, ms: float, imad_peak: dict, key: str, workload: str = None) -> dict:
+    """Multiplies executed per second against the rates of those multiplies: the rates that the library's own register-only kernels
+    reached on this GPU (hikonv_pipe_rate), where they were measured; `frac_of_derived` divides by SMs x lanes per clock x maximum SM
+    clock instead.  `frac` is the time the multiplies take at these rates over the step's time, which holds the packing kernels, too;
+    where a layer multiplies in double precision, `peak` is the mean rate of the two kinds in these shares."""
+    muls, doubles = (sum(f[k] for f in forms) for k in ("multiplies", "double_multiplies"))
+    achieved = (muls + doubles) / (ms * 1e-3)
+
+    def rate(suffix):
+        return (muls + doubles) / (muls / imad_peak[key + suffix] + doubles / imad_peak["double" + suffix])
+
+    derived = rate("")
+    measured = rate("_measured") if key + "_measured" in imad_peak else None
     peak = measured if measured else derived
     out = {"bound": "alu", "achieved": achieved / 1e12, "peak": peak / 1e12, "unit": "T multiply-add/s",
            "frac": achieved / peak, "traffic": None,
            "peak_kind": "of measured (register-only multiply-add kernel, this run)" if measured else "of derived",
-           "frac_of_derived": achieved / derived, "derived_peak": derived / 1e12}
+           "frac_of_derived": achieved / derived, "derived_peak": derived / 1e12,
+           "integer_multiplies": muls, "double_precision_multiplies": doubles}
     # Issue model: a scheduler spends the measured cycles on every warp-wide multiply-add and on every other warp
     # instruction of the layer kernel (counted under ncu); the sum over the device's schedulers is the time the layer
     # kernel cannot go below with this instruction mix, to be read against the step (which also holds the packing launch).
@@ -759,9 +789,8 @@ def layer_workloads(torch, np, hk, inputs, network, dev, imad_peak):
         for key, algo in (("packed", hk.ALGO_PACKED32), ("unpacked", hk.ALGO_UNPACKED_IMAD)):
             ms = time_fn(lambda: hk.conv2d(d_x, d_w, shape["pad"], shape["p"], shape["q"], shape["x_signed"], shape["w_signed"],
                                            requant=rq, algo=algo, workspace=ws, out=o))
-            muls = hk.conv2d_multiplies(shape["B"], shape["Ci"], shape["H"], shape["W"], shape["Co"], shape["K"], shape["pad"],
-                                        shape["p"], shape["q"], shape["x_signed"], shape["w_signed"], algo)
-            rec[key] = {"ms": ms, "value": macs / (ms * 1e-3), "unit": UNIT, "roofline": alu_roofline(muls, ms, imad_peak, key, name)}
+            rec[key] = {"ms": ms, "value": macs / (ms * 1e-3), "unit": UNIT,
+                        "roofline": alu_roofline(layer_forms(hk, shape, algo), ms, imad_peak, key, name)}
         rec["layout"] = hk.conv2d_layout(shape["B"], shape["Ci"], shape["H"], shape["W"], shape["Co"], shape["K"], shape["pad"],
                                          shape["p"], shape["q"], shape["x_signed"], shape["w_signed"])
         rec["packed_over_unpacked"] = rec["unpacked"]["ms"] / rec["packed"]["ms"]
@@ -802,28 +831,15 @@ def layer_workloads(torch, np, hk, inputs, network, dev, imad_peak):
     x, layers, head_w = inputs.c5_network()
     d_x = torch.from_numpy(inputs.to_storage(x)).to(dev)
     net = network.CompactCnn(layers, head_w, device=dev)
-    macs = 0.0
-    H, W = x.shape[2], x.shape[3]
-    for L in layers:
-        Co, Ci, K, _ = L["w"].shape
-        macs += float(x.shape[0]) * Co * H * W * Ci * K * K
-        if L["pool"]:
-            H, W = H // 2, W // 2
-    macs += float(x.shape[0]) * head_w.shape[0] * H * W * head_w.shape[1]
-    rec = {"macs": macs}
+    rec = {}
     for key, algo in (("packed", hk.ALGO_PACKED32), ("unpacked", hk.ALGO_UNPACKED_IMAD)):
         untuned_ms = time_fn(lambda: net.forward(d_x, algo=algo), iters=5)
         tiles = net.tune_tiles(d_x, algo=algo)              # set-up: the network times tile shapes once per input shape
         ms = time_fn(lambda: net.forward(d_x, algo=algo), iters=5)
-        # multiplies the nine layer launches execute (positions incl. halo x Co x Ci x K x J, summed)
-        muls, Hl, Wl = 0.0, x.shape[2], x.shape[3]
-        for L, tile in zip(layers, tiles):
-            Co, Ci, K, _ = L["w"].shape
-            muls += hk.conv2d_multiplies(x.shape[0], Ci, Hl, Wl, Co, K, L["pad"], L["p"], L["q"], L["x_signed"], L["w_signed"], algo, tile)
-            if L["pool"]:
-                Hl, Wl = Hl // 2, Wl // 2
-        muls += hk.conv2d_multiplies(x.shape[0], head_w.shape[1], Hl, Wl, head_w.shape[0], 1, 0, 4, 4, False, True, algo)
-        rec[key] = {"ms": ms, "value": macs / (ms * 1e-3), "unit": UNIT, "roofline": alu_roofline(muls, ms, imad_peak, key),
+        forms, macs, _ = network_forms(hk, layers, head_w, x.shape[0], x.shape[2], x.shape[3], algo, tiles)
+        rec["macs"] = macs
+        rec[key] = {"ms": ms, "value": macs / (ms * 1e-3), "unit": UNIT, "roofline": alu_roofline(forms, ms, imad_peak, key),
+                    "launches": sum(f["launches"] for f in forms),
                     "ms_with_the_library_s_own_tiles": untuned_ms, "tuned_tiles": [t["tile"] if t else None for t in tiles]}
     rec["packed_over_unpacked"] = rec["unpacked"]["ms"] / rec["packed"]["ms"]
     out["c5"] = rec

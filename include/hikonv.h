@@ -415,7 +415,7 @@ double hikonv_conv2d_multiplies(int B, int Ci, int H, int W, int Co, int K, int 
                                 int x_signed, int w_signed, int algo, const hikonv_tuning_t *tune);
 
 /*
- * hikonv_pipe_rate - measured issue rate of one integer instruction, for the rooflines of the packed kernels.
+ * hikonv_pipe_rate - measured issue rate of one instruction, for the rooflines of the packed kernels.
  * (A measurement aid; the paper has no counterpart.)  The 2-D layer kernels are bound by the 32x32->64
  * multiply-add that implements Eq. 9, and no public table gives its rate on this GPU.  The call runs a
  * register-only kernel (four CTAs of 256 threads per SM, eight independent dependency chains per thread whose
@@ -432,9 +432,10 @@ typedef enum {
     HIKONV_PIPE_LOGIC = 3,        /* lop3.b32: masks of the split and of the carry-save moves    */
     HIKONV_PIPE_SHIFT = 4,        /* shf.r: the funnel shifts of the split                       */
     HIKONV_PIPE_PRMT = 5,         /* prmt.b32: code extraction and byte-aligned slot extraction  */
-    HIKONV_PIPE_MAD_WIDE_WITH_LOGIC = 6 /* mad.wide.u32 with one lop3.b32 (on other registers) per two of them:
+    HIKONV_PIPE_MAD_WIDE_WITH_LOGIC = 6, /* mad.wide.u32 with one lop3.b32 (on other registers) per two of them:
                                      the rate of the multiply-adds alone in that mix; against kind 0 it tells what an
                                      instruction of another pipe costs the stream of packed multiplies              */
+    HIKONV_PIPE_FMA_F64 = 7       /* fma of doubles: the multiply of words of three filters (HIKONV_FORM_FILTERS) */
 } hikonv_pipe_kind;
 int hikonv_pipe_rate(int kind, int iters, uint32_t *d_scratch_word, double *h_ops_per_second,
                      double *h_lanes_per_clock_per_sm, void *stream);

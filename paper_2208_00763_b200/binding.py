@@ -24,7 +24,7 @@ ALGO_PACKED32, ALGO_PACKED64EMU, ALGO_UNPACKED_IMAD, ALGO_DP4A = 0, 1, 2, 3
 FORM_TWO_LAUNCHES, FORM_ONE_LAUNCH, FORM_FILTERS, FORM_UNPACKED = 0, 1, 2, 3
 GB_SINGLE, GB_1D, GB_DNN = 0, 1, 2
 PIPE_KINDS = {"mad_wide_u32": 0, "mad_wide_s32": 1, "mad_lo_s32": 2, "logic": 3, "shift": 4, "prmt": 5,
-              "mad_wide_with_logic": 6}
+              "mad_wide_with_logic": 6, "fma_f64": 7}
 
 
 class HikonvError(RuntimeError):
@@ -479,7 +479,7 @@ def conv2d_multiplies(B, Ci, H, W, Co, K, pad, p, q, x_signed, w_signed, algo=AL
 
 
 def pipe_rate(kind: str, iters: int = 2048, device=None, stream=None) -> dict:
-    """Measured rate of one integer instruction (see ``PIPE_KINDS``): operations per second (instructions x 32
+    """Measured rate of one instruction (see ``PIPE_KINDS``): operations per second (instructions x 32
     lanes) and lanes per clock per SM at the device's maximum SM clock.  Synchronises."""
     word = torch.zeros(1, dtype=torch.int32, device=device or "cuda")
     ops, lanes = ctypes.c_double(0.0), ctypes.c_double(0.0)

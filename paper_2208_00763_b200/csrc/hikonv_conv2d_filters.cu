@@ -8,7 +8,7 @@
 // [2^52, 2^53), where doubles are the integers; its fraction bits are the slots.
 //
 // Where codes are wide the words of pixels and taps (hikonv_conv2d_strip.cuh) hold three products, too, at 4.8 cycles a warp-wide
-// multiplication in their loop; a double-precision one takes 2.05, and other instructions issue beside it.  The first layer of the
+// multiplication in their loop; a double-precision one takes 2.02 (hikonv_pipe_rate), and other instructions issue beside it.  The first layer of the
 // compact CNN spent three quarters of its instructions outside the multiplications (prologue, exchange of upper slots, split,
 // staging of bytes); here the split needs no neighbour and the 2x2 pool is a thread's own pixels.
 //
@@ -29,6 +29,27 @@ constexpr int kWords = 4;                // kernel words of a thread whose codes
 
 // 2^52 + byte b of v.
 __device__ __forceinline__ double byte_as_double(uint32_t v, int b) { return __hiloint2double(0x43300000, (int)extract_code<false>(v, b)); }
+
+// The aligned words that hold the four codes from column col0 on of an image row of W one-byte codes, which starts at code `row` of the
+// tensor x: the codes begin at byte `off` of lo and go on in hi.  Words without a code of the row are not read and left alone, and hi
+// is not needed where off is zero.  RAGGED: the tensor's ends need not be aligned, and the words that reach outside it are put
+// together from bytes (`codes`: all of the tensor).
+template <bool RAGGED>
+__device__ __forceinline__ void load_row_codes(const int8_t *x, int row, int codes, int W, int col0, uint32_t &lo, uint32_t &hi, uint32_t &off) {
+    const int8_t *src = x + (row + col0);
+    off = (uint32_t)(uintptr_t)src & 3u;
+    const uint32_t *al = reinterpret_cast<const uint32_t *>(src - off);
+    const int c = col0 - (int)off;                               // column at the start of lo
+    auto load = [&](int i, uint32_t &v) {
+        const int first = row + c + 4 * i;                       // code at the start of the word
+        if (!RAGGED || (first >= 0 && first <= codes - 4)) v = load_ordered(al + i);
+        else
+            for (int b = 0; b < 4; ++b)
+                if (c + 4 * i + b >= 0 && c + 4 * i + b < W) v |= (uint32_t)(uint8_t)load_ordered(x + first + b) << (8 * b);
+    };
+    if (c + 3 >= 0 && c < W) load(0, lo);
+    if (off != 0u && c + 7 >= 0 && c + 4 < W) load(1, hi);
+}
 
 // RAGGED: the input begins at any byte, or ends at any (an instantiation of its own: the branch for it cost aligned inputs 2 %).
 template <int NW, bool RAGGED>

@@ -109,27 +109,6 @@ __device__ __forceinline__ void pack_row_words(const int8_t *x, int row, int rag
     }
 }
 
-// The aligned words that hold the four codes from column col0 on of an image row of W one-byte codes, which starts at code `row` of the
-// tensor x: the codes begin at byte `off` of lo and go on in hi.  Words without a code of the row are not read and left alone, and hi
-// is not needed where off is zero.  RAGGED: the tensor's ends need not be aligned, and the words that reach outside it are put
-// together from bytes (`codes`: all of the tensor).
-template <bool RAGGED>
-__device__ __forceinline__ void load_row_codes(const int8_t *x, int row, int codes, int W, int col0, uint32_t &lo, uint32_t &hi, uint32_t &off) {
-    const int8_t *src = x + (row + col0);
-    off = (uint32_t)(uintptr_t)src & 3u;
-    const uint32_t *al = reinterpret_cast<const uint32_t *>(src - off);
-    const int c = col0 - (int)off;                               // column at the start of lo
-    auto load = [&](int i, uint32_t &v) {
-        const int first = row + c + 4 * i;                       // code at the start of the word
-        if (!RAGGED || (first >= 0 && first <= codes - 4)) v = load_ordered(al + i);
-        else
-            for (int b = 0; b < 4; ++b)
-                if (c + 4 * i + b >= 0 && c + 4 * i + b < W) v |= (uint32_t)(uint8_t)load_ordered(x + first + b) << (8 * b);
-    };
-    if (c + 3 >= 0 && c < W) load(0, lo);
-    if (off != 0u && c + 7 >= 0 && c + 4 < W) load(1, hi);
-}
-
 // Maxima of neighbouring bytes of two rows of eight bytes: four bytes.
 template <bool SIGNED>
 __device__ __forceinline__ uint32_t pool_pairs(uint32_t a0, uint32_t a1, uint32_t b0, uint32_t b1) {

@@ -1,4 +1,4 @@
-// hikonv_pipe_rate: measured issue rate of the integer instructions the packed kernels are made of.
+// hikonv_pipe_rate: measured issue rate of the instructions the packed kernels are made of.
 //
 // The roofline of the 2-D layer kernels is the rate of the 32x32->64 multiply-add (Eq. 9 is one such
 // instruction).  No public table gives that rate for this GPU, so the library measures it: every thread runs
@@ -9,6 +9,8 @@
 // wide multiply-adds and reports the rate of the multiply-adds alone: what an instruction of another pipe costs
 // the multiply-add stream (the layer kernels spend one to two such instructions per multiply-add on loads, carry-save
 // moves and the split).
+// HIKONV_PIPE_FMA_F64 is the double-precision multiply-add of the kernel on words of several filters, in the same eight chains; its
+// multiplier is a kernel argument, small enough that the chains hardly grow (held in a register it cost 8 % in register ports).
 // Grid: four CTAs of 256 threads per SM (eight warps per scheduler, 64 independent instructions in flight on
 // each), timed with CUDA events around the launch.
 #include "hikonv_cuda.cuh"
@@ -74,6 +76,24 @@ __global__ void __launch_bounds__(256) pipe_rate_kernel(int iters, uint32_t seed
     if (x == 0x9E3779B9u) sink[0] = x;                          // keeps the chains alive; practically never true
 }
 
+__global__ void __launch_bounds__(256) pipe_rate_f64_kernel(int iters, double b, uint32_t *sink) {
+    const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x;
+    double acc[kChains];
+#pragma unroll
+    for (int c = 0; c < kChains; ++c) acc[c] = (double)(tid + 977u * c + 1u);
+    for (int it = 0; it < iters; ++it) {
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u) {
+#pragma unroll
+            for (int c = 0; c < kChains; ++c) acc[c] = fma(acc[(c + 1) % kChains], b, acc[c]);
+        }
+    }
+    double x = 0.0;
+#pragma unroll
+    for (int c = 0; c < kChains; ++c) x += acc[c];
+    if (x == -1.0) sink[0] = 1u;                                // never: the chains are positive
+}
+
 template <int KIND>
 static int run_kind(int iters, unsigned grid, cudaStream_t st, uint32_t *d_sink) {
     return launch_plain(pipe_rate_kernel<KIND>, dim3(grid), dim3(256), 0, st, iters, 12345u, d_sink);
@@ -88,6 +108,7 @@ static int launch_kind(int kind, int iters, unsigned grid, cudaStream_t st, uint
         case HIKONV_PIPE_SHIFT: return run_kind<HIKONV_PIPE_SHIFT>(iters, grid, st, d_sink);
         case HIKONV_PIPE_PRMT: return run_kind<HIKONV_PIPE_PRMT>(iters, grid, st, d_sink);
         case HIKONV_PIPE_MAD_WIDE_WITH_LOGIC: return run_kind<HIKONV_PIPE_MAD_WIDE_WITH_LOGIC>(iters, grid, st, d_sink);
+        case HIKONV_PIPE_FMA_F64: return launch_plain(pipe_rate_f64_kernel, dim3(grid), dim3(256), 0, st, iters, 1.0 / (1 << 30), d_sink);
         default: return HIKONV_ERR_INVALID_ARG;
     }
 }
@@ -99,7 +120,7 @@ using namespace hikonv;
 extern "C" int hikonv_pipe_rate(int kind, int iters, uint32_t *d_scratch_word, double *h_ops_per_second,
                                 double *h_lanes_per_clock_per_sm, void *stream) {
     if (!d_scratch_word || !h_ops_per_second || iters < 1 || iters > (1 << 20)) return HIKONV_ERR_INVALID_ARG;
-    if (kind < HIKONV_PIPE_MAD_WIDE_U32 || kind > HIKONV_PIPE_MAD_WIDE_WITH_LOGIC) return HIKONV_ERR_INVALID_ARG;
+    if (kind < HIKONV_PIPE_MAD_WIDE_U32 || kind > HIKONV_PIPE_FMA_F64) return HIKONV_ERR_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)stream;
     int dev = 0, sms = 0, khz = 0;
     HIKONV_CUDA_TRY(cudaGetDevice(&dev));

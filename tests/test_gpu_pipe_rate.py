@@ -16,6 +16,8 @@ def test_every_kind_gives_a_plausible_rate():
         assert 16.0 < rates[kind]["lanes_per_clock_per_sm"] <= 33.0, (kind, rates[kind])
     for kind in ("mad_lo_s32", "logic", "shift", "prmt"):
         assert 32.0 < rates[kind]["lanes_per_clock_per_sm"] <= 66.0, (kind, rates[kind])
+    # 64 double-precision lanes
+    assert 32.0 < rates["fma_f64"]["lanes_per_clock_per_sm"] <= 66.0, rates["fma_f64"]
     # logic instructions between the multiply-adds do not come for free, and cannot cost more than their own issue slots
     mixed, pure = rates["mad_wide_with_logic"]["lanes_per_clock_per_sm"], rates["mad_wide_u32"]["lanes_per_clock_per_sm"]
     assert 0.6 * pure < mixed <= 1.02 * pure, (mixed, pure)

@@ -53,7 +53,7 @@ int main() {
 
 
 def test_row_codes_are_read_by_words_from_inside_the_tensor(tmp_path):
-    text = open(os.path.join(ROOT, "paper_2208_00763_b200", "csrc", "hikonv_conv2d_util.cuh")).read()
+    text = open(os.path.join(ROOT, "paper_2208_00763_b200", "csrc", "hikonv_conv2d_filters.cu")).read()
     part = re.search(r"template <bool RAGGED>\n__device__ __forceinline__ void load_row_codes\(.*?\n}\n", text, re.S)
     assert part
     src, exe = tmp_path / "harness.cpp", tmp_path / "harness"
