@@ -495,7 +495,12 @@ static SmallChoice choose_small(const StripProblem &q) {
 constexpr int kFiltersMaxCi = 6, kFiltersMinCo = 16;    // see plan_layer
 constexpr double kFiltersMinOutputs = 1.0e6;
 
-// The kernel whose words hold the weights of several filters: its tile and the modelled cycles of the call.
+// The kernel whose words hold the weights of several filters: its tile and the modelled SM cycles of the call.  The model is a sum: the launch,
+// the packing of the kernel words, the first fetch, then per tile the double-precision pipe (2.1 cycles a multiply-add; 190 per word for
+// the split; 119 per channel and row of four codes staged), a third of the passes through shared memory, and per channel and
+// step what a CTA waits for (latencies, the barrier).  Fitted to 3531 tiles of 237 layers (1 to 6 input channels, 16 to 128
+// filters, 1 to 1024 images, 4 to 1080 rows): 6 % rms.  The tiles it picks are 1.4 % slower than the best measured ones on average; a maximum of
+// pipe and latency in place of the sum picked tiles 5.7 % slower, and left some layers up to 29 % slower than in two launches.
 struct FiltersChoice {
     int NW, groups, TQ, NSEG, TS, pos_warps, CK, rows, PW, threads;
     size_t smem;
@@ -537,10 +542,10 @@ static FiltersChoice choose_filters(const StripProblem &q, const FiltersForced &
                 if (c.TQ == last_tq) continue;
                 last_tq = c.TQ;
                 if (c.TQ > warps_max * 32) continue;
-                // issue cycles of a warp for one tile's products, and the least that is beside them
-                const double products = q.Ci * KK * 4.0 * NW * 2.1, outside = q.Ci * 40.0 + 150 + 4.0 * NW * NS * 8.0;
-                auto hopeless = [&](double cycles) { return best.cost >= 0 && 1500 + cycles * (1.0 - 1e-9) >= best.cost; };
-                if (hopeless((double)(strips * c.NSEG * c.TQ * c.groups * c.gy) / (128.0 * q.sms) * (products + 0.6 * outside))) continue;
+                // a warp's multiply-adds and split
+                const double products = q.Ci * KK * 4.0 * NW * 2.1 + 190.0 * NW;
+                auto hopeless = [&](double cycles) { return best.cost >= 0 && 2530 + cycles * (1.0 - 1e-9) >= best.cost; };
+                if (hopeless((double)(strips * c.NSEG * c.TQ * c.groups * c.gy) / (128.0 * q.sms) * products)) continue;
                 const int ts_hi = (int)std::max<long long>(1, std::min<long long>(warps_max * 32 / c.TQ, strips));
                 for (c.TS = 1; c.TS <= ts_hi; ++c.TS) {
                     c.pos_warps = ceil_div(c.TS * c.TQ, 32);
@@ -551,15 +556,14 @@ static FiltersChoice choose_filters(const StripProblem &q, const FiltersForced &
                     const int by_regs = std::min(filters_resident(NW) * (kFiltersThreads / c.threads), 8);
                     const size_t plane = 8 * (size_t)c.rows * c.PW;
                     const double items = (double)c.rows * (c.PW / 4) / c.threads;      // rows of four codes that a thread stages per channel
-                    // all of it, and what a warp's own latencies leave a tile at least
-                    const double rest = outside + q.Ci * items * 45.0;
-                    const double alone = q.Ci * (KK * std::max(4.0 * NW * 2.1, 18.0) + 150 + std::max(0.0, items - 2.0) * 150) + 600;
                     const int per_sched = ceil_div(c.threads / 32, 4);
+                    // of a tile, by itself, and for every CTA that shares the SM
+                    const double busy = per_sched * (products + 119.0 * q.Ci * items) + 0.36 * (c.threads / 32) * q.Ci * (32 + KK * NW / 2.0 + 8 * items);
+                    auto waits = [&](int CK) { return 294.0 * q.Ci + 1020.0 * ceil_div(q.Ci, CK); };
                     // what comes before the first tile, with n warps on a scheduler: packing the kernel words, fetching the first step's CK channels
                     const double word_rounds = std::ceil((double)q.Ci * KK * WT / (4.0 * c.threads));
-                    auto before = [&](double n, int CK) { return word_rounds * (500 + 150 * n) + std::ceil(CK * items / 2.0) * (400 + 100 * n); };
-                    const double share = (double)(c.tiles * c.gy) / q.sms;
-                    if (hopeless(before(per_sched, 1) + std::max(share * per_sched * (products + 0.6 * rest), alone))) continue;
+                    auto before = [&](double n, int CK) { return word_rounds * (1520 + 175 * n) + std::ceil(CK * items / 2.0) * 440; };
+                    if (hopeless(before(per_sched, 1) + (double)(c.tiles * c.gy) / q.sms * busy + waits(q.Ci))) continue;
                     for (int want = 1; want <= by_regs; ++want) {
                         if (want > 1 && c.tiles * c.gy <= (long long)(want - 1) * q.sms) break;
                         c.gx = std::max<long long>(1, std::min<long long>(c.tiles, (long long)want * q.sms / c.gy));
@@ -568,8 +572,8 @@ static FiltersChoice choose_filters(const StripProblem &q, const FiltersForced &
                         c.gx = (c.tiles + per_cta - 1) / per_cta;
                         const double resident = std::max(1.0, std::min((double)want, std::ceil((double)(c.gx * c.gy) / q.sms)));
                         const double rounds = std::ceil((double)(c.gx * c.gy) / (resident * q.sms));
-                        const double n = resident * per_sched, tiles_alone = per_cta * std::max(n * (products + 0.6 * rest), alone);
-                        if (hopeless(before(n, 1) + rounds * tiles_alone)) continue;
+                        const double n = resident * per_sched, tiles_of_sm = rounds * per_cta;
+                        if (hopeless(before(n, 1) + tiles_of_sm * (resident * busy + waits(q.Ci)))) continue;
                         const size_t room = std::min<size_t>(kSmemPerCta, kSmemPerSm / want - 1024);
                         for (int part = 1, CK = 0; part <= 8; part *= 2) {
                             const int divided = force.CK > 0 ? std::min(force.CK, q.Ci) : ceil_div(q.Ci, part);
@@ -577,7 +581,7 @@ static FiltersChoice choose_filters(const StripProblem &q, const FiltersForced &
                             CK = divided;
                             const size_t smem = word_bytes + 2 * CK * plane;
                             if (smem > room) continue;
-                            c.cost = 1500 + before(n, CK) + rounds * (tiles_alone + (double)per_cta * ceil_div(q.Ci, CK) * 150);
+                            c.cost = 2530 + before(n, CK) + tiles_of_sm * (resident * busy + waits(CK));
                             c.CK = CK;
                             c.smem = smem;
                             if (best.cost < 0 || c.cost < best.cost * (1.0 - 1e-9)) best = c;
@@ -711,10 +715,13 @@ static int plan_layer(int B, int Ci, int H, int W, int Co, int K, int stride, in
         // Words of several filters (tune->tile == -3: wherever the layer fits them, and more digits in front force parts of its tile): the slots hold the sums of the whole layer.  They are
         // the faster ones for pooled layers of few input channels whose words of pixels hold three products at best (N = 2, two words
         // per kernel row): the pool is then a thread's own pixels.  As graphs, two launches / this kernel: 3 -> 16 channels u8 x s4 on
-        // 160x320 maps, 1 / 2 / 4 / 16 / 64 images 7.0 / 9.7 / 12.5 / 34.5 / 123.7 against 6.9 / 8.1 / 9.7 / 29.8 / 81.9 us, sixteen
-        // 48x48 maps 5.4 / 5.8 (0.6 million sums: the line lies at a million); 3 -> 32 and 3 -> 64 on sixteen 160x320 maps 63.7 / 48.6 and
-        // 119 / 79.9; 6 -> 32 at 6 bits 95.2 / 77.9; 3 -> 8 (three of four words used) 19.7 / 21.9.  Without a pool the other form's stores
-        // are direct: 3 -> 32 on 64 112x112 maps 55.7 / 79.4, four 160x320 maps 11.1 / 11.2.
+        // 160x320 maps, 2 / 4 / 16 / 64 images 9.5 / 12.2 / 34.1 / 123.6 against 6.9 / 8.9 / 24.7 / 82.2 us; sixty-four and 256 32x32 maps
+        // 6.5 / 13.1 against 5.8 / 10.0; 1 -> 16 on 1024 8x8 and 28x28 maps 5.9 / 32.3 against 4.4 / 14.7; 3 -> 32 on sixty-four 112x112 maps
+        // 58.5 / 50.4; 6 -> 96 at 6 bits on thirty-two 160x320 maps 522 / 343.  Over 413 layers that the rule takes (every width it allows, 1 to
+        // 6 channels, 16 to 128 filters, a million sums to 4e8) 0.63 of the time, one of them slower (3.7 %: 6 -> 39 on six 52x120 maps).
+        // Below a million sums 15 of 107 were slower, by up to 10 %, and what these calls take is launch and first fetch, which the models of
+        // the forms do not tell apart (by their comparison 7 would still be slower): the line lies there.  3 -> 8 (three of four words used)
+        // 19.7 / 21.9.  Without a pool the other form's stores are direct: 3 -> 32 on sixty-four 112x112 maps 55.7 / 79.4, four 160x320 maps 11.1 / 11.2.
         const bool own_layout = tune && (tune->N || tune->S || tune->M || tune->tile);
         const bool force_filters = tune && tune->tile <= -3 && tune->tile % 10 == -3 && !tune->N && !tune->S && !tune->M;
         if (K == kFiltersK && out.byte_inputs && out.out_bits == 8 && (!own_layout || force_filters)) {
