@@ -1,6 +1,6 @@
 // The 1-D packed kernel for long filters: kernels that are cut into more chunks than the register-resident kernels are built for.
 //
-// A CTA computes kThreads x R consecutive blocks of N outputs.  It packs the blocks' codes once into shared memory (Eq. 5; four
+// A CTA computes THREADS x R consecutive blocks of N outputs.  It packs the blocks' codes once into shared memory (Eq. 5; four
 // words per thread from N aligned 32-bit loads, permutes and multiply-adds), then every thread forms R neighbouring
 //     Q_x = bias + sum_j A_{x-j} B_j                                                                   (Eq. 9)
 // in registers, four chunks at a time: the R + 3 words they need are read from shared memory (R is odd, so a warp's reads fall
@@ -14,24 +14,25 @@
 namespace hikonv {
 
 // Threads of a CTA.  At two codes per word half of 256, with twice the CTAs per SM: the same warps, but a barrier holds up four of them and
-// the phases of more CTAs (load and pack, multiply, store) lie beside each other: 4.2 M 8-bit codes, 24 taps 8.9 -> 8.06 us a call.  At
-// three codes it changed nothing (31 taps 6.93 / 6.93), at four and more it cost 5 % (20 taps at 2 bits 5.15 -> 5.4).
+// the phases of more CTAs (load and pack, multiply, store) lie beside each other.  As graphs, 8 x 8 bits, 24 taps: 300 000 / 1 M / 2 M / 4.2 M
+// codes 3.56 / 4.78 / 6.12 / 8.71 -> 3.07 / 4.67 / 5.80 / 7.95 us; 384 signals of 2000 to 4.2 M codes, 9 to 32 taps and eight widths took 0.5 to 16 % less, all of
+// them.  At three codes it changed nothing (31 taps 6.93 / 6.93), at four and more it cost 5 % (20 taps at 2 bits 5.15 -> 5.4).
 __host__ __device__ constexpr int long_threads(int N) { return N == 2 ? 128 : 256; }
+// Resident CTAs that the registers leave room for: a signal of a few million codes is about one wave of them, with a tail of a few per
+// cent at five CTAs of 256 threads per SM and none at six, which N = 3 reaches without spilling (4.2 M codes, 12 / 16 / 31 taps:
+// 6.3 / 7.0 / 7.7 -> 5.5 / 6.3 / 7.3 us for a launch by itself; the other block sizes lost 2 to 20 % at five or six).
 __host__ __device__ constexpr int long_resident(int N) { return N == 3 || N == 2 ? 6 : 3; }
 constexpr int kLongJ = (kMaxJ + 3) / 4 * 4;                    // chunks, rounded up to whole groups of four
 // Blocks per thread: odd, and at most 28 outputs.
 __host__ __device__ constexpr int long_run(int N) { return N == 1 ? 15 : N == 2 ? 11 : N <= 4 ? 7 : N == 5 ? 5 : 3; }
 
-// Resident CTAs: a signal of a few million codes is about one wave of them, with a tail of a few per cent at five CTAs per SM
-// and none at six, which N = 3 reaches without spilling (4.2 M codes, 12 / 16 / 31 taps: 6.3 / 7.0 / 7.7 -> 5.5 / 6.3 / 7.3 us for
-// a launch by itself; the other block sizes lost 2 to 20 % at five or six).
 template <int N, bool SP, bool FS>
 __global__ void __launch_bounds__(long_threads(N), long_resident(N)) conv1d_long_kernel(const Conv1dTcParams p) {
-    constexpr int kLongThreads = long_threads(N), R = long_run(N), TILE = kLongThreads * R, FRONT = kLongJ;   // blocks per tile; packed words in front of it
+    constexpr int THREADS = long_threads(N), R = long_run(N), TILE = THREADS * R, FRONT = kLongJ;   // blocks per tile; packed words in front of it
     static_assert(TILE % 4 == 0 && FRONT % 4 == 0 && FRONT > kMaxJ - 1, "groups of four words");
     __shared__ __align__(16) uint32_t s_A[FRONT + TILE];
     __shared__ __align__(16) uint32_t s_B[kLongJ];
-    __shared__ uint32_t s_hi[kLongThreads + 1];                // [1 + t]: what thread t's last block hands on; [0]: the block before the tile
+    __shared__ uint32_t s_hi[THREADS + 1];                // [1 + t]: what thread t's last block hands on; [0]: the block before the tile
     __shared__ __align__(16) int32_t s_out[TILE * N];
     const int tid = threadIdx.x;
     const long long x0 = (long long)blockIdx.x * TILE;         // first block of the tile
@@ -50,7 +51,7 @@ __global__ void __launch_bounds__(long_threads(N), long_resident(N)) conv1d_long
         s_B[tid] = b;
     }
     const uint32_t step = 1u << p.S;
-    for (int q = tid; q < (FRONT + TILE) / 4; q += kLongThreads) {
+    for (int q = tid; q < (FRONT + TILE) / 4; q += THREADS) {
         const long long e0 = (x0 - FRONT + 4 * q) * N;         // first code of the four words
         uint32_t w[N];
         if (p.aligned && e0 >= 0 && e0 + 4 * N <= p.len) {
@@ -118,9 +119,9 @@ __global__ void __launch_bounds__(long_threads(N), long_resident(N)) conv1d_long
     const long long y0 = x0 * N;
     if (p.aligned && y0 + TILE * N <= p.n_out) {
         int4 *dst = reinterpret_cast<int4 *>(p.y + y0);
-        for (int i = tid; i < TILE * N / 4; i += kLongThreads) __stcs(dst + i, reinterpret_cast<const int4 *>(s_out)[i]);
+        for (int i = tid; i < TILE * N / 4; i += THREADS) __stcs(dst + i, reinterpret_cast<const int4 *>(s_out)[i]);
     } else {
-        for (int i = tid; i < TILE * N; i += kLongThreads)
+        for (int i = tid; i < TILE * N; i += THREADS)
             if (y0 + i < p.n_out) p.y[y0 + i] = s_out[i];
     }
 }

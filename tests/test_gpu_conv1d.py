@@ -68,8 +68,8 @@ def test_extreme_codes(signed, algo):
 
 @pytest.mark.parametrize("K", [9, 13, 16, 24, 31, 32])
 def test_long_filters(K):
-    # kernels cut into more chunks than the register-resident kernels take: every width and sign, lengths around a tile of
-    # 256 threads x R blocks, extreme codes, buffers off their alignment, and every block size the kernel is built for
+    # kernels cut into more chunks than the register-resident kernels take: every width and sign, lengths around tiles of
+    # 256 threads x R blocks (the second and fourth tile's ends at two codes per word), extreme codes, buffers off their alignment, and every block size the kernel is built for
     rng = np.random.default_rng(600 + K)
     run = {1: 15, 2: 11, 3: 7, 4: 7, 5: 5, 6: 3, 7: 3, 8: 3}
     for p in range(1, 9):
@@ -96,6 +96,25 @@ def test_long_filters(K):
             assert err.status == hk.ERR_NO_FIT
             continue
         assert_exact(got, direct.conv1d_full(f, g), "N=%d" % n_forced)
+
+
+@pytest.mark.parametrize("K", [9, 24, 32])
+def test_long_filters_at_the_ends_of_the_smaller_tiles(K):
+    # two codes per word: tiles of 128 threads x 11 blocks; outputs that end one before, at and one past the end of the first and third tile,
+    # and within it, on aligned and unaligned buffers
+    rng = np.random.default_rng(700 + K)
+    per_tile = 128 * 11 * 2
+    for (p, q, fs, gs) in ((8, 8, False, False), (8, 8, True, True), (8, 4, False, True), (6, 8, True, False)):
+        assert hk.conv1d_layout(p, q, fs, gs, K)["N"] == 2
+        g = inputs.uniform_codes(rng, (K,), q, gs)
+        for n_out in (per_tile - 1, per_tile, per_tile + 1, 3 * per_tile - 1, 3 * per_tile, 3 * per_tile + 1, 2 * per_tile - 700):
+            f = inputs.uniform_codes(rng, (n_out - K + 1,), p, fs)
+            ref = direct.conv1d_full(f, g)
+            assert_exact(_run(f, g, p, q, fs, gs, hk.ALGO_PACKED32), ref, "p=%d q=%d n_out=%d" % (p, q, n_out))
+            buf, y = torch.zeros(f.size + 8, dtype=torch.int8, device="cuda"), torch.full((n_out + 8,), 77, dtype=torch.int32, device="cuda")
+            d_f = buf[3:3 + f.size].copy_(dev(f))
+            assert_exact(hk.conv1d(d_f, dev(g), p, q, fs, gs, out=y[1:1 + n_out]), ref, "unaligned n_out=%d" % n_out)
+            assert bool((y[:1] == 77).all()) and bool((y[1 + n_out:] == 77).all())
 
 
 @pytest.mark.parametrize("algo", ALGOS)
