@@ -719,10 +719,12 @@ static int plan_layer(int B, int Ci, int H, int W, int Co, int K, int stride, in
         // 6.5 / 13.1 against 5.8 / 10.0; 1 -> 16 on 1024 8x8 and 28x28 maps 5.9 / 32.3 against 4.4 / 14.7; 3 -> 32 on sixty-four 112x112 maps
         // 58.5 / 50.4; 6 -> 96 at 6 bits on thirty-two 160x320 maps 522 / 343.  Over 413 layers that the rule takes (every width it allows, 1 to
         // 6 channels, 16 to 128 filters, a million sums to 4e8) 0.63 of the time, one of them slower (3.7 %: 6 -> 39 on six 52x120 maps).
-        // Below a million sums 15 of 107 were slower, by up to 10 %, and what these calls take is launch and first fetch, which the models of
-        // the forms do not tell apart (by their comparison 7 would still be slower): the line lies there.  3 -> 8 (three of four words used)
-        // 19.7 / 21.9.  Layers without a pool are not taken: over forty of them 0.64 to 1.28 of the time (sums and codes alike: 3 -> 16 on forty-eight
-        // 48x320 maps 30.4 / 32.6, 6 -> 39 on six 52x120 maps 10.0 / 11.1, 6 -> 36 on 129 18x278 maps 110 / 71), and no line drawn between them yet.
+        // Below a million sums 14 of 107 were slower by more than half a per cent, up to 10 %, and what these calls take is launch and first
+        // fetch, which the models of the forms do not tell apart (by their comparison 7 would still be slower): the line lies there.  The line
+        // at 16 filters is older than the present tiles: 3 -> 8 and 3 -> 12 on sixteen 160x320 maps 19.5 / 17.8 and 33.9 / 19.2, on
+        // sixty-four 68.1 / 57.7 and 121.6 / 62.5 would gain, too.  Nor are layers without a pool taken: over forty of them 0.64 to 1.28 of the
+        // time, sums and codes alike (3 -> 16 on forty-eight 48x320 maps 30.4 / 32.6, 6 -> 39 on six 52x120 maps 10.0 / 11.1, 6 -> 36 on
+        // 129 18x278 maps 110 / 71), and no line drawn between them.
         const bool own_layout = tune && (tune->N || tune->S || tune->M || tune->tile);
         const bool force_filters = tune && tune->tile <= -3 && tune->tile % 10 == -3 && !tune->N && !tune->S && !tune->M;
         if (K == kFiltersK && out.byte_inputs && out.out_bits == 8 && (!own_layout || force_filters)) {

@@ -16,8 +16,10 @@
 // a warp.  CTAs stay: each packs the weights of its filters once and walks over tiles; while it multiplies one step (a tile's
 // activations as doubles in shared memory) its threads fetch the next one's, a few rows of four codes beside every channel, into the
 // other buffer.  A layer is one launch and writes no packed activations.
-// First layer of the network (64x3x160x320 -> 16 channels, u8 x s4, pooled), packing launch included, as a graph: 122.9 -> 81.8 us.
-// Without the walk over tiles (one tile a CTA, staged before it multiplies) 97.5 us, 30 % of the cycles waiting for the staging.
+// First layer of the network (64x3x160x320 -> 16 channels, u8 x s4, pooled), packing launch included, as a graph: 122.9 -> 82 us (97.5 with one
+// tile a CTA, staged before it multiplies).  What bounds it: instructions around the multiplies.  Of 54.3 M warp instructions 17.0 M are
+// double-precision; the schedulers issue in 59 % of the cycles, the pipe is busy in 37 %, and warps wait for results of their own
+// and for their turn, hardly for the barrier or for loads.
 #include "hikonv_cuda.cuh"
 #include "hikonv_conv2d_filters.h"
 #include "hikonv_conv2d_util.cuh"

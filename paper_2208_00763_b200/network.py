@@ -90,7 +90,7 @@ class CompactCnn:
     def forward(self, d_x: torch.Tensor, algo: int = hk.ALGO_PACKED32, keep_activations: bool = False, stream=None,
                 fused_pool: bool = True):
         """``fused_pool``: layers followed by a pool run it inside their epilogue (``hikonv_conv2d_dense`` with one code
-        per byte; the default: four launches fewer, 0.471 against 0.496 ms on the benchmark network); otherwise the pool
+        per byte; the default: five launches fewer, 0.441 against 0.501 ms on the benchmark network); otherwise the pool
         is a launch of its own."""
         self._ensure_workspace(d_x.shape)
         tiles = self._tiles.get((algo, bool(fused_pool), tuple(d_x.shape)))
